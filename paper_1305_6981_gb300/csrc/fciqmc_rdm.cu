@@ -1,14 +1,22 @@
 // Energy functional E(h, V; c) = c^T H c / c^T c over a fixed determinant list, and its gradient with
 // respect to the one- and two-electron integrals (the 1- and 2-RDMs of c divided by c^T c).
 //
-// Pairs of determinants that H connects (differing in at most two spin orbitals) are found without a
-// sort: every determinant I emits, for each pair {x, y} of its occupied spin orbitals, the key
-// I - {x, y}. Two distinct determinants share a key exactly when they differ by a double excitation
-// (one shared key, their hole sets removed) or a single excitation (one shared key per common
-// electron; the pair is kept only in the bucket of the lowest common electron). Keys are grouped in
-// an open-addressing table (128-bit compare-and-swap for two-word determinants), buckets with two or
-// more members get contiguous member segments (sorted by determinant index, so sums are
-// deterministic), and each thread then evaluates one candidate pair.
+// The pair structure. Every determinant I emits, for each pair {x < y} of its occupied spin orbitals, the key
+// K = I - {x, y}. With v_K(xy) = +-c_I, the sign being that of a_y a_x |I>, the off-diagonal part of the
+// energy is a sum over keys of small quadratic forms,
+//   c^T H c - diagonal = sum_K sum_{xy != zw} v_K(xy) v_K(zw) <xy|T|zw>,
+//   T = the antisymmetrised two-electron integral + (one-electron elements) / (N - 1),
+// because two determinants that differ by a double excitation share one key and two that differ by a single
+// share N - 1 of them, whose T elements add up to the whole Slater-Condon element (its spectator sum runs
+// over the keys). So no pair needs to be decoded: a member of a key's group is (pair code, signed
+// amplitude), T is a table over pair codes, and a pair of members costs one table read and one FMA. The
+// two-body density matrix is the same sum with T's element replaced by its index.
+// Only keys shared by two or more determinants matter; the diagonal comes from the occupation-pair sums
+// O_pq = sum_I c_I^2 n_p n_q.
+//
+// Grouping is a radix partition by a 64-bit XOR hash of the key (one word per spin orbital, so a key's hash
+// is the determinant's with two words taken out): keys are 8-byte records, scattered once into partitions
+// that fit in shared memory, where one block groups them exactly (the hash only routes; determinants decide).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -20,25 +28,48 @@
 
 namespace {
 
-using fq::Params;
-
 constexpr int kThreads = 256;
-constexpr int kMaxGrid = 4096;
-constexpr unsigned long long kSaltKey = 0x2545F4914F6CDD1Dull;
+constexpr int kPartMax = 1 << 15;     // most partitions (their counters fill 128 KB of shared memory)
+constexpr int kBins = 1024;           // most bins of one scatter pass
+constexpr int kFineBits = 7;          // bins of the second pass, where one pass is not enough
+constexpr int kTileKeys = 4096;       // keys scattered at a time by one block (two blocks fit on an SM)
+constexpr int kCursorStride = 16;     // first-pass cursors, one per 64 bytes: every tile of every block takes room there
+constexpr int kHashThreads = 1024;    // threads of the passes over the keys
+static_assert(kBins == kHashThreads, "the first scatter pass has one thread per bin");
+constexpr int kGroupThreads = 512;
+// Records grouped at a time by one block and slots of its table: 110 KB of shared memory, so two blocks fit on
+// an SM. An average partition holds at most about 3,700 records up to 1.2e8 keys; longer ones are taken in
+// several parts.
+constexpr int kGroupCap = 4608;
+constexpr int kGroupSlots = 8192;
+constexpr int kBigLeaders = 16;       // distinct keys of one hash value that the oversized path tells apart
+constexpr int kTriangle = 48;         // groups from this size on are walked as a triangle (see row_range)
+constexpr int kMergeThreads = 128;
 
-struct RdmLayout {
-    size_t dets, c, keys, counts, cursor, moff, poff, members, bsum, partial, state, gh, ge, npair_tab, wpair, scan_tmp;
-    size_t total;
+// A determinant in the group of a key: its signed amplitude, its pair code (bits 0..12 the index within the
+// class, 13..14 the class: 0 alpha alpha, 1 beta beta, 2 mixed; bits 15..20 the group size, 63 from kTriangle
+// on), and the position of the group's first member in the partition.
+struct alignas(16) Member {
+    double v;
+    unsigned code;
+    unsigned first;
 };
 
 struct RdmState {
     unsigned long long n_buckets;
     unsigned long long n_members;  // members of buckets with two or more entries
     unsigned long long n_pairs;    // candidate pairs
-    unsigned long long n_single, n_double;
+    unsigned long long n_shared;   // pairs of members that share one spin orbital (counted on request)
+    unsigned long long n_apart;    // pairs that share none
     double norm;
     int status;
     int pad;
+};
+
+struct RdmLayout {
+    size_t dets, c, total_p, base_p, cursor_p, coarse_p, count_p, records, members, state, gh, ge, table, occ_part,
+        occ_pair, partial;
+    size_t total;
 };
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
@@ -53,9 +84,17 @@ int log2i(long long x) {
     return b;
 }
 
+constexpr int kSms = 152;                     // blocks of the passes that take one block per SM
+constexpr int kPairGrid = kSms * 8;           // blocks of the pair passes
+constexpr int kNormGrid = kSms;
+
 struct Dims {
-    int n_elec, n_orb, W, npairs;
-    long long n, n_keys, kcap, n_eri;
+    int n_elec, n_orb, n_so, W, npairs;
+    int n1, n2;          // pair codes of one spin (p < q) and of mixed spin (p, q)
+    int parts, pbits;    // partitions of the key records
+    int tbits;           // bits of a key's number
+    int hash_blocks;     // blocks of the passes over the determinants
+    long long n, n_keys, n_eri;
 };
 
 bool dims_of(int n_elec, int n_orb, long long n, Dims &d) {
@@ -63,11 +102,19 @@ bool dims_of(int n_elec, int n_orb, long long n, Dims &d) {
         return false;
     d.n_elec = n_elec;
     d.n_orb = n_orb;
+    d.n_so = 2 * n_orb;
     d.W = (2 * n_orb + 63) / 64;
     d.npairs = n_elec * (n_elec - 1) / 2;
+    d.n1 = n_orb * (n_orb - 1) / 2;
+    d.n2 = n_orb * n_orb;
     d.n = n;
     d.n_keys = n * d.npairs;
-    d.kcap = next_pow2(std::max<long long>(2 * d.n_keys, 1 << 12));
+    // about 4096 records a partition; small lists get up to 512 partitions of at least 256, to spread over the SMs
+    d.parts = (int)std::min<long long>(
+        kPartMax, next_pow2(std::max<long long>(d.n_keys / 4096, std::min<long long>(512, std::max<long long>(1, d.n_keys / 256)))));
+    d.pbits = log2i(d.parts);
+    d.tbits = std::max(1, log2i(d.n_keys));
+    d.hash_blocks = (int)std::min<long long>(kSms, (n + 31) / 32);
     long long np = (long long)n_orb * (n_orb + 1) / 2;
     d.n_eri = np * (np + 1) / 2;
     return d.n_keys < (1LL << 31);
@@ -81,23 +128,22 @@ RdmLayout layout_of(const Dims &d) {
         off = align256(off + b);
         return o;
     };
-    const int stride = d.W == 1 ? 2 : 4;
     L.dets = take(sizeof(unsigned long long) * d.W * d.n);
     L.c = take(sizeof(double) * d.n);
-    L.keys = take(sizeof(unsigned long long) * stride * d.kcap);
-    L.counts = take(sizeof(unsigned) * d.n_keys);
-    L.cursor = take(sizeof(unsigned) * d.n_keys);
-    L.moff = take(sizeof(unsigned long long) * (d.n_keys + 1));
-    L.poff = take(sizeof(unsigned long long) * (d.n_keys + 1));
-    L.members = take(sizeof(unsigned long long) * d.n_keys);
-    L.bsum = take(sizeof(unsigned long long) * 2 * (kMaxGrid + 1));
-    L.partial = take(sizeof(double) * 4 * kMaxGrid);
+    L.total_p = take(sizeof(unsigned) * d.parts);
+    L.base_p = take(sizeof(unsigned) * (d.parts + 1));
+    L.cursor_p = take(sizeof(unsigned) * d.parts);
+    L.coarse_p = take(sizeof(unsigned) * kBins * kCursorStride);
+    L.count_p = take(sizeof(unsigned) * d.parts);
+    L.records = take(sizeof(unsigned long long) * d.n_keys);
+    L.members = take(sizeof(Member) * d.n_keys);
     L.state = take(sizeof(RdmState));
     L.gh = take(sizeof(double) * d.n_orb * d.n_orb);
     L.ge = take(sizeof(double) * d.n_eri);
-    L.npair_tab = take(sizeof(double) * 2 * fq::MAXSO * fq::MAXSO);
-    L.wpair = take(sizeof(double) * 2 * d.n_orb * d.n_orb);
-    L.scan_tmp = take(sizeof(unsigned long long) * 4);
+    L.table = take(sizeof(double) * ((size_t)d.n1 * d.n1 + (size_t)d.n2 * d.n2));
+    L.occ_part = take(sizeof(double) * kSms * ((size_t)d.n_so * (d.n_so + 1) / 2));
+    L.occ_pair = take(sizeof(double) * ((size_t)d.n_so * (d.n_so + 1) / 2));
+    L.partial = take(sizeof(double) * 2 * (kPairGrid + kNormGrid));
     L.total = off;
     return L;
 }
@@ -105,235 +151,603 @@ RdmLayout layout_of(const Dims &d) {
 // ------------------------------------------------------------------------------------ device helpers
 template <int W>
 __device__ __forceinline__ void load_det(const unsigned long long *dets, long long i, unsigned long long (&d)[W]) {
-#pragma unroll
-    for (int w = 0; w < W; ++w) d[w] = dets[i * W + w];
-}
-
-// x-th occupied spin orbital (ascending) of d
-template <int W>
-__device__ __forceinline__ int nth_occ(const unsigned long long (&d)[W], int x) {
-    return fq::select_bit<W>(d, x);
-}
-
-// member word: determinant index (bits 0..31), removed orbitals x (32..39) and y (40..47)
-__device__ __forceinline__ unsigned long long pack_member(unsigned I, int x, int y) {
-    return (unsigned long long)I | ((unsigned long long)x << 32) | ((unsigned long long)y << 40);
-}
-
-template <int W>
-__device__ __forceinline__ long long key_lookup(const unsigned long long *tab, long long kcap, int kbits,
-                                                const unsigned long long (&key)[W]) {
-    constexpr int S = fq::Stride<W>::v;
-    unsigned long long h = fq::table_hash<W>(key, kSaltKey) >> (64 - kbits);
-    for (long long probe = 0; probe < kcap; ++probe) {
-        const unsigned long long *e = tab + h * S;
-        bool match = true, empty = true;
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-            match = match && (e[w] == key[w]);
-            empty = empty && (e[w] == fq::EMPTY);
-        }
-        if (match) return (long long)h;
-        if (empty) return -1;
-        h = (h + 1ull) & ((unsigned long long)kcap - 1ull);
+    if (W == 2) {
+        const ulonglong2 x = __ldg(reinterpret_cast<const ulonglong2 *>(dets) + i);
+        d[0] = x.x;
+        d[W - 1] = x.y;
+    } else {
+        d[0] = __ldg(dets + i);
     }
-    return -1;
+}
+
+// The hash word of a spin orbital.
+__device__ __forceinline__ unsigned long long orbital_word(int k) { return fq::mix64(0x9E3779B97F4A7C15ull * (unsigned long long)(k + 1)); }
+
+// Electron pairs in order k = y (y - 1) / 2 + x, x < y, packed x | y << 8.
+__device__ __forceinline__ void triangle_of(int k, int &x, int &y) {  // k = y (y - 1) / 2 + x, x < y
+    y = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)k)) * 0.5f);
+    while (y > 1 && y * (y - 1) / 2 > k) --y;
+    while ((y + 1) * y / 2 <= k) ++y;
+    x = k - y * (y - 1) / 2;
+}
+__device__ __forceinline__ void fill_pairs(int n_elec, unsigned short *pairs) {
+    for (int k = threadIdx.x; k < n_elec * (n_elec - 1) / 2; k += blockDim.x) {
+        int x, y;
+        triangle_of(k, x, y);
+        pairs[k] = (unsigned short)(x | (y << 8));
+    }
+}
+
+// A key record: the low tbits bits are the emitting (determinant, pair) t = I npairs + k, the others the hash bits after
+// those that chose the partition (64 - tbits of them, at least 33; tbits = bits of the number of keys).
+__device__ __forceinline__ unsigned rec_t(unsigned long long r, int tbits) { return (unsigned)r & ((1u << tbits) - 1u); }
+__device__ __forceinline__ unsigned long long rec_hash(unsigned long long r, int tbits) { return r >> tbits; }
+__device__ __forceinline__ unsigned long long make_rec(unsigned long long hash, int used, int tbits, unsigned t) {
+    return (((hash << used) >> tbits) << tbits) | (unsigned long long)t;
+}
+
+// Key and removed spin orbitals of a record.
+struct KeyOf {
+    unsigned I;
+    int k, ox, oy;
+};
+template <int W>
+__device__ __forceinline__ KeyOf key_of(const unsigned long long *dets, const unsigned short *pairs, int npairs, unsigned t,
+                                        unsigned long long (&key)[W]) {
+    KeyOf q;
+    q.I = t / (unsigned)npairs;
+    q.k = (int)(t - q.I * (unsigned)npairs);
+    const unsigned short pr = pairs[q.k];
+    load_det<W>(dets, q.I, key);
+    q.ox = fq::select_bit<W>(key, pr & 0xFF);
+    q.oy = fq::select_bit<W>(key, pr >> 8);
+    fq::flip<W>(key, q.ox);
+    fq::flip<W>(key, q.oy);
+    return q;
+}
+
+// Code of the pair ox < oy: class << 13 | index. Mixed pairs are indexed alpha first. kNoPair for orbitals outside the
+// basis or out of order (a determinant that is none of the run's): such members carry no amplitude.
+constexpr unsigned kNoPair = 0x7FFFu;
+__device__ __forceinline__ unsigned pair_code(int ox, int oy, int n_orb) {
+    if (ox >= oy || oy >= 2 * n_orb) return kNoPair;
+    const int p = ox >> 1, q = oy >> 1, sx = ox & 1, sy = oy & 1;
+    if (sx == sy) return ((unsigned)sx << 13) | (unsigned)(q * (q - 1) / 2 + p);
+    return (2u << 13) | (unsigned)(sx == 0 ? p * n_orb + q : q * n_orb + p);
 }
 
 // ------------------------------------------------------------------------------------ construction kernels
-// Empty key table: EMPTY key words, zero payloads.
-__global__ void k_key_init(unsigned long long *tab, long long kcap, int W) {
-    const int S = W == 1 ? 2 : 4;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < kcap; e += (long long)gridDim.x * blockDim.x) {
-        for (int w = 0; w < W; ++w) tab[e * S + w] = fq::EMPTY;
-        tab[e * S + W] = 0ull;
-    }
+// The keys of determinants [lo, hi), one determinant per warp at a time: the lanes decode it together (each set bit's
+// rank is a population count) and then take its pairs. f(pair's key number t, its 64-bit hash).
+struct HashShared {
+    unsigned long long z[fq::MAXSO];
+    unsigned long long zo[kHashThreads / 32][fq::MAXN];
+    unsigned short pairs[fq::MAXPAIRS];
+};
+__device__ __forceinline__ void hash_setup(HashShared &s, int n_elec) {
+    fill_pairs(n_elec, s.pairs);
+    for (int k = threadIdx.x; k < fq::MAXSO; k += blockDim.x) s.z[k] = orbital_word(k);
 }
-
-// Key table entries: key words, then (bucket id << 32) + number of determinants with that key.
-template <int W>
-__global__ void k_keys(const unsigned long long *dets, long long n, int n_elec, unsigned long long *tab, long long kcap,
-                       int kbits, RdmState *st) {
-    constexpr int S = fq::Stride<W>::v;
+template <int W, typename F>
+__device__ __forceinline__ void for_keys(HashShared &s, const unsigned long long *dets, long long lo, long long hi, int n_elec, F f) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long *zo = s.zo[warp];
     const int npairs = n_elec * (n_elec - 1) / 2;
-    const long long total = n * npairs;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
-        const long long I = t / npairs;
-        int k = (int)(t - I * npairs);
-        int y = 1;
-        while ((y + 1) * y / 2 <= k) ++y;
-        const int x = k - y * (y - 1) / 2;
+    for (long long I = lo + warp; I < hi; I += kHashThreads / 32) {
         unsigned long long d[W];
         load_det<W>(dets, I, d);
-        unsigned long long key[W];
+        unsigned long long z = 0;
+        int base = 0;
+        __syncwarp();
 #pragma unroll
-        for (int w = 0; w < W; ++w) key[w] = d[w];
-        fq::flip<W>(key, nth_occ<W>(d, x));
-        fq::flip<W>(key, nth_occ<W>(d, y));
-        unsigned long long h = fq::table_hash<W>(key, kSaltKey) >> (64 - kbits);
-        bool done = false;
-        for (long long probe = 0; probe < kcap && !done; ++probe) {
-            unsigned long long *e = tab + h * S;
-            int r = fq::probe_key<W>(e, key);
-            if (r == 1) {
-                atomicAdd(e + W, 1ull);
-                done = true;
-            } else if (r == 2) {
-                bool claimed;
-                if (fq::claim_key<W>(e, key, claimed)) {
-                    unsigned long long add = 1ull;
-                    if (claimed) add += atomicAdd(&st->n_buckets, 1ull) << 32;
-                    atomicAdd(e + W, add);
-                    done = true;
-                }
+        for (int c = 0; c < 2 * W; ++c) {
+            const unsigned bits = (unsigned)(d[c >> 1] >> (32 * (c & 1)));
+            if ((bits >> lane) & 1u) {
+                const int r = base + __popc(bits & ((1u << lane) - 1u));
+                const unsigned long long w = s.z[32 * c + lane];
+                z ^= w;
+                if (r < fq::MAXN) zo[r] = w;
             }
-            if (!done) h = (h + 1ull) & ((unsigned long long)kcap - 1ull);
+            base += __popc(bits);
         }
-        if (!done) atomicCAS(&st->status, 0, FCIQMC_ERR_CAPACITY);
+        for (int r = base + lane; r < n_elec; r += 32) zo[r] = 0ull;  // (a determinant short of electrons)
+        const unsigned zl = __reduce_xor_sync(0xFFFFFFFFu, (unsigned)z), zh = __reduce_xor_sync(0xFFFFFFFFu, (unsigned)(z >> 32));
+        const unsigned long long H = (unsigned long long)zl | ((unsigned long long)zh << 32);
+        __syncwarp();
+        const unsigned t0 = (unsigned)(I * npairs);
+        for (int k = lane; k < npairs; k += 32) {
+            const unsigned short pr = s.pairs[k];
+            f(t0 + (unsigned)k, H ^ zo[pr & 0xFF] ^ zo[pr >> 8]);
+        }
     }
 }
 
+// Keys per partition, counted in shared memory.
 template <int W>
-__global__ void k_counts(const unsigned long long *tab, long long kcap, unsigned *counts) {
-    constexpr int S = fq::Stride<W>::v;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < kcap; e += (long long)gridDim.x * blockDim.x) {
-        bool empty = true;
-#pragma unroll
-        for (int w = 0; w < W; ++w) empty = empty && (tab[e * S + w] == fq::EMPTY);
-        if (empty) continue;
-        const unsigned long long v = tab[e * S + W];
-        counts[v >> 32] = (unsigned)(v & 0xFFFFFFFFull);
+__global__ void __launch_bounds__(kHashThreads) k_key_hist(const unsigned long long *dets, long long n, int n_elec, int parts,
+                                                           int pbits, unsigned *total_p) {
+    extern __shared__ unsigned s_count[];
+    __shared__ HashShared s_h;
+    hash_setup(s_h, n_elec);
+    for (int p = threadIdx.x; p < parts; p += blockDim.x) s_count[p] = 0;
+    __syncthreads();
+    for_keys<W>(s_h, dets, n * blockIdx.x / gridDim.x, n * (blockIdx.x + 1) / gridDim.x, n_elec, [&](unsigned, unsigned long long h) {
+        atomicAdd(&s_count[pbits ? (unsigned)(h >> (64 - pbits)) : 0u], 1u);
+    });
+    __syncthreads();
+    for (int p = threadIdx.x; p < parts; p += blockDim.x) {
+        const unsigned m = s_count[p];
+        if (m) atomicAdd(&total_p[p], m);
     }
 }
 
-// Exclusive scans over buckets b < nb of m_b = count if count >= 2 else 0 (member offsets) and of
-// p_b = C(m_b, 2) (pair offsets), in three passes: per-block sums, a scan of the block sums, then
-// per-element offsets. Both outputs have nb + 1 entries.
-__global__ void k_scan_blocks(const unsigned *counts, long long nb, long long per_block, unsigned long long *bsum) {
-    __shared__ unsigned long long s_m[kThreads], s_p[kThreads];
-    const long long lo = (long long)blockIdx.x * per_block, hi = min(lo + per_block, nb);
-    unsigned long long m = 0, p = 0;
-    for (long long b = lo + threadIdx.x; b < hi; b += blockDim.x) {
-        const unsigned long long c = counts[b] >= 2 ? counts[b] : 0;
-        m += c;
-        p += c * (c - 1) / 2;
+// First record of every partition and of every bin of the first scatter pass (one block).
+__global__ void __launch_bounds__(1024) k_part_scan(const unsigned *total_p, int parts, int fine, unsigned *base_p, unsigned *cursor_p,
+                                                    unsigned *coarse_p) {
+    __shared__ unsigned s_w[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned carry = 0;
+    for (int p0 = 0; p0 < parts; p0 += 4096) {  // four neighbouring partitions per thread, so loads are coalesced
+        unsigned m[4], sum = 0;
+        const int p = p0 + 4 * (int)threadIdx.x;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            m[k] = p + k < parts ? total_p[p + k] : 0u;
+            sum += m[k];
+        }
+        unsigned x = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        __syncthreads();
+        if (lane == 31) s_w[warp] = x;
+        __syncthreads();
+        unsigned off = carry + x - sum, all = 0;
+#pragma unroll
+        for (int w = 0; w < 32; ++w) {
+            const unsigned y = s_w[w];
+            off += w < warp ? y : 0u;
+            all += y;
+        }
+        carry += all;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (p + k < parts) {
+                base_p[p + k] = off;
+                cursor_p[p + k] = off;
+                if (((p + k) & ((1 << fine) - 1)) == 0) coarse_p[((p + k) >> fine) * kCursorStride] = off;
+            }
+            off += m[k];
+        }
     }
-    s_m[threadIdx.x] = m;
-    s_p[threadIdx.x] = p;
-    __syncthreads();
-    for (int o = kThreads / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) {
-            s_m[threadIdx.x] += s_m[threadIdx.x + o];
-            s_p[threadIdx.x] += s_p[threadIdx.x + o];
+    if (threadIdx.x == 0) base_p[parts] = carry;
+}
+
+// Scatter of the key records to their partitions, a tile of up to kTileKeys at a time: the block counts the tile's
+// bins, takes room for each with one atomic, sorts the tile by bin in shared memory and writes it in that order, so
+// that neighbouring lanes write neighbouring records. (One store per lane wherever its record belongs took 2.4 ms
+// for 1.2e8 keys and 256 bins, every warp touching 32 pages; all 32,768 partitions at once took 4.5 ms.) Up to kBins
+// partitions one pass does; beyond, this pass takes the leading bits and k_refine the rest.
+// First pass: the records are made from the determinants. bits: of the bin number.
+struct ScatterShared {
+    HashShared h;
+    unsigned long long hash[kTileKeys];
+    unsigned long long rec[kTileKeys];
+    unsigned short bin[kTileKeys];
+    unsigned at[kBins];      // a bin's next place in the tile
+    unsigned to[kBins];      // where the tile's first record would go if it belonged to the bin
+    unsigned scan[kHashThreads / 32];
+};
+template <int W>
+__global__ void __launch_bounds__(kHashThreads, 2) k_key_scatter(const unsigned long long *dets, long long n, int n_elec,
+                                                                 int bits, int tbits, unsigned *cursor, unsigned long long *out) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    ScatterShared &s = *reinterpret_cast<ScatterShared *>(s_raw);
+    hash_setup(s.h, n_elec);
+    const int npairs = n_elec * (n_elec - 1) / 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = max(1, kTileKeys / npairs);  // determinants of a tile (npairs <= MAXPAIRS < kTileKeys)
+    for (long long lo = (long long)blockIdx.x * per; lo < n; lo += (long long)gridDim.x * per) {
+        const long long hi = min(lo + per, n);
+        const int m = (int)((hi - lo) * npairs);
+        s.at[threadIdx.x] = 0;  // kBins = kHashThreads
+        __syncthreads();
+        const unsigned t0 = (unsigned)(lo * npairs);
+        for_keys<W>(s.h, dets, lo, hi, n_elec, [&](unsigned t, unsigned long long h) {
+            s.hash[t - t0] = h;
+            atomicAdd(&s.at[bits ? (unsigned)(h >> (64 - bits)) : 0u], 1u);
+        });
+        __syncthreads();
+        const unsigned c = s.at[threadIdx.x];
+        unsigned x = c;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s.scan[warp] = x;
+        __syncthreads();
+        unsigned off = x - c;
+#pragma unroll
+        for (int w = 0; w < kHashThreads / 32; ++w) off += w < warp ? s.scan[w] : 0u;
+        s.at[threadIdx.x] = off;
+        s.to[threadIdx.x] = c ? atomicAdd(&cursor[threadIdx.x * kCursorStride], c) - off : 0u;
+        __syncthreads();
+        for (int k = threadIdx.x; k < m; k += kHashThreads) {
+            const unsigned long long h = s.hash[k];
+            const unsigned b = bits ? (unsigned)(h >> (64 - bits)) : 0u, at = atomicAdd(&s.at[b], 1u);
+            s.rec[at] = make_rec(h, bits, tbits, t0 + (unsigned)k);
+            s.bin[at] = (unsigned short)b;
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < m; k += kHashThreads) out[s.to[s.bin[k]] + (unsigned)k] = s.rec[k];
+        __syncthreads();
+    }
+}
+
+// Second pass: the records of coarse bin blockIdx.y to its 2^kFineBits partitions, by their hash's leading bits, which
+// are shifted out (the last kFineBits of the hash become zero).
+__global__ void __launch_bounds__(kHashThreads) k_refine(const unsigned long long *in, int tbits, const unsigned *base_p, unsigned *cursor_p,
+                                                         unsigned long long *out) {
+    constexpr int kFine = 1 << kFineBits;
+    __shared__ unsigned long long s_rec[4096];
+    __shared__ unsigned s_at[kFine];
+    const unsigned lo = base_p[blockIdx.y << kFineBits], hi = base_p[(blockIdx.y + 1) << kFineBits];
+    unsigned *cursor = cursor_p + (blockIdx.y << kFineBits);
+    for (unsigned long long t = (unsigned long long)lo + blockIdx.x * 4096ull; t < hi; t += gridDim.x * 4096ull) {
+        const int m = (int)min(4096ull, hi - t);
+        if (threadIdx.x < kFine) s_at[threadIdx.x] = 0;
+        __syncthreads();
+        for (int k = threadIdx.x; k < m; k += blockDim.x) {
+            const unsigned long long r = in[t + k];
+            s_rec[k] = r;
+            atomicAdd(&s_at[(unsigned)(r >> (64 - kFineBits))], 1u);
+        }
+        __syncthreads();
+        if (threadIdx.x < kFine) {
+            const unsigned c = s_at[threadIdx.x];
+            s_at[threadIdx.x] = c ? atomicAdd(&cursor[threadIdx.x], c) : 0u;
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < m; k += blockDim.x) {
+            const unsigned long long r = s_rec[k];
+            out[atomicAdd(&s_at[(unsigned)(r >> (64 - kFineBits))], 1u)] = make_rec(rec_hash(r, tbits) << tbits, kFineBits, tbits, rec_t(r, tbits));
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        bsum[2 * blockIdx.x] = s_m[0];
-        bsum[2 * blockIdx.x + 1] = s_p[0];
-    }
-}
-
-__global__ void k_scan_top(unsigned long long *bsum, int nblocks, RdmState *st) {
-    if (threadIdx.x != 0) return;
-    unsigned long long m = 0, p = 0;
-    for (int b = 0; b < nblocks; ++b) {
-        const unsigned long long bm = bsum[2 * b], bp = bsum[2 * b + 1];
-        bsum[2 * b] = m;
-        bsum[2 * b + 1] = p;
-        m += bm;
-        p += bp;
-    }
-    st->n_members = m;
-    st->n_pairs = p;
-}
-
-__global__ void k_scan_out(const unsigned *counts, long long nb, long long per_block, const unsigned long long *bsum,
-                           unsigned long long *moff, unsigned long long *poff, const RdmState *st) {
-    if (threadIdx.x != 0) return;  // one thread per block walks its range in order
-    const long long lo = (long long)blockIdx.x * per_block, hi = min(lo + per_block, nb);
-    unsigned long long m = bsum[2 * blockIdx.x], p = bsum[2 * blockIdx.x + 1];
-    for (long long b = lo; b < hi; ++b) {
-        moff[b] = m;
-        poff[b] = p;
-        const unsigned long long c = counts[b] >= 2 ? counts[b] : 0;
-        m += c;
-        p += c * (c - 1) / 2;
-    }
-    if (hi == nb && lo < hi) {
-        moff[nb] = st->n_members;
-        poff[nb] = st->n_pairs;
-    }
 }
 
 template <int W>
-__global__ void k_members(const unsigned long long *dets, long long n, int n_elec, const unsigned long long *tab,
-                          long long kcap, int kbits, const unsigned *counts, unsigned *cursor,
-                          const unsigned long long *moff, unsigned long long *members) {
-    constexpr int S = fq::Stride<W>::v;
-    const int npairs = n_elec * (n_elec - 1) / 2;
-    const long long total = n * npairs;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
-        const long long I = t / npairs;
-        int k = (int)(t - I * npairs);
-        int y = 1;
-        while ((y + 1) * y / 2 <= k) ++y;
-        const int x = k - y * (y - 1) / 2;
-        unsigned long long d[W];
-        load_det<W>(dets, I, d);
-        unsigned long long key[W];
+__device__ __forceinline__ bool same_key(const unsigned long long (&a)[W], const unsigned long long (&b)[W]) {
+    bool e = true;
 #pragma unroll
-        for (int w = 0; w < W; ++w) key[w] = d[w];
-        const int ox = nth_occ<W>(d, x), oy = nth_occ<W>(d, y);
-        fq::flip<W>(key, ox);
-        fq::flip<W>(key, oy);
-        const long long e = key_lookup<W>(tab, kcap, kbits, key);
-        if (e < 0) continue;
-        const unsigned long long b = tab[e * S + W] >> 32;
-        if (counts[b] < 2) continue;
-        const unsigned pos = atomicAdd(&cursor[b], 1u);
-        members[moff[b] + pos] = pack_member((unsigned)I, ox, oy);
-    }
+    for (int w = 0; w < W; ++w) e = e && a[w] == b[w];
+    return e;
 }
 
-// Sorts each bucket's members by determinant index (insertion sort; buckets are small).
-__global__ void k_sort_members(long long nb, const unsigned *counts, const unsigned long long *moff,
-                               unsigned long long *members) {
-    for (long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += (long long)gridDim.x * blockDim.x) {
-        const unsigned c = counts[b];
-        if (c < 2) continue;
-        unsigned long long *m = members + moff[b];
-        for (unsigned i = 1; i < c; ++i) {
-            const unsigned long long v = m[i];
-            unsigned j = i;
-            while (j > 0 && (m[j - 1] & 0xFFFFFFFFull) > (v & 0xFFFFFFFFull)) {
-                m[j] = m[j - 1];
-                --j;
+// Exclusive block scan of a 64-bit value (packed 16-bit fields); total in `sum`.
+__device__ __forceinline__ unsigned long long block_scan64(unsigned long long v, unsigned long long *s_w, unsigned long long &sum) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long x = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x += y;
+    }
+    __syncthreads();
+    if (lane == 31) s_w[warp] = x;
+    __syncthreads();
+    unsigned long long off = 0, tot = 0;
+#pragma unroll
+    for (int w = 0; w < kGroupThreads / 32; ++w) {
+        const unsigned long long y = s_w[w];
+        off += w < warp ? y : 0ull;
+        tot += y;
+    }
+    sum = tot;
+    return x - v + off;
+}
+
+// Signed amplitude of a member: the parity of removing the x-th and y-th electron, and one more exchange when a
+// mixed pair has its beta orbital first (pair codes put alpha first).
+__device__ __forceinline__ double signed_c(const double *c, unsigned I, unsigned short pr, int ox, int oy) {
+    const double v = __ldg(c + I);
+    const int par = ((pr & 0xFF) + (pr >> 8) + (((ox ^ oy) & ox) & 1)) & 1;
+    return par ? -v : v;
+}
+
+template <int W>
+struct GroupShared {
+    unsigned long long rec[kGroupCap];
+    unsigned table[kGroupSlots];       // (leading record << 16) | count, later (start << 16) | members placed
+    unsigned short slot[kGroupCap];    // a record's slot
+    unsigned short order[kGroupCap];   // record at each place of the kept members
+    unsigned short code[kGroupCap];    // of the member at a place: pair code, bit 15: negative sign
+    unsigned short orb[kGroupCap];     // its spin orbitals, x | y << 8
+    unsigned short pairs[fq::MAXPAIRS];
+    unsigned long long scan[kGroupThreads / 32];
+    unsigned long long lo, hi;         // smallest and largest hash of a selection
+    unsigned long long leader[kBigLeaders][W];
+    unsigned long long acc[3];
+    unsigned n, min_t, kept, bad;
+};
+
+// Records s.rec[0, s.n) grouped by key; groups of two and more go to out + s.kept, longer groups first (four size
+// classes), members in the order of their codes, so that the lanes of the pair passes have rows of similar length
+// and neighbouring table columns. Grouping goes by the hash bits; every member's key is then compared with its
+// group's first, and in the rare case that two keys share the hash, false is returned and nothing is written:
+// called again with `exact`, the keys themselves are compared on insertion.
+template <int W>
+__device__ __forceinline__ bool group_shared(GroupShared<W> &s, const unsigned long long *dets, const double *c, int npairs,
+                                             int n_orb, int tbits, Member *out, bool exact) {
+    constexpr unsigned kFree = 0xFFFFFFFFu;
+    const unsigned n = s.n;
+    for (int h = threadIdx.x; h < kGroupSlots; h += kGroupThreads) s.table[h] = kFree;
+    if (threadIdx.x == 0) s.bad = 0;
+    __syncthreads();
+    for (unsigned i = threadIdx.x; i < n; i += kGroupThreads) {
+        const unsigned long long r = s.rec[i];
+        unsigned h = (unsigned)(rec_hash(r, tbits) >> kFineBits) & (kGroupSlots - 1);
+        for (int probe = 0; probe < kGroupSlots; ++probe) {  // ends earlier: the table has more slots than records
+            unsigned e = *(volatile unsigned *)&s.table[h];
+            if (e == kFree) {
+                e = atomicCAS(&s.table[h], kFree, (i << 16) | 1u);
+                if (e == kFree) {
+                    s.slot[i] = (unsigned short)h;
+                    break;
+                }
             }
-            m[j] = v;
+            const unsigned long long q = s.rec[e >> 16];
+            bool match = rec_hash(q, tbits) == rec_hash(r, tbits);
+            if (exact && match) {
+                unsigned long long key[W], other[W];
+                key_of<W>(dets, s.pairs, npairs, rec_t(r, tbits), key);
+                key_of<W>(dets, s.pairs, npairs, rec_t(q, tbits), other);
+                match = same_key<W>(key, other);
+            }
+            if (match) {
+                atomicAdd(&s.table[h], 1u);
+                s.slot[i] = (unsigned short)h;
+                break;
+            }
+            h = (h + 1) & (kGroupSlots - 1);
         }
     }
-}
-
-__global__ void k_norm(const double *c, long long n, double *partial) {
-    __shared__ double s[kThreads];
-    double v = 0.0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        v = __dadd_rn(v, __dmul_rn(c[i], c[i]));
-    s[threadIdx.x] = v;
+    __syncthreads();
+    // member places by size class: 32 and more, 8.., 3.., 2 (16-bit fields of one scan)
+    constexpr int kPer = kGroupSlots / kGroupThreads;
+    unsigned long long mine = 0, buckets = 0, pairs = 0;
+    for (int k = 0; k < kPer; ++k) {
+        const unsigned e = s.table[k * kGroupThreads + threadIdx.x];
+        if (e == kFree) continue;
+        const unsigned m = e & 0xFFFFu;
+        ++buckets;
+        if (m < 2) continue;
+        pairs += (unsigned long long)m * (m - 1) / 2;
+        mine += (unsigned long long)m << (m >= 32 ? 0 : m >= 8 ? 16 : m >= 3 ? 32 : 48);
+    }
+    unsigned long long total = 0;
+    unsigned long long off = block_scan64(mine, s.scan, total);
+    const unsigned t0 = (unsigned)(total & 0xFFFF), t1 = (unsigned)((total >> 16) & 0xFFFF), t2 = (unsigned)((total >> 32) & 0xFFFF),
+                   t3 = (unsigned)(total >> 48);
+    const unsigned placed = t0 + t1 + t2 + t3;
+    off += ((unsigned long long)t0 << 16) + ((unsigned long long)(t0 + t1) << 32) + ((unsigned long long)(t0 + t1 + t2) << 48);
+    for (int k = 0; k < kPer; ++k) {
+        const unsigned h = k * kGroupThreads + threadIdx.x, e = s.table[h];
+        if (e == kFree) continue;
+        const unsigned m = e & 0xFFFFu;
+        if (m < 2) {
+            s.table[h] = kFree;  // a key of one determinant: dropped
+        } else {
+            const int sh = m >= 32 ? 0 : m >= 8 ? 16 : m >= 3 ? 32 : 48;
+            s.table[h] = (unsigned)((off >> sh) & 0xFFFF) << 16;
+            off += (unsigned long long)m << sh;
+        }
+    }
+    __syncthreads();
+    for (unsigned i = threadIdx.x; i < n; i += kGroupThreads) {
+        const unsigned h = s.slot[i];
+        if (s.table[h] == kFree) continue;
+        const unsigned e = atomicAdd(&s.table[h], 1u);
+        s.order[(e >> 16) + (e & 0xFFFFu)] = (unsigned short)i;
+    }
+    __syncthreads();
+    for (unsigned at = threadIdx.x; at < placed; at += kGroupThreads) {
+        unsigned long long key[W];
+        const KeyOf q = key_of<W>(dets, s.pairs, npairs, rec_t(s.rec[s.order[at]], tbits), key);
+        const unsigned short pr = s.pairs[q.k];
+        const unsigned par = ((pr & 0xFF) + (pr >> 8) + (((q.ox ^ q.oy) & q.ox) & 1)) & 1;
+        s.code[at] = (unsigned short)(pair_code(q.ox, q.oy, n_orb) | (par << 15));
+        s.orb[at] = (unsigned short)(q.ox | (q.oy << 8));
+    }
+    __syncthreads();
+    if (!exact) {
+        // the same key: the determinants differ by the two pairs
+        for (unsigned at = threadIdx.x; at < placed; at += kGroupThreads) {
+            const unsigned i = s.order[at], first = s.table[s.slot[i]] >> 16;
+            if (first == at) continue;
+            unsigned long long a[W], b[W];
+            load_det<W>(dets, rec_t(s.rec[i], tbits) / (unsigned)npairs, a);
+            load_det<W>(dets, rec_t(s.rec[s.order[first]], tbits) / (unsigned)npairs, b);
+            const unsigned x = s.orb[at], y = s.orb[first];
+            fq::flip<W>(a, x & 0xFF);
+            fq::flip<W>(a, x >> 8);
+            fq::flip<W>(b, y & 0xFF);
+            fq::flip<W>(b, y >> 8);
+            if (!same_key<W>(a, b)) s.bad = 1;
+        }
+        __syncthreads();
+        if (s.bad) return false;
+    }
+    const unsigned kept = s.kept;
+    for (unsigned at = threadIdx.x; at < placed; at += kGroupThreads) {
+        const unsigned i = s.order[at], e = s.table[s.slot[i]];
+        const unsigned first = e >> 16, m = e & 0xFFFFu, ci = s.code[at], code = ci & 0x7FFFu;
+        unsigned rank = 0;
+        for (unsigned j = first; j < first + m; ++j) {
+            const unsigned cj = s.code[j] & 0x7FFFu;
+            rank += (cj < code || (cj == code && j < at)) ? 1u : 0u;
+        }
+        const double v = __ldg(c + rec_t(s.rec[i], tbits) / (unsigned)npairs);
+        Member o;
+        o.v = code == kNoPair ? 0.0 : (ci & 0x8000u) ? -v : v;
+        o.code = (code == kNoPair ? 0u : code) | ((m >= kTriangle ? 63u : m) << 15);
+        o.first = kept + first;
+        out[kept + first + rank] = o;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        buckets += __shfl_down_sync(0xFFFFFFFFu, buckets, o);
+        pairs += __shfl_down_sync(0xFFFFFFFFu, pairs, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&s.acc[0], buckets);
+        atomicAdd(&s.acc[2], pairs);
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int k = 0; k < kThreads; ++k) t = __dadd_rn(t, s[k]);
-        partial[blockIdx.x] = t;
+        s.kept = kept + placed;
+        s.acc[1] += placed;
+    }
+    __syncthreads();
+    return true;
+}
+
+// More than kGroupCap records of one partition with the same hash bits (a key shared by thousands of
+// determinants): the distinct keys are taken one after another (smallest record first), each in two passes
+// over the partition; its members are written in the order the threads meet them.
+template <int W>
+__device__ void group_big(GroupShared<W> &s, const unsigned long long *rec, unsigned size, unsigned long long hash,
+                          const unsigned long long *dets, const double *c, int npairs, int n_orb, int tbits, Member *out, RdmState *st) {
+    for (int nl = 0;; ++nl) {
+        if (threadIdx.x == 0) {
+            s.min_t = 0xFFFFFFFFu;
+            s.n = 0;
+        }
+        __syncthreads();
+        for (unsigned i = threadIdx.x; i < size; i += kGroupThreads) {
+            const unsigned long long r = rec[i];
+            if (rec_hash(r, tbits) != hash) continue;
+            unsigned long long key[W];
+            key_of<W>(dets, s.pairs, npairs, rec_t(r, tbits), key);
+            bool seen = false;
+            for (int l = 0; l < nl; ++l) seen = seen || same_key<W>(key, s.leader[l]);
+            if (!seen) atomicMin(&s.min_t, rec_t(r, tbits));
+        }
+        __syncthreads();
+        const unsigned t = s.min_t;
+        if (t == 0xFFFFFFFFu) return;
+        if (nl >= kBigLeaders) {
+            if (threadIdx.x == 0) atomicCAS(&st->status, 0, FCIQMC_ERR_CAPACITY);
+            return;
+        }
+        unsigned long long lead[W];
+        key_of<W>(dets, s.pairs, npairs, t, lead);
+        if (threadIdx.x == 0)
+            for (int w = 0; w < W; ++w) s.leader[nl][w] = lead[w];
+        for (unsigned i = threadIdx.x; i < size; i += kGroupThreads) {
+            const unsigned long long r = rec[i];
+            if (rec_hash(r, tbits) != hash) continue;
+            unsigned long long key[W];
+            key_of<W>(dets, s.pairs, npairs, rec_t(r, tbits), key);
+            if (same_key<W>(key, lead)) atomicAdd(&s.n, 1u);
+        }
+        __syncthreads();
+        const unsigned m = s.n, kept = s.kept;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s.acc[0] += 1;
+            s.n = 0;
+            if (m >= 2) {
+                s.acc[1] += m;
+                s.acc[2] += (unsigned long long)m * (m - 1) / 2;
+                s.kept = kept + m;
+            }
+        }
+        __syncthreads();
+        if (m < 2) continue;
+        for (unsigned i = threadIdx.x; i < size; i += kGroupThreads) {
+            const unsigned long long r = rec[i];
+            if (rec_hash(r, tbits) != hash) continue;
+            unsigned long long key[W];
+            const KeyOf q = key_of<W>(dets, s.pairs, npairs, rec_t(r, tbits), key);
+            if (!same_key<W>(key, lead)) continue;
+            Member o;
+            const unsigned code = pair_code(q.ox, q.oy, n_orb);
+            o.v = code == kNoPair ? 0.0 : signed_c(c, q.I, s.pairs[q.k], q.ox, q.oy);
+            o.code = (code == kNoPair ? 0u : code) | ((m >= kTriangle ? 63u : m) << 15);
+            o.first = kept;
+            out[kept + atomicAdd(&s.n, 1u)] = o;
+        }
+        __syncthreads();
     }
 }
 
-__global__ void k_sum_partials(const double *partial, int n, double *out) {
-    if (threadIdx.x != 0) return;
-    double t = 0.0;
-    for (int b = 0; b < n; ++b) t = __dadd_rn(t, partial[b]);
-    *out = t;
+// One block per partition: its records in shared memory (in parts by further hash bits when there are more than
+// fit), grouped by key, the groups of two and more written as members at the partition's place.
+template <int W>
+__global__ void __launch_bounds__(kGroupThreads, 2) k_group(const unsigned long long *dets, const double *c, int n_elec, int n_orb,
+                                                            int tbits, const unsigned long long *records, const unsigned *base_p,
+                                                            Member *members, unsigned *count_p, RdmState *st) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    GroupShared<W> &s = *reinterpret_cast<GroupShared<W> *>(s_raw);
+    const int npairs = n_elec * (n_elec - 1) / 2;
+    fill_pairs(n_elec, s.pairs);
+    if (threadIdx.x < 3) s.acc[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s.kept = 0;
+    const unsigned base = base_p[blockIdx.x], size = base_p[blockIdx.x + 1] - base;
+    const unsigned long long *rec = records + base;
+    Member *out = members + base;
+    if (size <= (unsigned)kGroupCap) {
+        for (unsigned i = threadIdx.x; i < size; i += kGroupThreads) s.rec[i] = rec[i];
+        if (threadIdx.x == 0) s.n = size;
+        __syncthreads();
+        if (size && !group_shared<W>(s, dets, c, npairs, n_orb, tbits, out, false)) group_shared<W>(s, dets, c, npairs, n_orb, tbits, out, true);
+    } else {
+        // sub-partitions by the leading `depth` bits of the hash, deeper where one is still too long
+        int d0 = 1;
+        while (((unsigned)kGroupCap / 2) << d0 < size && d0 < 20) ++d0;
+        int depth = d0;
+        unsigned long long sub = 0;
+        while (sub < (1ull << depth)) {
+            if (threadIdx.x == 0) {
+                s.n = 0;
+                s.lo = ~0ull;
+                s.hi = 0;
+            }
+            __syncthreads();
+            for (unsigned i = threadIdx.x; i < size; i += kGroupThreads) {
+                const unsigned long long r = rec[i];
+                if (rec_hash(r, tbits) >> (64 - tbits - depth) != sub) continue;
+                const unsigned k = atomicAdd(&s.n, 1u);
+                if (k < (unsigned)kGroupCap) s.rec[k] = r;
+                atomicMin(&s.lo, rec_hash(r, tbits));
+                atomicMax(&s.hi, rec_hash(r, tbits));
+            }
+            __syncthreads();
+            const unsigned m = s.n;
+            if (m > (unsigned)kGroupCap && s.lo != s.hi) {  // two hashes share these bits, so there are more
+                ++depth;
+                sub <<= 1;
+                __syncthreads();
+                continue;
+            }
+            const unsigned long long hash = s.lo;
+            __syncthreads();
+            if (m > (unsigned)kGroupCap) group_big<W>(s, rec, size, hash, dets, c, npairs, n_orb, tbits, out, st);
+            else if (m && !group_shared<W>(s, dets, c, npairs, n_orb, tbits, out, false)) group_shared<W>(s, dets, c, npairs, n_orb, tbits, out, true);
+            __syncthreads();
+            ++sub;
+            while (depth > d0 && !(sub & 1ull)) {
+                sub >>= 1;
+                --depth;
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        count_p[blockIdx.x] = s.kept;
+        if (s.acc[0]) atomicAdd(&st->n_buckets, s.acc[0]);
+        if (s.acc[1]) atomicAdd(&st->n_members, s.acc[1]);
+        if (s.acc[2]) atomicAdd(&st->n_pairs, s.acc[2]);
+    }
 }
 
 // ------------------------------------------------------------------------------------ compensated sums
@@ -363,378 +777,369 @@ __device__ __forceinline__ CSum warp_csum(CSum a) {
     }
     return a;  // lane 0 holds the warp's sum
 }
-// Block sum of every thread's acc into out[0] (sum) and out[1] (running error); s: kThreads / 32 slots.
-__device__ __forceinline__ void block_csum(CSum acc, CSum *s, double *out) {
+// Block sum of every thread's acc, in thread 0; s: one slot per warp.
+__device__ __forceinline__ CSum block_csum(CSum acc, CSum *s) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     acc = warp_csum(acc);
     if (lane == 0) s[warp] = acc;
     __syncthreads();
+    CSum x{0.0, 0.0};
     if (warp == 0) {
-        CSum x = lane < kThreads / 32 ? s[lane] : CSum{0.0, 0.0};
+        if (lane < (int)(blockDim.x >> 5)) x = s[lane];
         x = warp_csum(x);
-        if (lane == 0) {
-            out[0] = x.s;
-            out[1] = x.c;
+    }
+    __syncthreads();
+    return x;
+}
+
+// ------------------------------------------------------------------------------------ diagonal
+// Occupation-pair sums over spin orbitals p <= q, O_pq = sum_I c_I^2 n_p n_q at q (q + 1) / 2 + p (p == q: the
+// occupations). One determinant per warp at a time: the lanes hold its occupied list and take its pairs, which are
+// distinct, so each warp adds into a copy of its own in shared memory without atomics (shared FP64 atomics are
+// compare-and-swap loops, and the core pairs, occupied in nearly every determinant, made all lanes retry on
+// one word). Block copies are added up in warp order into occ_part[block].
+template <int W>
+__global__ void __launch_bounds__(256) k_occ_pairs(const unsigned long long *dets, const double *c, long long n, int n_elec,
+                                                   int n_so, double *occ_part) {
+    extern __shared__ double s_o[];
+    __shared__ unsigned short s_pairs[fq::MAXPAIRS];
+    fill_pairs(n_elec, s_pairs);
+    const int nent = n_so * (n_so + 1) / 2, npairs = n_elec * (n_elec - 1) / 2;
+    const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int k = threadIdx.x; k < nent * nw; k += blockDim.x) s_o[k] = 0.0;
+    __syncthreads();
+    double *o = s_o + nent * warp;
+    const long long step = (long long)gridDim.x * nw;
+    long long I = (long long)blockIdx.x * nw + warp;
+    // the lane's occupied orbitals (ranks lane and lane + 32; ranks beyond the electrons are not used) and c^2, of the
+    // next determinant while the current one's sums are in flight
+    auto decode = [&](long long i, int &k0, int &k1, double &c2) {
+        unsigned long long d[W];
+        load_det<W>(dets, i, d);
+        const double ci = __ldg(c + i);
+        k0 = fq::select_bit<W>(d, lane);
+        k1 = n_elec > 32 ? fq::select_bit<W>(d, lane + 32) : 0;
+        c2 = __dmul_rn(ci, ci);
+    };
+    int k0 = 0, k1 = 0, nk0 = 0, nk1 = 0;
+    double c2 = 0.0, nc2 = 0.0;
+    if (I < n) decode(I, k0, k1, c2);
+    for (; I < n; I += step, k0 = nk0, k1 = nk1, c2 = nc2) {
+        if (I + step < n) decode(I + step, nk0, nk1, nc2);
+        // four pairs of a lane at a time: their words are distinct, so the loads need not wait for the stores
+        for (int k0s = 0; k0s < npairs; k0s += 128) {
+            double *e[4], x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = k0s + 32 * u + lane;
+                const unsigned short pr = k < npairs ? s_pairs[k] : 0;
+                const int rx = pr & 0xFF, ry = pr >> 8;
+                int p = __shfl_sync(0xFFFFFFFFu, k0, rx & 31), q = __shfl_sync(0xFFFFFFFFu, k0, ry & 31);
+                if (n_elec > 32) {
+                    const int p1 = __shfl_sync(0xFFFFFFFFu, k1, rx & 31), q1 = __shfl_sync(0xFFFFFFFFu, k1, ry & 31);
+                    if (rx >= 32) p = p1;
+                    if (ry >= 32) q = q1;
+                }
+                e[u] = k < npairs && p <= q && q < n_so ? o + q * (q + 1) / 2 + p : nullptr;
+                x[u] = e[u] ? *e[u] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (e[u]) *e[u] = __dadd_rn(x[u], c2);
         }
+        if (lane < n_elec && k0 < n_so) {
+            double *e = o + k0 * (k0 + 1) / 2 + k0;
+            *e = __dadd_rn(*e, c2);
+        }
+        if (lane + 32 < n_elec && k1 < n_so) {
+            double *e = o + k1 * (k1 + 1) / 2 + k1;
+            *e = __dadd_rn(*e, c2);
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < nent; k += blockDim.x) {
+        double t = 0.0;
+        for (int w = 0; w < nw; ++w) t = __dadd_rn(t, s_o[nent * w + k]);
+        occ_part[(size_t)blockIdx.x * nent + k] = t;
+    }
+}
+
+// Sums of the blocks' occupation pairs (compensated, in block order); the last block adds the partial sums of c^2.
+__global__ void __launch_bounds__(kMergeThreads) k_occ_merge(const double *occ_part, int nblocks, int nent, double *occ_pair,
+                                                             const double *norm_part, int n_norm, RdmState *st) {
+    if (blockIdx.x == gridDim.x - 1) {
+        __shared__ CSum s[kMergeThreads / 32];
+        CSum a{0.0, 0.0};
+        for (int b = threadIdx.x; b < n_norm; b += kMergeThreads) csum_merge(a, CSum{norm_part[2 * b], norm_part[2 * b + 1]});
+        a = block_csum(a, s);
+        if (threadIdx.x == 0) st->norm = __dadd_rn(a.s, a.c);
+        return;
+    }
+    const int k = blockIdx.x * kMergeThreads + threadIdx.x;
+    if (k >= nent) return;
+    CSum a{0.0, 0.0};
+    for (int b = 0; b < nblocks; ++b) csum_add(a, occ_part[(size_t)b * nent + k]);
+    occ_pair[k] = __dadd_rn(a.s, a.c);
+}
+
+__global__ void __launch_bounds__(kThreads) k_norm(const double *c, long long n, double *partial) {
+    __shared__ CSum s[kThreads / 32];
+    CSum v{0.0, 0.0};
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        csum_add(v, __dmul_rn(c[i], c[i]));
+    v = block_csum(v, s);
+    if (threadIdx.x == 0) {
+        partial[2 * blockIdx.x] = v.s;
+        partial[2 * blockIdx.x + 1] = v.c;
     }
 }
 
 // ------------------------------------------------------------------------------------ pairs
-struct PairInfo {
-    long long I, J;
-    int kind;            // 0: skip, 1: single i -> a (from I), 2: double (i<j) -> (a<b) (from I)
-    int i, j, a, b;
+// T over pair codes: the same-spin block (n1 x n1, rows and columns p < q), then the mixed block (n2 x n2, alpha
+// first); the diagonals stay zero (the diagonal of H comes from the occupation-pair sums).
+__global__ void __launch_bounds__(kThreads) k_pair_table(const double *h, const double *eri, int n_orb, int n1, int n2, double inv,
+                                                         double *table) {
+    const int row = blockIdx.y;
+    if (row < n1) {
+        int p, q;
+        triangle_of(row, p, q);
+        for (int col = blockIdx.x * blockDim.x + threadIdx.x; col < n1; col += gridDim.x * blockDim.x) {
+            int r, s;
+            triangle_of(col, r, s);
+            double v = 0.0;
+            if (col != row) {
+                v = __dsub_rn(__ldg(eri + fq::eidx(p, r, q, s)), __ldg(eri + fq::eidx(p, s, q, r)));
+                if (q == s) v = __dadd_rn(v, __dmul_rn(inv, __ldg(h + p * n_orb + r)));
+                if (p == r) v = __dadd_rn(v, __dmul_rn(inv, __ldg(h + q * n_orb + s)));
+                if (q == r) v = __dsub_rn(v, __dmul_rn(inv, __ldg(h + p * n_orb + s)));
+                if (p == s) v = __dsub_rn(v, __dmul_rn(inv, __ldg(h + q * n_orb + r)));
+            }
+            table[(size_t)row * n1 + col] = v;
+        }
+    } else {
+        const int row2 = row - n1, p = row2 / n_orb, q = row2 - p * n_orb;
+        for (int col = blockIdx.x * blockDim.x + threadIdx.x; col < n2; col += gridDim.x * blockDim.x) {
+            const int r = col / n_orb, s = col - r * n_orb;
+            double v = 0.0;
+            if (col != row2) {
+                v = __ldg(eri + fq::eidx(p, r, q, s));
+                if (q == s) v = __dadd_rn(v, __dmul_rn(inv, __ldg(h + p * n_orb + r)));
+                if (p == r) v = __dadd_rn(v, __dmul_rn(inv, __ldg(h + q * n_orb + s)));
+            }
+            table[(size_t)n1 * n1 + (size_t)row2 * n2 + col] = v;
+        }
+    }
+}
+
+// The partners of member j of a group of m starting at `first`, so that every pair is met once: small groups
+// cyclically (each member takes about half of the others, so the lanes of a warp, in groups of similar size,
+// finish together), large ones (m >= kTriangle) as a triangle, in which the lanes of a warp meet the same partner
+// at the same time and read neighbouring columns of its table row.
+struct RowRange {
+    int n;        // partners
+    int at;       // first partner, counted from the group's start
+    int wrap;     // group size for the cyclic walk (never reached by the triangle)
 };
-
-// Last bucket b in [lo, hi] with poff[b] <= x.
-__device__ __forceinline__ long long bucket_search(const unsigned long long *poff, unsigned long long x, long long lo,
-                                                   long long hi) {
-    while (lo < hi) {
-        const long long mid = (lo + hi + 1) >> 1;
-        if (poff[mid] <= x) lo = mid; else hi = mid - 1;
-    }
-    return lo;
+__device__ __forceinline__ RowRange row_range(unsigned packed, int local) {
+    const int m = (int)(packed >> 15);
+    if (m == 63) return RowRange{local, 0, 0x7FFFFFFF};
+    const int half = (m - 1) >> 1, even = (m & 1) == 0 && local < (m >> 1) ? 1 : 0;
+    return RowRange{half + even, local + 1 < m ? local + 1 : 0, m};
 }
 
-// Bucket of pair k * 2^kPairIndexShift for every k (the coarse index of the bucket search).
-constexpr int kPairIndexShift = 8;
-__global__ void k_pair_index(const unsigned long long *poff, long long nb, const RdmState *st, unsigned *idx) {
-    const unsigned long long nk = (st->n_pairs >> kPairIndexShift) + 1;
-    for (unsigned long long k = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; k < nk;
-         k += (unsigned long long)gridDim.x * blockDim.x)
-        idx[k] = (unsigned)bucket_search(poff, k << kPairIndexShift, 0, nb - 1);
-}
-
-// Candidate pair t: bucket by binary search over pair offsets, narrowed by the coarse index when there is
-// one, (u < v) by inverse triangular index (the float square root is a first guess that the integer
-// steps correct).
-template <int W>
-__device__ __forceinline__ PairInfo pair_of(unsigned long long t, unsigned long long np, long long nb,
-                                            const unsigned long long *poff, const unsigned *pidx,
-                                            const unsigned long long *moff, const unsigned long long *members,
-                                            const unsigned long long *dets, unsigned long long (&dI)[W],
-                                            unsigned long long (&dJ)[W]) {
-    PairInfo P{};
-    long long b_lo = 0, b_hi = nb - 1;
-    if (pidx) {
-        const unsigned long long k = t >> kPairIndexShift;
-        b_lo = pidx[k];
-        if (((k + 1) << kPairIndexShift) < np) b_hi = pidx[k + 1];
-    }
-    const long long lo = bucket_search(poff, t, b_lo, b_hi);
-    const unsigned long long l = t - poff[lo];
-    unsigned long long v = (unsigned long long)((1.0f + sqrtf(1.0f + 8.0f * (float)l)) * 0.5f);
-    while (v > 1 && v * (v - 1) / 2 > l) --v;
-    while ((v + 1) * v / 2 <= l) ++v;
-    const unsigned long long u = l - v * (v - 1) / 2;
-    const unsigned long long mu = members[moff[lo] + u], mv = members[moff[lo] + v];
-    P.I = (long long)(mu & 0xFFFFFFFFull);
-    P.J = (long long)(mv & 0xFFFFFFFFull);
-    load_det<W>(dets, P.I, dI);
-    load_det<W>(dets, P.J, dJ);
-    int nd = 0;
-    unsigned long long holes[W], parts[W], common[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-        holes[w] = dI[w] & ~dJ[w];
-        parts[w] = dJ[w] & ~dI[w];
-        common[w] = dI[w] & dJ[w];
-        nd += __popcll(holes[w]);
-    }
-    if (nd == 2) {
-        P.kind = 2;
-        P.i = fq::select_bit<W>(holes, 0);
-        P.j = fq::select_bit<W>(holes, 1);
-        P.a = fq::select_bit<W>(parts, 0);
-        P.b = fq::select_bit<W>(parts, 1);
-    } else if (nd == 1) {
-        // single: kept only in the bucket whose shared removed orbital is the lowest common electron
-        const int xu = (int)((mu >> 32) & 0xFF), yu = (int)((mu >> 40) & 0xFF);
-        const int hole = fq::select_bit<W>(holes, 0);
-        const int shared = xu == hole ? yu : xu;
-        if (shared == fq::select_bit<W>(common, 0)) {
-            P.kind = 1;
-            P.i = hole;
-            P.a = fq::select_bit<W>(parts, 0);
-        }
-    }
-    return P;
-}
-
-template <int W>
-__device__ __forceinline__ double single_h(const Params &P, const unsigned long long (&d)[W], int i, int a) {
-    const int I = i >> 1, A = a >> 1;
-    double v = P.h[I * P.n_orb + A];
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-        unsigned long long m = d[w];
-        while (m) {
-            const int j = 64 * w + __ffsll((long long)m) - 1;
-            m &= m - 1;
-            if (j == i) continue;
-            const int J = j >> 1;
-            v = __dadd_rn(v, fq::eri_d(P, I, A, J, J));
-            if ((j & 1) == (i & 1)) v = __dsub_rn(v, fq::eri_d(P, I, J, J, A));
-        }
-    }
-    return (fq::count_between<W>(d, i, a) & 1) ? -v : v;
-}
-
-// Single-excitation pairs are a few percent of the candidates, and each costs an O(N) FP64 loop: a warp
-// queues its lanes' singles (pair I, J and orbitals i -> a) and evaluates them 32 at a time, so the loop
-// never runs for one lane while 31 wait. The queue order is fixed by the warp's schedule.
-struct SingleQueue {
-    unsigned long long ij[64];  // I | J << 32
-    unsigned short ia[64];      // i | a << 8
-    unsigned n;
-};
-__device__ __forceinline__ void queue_single(SingleQueue &q, bool single, const PairInfo &p) {
-    const unsigned m = __ballot_sync(0xFFFFFFFFu, single);
-    const int lane = threadIdx.x & 31;
-    const unsigned n = q.n;
-    if (single) {
-        const unsigned k = n + __popc(m & ((1u << lane) - 1u));
-        q.ij[k] = (unsigned long long)p.I | ((unsigned long long)p.J << 32);
-        q.ia[k] = (unsigned short)(p.i | (p.a << 8));
-    }
-    __syncwarp();
-    if (lane == 0) q.n = n + __popc(m);
-    __syncwarp();
-}
-// Takes up to 32 queued singles (all when `all`, else only once 32 are queued): lane k gets entry k
-// (take = false for the others); the rest moves to the front.
-__device__ __forceinline__ bool pop_single(SingleQueue &q, bool all, long long &I, long long &J, int &i, int &a) {
-    const int lane = threadIdx.x & 31;
-    const unsigned n = q.n;
-    if (n == 0 || (!all && n < 32)) return false;
-    const unsigned take = min(n, 32u);
-    bool got = false;
-    if ((unsigned)lane < take) {
-        I = (long long)(q.ij[lane] & 0xFFFFFFFFull);
-        J = (long long)(q.ij[lane] >> 32);
-        i = q.ia[lane] & 0xFF;
-        a = q.ia[lane] >> 8;
-        got = true;
-    }
-    __syncwarp();
-    const unsigned rest = n - take;
-    if ((unsigned)lane < rest) {
-        q.ij[lane] = q.ij[take + lane];
-        q.ia[lane] = q.ia[take + lane];
-    }
-    __syncwarp();
-    if (lane == 0) q.n = rest;
-    __syncwarp();
-    return got;
-}
-
-// 2 c_I c_J H_IJ summed over candidate pairs, per block in a fixed order (compensated).
-template <int W>
-__global__ void __launch_bounds__(kThreads) k_pair_energy(Params P, const unsigned long long *dets, const double *c,
-                                                          long long nb, const unsigned long long *poff,
-                                                          const unsigned *pidx, const unsigned long long *moff,
-                                                          const unsigned long long *members, const RdmState *st,
-                                                          double *partial) {
-    __shared__ CSum s[kThreads / 32];
-    __shared__ SingleQueue s_q[kThreads / 32];
-    SingleQueue &sq = s_q[threadIdx.x >> 5];
-    if ((threadIdx.x & 31) == 0) sq.n = 0;
-    __syncwarp();
-    const unsigned long long np = st->n_pairs;
+// 2 c_I c_J H_IJ summed over the pairs of members, without the factor 2: per thread the rows of its members, plain
+// within one partition (a handful of rows), compensated across partitions, the blocks' sums in a fixed tree. A
+// row is an FMA chain of at most half a small group, or of eight partners of a large one at a time.
+// Bound by the FP64 pipe (one FMA per pair, charged per warp instruction) and the table reads from L2.
+__global__ void __launch_bounds__(kThreads) k_pair_energy(const Member *members, const unsigned *base_p, const unsigned *count_p,
+                                                          int parts, int n1, int n2, const double *table, double *partial) {
+    __shared__ CSum s_red[kThreads / 32];
     CSum acc{0.0, 0.0};
-    auto add_single = [&](bool all) {
-        long long I = 0, J = 0;
-        int i = 0, a = 0;
-        if (pop_single(sq, all, I, J, i, a)) {
-            unsigned long long dI[W];
-            load_det<W>(dets, I, dI);
-            csum_add(acc, __dmul_rn(__dmul_rn(2.0, __dmul_rn(c[I], c[J])), single_h<W>(P, dI, i, a)));
+    const double *mixed = table + (size_t)n1 * n1;
+    for (int p = blockIdx.x; p < parts; p += gridDim.x) {
+        const Member *mem = members + base_p[p];
+        const int cnt = (int)count_p[p];
+        if ((int)threadIdx.x >= cnt) continue;
+        double sum = 0.0;
+        for (int j = threadIdx.x; j < cnt; j += kThreads) {
+            const Member u = mem[j];
+            const Member *grp = mem + u.first;
+            const RowRange r = row_range(u.code, j - (int)u.first);
+            const unsigned cls = (u.code >> 13) & 3u, cu = u.code & 0x1FFFu;
+            const double *col = (cls == 2u ? mixed : table) + cu;
+            const int stride = cls == 2u ? n2 : n1;
+            double row = 0.0;
+            int at = r.at;
+            for (int k0 = 0; k0 < r.n; k0 += 8) {
+                double part = 0.0;
+                const int k1 = min(k0 + 8, r.n);
+#pragma unroll 4
+                for (int k = k0; k < k1; ++k) {
+                    const Member w = grp[at];
+                    at = at + 1 == r.wrap ? 0 : at + 1;
+                    if (((w.code >> 13) & 3u) == cls) part = __fma_rn(__ldg(col + (size_t)(w.code & 0x1FFFu) * stride), w.v, part);
+                }
+                row = __dadd_rn(row, part);
+            }
+            sum = __fma_rn(u.v, row, sum);
         }
-    };
-    // warp-uniform loop: lane k takes pair base + k
-    for (unsigned long long base = (unsigned long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < np;
-         base += (unsigned long long)gridDim.x * blockDim.x) {
-        const unsigned long long t = base + (threadIdx.x & 31);
-        PairInfo q{};
-        if (t < np) {
-            unsigned long long dI[W], dJ[W];
-            q = pair_of<W>(t, np, nb, poff, pidx, moff, members, dets, dI, dJ);
-            if (q.kind == 2)
-                csum_add(acc, __dmul_rn(__dmul_rn(2.0, __dmul_rn(c[q.I], c[q.J])),
-                                        fq::hij_double<W>(P, dI, q.i, q.j, q.a, q.b)));
-        }
-        queue_single(sq, q.kind == 1, q);
-        add_single(false);
+        csum_add(acc, sum);
     }
-    add_single(true);  // fewer than 32 remain
-    block_csum(acc, s, partial + 2 * blockIdx.x);
+    acc = block_csum(acc, s_red);
+    if (threadIdx.x == 0) {
+        partial[2 * blockIdx.x] = acc.s;
+        partial[2 * blockIdx.x + 1] = acc.c;
+    }
 }
 
-// c_I^2 H_II per block (pair-term table in shared memory, compensated).
-template <int W>
-__global__ void __launch_bounds__(kThreads) k_diag_energy(Params P, const unsigned long long *dets, const double *c,
-                                                          long long n, double *partial) {
-    extern __shared__ double s_w[];
-    __shared__ CSum s[kThreads / 32];
-    const int M = P.n_orb;
-    for (int k = threadIdx.x; k < 2 * M * M; k += blockDim.x) s_w[k] = P.wpair[k];
-    for (int k = threadIdx.x; k < M; k += blockDim.x) s_w[2 * M * M + k] = P.h[k * M + k];
-    __syncthreads();
-    CSum acc{0.0, 0.0};
-    for (long long I = (long long)blockIdx.x * blockDim.x + threadIdx.x; I < n; I += (long long)gridDim.x * blockDim.x) {
-        unsigned long long d[W];
-        load_det<W>(dets, I, d);
-        csum_add(acc, __dmul_rn(__dmul_rn(c[I], c[I]), fq::hdiag<W>(P, d, s_w, s_w + 2 * M * M)));
-    }
-    block_csum(acc, s, partial + 2 * blockIdx.x);
-}
-
-// One warp: lane k merges the block partials k, k + 32, ... (diagonal, then pairs), then a fixed tree.
-__global__ void k_energy_finish(const double *pp, int npp, const double *pd, int npd, const RdmState *st, double *e) {
-    const int lane = threadIdx.x & 31;
-    if (threadIdx.x >= 32) return;
+// One block: the pair sums (twice: both orders of a pair), then the diagonal from the occupation pairs,
+// sum_p O_pp h_pp + sum_{p<q} O_pq ((pp|qq) - delta_spin (pq|qp)), all compensated in a fixed order; over c^T c.
+__global__ void __launch_bounds__(1024) k_energy_finish(const double *pp, int npp, const double *occ_pair, const double *h,
+                                                        const double *eri, int n_orb, const RdmState *st, double *e) {
+    __shared__ CSum s_red[32];
     CSum tot{0.0, 0.0};
-    for (int b = lane; b < npd; b += 32) csum_merge(tot, CSum{pd[2 * b], pd[2 * b + 1]});
-    for (int b = lane; b < npp; b += 32) csum_merge(tot, CSum{pp[2 * b], pp[2 * b + 1]});
-    tot = warp_csum(tot);
-    if (lane == 0) *e = __ddiv_rn(__dadd_rn(tot.s, tot.c), st->norm);
+    for (int b = threadIdx.x; b < npp; b += blockDim.x) csum_merge(tot, CSum{2.0 * pp[2 * b], 2.0 * pp[2 * b + 1]});
+    const int nent = n_orb * (2 * n_orb + 1);
+    for (int k = threadIdx.x; k < nent; k += blockDim.x) {
+        int q = (int)((sqrtf(8.0f * (float)k + 1.0f) - 1.0f) * 0.5f);
+        while (q * (q + 1) / 2 > k) --q;
+        while ((q + 1) * (q + 2) / 2 <= k) ++q;
+        const int p = k - q * (q + 1) / 2;
+        const double o = occ_pair[k];
+        const int P = p >> 1, Q = q >> 1;
+        double x;
+        if (p == q) {
+            x = __ldg(h + P * n_orb + P);
+        } else {
+            x = __ldg(eri + fq::eidx(P, P, Q, Q));
+            if ((p & 1) == (q & 1)) x = __dsub_rn(x, __ldg(eri + fq::eidx(P, Q, Q, P)));
+        }
+        csum_add(tot, __dmul_rn(o, x));
+    }
+    tot = block_csum(tot, s_red);
+    if (threadIdx.x == 0) *e = __ddiv_rn(__dadd_rn(tot.s, tot.c), st->norm);
 }
 
-__global__ void k_pair_wpair(Params P, double *wpair) {
-    const int M = P.n_orb;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < M * M; k += gridDim.x * blockDim.x) {
-        const int p = k / M, q = k % M;
-        const double j = fq::eri_d(P, p, p, q, q);
-        wpair[k] = j;
-        wpair[M * M + k] = __dsub_rn(j, fq::eri_d(P, p, q, q, p));
+// The two-body density matrix over pair codes: v v' of every pair of members added at (smaller code, larger code) with
+// one FP64 reduction in L2. Large groups walk a triangle, so a warp's reductions fall in one table row.
+__global__ void __launch_bounds__(kThreads) k_pair_grad(const Member *members, const unsigned *base_p, const unsigned *count_p,
+                                                        int parts, int n1, int n2, double *table) {
+    double *mixed = table + (size_t)n1 * n1;
+    for (int p = blockIdx.x; p < parts; p += gridDim.x) {
+        const Member *mem = members + base_p[p];
+        const int cnt = (int)count_p[p];
+        for (int j = threadIdx.x; j < cnt; j += kThreads) {
+            const Member u = mem[j];
+            const Member *grp = mem + u.first;
+            const RowRange r = row_range(u.code, j - (int)u.first);
+            const unsigned cls = (u.code >> 13) & 3u, cu = u.code & 0x1FFFu;
+            double *t = cls == 2u ? mixed : table;
+            const int stride = cls == 2u ? n2 : n1;
+            int at = r.at;
+#pragma unroll 4
+            for (int k = 0; k < r.n; ++k) {
+                const Member w = grp[at];
+                at = at + 1 == r.wrap ? 0 : at + 1;
+                const unsigned cw = w.code & 0x1FFFu;
+                if (((w.code >> 13) & 3u) == cls)
+                    atomicAdd(t + (size_t)min(cu, cw) * stride + max(cu, cw), __dmul_rn(u.v, w.v));
+            }
+        }
     }
 }
 
-// Gradient contributions of the connected pairs (atomics into the unscaled RDM arrays).
-template <int W>
-__global__ void __launch_bounds__(kThreads) k_pair_grad(int n_orb, const unsigned long long *dets, const double *c,
-                                                        long long nb, const unsigned long long *poff,
-                                                        const unsigned *pidx, const unsigned long long *moff,
-                                                        const unsigned long long *members, RdmState *st, double *gh,
-                                                        double *ge) {
-    __shared__ SingleQueue s_q[kThreads / 32];
-    SingleQueue &sq = s_q[threadIdx.x >> 5];
-    if ((threadIdx.x & 31) == 0) sq.n = 0;
-    __syncwarp();
-    const unsigned long long np = st->n_pairs;
-    unsigned long long ns = 0, ndb = 0;
-    auto add_single = [&](bool all) {
-        long long Id = 0, Jd = 0;
-        int i = 0, a = 0;
-        if (pop_single(sq, all, Id, Jd, i, a)) {
-            ++ns;
-            unsigned long long dI[W];
-            load_det<W>(dets, Id, dI);
-            const double cc = c[Id] * c[Jd];
-            const double sg = (fq::count_between<W>(dI, i, a) & 1) ? -cc : cc;
-            const int I = i >> 1, A = a >> 1;
-            atomicAdd(&gh[I * n_orb + A], sg);
-            atomicAdd(&gh[A * n_orb + I], sg);
-#pragma unroll
-            for (int w = 0; w < W; ++w) {
-                unsigned long long m = dI[w];
-                while (m) {
-                    const int j = 64 * w + __ffsll((long long)m) - 1;
-                    m &= m - 1;
-                    if (j == i) continue;
-                    const int J = j >> 1;
-                    atomicAdd(&ge[fq::eidx(I, A, J, J)], 2.0 * sg);
-                    if ((j & 1) == (i & 1)) atomicAdd(&ge[fq::eidx(I, J, J, A)], -2.0 * sg);
-                }
+// Maps the density matrix over pair codes (rows < columns) and the occupation-pair sums onto h and the packed ERIs.
+__global__ void __launch_bounds__(kThreads) k_fold(const double *table, const double *occ_pair, int n_orb, int n1, int n2, double inv,
+                                                   double *gh, double *ge) {
+    auto one_body = [&](int a, int b, double v) {  // both h[a][b] and h[b][a]
+        atomicAdd(&gh[a * n_orb + b], v);
+        atomicAdd(&gh[b * n_orb + a], v);
+    };
+    const int row = blockIdx.y;
+    if (row < n1) {
+        int p, q;
+        triangle_of(row, p, q);
+        for (int col = row + 1 + blockIdx.x * blockDim.x + threadIdx.x; col < n1; col += gridDim.x * blockDim.x) {
+            const double g = table[(size_t)row * n1 + col];
+            if (g == 0.0) continue;
+            int r, s;
+            triangle_of(col, r, s);
+            const double g1 = __dmul_rn(inv, g);
+            atomicAdd(&ge[fq::eidx(p, r, q, s)], 2.0 * g);
+            atomicAdd(&ge[fq::eidx(p, s, q, r)], -2.0 * g);
+            if (q == s) one_body(p, r, g1);
+            if (p == r) one_body(q, s, g1);
+            if (q == r) one_body(p, s, -g1);
+            if (p == s) one_body(q, r, -g1);
+        }
+    } else if (row < n1 + n2) {
+        const int row2 = row - n1, p = row2 / n_orb, q = row2 - p * n_orb;
+        for (int col = row2 + 1 + blockIdx.x * blockDim.x + threadIdx.x; col < n2; col += gridDim.x * blockDim.x) {
+            const double g = table[(size_t)n1 * n1 + (size_t)row2 * n2 + col];
+            if (g == 0.0) continue;
+            const int r = col / n_orb, s = col - r * n_orb;
+            const double g1 = __dmul_rn(inv, g);
+            atomicAdd(&ge[fq::eidx(p, r, q, s)], 2.0 * g);
+            if (q == s) one_body(p, r, g1);
+            if (p == r) one_body(q, s, g1);
+        }
+    } else if (blockIdx.x == 0) {  // spin orbital q: O_pq for p <= q
+        const int q = row - n1 - n2, Q = q >> 1;
+        for (int p = threadIdx.x; p <= q; p += blockDim.x) {
+            const double v = occ_pair[q * (q + 1) / 2 + p];
+            if (v == 0.0) continue;
+            const int P = p >> 1;
+            if (p == q) {
+                atomicAdd(&gh[P * n_orb + P], v);
+            } else {
+                atomicAdd(&ge[fq::eidx(P, P, Q, Q)], v);
+                if ((p & 1) == (q & 1)) atomicAdd(&ge[fq::eidx(P, Q, Q, P)], -v);
             }
+        }
+    }
+}
+
+// Connected pairs for fciqmc_rdm_info: pairs of members with one spin orbital in common (each single excitation
+// N - 1 times, once per shared key) and with none (the double excitations).
+__global__ void __launch_bounds__(kThreads) k_pair_count(const Member *members, const unsigned *base_p, const unsigned *count_p,
+                                                         int parts, int n_orb, RdmState *st) {
+    unsigned long long shared_n = 0, apart = 0;
+    auto orbitals = [&](unsigned code, int &x, int &y) {
+        const unsigned cls = (code >> 13) & 3u, c = code & 0x1FFFu;
+        if (cls == 2u) {
+            x = 2 * (int)(c / (unsigned)n_orb);
+            y = 2 * (int)(c % (unsigned)n_orb) + 1;
+        } else {
+            int p, q;
+            triangle_of((int)c, p, q);
+            x = 2 * p + (int)cls;
+            y = 2 * q + (int)cls;
         }
     };
-    // warp-uniform loop: lane k takes pair base + k
-    for (unsigned long long base = (unsigned long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < np;
-         base += (unsigned long long)gridDim.x * blockDim.x) {
-        const unsigned long long t = base + (threadIdx.x & 31);
-        PairInfo q{};
-        unsigned long long dI[W], dJ[W];
-        if (t < np) q = pair_of<W>(t, np, nb, poff, pidx, moff, members, dets, dI, dJ);
-        queue_single(sq, q.kind == 1, q);
-        add_single(false);
-        if (q.kind == 2) {
-            const double cc = c[q.I] * c[q.J];
-            ++ndb;
-            const double sg = fq::double_parity<W>(dI, q.i, q.j, q.a, q.b) ? -cc : cc;
-            if ((q.i & 1) == (q.a & 1) && (q.j & 1) == (q.b & 1))
-                atomicAdd(&ge[fq::eidx(q.i >> 1, q.a >> 1, q.j >> 1, q.b >> 1)], 2.0 * sg);
-            if ((q.i & 1) == (q.b & 1) && (q.j & 1) == (q.a & 1))
-                atomicAdd(&ge[fq::eidx(q.i >> 1, q.b >> 1, q.j >> 1, q.a >> 1)], -2.0 * sg);
-        }
-    }
-    add_single(true);  // fewer than 32 remain
-    if (ns) atomicAdd(&st->n_single, ns);
-    if (ndb) atomicAdd(&st->n_double, ndb);
-}
-
-// Diagonal contributions: occupation-pair sums O_pq = sum_I c_I^2 n_p n_q over spin orbitals p <= q
-// (p == q gives sum_I c_I^2 n_p). Each thread walks the occupied pairs of its determinants and adds c_I^2
-// into a block copy of the triangle in shared memory (index q (q + 1) / 2 + p), flushed once per block.
-// O is stored at p * n_so + q.
-template <int W>
-__global__ void __launch_bounds__(kThreads) k_diag_grad(int n_so, const unsigned long long *dets, const double *c,
-                                                        long long n, double *occ_pair) {
-    extern __shared__ double s_o[];
-    const int nent = n_so * (n_so + 1) / 2;
-    for (int k = threadIdx.x; k < nent; k += blockDim.x) s_o[k] = 0.0;
-    __syncthreads();
-    for (long long I = (long long)blockIdx.x * blockDim.x + threadIdx.x; I < n; I += (long long)gridDim.x * blockDim.x) {
-        unsigned long long d[W];
-        load_det<W>(dets, I, d);
-        const double c2 = c[I] * c[I];
-#pragma unroll
-        for (int wq = 0; wq < W; ++wq) {
-            unsigned long long mq = d[wq];
-            while (mq) {
-                const int q = 64 * wq + __ffsll((long long)mq) - 1;
-                mq &= mq - 1;
-                const int row = q * (q + 1) / 2;
-#pragma unroll
-                for (int wp = 0; wp <= wq; ++wp) {
-                    unsigned long long mp = d[wp];
-                    if (wp == wq) mp &= (q & 63) == 63 ? ~0ull : ((2ull << (q & 63)) - 1ull);  // p <= q
-                    while (mp) {
-                        const int p = 64 * wp + __ffsll((long long)mp) - 1;
-                        mp &= mp - 1;
-                        atomicAdd(&s_o[row + p], c2);
-                    }
-                }
+    for (int p = blockIdx.x; p < parts; p += gridDim.x) {
+        const Member *mem = members + base_p[p];
+        const int cnt = (int)count_p[p];
+        for (int j = threadIdx.x; j < cnt; j += kThreads) {
+            const Member u = mem[j];
+            int ux, uy;
+            orbitals(u.code, ux, uy);
+            for (int k = (int)u.first; k < j; ++k) {
+                int wx, wy;
+                orbitals(mem[k].code, wx, wy);
+                const int same = (ux == wx) + (ux == wy) + (uy == wx) + (uy == wy);
+                if (same == 1) ++shared_n;
+                else if (same == 0) ++apart;
             }
         }
     }
-    __syncthreads();
-    for (int k = threadIdx.x; k < nent; k += blockDim.x) {
-        const double v = s_o[k];
-        if (v != 0.0) {
-            int q = 0;
-            while ((q + 1) * (q + 2) / 2 <= k) ++q;
-            atomicAdd(&occ_pair[(k - q * (q + 1) / 2) * n_so + q], v);
-        }
+    for (int o = 16; o > 0; o >>= 1) {
+        shared_n += __shfl_down_sync(0xFFFFFFFFu, shared_n, o);
+        apart += __shfl_down_sync(0xFFFFFFFFu, apart, o);
     }
-}
-
-// Maps the occupation-pair sums onto h and the packed ERIs and scales the whole RDM by 1 / c^T c.
-__global__ void k_diag_finish(int n_orb, const double *occ_pair, double *gh, double *ge, const RdmState *st) {
-    if (blockIdx.x != 0) return;
-    const int n_so = 2 * n_orb;
-    for (int e = threadIdx.x; e < n_so * n_so; e += blockDim.x) {
-        const int p = e / n_so, q = e % n_so;
-        if (q < p) continue;
-        const double v = occ_pair[e];
-        if (v == 0.0) continue;
-        const int P = p >> 1, Q = q >> 1;
-        if (p == q) {
-            atomicAdd(&gh[P * n_orb + P], v);
-        } else {
-            atomicAdd(&ge[fq::eidx(P, P, Q, Q)], v);
-            if ((p & 1) == (q & 1)) atomicAdd(&ge[fq::eidx(P, Q, Q, P)], -v);
-        }
+    if ((threadIdx.x & 31) == 0) {
+        if (shared_n) atomicAdd(&st->n_shared, shared_n);
+        if (apart) atomicAdd(&st->n_apart, apart);
     }
 }
 
@@ -754,117 +1159,97 @@ struct fciqmc_rdm {
     RdmLayout L;
     char *ws;
     cudaStream_t s;
-    int grid;
-    int sms;
-    long long nb;  // buckets (host copy after construction)
-    bool pidx_ok;  // the coarse index of the bucket search is built (in the member-cursor buffer)
     RdmState host;
     bool rdm_ready;  // unscaled density matrices computed
 };
 
 namespace {
 template <typename T>
-T *ptr(fciqmc_rdm *r, size_t off) {
+T *ptr(const fciqmc_rdm *r, size_t off) {
     return reinterpret_cast<T *>(r->ws + off);
 }
-Params params_for(fciqmc_rdm *r, const double *h, const double *eri) {
-    Params P{};
-    P.n_elec = r->d.n_elec;
-    P.n_orb = r->d.n_orb;
-    P.n_so = 2 * r->d.n_orb;
-    P.h = h;
-    P.eri = eri;
-    P.wpair = ptr<double>(r, r->L.wpair);
-    return P;
+
+// Warps of a k_occ_pairs block: as many copies of the occupation triangle as fit in 208 KB, at most eight.
+int occ_warps(const Dims &d) {
+    const size_t nent = (size_t)d.n_so * (d.n_so + 1) / 2;
+    return (int)std::max<size_t>(1, std::min<size_t>(8, (208u << 10) / (sizeof(double) * nent)));
 }
 
 template <int W>
 int construct(fciqmc_rdm *r) {
     const Dims &d = r->d;
     cudaStream_t s = r->s;
-    const int stride = W == 1 ? 2 : 4;
-    const int g = r->grid;
     RdmState *st = ptr<RdmState>(r, r->L.state);
-    unsigned long long *tab = ptr<unsigned long long>(r, r->L.keys);
-    (void)stride;
-    k_key_init<<<g, kThreads, 0, s>>>(tab, d.kcap, W);
+    const unsigned long long *dets = ptr<unsigned long long>(r, r->L.dets);
+    const double *c = ptr<double>(r, r->L.c);
+    unsigned *total = ptr<unsigned>(r, r->L.total_p), *base = ptr<unsigned>(r, r->L.base_p);
+    unsigned *cursor = ptr<unsigned>(r, r->L.cursor_p), *coarse = ptr<unsigned>(r, r->L.coarse_p);
+    unsigned long long *records = ptr<unsigned long long>(r, r->L.records);
+    const size_t sm_hist = sizeof(unsigned) * d.parts, sm_group = sizeof(GroupShared<W>);
+    const size_t sm_scatter = sizeof(ScatterShared);
+    const size_t nent = (size_t)d.n_so * (d.n_so + 1) / 2, sm_occ = sizeof(double) * nent * occ_warps(d);
+    if (cudaFuncSetAttribute(k_key_hist<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(unsigned) * kPartMax)) != cudaSuccess ||
+        cudaFuncSetAttribute(k_key_scatter<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_scatter) != cudaSuccess ||
+        cudaFuncSetAttribute(k_group<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_group) != cudaSuccess ||
+        cudaFuncSetAttribute(k_occ_pairs<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 << 10) != cudaSuccess)
+        return FCIQMC_ERR_CUDA;
     cudaMemsetAsync(st, 0, sizeof(RdmState), s);
-    k_keys<W><<<g, kThreads, 0, s>>>(ptr<unsigned long long>(r, r->L.dets), d.n, d.n_elec, tab, d.kcap, log2i(d.kcap), st);
-    if (cudaMemcpyAsync(&r->host, st, sizeof(RdmState), cudaMemcpyDeviceToHost, s) != cudaSuccess) return FCIQMC_ERR_CUDA;
-    if (cudaStreamSynchronize(s) != cudaSuccess) return FCIQMC_ERR_CUDA;
-    if (r->host.status) return r->host.status;
-    const long long nb = (long long)r->host.n_buckets;
-    r->nb = nb;
-    unsigned *counts = ptr<unsigned>(r, r->L.counts);
-    k_counts<W><<<g, kThreads, 0, s>>>(tab, d.kcap, counts);
-    const int nblk = (int)std::min<long long>(kMaxGrid, std::max<long long>(1, (nb + 4095) / 4096));
-    const long long per_block = (nb + nblk - 1) / nblk;
-    unsigned long long *bsum = ptr<unsigned long long>(r, r->L.bsum);
-    unsigned long long *moff = ptr<unsigned long long>(r, r->L.moff), *poff = ptr<unsigned long long>(r, r->L.poff);
-    k_scan_blocks<<<nblk, kThreads, 0, s>>>(counts, nb, per_block, bsum);
-    k_scan_top<<<1, 32, 0, s>>>(bsum, nblk, st);
-    k_scan_out<<<nblk, 32, 0, s>>>(counts, nb, per_block, bsum, moff, poff, st);
-    unsigned *cursor = ptr<unsigned>(r, r->L.cursor);
-    cudaMemsetAsync(cursor, 0, sizeof(unsigned) * nb, s);
-    unsigned long long *members = ptr<unsigned long long>(r, r->L.members);
-    k_members<W><<<g, kThreads, 0, s>>>(ptr<unsigned long long>(r, r->L.dets), d.n, d.n_elec, tab, d.kcap, log2i(d.kcap),
-                                        counts, cursor, moff, members);
-    k_sort_members<<<g, kThreads, 0, s>>>(nb, counts, moff, members);
-    double *partial = ptr<double>(r, r->L.partial);
-    k_norm<<<g, kThreads, 0, s>>>(ptr<double>(r, r->L.c), d.n, partial);
-    k_sum_partials<<<1, 32, 0, s>>>(partial, g, &st->norm);
+    cudaMemsetAsync(total, 0, sizeof(unsigned) * d.parts, s);
+    k_key_hist<W><<<d.hash_blocks, kHashThreads, sm_hist, s>>>(dets, d.n, d.n_elec, d.parts, d.pbits, total);
+    const int fine = d.parts > kBins ? kFineBits : 0, cbits = d.pbits - fine;  // bits of the two scatter passes
+    k_part_scan<<<1, 1024, 0, s>>>(total, d.parts, fine, base, cursor, coarse);
+    const long long per = std::max(1, kTileKeys / d.npairs);
+    const int gs = (int)std::min<long long>(2 * kSms, (d.n + per - 1) / per);
+    // with two passes the first one's records lie where the members will be written last
+    unsigned long long *first = fine ? reinterpret_cast<unsigned long long *>(ptr<Member>(r, r->L.members)) : records;
+    k_key_scatter<W><<<gs, kHashThreads, sm_scatter, s>>>(dets, d.n, d.n_elec, cbits, d.tbits, coarse, first);
+    if (fine) {
+        const long long tiles = ((d.n_keys >> cbits) + 4095) / 4096;  // of an average coarse bin
+        k_refine<<<dim3((unsigned)std::min<long long>(tiles + 1, 1024), 1u << cbits), kHashThreads, 0, s>>>(first, d.tbits, base, cursor, records);
+    }
+    k_group<W><<<d.parts, kGroupThreads, sm_group, s>>>(dets, c, d.n_elec, d.n_orb, d.tbits, records, base, ptr<Member>(r, r->L.members),
+                                                        ptr<unsigned>(r, r->L.count_p), st);
+    double *norm_part = ptr<double>(r, r->L.partial) + 2 * kPairGrid;
+    const int nw = occ_warps(d);
+    const int go = (int)std::min<long long>(kSms, (d.n + nw - 1) / nw), gn = (int)std::min<long long>(kNormGrid, (d.n + kThreads - 1) / kThreads);
+    k_norm<<<gn, kThreads, 0, s>>>(c, d.n, norm_part);
+    k_occ_pairs<W><<<go, 32 * nw, sm_occ, s>>>(dets, c, d.n, d.n_elec, d.n_so, ptr<double>(r, r->L.occ_part));
+    k_occ_merge<<<(unsigned)((nent + kMergeThreads - 1) / kMergeThreads) + 1, kMergeThreads, 0, s>>>(
+        ptr<double>(r, r->L.occ_part), go, (int)nent, ptr<double>(r, r->L.occ_pair), norm_part, gn, st);
     if (cudaGetLastError() != cudaSuccess) return FCIQMC_ERR_CUDA;
     if (cudaMemcpyAsync(&r->host, st, sizeof(RdmState), cudaMemcpyDeviceToHost, s) != cudaSuccess) return FCIQMC_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return FCIQMC_ERR_CUDA;
-    // coarse index of the bucket search, in the member cursors (no longer needed)
-    r->pidx_ok = r->host.status == 0 && nb > 0 &&
-                 (long long)(r->host.n_pairs >> kPairIndexShift) + 2 <= d.n_keys;
-    if (r->pidx_ok) {
-        k_pair_index<<<g, kThreads, 0, s>>>(poff, nb, st, cursor);
-        if (cudaGetLastError() != cudaSuccess) return FCIQMC_ERR_CUDA;
-    }
     return r->host.status;
 }
 
-template <int W>
-void launch_energy(fciqmc_rdm *r, const Params &P, double *e) {
+dim3 table_grid(const Dims &d, int extra_rows) {
+    return dim3((unsigned)std::max(1, (std::max(d.n1, d.n2) + 4 * kThreads - 1) / (4 * kThreads)), (unsigned)(d.n1 + d.n2 + extra_rows));
+}
+int pair_grid(const Dims &d) { return std::min(kPairGrid, d.parts); }
+
+void launch_energy(fciqmc_rdm *r, const double *h, const double *eri, double *e) {
     const Dims &d = r->d;
     cudaStream_t s = r->s;
-    const int g = r->grid;
-    RdmState *st = ptr<RdmState>(r, r->L.state);
-    double *partial = ptr<double>(r, r->L.partial);
-    const int gd = std::min(g, kMaxGrid / 2);
-    const size_t smem = sizeof(double) * (2 * d.n_orb * d.n_orb + d.n_orb);
-    k_pair_wpair<<<8, kThreads, 0, s>>>(P, const_cast<double *>(P.wpair));
-    k_diag_energy<W><<<gd, kThreads, smem, s>>>(P, ptr<unsigned long long>(r, r->L.dets), ptr<double>(r, r->L.c), d.n,
-                                                partial);
-    const unsigned *pidx = r->pidx_ok ? ptr<unsigned>(r, r->L.cursor) : nullptr;
-    k_pair_energy<W><<<gd, kThreads, 0, s>>>(P, ptr<unsigned long long>(r, r->L.dets), ptr<double>(r, r->L.c), r->nb,
-                                             ptr<unsigned long long>(r, r->L.poff), pidx,
-                                             ptr<unsigned long long>(r, r->L.moff),
-                                             ptr<unsigned long long>(r, r->L.members), st, partial + 2 * gd);
-    k_energy_finish<<<1, 32, 0, s>>>(partial + 2 * gd, gd, partial, gd, st, e);
+    const RdmState *st = ptr<RdmState>(r, r->L.state);
+    double *partial = ptr<double>(r, r->L.partial), *table = ptr<double>(r, r->L.table);
+    const int g = pair_grid(d);
+    k_pair_table<<<table_grid(d, 0), kThreads, 0, s>>>(h, eri, d.n_orb, d.n1, d.n2, 1.0 / (d.n_elec - 1), table);
+    k_pair_energy<<<g, kThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p), ptr<unsigned>(r, r->L.count_p),
+                                         d.parts, d.n1, d.n2, table, partial);
+    k_energy_finish<<<1, 1024, 0, s>>>(partial, g, ptr<double>(r, r->L.occ_pair), h, eri, d.n_orb, st, e);
 }
 
-template <int W>
 void launch_rdm(fciqmc_rdm *r) {
     const Dims &d = r->d;
     cudaStream_t s = r->s;
-    const int g = r->grid;
-    RdmState *st = ptr<RdmState>(r, r->L.state);
-    double *gh = ptr<double>(r, r->L.gh), *ge = ptr<double>(r, r->L.ge);
-    double *occ_pair = ptr<double>(r, r->L.npair_tab);
+    double *gh = ptr<double>(r, r->L.gh), *ge = ptr<double>(r, r->L.ge), *table = ptr<double>(r, r->L.table);
     cudaMemsetAsync(gh, 0, sizeof(double) * d.n_orb * d.n_orb, s);
     cudaMemsetAsync(ge, 0, sizeof(double) * d.n_eri, s);
-    cudaMemsetAsync(occ_pair, 0, sizeof(double) * 4 * d.n_orb * d.n_orb, s);
-    const unsigned *pidx = r->pidx_ok ? ptr<unsigned>(r, r->L.cursor) : nullptr;
-    k_pair_grad<W><<<g, kThreads, 0, s>>>(d.n_orb, ptr<unsigned long long>(r, r->L.dets), ptr<double>(r, r->L.c), r->nb,
-                                          ptr<unsigned long long>(r, r->L.poff), pidx, ptr<unsigned long long>(r, r->L.moff),
-                                          ptr<unsigned long long>(r, r->L.members), st, gh, ge);
-    k_diag_grad<W><<<std::min<long long>(g, (d.n + kThreads - 1) / kThreads), kThreads,
-                     sizeof(double) * d.n_orb * (2 * d.n_orb + 1), s>>>(
-        2 * d.n_orb, ptr<unsigned long long>(r, r->L.dets), ptr<double>(r, r->L.c), d.n, occ_pair);
-    k_diag_finish<<<1, kThreads, 0, s>>>(d.n_orb, occ_pair, gh, ge, st);
+    cudaMemsetAsync(table, 0, sizeof(double) * ((size_t)d.n1 * d.n1 + (size_t)d.n2 * d.n2), s);
+    k_pair_grad<<<pair_grid(d), kThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p),
+                                                  ptr<unsigned>(r, r->L.count_p), d.parts, d.n1, d.n2, table);
+    k_fold<<<table_grid(d, d.n_so), kThreads, 0, s>>>(table, ptr<double>(r, r->L.occ_pair), d.n_orb, d.n1, d.n2,
+                                                      1.0 / (d.n_elec - 1), gh, ge);
 }
 }  // namespace
 
@@ -892,21 +1277,6 @@ int fciqmc_rdm_create(int n_elec, int n_orb, const uint64_t *dets_dev, const dou
     r->L = L;
     r->ws = static_cast<char *>(workspace);
     r->s = static_cast<cudaStream_t>(cuda_stream);
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&r->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-        delete r;
-        return FCIQMC_ERR_CUDA;
-    }
-    r->grid = std::min(kMaxGrid, r->sms * 8);
-    const size_t smem = sizeof(double) * (2 * d.n_orb * d.n_orb + d.n_orb);
-    const size_t smem_o = sizeof(double) * d.n_orb * (2 * d.n_orb + 1);  // occupation-pair triangle
-    if (cudaFuncSetAttribute(k_diag_energy<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaFuncSetAttribute(k_diag_energy<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaFuncSetAttribute(k_diag_grad<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_o) != cudaSuccess ||
-        cudaFuncSetAttribute(k_diag_grad<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_o) != cudaSuccess) {
-        delete r;
-        return FCIQMC_ERR_CUDA;
-    }
     if (cudaMemcpyAsync(ptr<unsigned long long>(r, L.dets), dets_dev, sizeof(uint64_t) * d.W * d.n, cudaMemcpyDeviceToDevice, r->s) != cudaSuccess ||
         cudaMemcpyAsync(ptr<double>(r, L.c), c_dev, sizeof(double) * d.n, cudaMemcpyDeviceToDevice, r->s) != cudaSuccess) {
         delete r;
@@ -923,37 +1293,40 @@ int fciqmc_rdm_create(int n_elec, int n_orb, const uint64_t *dets_dev, const dou
 
 int fciqmc_rdm_energy(fciqmc_rdm *r, const double *h_dev, const double *eri_dev, double *e_dev) {
     if (!r || !h_dev || !eri_dev || !e_dev) return FCIQMC_ERR_INVALID_ARG;
-    Params P = params_for(r, h_dev, eri_dev);
-    if (r->d.W == 1) launch_energy<1>(r, P, e_dev);
-    else launch_energy<2>(r, P, e_dev);
+    launch_energy(r, h_dev, eri_dev, e_dev);
     return cudaGetLastError() == cudaSuccess ? FCIQMC_OK : FCIQMC_ERR_CUDA;
 }
 
 int fciqmc_rdm_gradient(fciqmc_rdm *r, const double *scale_dev, double *grad_h_dev, double *grad_eri_dev) {
     if (!r || !scale_dev || !grad_h_dev || !grad_eri_dev) return FCIQMC_ERR_INVALID_ARG;
-    RdmState *st = ptr<RdmState>(r, r->L.state);
     if (!r->rdm_ready) {
-        if (r->d.W == 1) launch_rdm<1>(r);
-        else launch_rdm<2>(r);
+        launch_rdm(r);
         r->rdm_ready = true;
     }
     const long long nh = (long long)r->d.n_orb * r->d.n_orb;
-    k_scale_out<<<std::min(r->grid, 1024), kThreads, 0, r->s>>>(ptr<double>(r, r->L.gh), ptr<double>(r, r->L.ge), nh,
-                                                                r->d.n_eri, scale_dev, st, grad_h_dev, grad_eri_dev);
+    const int g = (int)std::min<long long>(kSms * 4, (nh + r->d.n_eri + kThreads - 1) / kThreads);
+    k_scale_out<<<g, kThreads, 0, r->s>>>(ptr<double>(r, r->L.gh), ptr<double>(r, r->L.ge), nh, r->d.n_eri, scale_dev,
+                                          ptr<RdmState>(r, r->L.state), grad_h_dev, grad_eri_dev);
     return cudaGetLastError() == cudaSuccess ? FCIQMC_OK : FCIQMC_ERR_CUDA;
 }
 
 int fciqmc_rdm_info(fciqmc_rdm *r, int64_t *counts) {
     if (!r || !counts) return FCIQMC_ERR_INVALID_ARG;
+    RdmState *st = ptr<RdmState>(r, r->L.state);
     RdmState h;
-    if (cudaMemcpyAsync(&h, ptr<RdmState>(r, r->L.state), sizeof(RdmState), cudaMemcpyDeviceToHost, r->s) != cudaSuccess ||
+    if (r->rdm_ready) {
+        if (cudaMemsetAsync(&st->n_shared, 0, 2 * sizeof(unsigned long long), r->s) != cudaSuccess) return FCIQMC_ERR_CUDA;
+        k_pair_count<<<pair_grid(r->d), kThreads, 0, r->s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p),
+                                                            ptr<unsigned>(r, r->L.count_p), r->d.parts, r->d.n_orb, st);
+    }
+    if (cudaMemcpyAsync(&h, st, sizeof(RdmState), cudaMemcpyDeviceToHost, r->s) != cudaSuccess ||
         cudaStreamSynchronize(r->s) != cudaSuccess)
         return FCIQMC_ERR_CUDA;
     counts[0] = (int64_t)h.n_buckets;
     counts[1] = (int64_t)h.n_members;
     counts[2] = (int64_t)h.n_pairs;
-    counts[3] = (int64_t)h.n_single;
-    counts[4] = (int64_t)h.n_double;
+    counts[3] = (int64_t)(h.n_shared / (unsigned long long)(r->d.n_elec - 1));
+    counts[4] = (int64_t)h.n_apart;
     return h.status;
 }
 

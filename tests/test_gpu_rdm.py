@@ -153,3 +153,56 @@ def test_full_size_million_determinants():
         fd = (float(f.energy(h0, v0 + d)) - float(f.energy(h0, v0 - d))) / (2 * eps)
         assert abs(fd - gen[k]) < 1e-8
     f.close()
+
+
+def _some_pairs(n_orb, n_elec, n, seed, sz=None):
+    """n distinct determinants of n_elec electrons, all spins mixed (or n_alpha - n_beta = sz)."""
+    rng = np.random.default_rng(seed)
+    out = set()
+    while len(out) < n:
+        if sz is None:
+            occ = rng.choice(2 * n_orb, n_elec, replace=False)
+        else:
+            na = (n_elec + sz) // 2
+            occ = np.concatenate([2 * rng.choice(n_orb, na, replace=False), 2 * rng.choice(n_orb, n_elec - na, replace=False) + 1])
+        out.add(sum(1 << int(k) for k in occ))
+    return sorted(out)
+
+
+def _grouping_cases():
+    # two electrons share one key: whole lists in one group, below and above the records a block groups at a time,
+    # and just around the size from which groups are walked as a triangle
+    for n in (2, 3, 47, 48, 49, 700):
+        yield f"2e-{n}", 20, 2, _some_pairs(20, 2, n, n)
+    yield "2e-whole-52-orbitals", 52, 2, [(1 << a) | (1 << b) for a in range(104) for b in range(a)]
+    # one key of 5,151 determinants beside keys of a hundred: an oversized partition taken in parts
+    yield "3e-one-orbital-common", 52, 3, [1 | (1 << a) | (1 << b) for a in range(1, 103) for b in range(1, a)]
+    # one word, all spins, the whole space; two words, many electrons, odd counts
+    yield "3e-5o-whole", 5, 3, [d for d in range(1 << 10) if bin(d).count("1") == 3]
+    yield "33e-40o", 40, 33, _some_pairs(40, 33, 40, 1, 1)
+    yield "64e-64o-near", 64, 64, sorted({((1 << 64) - 1) ^ (1 << i) ^ (1 << (64 + a)) for i in range(0, 64, 9) for a in range(0, 64, 9)})
+
+
+@pytest.mark.parametrize("case", list(_grouping_cases()), ids=lambda c: c[0])
+def test_grouping_edges_match_oracle(case):
+    """E and both density matrices at the sizes where the grouping changes its path, against the oracle's density
+    matrices (built from operators, so lists of several S_z are right as well) and the energy they give. Every term
+    is a product of two amplitudes of a unit vector and one integral: 64-bit sums of up to 1e7 terms in another order
+    agree well within 1e7^(1/2) 2^-53 = 4e-13 of the largest term."""
+    _, n_orb, n_elec, ints = case
+    s = synth.make_system(n_orb, n_elec, seed=n_orb + n_elec, n_chol=8, fock_diagonal=False)
+    W = (2 * n_orb + 63) // 64
+    dets = np.array([bf.to_words(d, W) for d in ints], dtype=np.uint64)
+    c = np.random.default_rng(len(ints)).normal(size=len(ints))
+    c /= np.linalg.norm(c)
+    f = _functional(s, dets, c)
+    E = float(f.energy(_dev(s.h), _dev(s.eri_s8)))
+    gh, ge = f.gradient(torch.ones((), dtype=torch.float64, device="cuda"))
+    _, ghq, geq = Oracle(s, tau=0.01, ms2=n_elec % 2).rdm_energy(dets, c)
+    Eq = float((s.h * ghq).sum() + (s.eri_s8 * geq).sum())
+    assert abs(E - Eq) <= 1e-12 * max(1.0, abs(Eq))
+    assert np.abs(gh.cpu().numpy() - ghq).max() < 1e-12 and np.abs(ge.cpu().numpy() - geq).max() < 1e-12
+    info = f.info()
+    if len(ints) <= 1000:  # connected or not: the counts are of pairs one and two spin orbitals apart
+        assert (info["single_pairs"], info["double_pairs"]) == _count_pairs(dets)
+    f.close()
