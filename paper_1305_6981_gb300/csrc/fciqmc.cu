@@ -184,7 +184,7 @@ struct fciqmc_handle {
     cudaStream_t stream;
     fciqmc_info info;
     int sweep_grid, heavy_grid, ann_grid, diag_grid, small_grid;
-    size_t smem_w;
+    size_t smem_w, smem_d;   // dynamic shared memory: pair terms; pair terms and occupied lists
     double e_core;
     cudaGraph_t graph_tmpl;  // one iteration, kept for composing batch graphs
     cudaGraphExec_t graph;
@@ -206,9 +206,11 @@ T *at(fciqmc_handle *h, size_t off) {
 
 template <int W>
 int configure_kernels(fciqmc_handle *h) {
-    FQ_CUDA(cudaFuncSetAttribute(fq::k_new_diag<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem_w));
-    FQ_CUDA(cudaFuncSetAttribute(fq::k_prepare_list<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem_w));
-    FQ_CUDA(cudaFuncSetAttribute(fq::k_reference_energy<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem_w));
+    // the largest basis's sizes: the attribute belongs to the kernel, not to one run
+    constexpr int kMostDiag = (int)fq::diag_bytes(64, fq::MAXN);
+    FQ_CUDA(cudaFuncSetAttribute(fq::k_new_diag<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostDiag));
+    FQ_CUDA(cudaFuncSetAttribute(fq::k_prepare_list<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostDiag));
+    FQ_CUDA(cudaFuncSetAttribute(fq::k_reference_energy<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostDiag));
     int dev = 0, sms = 0, per_sm = 0;
     FQ_CUDA(cudaGetDevice(&dev));
     FQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -219,7 +221,7 @@ int configure_kernels(fciqmc_handle *h) {
     // k_new_diag: as many blocks as fit at once (one new slot per thread up to that many; each thread's H_ii
     // is a long chain of dependent FP64 adds, so more resident warps hide its latency; blocks with no new
     // slot return before loading the pair terms)
-    FQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fq::k_new_diag<W>, 256, h->smem_w));
+    FQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fq::k_new_diag<W>, fq::kDiagThreads, h->smem_d));
     h->diag_grid = std::min(kMaxGrid, std::max(1, sms * std::max(per_sm, 1)));
     h->heavy_grid = std::min(kMaxGrid, sms * 4);
     if (h->grid_request > 0) {
@@ -270,7 +272,7 @@ void enqueue_iteration(fciqmc_handle *h, cudaStream_t s) {
     fq::k_compact_finish<<<1, 32, 0, s>>>(P);
     launch_spawning<W>(h, s);
     fq::k_annihilate<W><<<h->ann_grid, 256, 0, s>>>(P);
-    fq::k_new_diag<W><<<h->diag_grid, 256, h->smem_w, s>>>(P);
+    fq::k_new_diag<W><<<h->diag_grid, fq::kDiagThreads, h->smem_d, s>>>(P);
     if (P.occ_units > 1) fq::k_round<W><<<h->small_grid, 256, 0, s>>>(P);
     fq::k_finish<<<1, 32, 0, s>>>(P);
 }
@@ -306,9 +308,9 @@ void launch_index_rebuild(fciqmc_handle *h) {
 
 template <int W>
 void launch_prepare(fciqmc_handle *h, int b, long long n, int compute) {  // slots [0, n)
-    long long blocks = std::min<long long>((n + 255) / 256, h->small_grid);
+    long long blocks = std::min<long long>((n + fq::kDiagThreads - 1) / fq::kDiagThreads, h->small_grid);
     if (blocks < 1) blocks = 1;
-    fq::k_prepare_list<W><<<(unsigned)blocks, 256, h->smem_w, h->stream>>>(h->P, b, 0, n, compute);
+    fq::k_prepare_list<W><<<(unsigned)blocks, fq::kDiagThreads, h->smem_d, h->stream>>>(h->P, b, 0, n, compute);
 }
 
 // The helper streams of set_walkers and their events, created together (nothing is kept if one fails).
@@ -368,9 +370,10 @@ int load_stage(fciqmc_handle *h, const DevState &cur, const uint64_t *dets, cons
             FQ_CUDA(cudaStreamWaitEvent(a, h->ev_chunk[k], 0));
             const unsigned ib = (unsigned)std::max<long long>(1, std::min<long long>((hi - lo + 255) / 256, h->small_grid));
             fq::k_index_insert<W><<<ib, 256, 0, a>>>(P, b, lo, hi);
+            const unsigned pb = (unsigned)std::max<long long>(1, std::min<long long>((hi - lo + fq::kDiagThreads - 1) / fq::kDiagThreads, 2ll * h->small_grid));
             // the chunk's derived words on the second helper stream, beside the index work
             FQ_CUDA(cudaStreamWaitEvent(h->aux2, h->ev_chunk[k], 0));
-            fq::k_prepare_list<W><<<ib, 256, 0, h->aux2>>>(P, b, lo, hi, 0);
+            fq::k_prepare_list<W><<<pb, fq::kDiagThreads, (size_t)fq::kDiagThreads * P.ostride, h->aux2>>>(P, b, lo, hi, 0);
         }
     }
     FQ_CUDA(cudaGetLastError());
@@ -535,6 +538,7 @@ int fciqmc_create(const double *h1, const double *eri_s8, double e_core, int n_e
     h->graph_tmpl = nullptr;
     h->grid_request = o.grid_blocks;
     h->smem_w = sizeof(double) * (2 * n_orb * n_orb + n_orb);
+    h->smem_d = fq::diag_bytes(n_orb, z.ostride);
     h->opt = o;
     h->tau = tau;
     h->init_thr = initiator_threshold < 0 ? -1 : initiator_threshold;
@@ -849,7 +853,7 @@ int fciqmc_profile(fciqmc_handle *h, int32_t n_iterations, double *kernel_ms) {
                     case 5: launch_heavy<1>(h, s); break;
                     case 6:
                         fq::k_annihilate<1><<<h->ann_grid, 256, 0, s>>>(P);
-                        fq::k_new_diag<1><<<h->diag_grid, 256, h->smem_w, s>>>(P);
+                        fq::k_new_diag<1><<<h->diag_grid, fq::kDiagThreads, h->smem_d, s>>>(P);
                         if (P.occ_units > 1) fq::k_round<1><<<h->small_grid, 256, 0, s>>>(P);
                         break;
                     default: fq::k_finish<<<1, 32, 0, s>>>(P); break;
@@ -871,7 +875,7 @@ int fciqmc_profile(fciqmc_handle *h, int32_t n_iterations, double *kernel_ms) {
                     case 5: launch_heavy<2>(h, s); break;
                     case 6:
                         fq::k_annihilate<2><<<h->ann_grid, 256, 0, s>>>(P);
-                        fq::k_new_diag<2><<<h->diag_grid, 256, h->smem_w, s>>>(P);
+                        fq::k_new_diag<2><<<h->diag_grid, fq::kDiagThreads, h->smem_d, s>>>(P);
                         if (P.occ_units > 1) fq::k_round<2><<<h->small_grid, 256, 0, s>>>(P);
                         break;
                     default: fq::k_finish<<<1, 32, 0, s>>>(P); break;
@@ -1247,7 +1251,7 @@ void enqueue_group_iteration(fciqmc_group *g, cudaStream_t s) {
     for (fciqmc_handle *h : g->parts) fq::k_receive<W><<<h->ann_grid, 256, 0, s>>>(h->P, g->links);
     for (fciqmc_handle *h : g->parts) {
         fq::k_annihilate<W><<<h->ann_grid, 256, 0, s>>>(h->P);
-        fq::k_new_diag<W><<<h->diag_grid, 256, h->smem_w, s>>>(h->P);
+        fq::k_new_diag<W><<<h->diag_grid, fq::kDiagThreads, h->smem_d, s>>>(h->P);
         if (h->P.occ_units > 1) fq::k_round<W><<<h->small_grid, 256, 0, s>>>(h->P);
     }
     const Params &P0 = g->parts[0]->P;

@@ -121,11 +121,38 @@ __global__ void __launch_bounds__(256) k_annihilate(Params P) {
     flush_counters<256, 4>(accv, dst, s_red);
 }
 
-// H_ii - E0 (and its nearest float) of the slots placed by k_annihilate this iteration, one per thread in
-// the FP64 order of hdiag / hphf_hdiag, with the pair terms in shared memory.
+// Threads of the kernels that evaluate diagonal elements, and their dynamic shared memory: the pair terms and h_pp, then
+// one occupied list per thread. H_ii is a chain of N + N (N - 1) / 2 dependent FP64 additions (its order is fixed),
+// and an SM issues one FP64 warp instruction in about 20 clocks, so a few hundred new slots finish soonest when spread
+// over as many SMs as possible: four warps a block, one per scheduler.
+constexpr int kDiagThreads = 128;
+__host__ __device__ constexpr size_t diag_bytes(int n_orb, int ostride) {
+    return sizeof(double) * ((size_t)2 * n_orb * n_orb + n_orb) + (size_t)kDiagThreads * ostride;
+}
+// Copies the pair terms and h_pp to shared memory (16 bytes at a time); returns the thread's occupied list.
+__device__ __forceinline__ unsigned char *load_diag_tables(const Params &P, double *s_w) {
+    const int M = P.n_orb;
+    const double2 *src = reinterpret_cast<const double2 *>(P.wpair);
+    double2 *dst = reinterpret_cast<double2 *>(s_w);
+#pragma unroll 4
+    for (int k = threadIdx.x; k < M * M; k += blockDim.x) dst[k] = src[k];
+    for (int k = threadIdx.x; k < M; k += blockDim.x) s_w[2 * M * M + k] = P.h[k * M + k];
+    return reinterpret_cast<unsigned char *>(s_w + 2 * M * M + M) + threadIdx.x * P.ostride;
+}
+// H_ii - E0 of a determinant with its occupied list.
 template <int W>
-__global__ void __launch_bounds__(256) k_new_diag(Params P) {
-    extern __shared__ double s_w[];  // [2][M][M] pair terms, then M diagonal h_pp
+__device__ __forceinline__ double diag_element(const Params &P, const unsigned long long (&d)[W], const unsigned char *occ, const double *s_w) {
+    const int M = P.n_orb;
+    double v = hdiag_occ(P.n_elec, M, occ, s_w, s_w + 2 * M * M);
+    if (P.hphf) v = hphf_hdiag<W>(P, d, v);
+    return __dsub_rn(v, P.E0);
+}
+
+// H_ii - E0 (and its nearest float) and the derived data of the slots placed by k_annihilate this iteration, one per
+// thread in the FP64 order of hdiag / hphf_hdiag, with the pair terms in shared memory.
+template <int W>
+__global__ void __launch_bounds__(kDiagThreads) k_new_diag(Params P) {
+    extern __shared__ __align__(16) double s_w[];
     DevState *st = P.st;
     if (st->status) return;
     const long long n = (long long)st->n_new;
@@ -133,8 +160,7 @@ __global__ void __launch_bounds__(256) k_new_diag(Params P) {
     const int M = P.n_orb;
     __shared__ Tables T;
     load_tables(P, T);
-    for (int k = threadIdx.x; k < 2 * M * M; k += blockDim.x) s_w[k] = P.wpair[k];
-    for (int k = threadIdx.x; k < M; k += blockDim.x) s_w[2 * M * M + k] = P.h[k * M + k];
+    unsigned char *occ = load_diag_tables(P, s_w);
     __syncthreads();
     const int lb = st->lb, pp = st->pp;
     const int *new_slots = P.pop[lb][pp];
@@ -143,11 +169,10 @@ __global__ void __launch_bounds__(256) k_new_diag(Params P) {
         unsigned long long key[W];
 #pragma unroll
         for (int w = 0; w < W; ++w) key[w] = P.det[lb][s * W + w];
-        const double v = P.hphf ? hphf_hdiag<W>(P, key, s_w, s_w + 2 * M * M) : hdiag<W>(P, key, s_w, s_w + 2 * M * M);
-        const double hdv = __dsub_rn(v, P.E0);
+        store_derived<W>(P, T, lb, s, key, occ);
+        const double hdv = diag_element<W>(P, key, occ, s_w);
         P.hd[lb][s] = hdv;
         P.hdf[lb][s] = __double2float_rn(hdv);
-        store_derived<W>(P, T, lb, s, key);
     }
 }
 
@@ -732,24 +757,20 @@ __global__ void k_index_clear_at(Params P, const int *pos, long long n) {
 // Slots [lo, n) of list buffer b as loaded: their derived words and occupied lists, and with compute their
 // diagonal elements (H_ii - E0 and its nearest float; without, the float copies are made by the check).
 template <int W>
-__global__ void __launch_bounds__(256) k_prepare_list(Params P, int b, long long lo, long long n, int compute) {
-    extern __shared__ double s_w[];
+__global__ void __launch_bounds__(kDiagThreads) k_prepare_list(Params P, int b, long long lo, long long n, int compute) {
+    extern __shared__ __align__(16) double s_w[];
     __shared__ Tables T;
     load_tables(P, T);
-    const int M = P.n_orb;
-    if (compute) {
-        for (int k = threadIdx.x; k < 2 * M * M; k += blockDim.x) s_w[k] = P.wpair[k];
-        for (int k = threadIdx.x; k < M; k += blockDim.x) s_w[2 * M * M + k] = P.h[k * M + k];
-    }
+    unsigned char *occ = compute ? load_diag_tables(P, s_w)
+                                 : reinterpret_cast<unsigned char *>(s_w) + threadIdx.x * P.ostride;
     __syncthreads();
     for (long long s = lo + (long long)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
         unsigned long long d[W];
 #pragma unroll
         for (int w = 0; w < W; ++w) d[w] = P.det[b][s * W + w];
-        store_derived<W>(P, T, b, s, d);
+        store_derived<W>(P, T, b, s, d, occ);
         if (compute) {
-            const double v = __dsub_rn(P.hphf ? hphf_hdiag<W>(P, d, s_w, s_w + 2 * M * M) : hdiag<W>(P, d, s_w, s_w + 2 * M * M),
-                                       P.E0);
+            const double v = diag_element<W>(P, d, occ, s_w);
             P.hd[b][s] = v;
             P.hdf[b][s] = __double2float_rn(v);
         }

@@ -499,11 +499,28 @@ __device__ double hdiag(const Params &P, const unsigned long long (&d)[W], const
     return v;
 }
 
+// hdiag of a determinant whose occupied list (ascending) is at hand: the same sums in the same order, on loops that
+// run alike in every lane of a warp, with the table reads ahead of the chain of dependent additions.
+__device__ __forceinline__ double hdiag_occ(int n_elec, int M, const unsigned char *occ, const double *w, const double *hdiag_tab) {
+    double v = 0.0;
+    for (int x = 0; x < n_elec; ++x) v = __dadd_rn(v, hdiag_tab[occ[x] >> 1]);
+    for (int x = 0; x + 1 < n_elec; ++x) {
+        const int p = occ[x];
+        const double *row = w + (p >> 1) * M;
+#pragma unroll 4
+        for (int y = x + 1; y < n_elec; ++y) {
+            const int q = occ[y];
+            v = __dadd_rn(v, row[(((p ^ q) & 1) ? 0 : M * M) + (q >> 1)]);
+        }
+    }
+    return v;
+}
+
 // <Phi_d|H|Phi_d> of a stored spin-coupled function: H_dd + sigma pi_d <d|H|dbar>, the second term only
 // for two open shells (d and dbar then differ by a double excitation).
+// (v: H_dd).
 template <int W>
-__device__ double hphf_hdiag(const Params &P, const unsigned long long (&d)[W], const double *w, const double *hdiag_tab) {
-    double v = hdiag<W>(P, d, w, hdiag_tab);
+__device__ double hphf_hdiag(const Params &P, const unsigned long long (&d)[W], double v) {
     const int no = n_open<W>(d);
     if (no == 2) {
         unsigned long long db[W];

@@ -243,20 +243,19 @@ __device__ __forceinline__ void prepare_det(const Params &P, const Tables &T, De
     fill_view<W>(P, v, pre, c);
 }
 
-// Derived words and occupied list of slot s of list buffer b, computed and stored.
+// Derived words and occupied list of slot s of list buffer b, computed and stored; the list is left in occ
+// (P.ostride bytes, 4-byte aligned).
 template <int W>
 __device__ __forceinline__ void store_derived(const Params &P, const Tables &T, int b, long long s,
-                                              const unsigned long long (&d)[W]) {
+                                              const unsigned long long (&d)[W], unsigned char *occ) {
     unsigned long long pre[PRE_WORDS];
-    unsigned char occ[MAXN] = {};
+    for (int k = P.n_elec; k < P.ostride; ++k) occ[k] = 0;
     derive_det<W>(P, T, d, pre, occ);
     ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(P.pre[b] + s * PRE_WORDS);
     dst[0] = make_ulonglong2(pre[0], pre[1]);
     dst[1] = make_ulonglong2(pre[2], pre[3]);
     unsigned *od = reinterpret_cast<unsigned *>(P.occa[b] + s * P.ostride);
-    for (int k = 0; k < P.ostride / 4; ++k)
-        od[k] = (unsigned)occ[4 * k] | ((unsigned)occ[4 * k + 1] << 8) | ((unsigned)occ[4 * k + 2] << 16) |
-                ((unsigned)occ[4 * k + 3] << 24);
+    for (int k = 0; k < P.ostride / 4; ++k) od[k] = reinterpret_cast<const unsigned *>(occ)[k];
 }
 
 // ---------------------------------------------------------------------------- one spawning attempt
