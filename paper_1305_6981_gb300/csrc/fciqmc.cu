@@ -84,11 +84,16 @@ bool sizes_of(int n_elec, int n_orb, const fciqmc_options &o, Sizes &z) {
 }
 
 struct Layout {
-    size_t state, h, h_f, eri, eri_f, wpair, map1, cmask, unionm, irrep, pairs, recip, rcpf, ref_occ, facts, e0;
+    size_t state, h, h_f, eri, eri_f, bnd, wpair, map1, cmask, unionm, irrep, pairs, recip, rcpf, ref_occ, facts, e0;
     size_t det[2], hd[2], hdf[2], pop[2][2], pre[2], occa[2], idx, mt, merged, heavy, heavy_occ, heavy_base, heavy_att, partial, hist;
     size_t ref_pinfo, ref_off2, ref_exc, outbox;
     size_t total;
 };
+
+// Most sweep tiles of a list of cap slots: full ones, or the small ones of a short list (next_tile).
+long long tiles_of(long long cap) {
+    return std::max<long long>((cap + fq::kTile - 1) / fq::kTile, (long long)kMaxGrid);
+}
 
 Layout layout_of(const Sizes &z, int n_orb) {
     Layout L{};
@@ -103,6 +108,7 @@ Layout layout_of(const Sizes &z, int n_orb) {
     L.h_f = take(sizeof(float) * n_orb * n_orb);
     L.eri = take(sizeof(double) * z.n_eri);
     L.eri_f = take(sizeof(float) * z.n_eri);
+    L.bnd = take(sizeof(float) * 2 * n_orb * n_orb * n_orb);
     L.wpair = take(sizeof(double) * 2 * n_orb * n_orb);
     L.map1 = take(sizeof(unsigned long long) * fq::MAXSO);
     L.cmask = take(sizeof(unsigned long long) * fq::NCLASS * fq::MAXW);
@@ -131,7 +137,7 @@ Layout layout_of(const Sizes &z, int n_orb) {
     L.heavy_occ = take((size_t)fq::MAXN * z.heavy_cap);
     L.heavy_base = take(sizeof(unsigned) * z.heavy_cap);
     L.heavy_att = take(sizeof(unsigned) * z.heavy_cap);
-    L.partial = take(sizeof(double) * (std::max<long long>((z.cap + fq::kTile - 1) / fq::kTile, kMaxGrid) + fq::kTileSums));
+    L.partial = take(sizeof(double) * (tiles_of(z.cap) + fq::kTileSums));
     L.hist = take(sizeof(fciqmc_row) * z.hist_cap);
     L.ref_pinfo = take(sizeof(unsigned) * std::max(z.npairs, 1));
     L.ref_off2 = take(sizeof(unsigned) * std::max<long long>((long long)z.npairs * z.n_so, 1));
@@ -567,6 +573,7 @@ int fciqmc_create(const double *h1, const double *eri_s8, double e_core, int n_e
     P.eri = at<double>(h, L.eri);
     P.eri_f = at<float>(h, L.eri_f);
     P.h_f = at<float>(h, L.h_f);
+    P.bnd = at<float>(h, L.bnd);
     P.wpair = at<double>(h, L.wpair);
     P.map1 = at<unsigned long long>(h, L.map1);
     P.cmask = at<unsigned long long>(h, L.cmask);
@@ -602,7 +609,7 @@ int fciqmc_create(const double *h1, const double *eri_s8, double e_core, int n_e
     P.heavy_cap = z.heavy_cap;
     P.rcpf = at<float>(h, L.rcpf);
     P.partial = at<double>(h, L.partial);
-    P.tiles_cap = std::max<long long>((z.cap + fq::kTile - 1) / fq::kTile, kMaxGrid);
+    P.tiles_cap = tiles_of(z.cap);
     P.hist = at<fciqmc_row>(h, L.hist);
     P.hist_cap = z.hist_cap;
     P.st = at<DevState>(h, L.state);
@@ -623,6 +630,16 @@ int fciqmc_create(const double *h1, const double *eri_s8, double e_core, int n_e
         cmask[cl * fq::MAXW + (k >> 6)] |= 1ull << (k & 63);
     }
     for (int p = 0; p < n_orb; ++p) irr[p] = orb_irrep ? (unsigned char)orb_irrep[p] : 0;
+    {
+        unsigned used = 0;
+        for (int p = 0; p < n_orb; ++p) used |= 1u << irr[p];
+        bool closed = true;
+        for (int g = 0; g < 8; ++g)
+            for (int k = 0; k < 8; ++k)
+                if (((used >> g) & 1u) && ((used >> k) & 1u) && !((used >> (g ^ k)) & 1u)) closed = false;
+        for (int g = 0; g < 8; ++g)
+            if (!closed || ((used >> g) & 1u)) P.full8 |= 0x80ull << (8 * g);
+    }
     std::vector<unsigned long long> unionm(2 * 256 * fq::MAXW, 0ull);
     for (int sp = 0; sp < 2; ++sp)
         for (int set = 0; set < 256; ++set)
@@ -702,6 +719,7 @@ int fciqmc_create(const double *h1, const double *eri_s8, double e_core, int n_e
                                              const_cast<float *>(P.eri_f), const_cast<double *>(P.recip), facts, e0);
             fq::k_reference_energy<2><<<1, 256, h->smem_w, s>>>(P, e0);
         }
+        fq::k_bounds<<<std::min(kMaxGrid, (2 * n_orb * n_orb * n_orb + 255) / 256), 256, 0, s>>>(P, const_cast<float *>(P.bnd));
         FQ_TRY(cudaGetLastError());
         long long hf[4];
         double E0;

@@ -157,7 +157,6 @@ __global__ void __launch_bounds__(kDiagThreads) k_new_diag(Params P) {
     if (st->status) return;
     const long long n = (long long)st->n_new;
     if ((long long)blockIdx.x * blockDim.x >= n) return;
-    const int M = P.n_orb;
     __shared__ Tables T;
     load_tables(P, T);
     unsigned char *occ = load_diag_tables(P, s_w);
@@ -275,13 +274,25 @@ __device__ __forceinline__ void shift_update(DevState *st, long long nw_out, lon
     }
 }
 
-// Heavy chunk size for the next iteration from its expected attempts: kChunk doubled while every k_heavy warp
-// still gets kChunksPerWarp chunks, up to kChunkGrowth kChunk (larger chunks: fewer table builds and batch
-// claims; small ones when the walkers are few, so that every warp has work).
+// Heavy chunk size for the next iteration from its expected attempts: the least that gives every k_heavy warp at most
+// one chunk, from kChunkLeast to kChunk (a warp that takes several small chunks pays for each claim: with eight chunks
+// per warp k_heavy took 112 us instead of 93 on 6e6 walkers of 24e/60o; chunks of 512 serial attempts for a
+// tenth of the warps took 90 instead of 47 on 3.6e4 walkers of 8e/8o), and on up to kChunkGrowth kChunk while every
+// warp gets kChunksPerWarp chunks (fewer table builds and batch claims).
 __device__ __forceinline__ unsigned next_chunk(long long attempts, long long warps) {
-    unsigned c = kChunk;
-    while (c < (unsigned)(kChunkGrowth * kChunk) && attempts >= 2ll * c * kChunksPerWarp * warps) c *= 2u;
+    unsigned c = kChunkLeast;
+    while (c < (unsigned)kChunk && attempts > (long long)c * warps) c *= 2u;
+    while (c >= (unsigned)kChunk && c < (unsigned)(kChunkGrowth * kChunk) && attempts >= 2ll * c * kChunksPerWarp * warps) c *= 2u;
     return c;
+}
+
+// Sweep tile for the next iteration: kTile, halved while there is not a tile for every fourth block, so that a list of
+// a few hundred determinants is spread over the SMs (8e/8o, 500 slots: 40 to 33 us). Longer lists keep whole tiles:
+// with two tiles for every block as the bound, 6e5 slots took 109 instead of 88 us.
+__device__ __forceinline__ int next_tile(long long slots, long long blocks) {
+    int t = kTile;
+    while (t > kTileLeast && (slots + t - 1) / t * 4 < blocks) t >>= 1;
+    return t;
 }
 
 // Makes the iteration's list the current one (new slots included, populations' parity flipped), decides a
@@ -305,6 +316,7 @@ __device__ __forceinline__ void commit_list(DevState *st, long long nd_out, long
     st->sweep_next = 0;
     st->heavy_next = 0;
     st->heavy_chunk = next_chunk(attempts, heavy_warps);
+    st->tile = next_tile(new_len, sweep_blocks);
     // a short list leaves most sweep blocks without a tile, and each tile's light attempts run in one block:
     // then the heavy path, whose chunks spread over every warp, takes determinants from 32 walkers on
     st->heavy_thr = (new_len + kTile - 1) / kTile * 4 < sweep_blocks ? (unsigned)kHeavyShort : (unsigned)kHeavy;
@@ -320,7 +332,8 @@ __global__ void __launch_bounds__(256) k_tile_sum(Params P) {
     __shared__ double s_red[256 / 32];
     DevState *st = P.st;
     if (st->status) return;
-    const long long n = (st->list_len + kTile - 1) / kTile;
+    const int tile = st->tile ? st->tile : kTile;
+    const long long n = (st->list_len + tile - 1) / tile;
     const long long lo = n * blockIdx.x / kTileSums, hi = n * (blockIdx.x + 1) / kTileSums;
     double v = 0.0;
     for (long long t = lo + threadIdx.x; t < hi; t += blockDim.x) v = __dadd_rn(v, P.partial[t]);
@@ -832,6 +845,25 @@ __global__ void __launch_bounds__(256) k_setup(Params P, long long n_eri, unsign
     if (threadIdx.x == 0) {
         facts[0] = (long long)s_ns;
         facts[1] = (long long)s_nd;
+    }
+}
+
+// Bounds of the doubles for attempt_screen: for spatial orbitals I, J and A, the largest |H| over the last virtual B
+// that an attempt I -> A, J -> B can have (parity left out), rounded up. Equal spins exclude B = A, I and J and opposite
+// spins B = J, none of which is unoccupied then. One thread per entry.
+__global__ void __launch_bounds__(256) k_bounds(Params P, float *bnd) {
+    const int M = P.n_orb;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 2 * M * M * M; k += gridDim.x * blockDim.x) {
+        const int A = k % M, J = k / M % M, I = k / (M * M) % M;
+        const bool equal = k >= M * M * M;
+        double m = 0.0;
+        for (int B = 0; B < M; ++B) {
+            if (B == J || (equal && (B == A || B == I))) continue;
+            double x = eri_d(P, I, A, J, B);
+            if (equal) x = __dsub_rn(x, eri_d(P, I, B, J, A));
+            m = fmax(m, fabs(x));
+        }
+        bnd[k] = __double2float_ru(m);
     }
 }
 

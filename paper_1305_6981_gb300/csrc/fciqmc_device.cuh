@@ -54,7 +54,8 @@ struct DevState {
     unsigned long long n_new;  // determinants placed in new slots this iteration (diagonal elements pending)
     unsigned long long sweep_next;  // next sweep tile to hand out (tiles are taken dynamically by the blocks)
     unsigned long long heavy_next;  // next batch of heavy chunks to hand out (taken dynamically by the warps)
-    unsigned heavy_chunk;           // attempts per heavy chunk this iteration (0: the smallest size)
+    unsigned heavy_chunk;           // attempts per heavy chunk this iteration (0: kChunk)
+    int tile;                       // determinants per sweep tile this iteration (0: kTile)
     unsigned heavy_thr;             // attempts above which a determinant takes the heavy path (0: kHeavy)
     unsigned long long ob_n[MAXPARTS];  // partitioned runs: spawns routed to each other partition this iteration
 };
@@ -91,6 +92,9 @@ struct Params {
     const double *eri;      // packed 8-fold
     const float *eri_f;     // same, rounded to float
     const float *h_f;       // h rounded to float
+    unsigned long long full8;  // bit 7 of byte g: irrep g is in use (of every byte when those are not closed under products)
+    const float *bnd;       // [2][n_orb][n_orb][n_orb]: over b, the largest |H| of the doubles I -> A, J -> b: [0] opposite
+                            // spins (A has the spin of I), [1] equal spins (k_bounds)
     const double *wpair;    // [2][n_orb][n_orb]: [0] opposite spin (pp|qq), [1] same spin (pp|qq) - (pq|qp)
     const unsigned long long *map1;   // n_so, orbital map of Algorithm 1
     const unsigned long long *cmask;  // [NCLASS][MAXW] spin orbitals of each (irrep, spin) class
@@ -171,13 +175,19 @@ __device__ __forceinline__ void set_status(DevState *st, int code) { atomicCAS(&
 #endif
 
 // ---------------------------------------------------------------------------
+// 32 x 32 -> 64 bits in one instruction (written as a low and a high product, a Philox block took 6% longer).
+__device__ __forceinline__ unsigned long long mul_wide(unsigned a, unsigned b) {
+    unsigned long long p;
+    asm("mul.wide.u32 %0, %1, %2;" : "=l"(p) : "r"(a), "r"(b));
+    return p;
+}
+
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11).
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        unsigned lo0 = 0xD2511F53u * c.x, hi0 = __umulhi(0xD2511F53u, c.x);
-        unsigned lo1 = 0xCD9E8D57u * c.z, hi1 = __umulhi(0xCD9E8D57u, c.z);
-        c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
+        const unsigned long long p0 = mul_wide(0xD2511F53u, c.x), p1 = mul_wide(0xCD9E8D57u, c.z);
+        c = make_uint4((unsigned)(p1 >> 32) ^ c.y ^ k.x, (unsigned)p1, (unsigned)(p0 >> 32) ^ c.w ^ k.y, (unsigned)p0);
         k.x += 0x9E3779B9u;
         k.y += 0xBB67AE85u;
     }
@@ -196,17 +206,15 @@ __device__ __forceinline__ void draw2(unsigned a, unsigned tag, unsigned long lo
 // in mixed radix: k = floor(R n / 2^75), uniform in [0, n), and R becomes R n mod 2^75. With
 // S = rh n + floor(rl n / 2^11) (at most 85 bits), k = floor(S / 2^64), the new rh = S mod 2^64 and the new
 // rl = rl n mod 2^11. Every radix is below 2^12 (at most MAXPAIRS = 2016 electron pairs, MAXSO spin
-// orbitals), so rl n fits 32 bits and (rh >> 32) n + 2^33 fits 64.
+// orbitals), so rl n fits 32 bits and both products with their carries fit 64.
 static_assert(MAXPAIRS < 4096 && MAXSO < 4096, "choice radices must stay below 2^12");
 __device__ __forceinline__ unsigned rank_next(unsigned long long &rh, unsigned &rl, unsigned n) {
-    const unsigned long long lo = (unsigned long long)(unsigned)rh * n;
-    const unsigned long long hi = (unsigned long long)(unsigned)(rh >> 32) * n;
     const unsigned q = rl * n;
-    const unsigned long long s0 = (lo & 0xFFFFFFFFull) + (q >> 11);
-    const unsigned long long sh = hi + (lo >> 32) + (s0 >> 32);
-    rh = (sh << 32) | (s0 & 0xFFFFFFFFull);
+    const unsigned long long lo = mul_wide((unsigned)rh, n) + (q >> 11);
+    const unsigned long long hi = mul_wide((unsigned)(rh >> 32), n) + (lo >> 32);
+    rh = (hi << 32) | (unsigned)lo;
     rl = q & 0x7FFu;
-    return (unsigned)(sh >> 32);
+    return (unsigned)(hi >> 32);
 }
 
 // ---------------------------------------------------------------------------

@@ -16,7 +16,7 @@
 
 namespace fq {
 
-constexpr int kTile = 256;          // determinants per sweep tile = threads per sweep block
+constexpr int kTile = 256;          // threads per sweep block = most determinants of a sweep tile
 constexpr int kTileSums = 32;       // range sums of the per-tile numerators (blocks of k_tile_sum)
 #ifndef FQ_SWEEP_MIN_BLOCKS
 #define FQ_SWEEP_MIN_BLOCKS 5          // resident sweep blocks per SM the register budget is sized for
@@ -29,7 +29,9 @@ constexpr int kHeavyShort = 32;  // the threshold for lists with fewer tiles tha
 #ifndef FQ_HEAVY_CHUNK
 #define FQ_HEAVY_CHUNK 512
 #endif
-constexpr int kChunk = FQ_HEAVY_CHUNK;  // smallest heavy chunk in attempts (one warp task)
+constexpr int kChunk = FQ_HEAVY_CHUNK;  // ordinary heavy chunk in attempts (one warp task)
+constexpr int kChunkLeast = 64;  // smallest, for runs with few walkers
+constexpr int kTileLeast = 32;
 #ifndef FQ_CHUNK_GROWTH
 #define FQ_CHUNK_GROWTH 4
 #endif
@@ -58,6 +60,7 @@ struct DetView {
     unsigned char nok;          // electrons with at least one symmetry-allowed single (N - delta_s)
     unsigned char flag;         // initiator
     unsigned char isref;        // the reference determinant
+    unsigned char full;         // every class keeps two unoccupied spin orbitals, so every unoccupied a is good
 };  // the occupied spin orbitals (ascending) are kept beside the view, n_elec bytes
 
 // Occupied spin orbitals of d in ascending order (for the exact FP64 paths, which run rarely); returns their
@@ -79,18 +82,22 @@ __device__ __forceinline__ int decode_occ(const unsigned long long (&d)[W], unsi
 // Bytes of one occupied list in the sweep's tile (the electron count rounded up to 4).
 __host__ __device__ constexpr int occ_stride(int n_elec) { return (n_elec + 3) & ~3; }
 
-struct Tables {
-    unsigned long long map1[MAXSO];
+// Tables of the spawning kernels, in the block's shared memory.
+struct AttemptTables {
     unsigned long long mask[NCLASS * MAXW];
     // spin orbitals of spin s in the irreps of a 4-bit set, for irreps 0..3 (half 0) and 4..7 (half 1):
     // uh[((s * 2 + half) * 16 + set) * MAXW + w]
     unsigned long long uh[2 * 2 * 16 * MAXW];
+    unsigned long long all[MAXW];  // every spin orbital of the basis
     unsigned char irrep[MAXSO / 2];
     unsigned short pairs[MAXPAIRS];
 };
+// With the orbital map of Algorithm 1, for the kernels that derive a determinant's data.
+struct Tables : AttemptTables {
+    unsigned long long map1[MAXSO];
+};
 
-__device__ __forceinline__ void load_tables(const Params &P, Tables &T) {
-    for (int k = threadIdx.x; k < P.n_so; k += blockDim.x) T.map1[k] = P.map1[k];
+__device__ __forceinline__ void load_tables(const Params &P, AttemptTables &T) {
     for (int k = threadIdx.x; k < NCLASS * MAXW; k += blockDim.x) T.mask[k] = P.cmask[k];
     for (int k = threadIdx.x; k < 2 * 2 * 16 * MAXW; k += blockDim.x) {
         const int w = k % MAXW, set = (k / MAXW) % 16, half = (k / (16 * MAXW)) % 2, s = k / (32 * MAXW);
@@ -99,8 +106,14 @@ __device__ __forceinline__ void load_tables(const Params &P, Tables &T) {
             if ((set >> b) & 1) u |= P.cmask[((4 * half + b) * 2 + s) * MAXW + w];
         T.uh[k] = u;
     }
+    for (int k = threadIdx.x; k < MAXW; k += blockDim.x) T.all[k] = k * 64 >= P.n_so ? 0ull : low_bits(min(P.n_so - 64 * k, 64));
     for (int k = threadIdx.x; k < P.n_orb; k += blockDim.x) T.irrep[k] = P.irrep[k];
     for (int k = threadIdx.x; k < P.npairs; k += blockDim.x) T.pairs[k] = P.pairs[k];
+}
+
+__device__ __forceinline__ void load_tables(const Params &P, Tables &T) {
+    for (int k = threadIdx.x; k < P.n_so; k += blockDim.x) T.map1[k] = P.map1[k];
+    load_tables(P, static_cast<AttemptTables &>(T));
 }
 
 // ---------------------------------------------------------------------------- float bounds
@@ -232,6 +245,8 @@ __device__ __forceinline__ void fill_view(const Params &P, DetView<W> &v, const 
     bool is_ref = det_eq<W>(v.d, P.ref);
     v.flag = (P.init_thr < 0 || ac > P.init_thr || is_ref) ? 1 : 0;
     v.isref = is_ref ? 1 : 0;
+    constexpr unsigned long long kTwo = 0x7E7E7E7E7E7E7E7Eull;  // counts <= 64: no byte carries
+    v.full = ((cb0 + kTwo) & (cb1 + kTwo) & P.full8) == P.full8 ? 1 : 0;
 }
 
 // The view of v.d (its bits already set), derived on the spot.
@@ -338,13 +353,17 @@ __device__ __forceinline__ float small_f(unsigned x) { return __int_as_float(0x4
 // Sec. VI B in ascending order and their number G; for each (irrep, spin) class its unoccupied spin
 // orbitals in ascending order, and the position of each unoccupied spin orbital in its class list.
 // Rows are padded by one 32-bit word so that the same position in different rows falls in different
-// shared-memory banks (the lanes of a warp read random rows).
+// shared-memory banks (the lanes of a warp read random rows). When every class keeps two unoccupied orbitals
+// (DetView::full) the good lists do not depend on the irrep: only rows 0, 8 and 16 are filled.
 struct HeavyTab {
     unsigned char glist[24][MAXSO + 4];
     unsigned char ulist[NCLASS][MAXSO / 2 + 4];
     unsigned char urank[MAXSO];
     unsigned char occ[MAXN];  // the determinant's occupied spin orbitals, ascending
-    unsigned short G[24];
+    unsigned short occ2[MAXN];  // the same with the orbital's irrep in the high byte
+    // per entry: its number of good a (x) and a bound of its doubles' 1 / P_gen factor (y): p <= |H| F (attempt_screen)
+    uint2 GF[24];
+    unsigned row_mask;  // entry -> filled row of glist
 };
 
 // Good a-orbitals for one (spin case, pair irrep): a of spin sa in irrep g is good when its class has
@@ -383,7 +402,7 @@ __device__ __forceinline__ unsigned good_set(const Params &P, const DetView<W> &
 // good_set with the union of the good classes' orbitals from the block's shared tables (two 4-irrep halves)
 // instead of the global 8-bit-set table.
 template <int W>
-__device__ __forceinline__ unsigned good_set_t(const Tables &T, const DetView<W> &v, int si, int sj, int gij,
+__device__ __forceinline__ unsigned good_set_t(const AttemptTables &T, const DetView<W> &v, int si, int sj, int gij,
                                                unsigned long long (&gm)[W]) {
     constexpr unsigned long long kOnes = 0x0101010101010101ull, kHigh = 0x8080808080808080ull;
     unsigned G = 0;
@@ -413,39 +432,59 @@ __device__ __forceinline__ unsigned good_set_t(const Tables &T, const DetView<W>
     return G;
 }
 
-// Builds tab for determinant v; called by all 32 lanes of a warp. Lanes 0..23 take one entry each,
-// lanes 24..31 two classes each.
+// Largest byte of a word of class counts.
+__device__ __forceinline__ unsigned max_byte(unsigned long long x) {
+    unsigned m = __vmaxu4((unsigned)x, (unsigned)(x >> 32));
+    m = __vmaxu4(m, m >> 16);
+    return __vmaxu4(m, m >> 8) & 0xFFu;
+}
+
+// Builds tab for determinant v; called by all 32 lanes of a warp. Lanes 0..23 take one entry's good set each; the
+// lists are written by all lanes together, a lane per spin orbital of a 32-orbital word, whose position is a
+// population count. (A lane per list, walking its bits one by one, took about 1500 instructions a build and left
+// runs of a few million walkers waiting for it: see k_heavy.)
 template <int W>
-__device__ __forceinline__ void build_heavy_tab(const Params &P, const Tables &T, const DetView<W> &v, HeavyTab &tab,
-                                                int lane) {
+__device__ __forceinline__ void build_heavy_tab(const Params &P, const AttemptTables &T, const DetView<W> &v,
+                                                const float *rcpf, HeavyTab &tab, int lane) {
+    const unsigned below = (1u << lane) - 1u;
+#pragma unroll
+    for (int c = 0; c < 2 * W; ++c) {
+        const int so = 32 * c + lane;
+        const unsigned long long un = ~v.d[c >> 1] & T.all[c >> 1];
+        if ((un >> (so & 63)) & 1ull) {
+            const int cl = T.irrep[so >> 1] * 2 + (so & 1);
+            int r = 0;
+#pragma unroll
+            for (int w = 0; w <= (c >> 1); ++w) {
+                unsigned long long m = ~v.d[w] & T.mask[cl * MAXW + w];
+                if (w == (c >> 1)) m &= (1ull << (so & 63)) - 1ull;
+                r += __popcll(m);
+            }
+            tab.ulist[cl][r] = (unsigned char)so;
+            tab.urank[so] = (unsigned char)r;
+        }
+    }
+    unsigned long long gm[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) gm[w] = 0ull;
     if (lane < 24) {
         const int sc = lane >> 3, gij = lane & 7;
         const int si = sc == 1 ? 1 : 0, sj = sc == 0 ? 0 : 1;
-        unsigned long long gm[W];
-        tab.G[lane] = (unsigned short)good_set<W>(P, v, si, sj, gij, gm);
-        int n = 0;
+        const unsigned G = good_set_t<W>(T, v, si, sj, gij, gm);
+        // M^(b|a) M^(a|b) / (M^(b|a) + M^(a|b)) grows with both counts: bounded at the largest classes of the spins
+        const unsigned ma = max_byte(v.cb8[si]), mb = max_byte(v.cb8[sj]);
+        const float F = ma && mb ? P.cdn_f * small_f(G) * small_f(ma) * small_f(mb) * rcpf[ma + mb] : 0.f;
+        tab.GF[lane] = make_uint2(G, __float_as_uint(F));
+    }
+    const unsigned stride = v.full ? 8u : 1u;
+    if (lane == 0) tab.row_mask = v.full ? 24u : 31u;
+    for (unsigned e = 0; e < 24; e += stride) {
+        int base = 0;
 #pragma unroll
-        for (int w = 0; w < W; ++w) {
-            unsigned long long m = gm[w];
-            while (m) {
-                tab.glist[lane][n++] = (unsigned char)(64 * w + __ffsll((long long)m) - 1);
-                m &= m - 1;
-            }
-        }
-    } else {
-        for (int c = lane - 24; c < NCLASS; c += 8) {
-            int n = 0;
-#pragma unroll
-            for (int w = 0; w < W; ++w) {
-                unsigned long long m = ~v.d[w] & T.mask[c * MAXW + w];
-                while (m) {
-                    const int so = 64 * w + __ffsll((long long)m) - 1;
-                    tab.ulist[c][n] = (unsigned char)so;
-                    tab.urank[so] = (unsigned char)n;
-                    ++n;
-                    m &= m - 1;
-                }
-            }
+        for (int c = 0; c < 2 * W; ++c) {
+            const unsigned m = __shfl_sync(0xFFFFFFFFu, (unsigned)(gm[c >> 1] >> (32 * (c & 1))), (int)e);
+            if ((m >> lane) & 1u) tab.glist[e][base + __popc(m & below)] = (unsigned char)(32 * c + lane);
+            base += __popc(m);
         }
     }
     __syncwarp();
@@ -551,7 +590,7 @@ __device__ float gen_prob_double_f(const Params &P, const DetView<W> &v, const H
     if (si == sj && ((a & 1) != si || (b & 1) != si)) return 0.f;
     long long G;
     if (tab) {  // the determinant's tables hold the good-set sizes
-        G = tab->G[(si == sj ? si : 2) * 8 + (gi ^ gj)];
+        G = tab->GF[(si == sj ? si : 2) * 8 + (gi ^ gj)].x;
     } else {
         unsigned long long gm[W];
         G = good_set<W>(P, v, si, sj, gi ^ gj, gm);
@@ -685,7 +724,7 @@ __device__ void hphf_attempt_end(const Params &P, const DetView<W> &v, const Hea
 // give the choices as mixed-radix digits (rank_next). A double is completed here; a single is
 // selected (electron i, virtual ao) and returned pending (true) for the warp to evaluate its element.
 template <int W, bool TAB, int MODE>
-__device__ __forceinline__ bool attempt_begin(const Params &P, const Tables &T, const DetView<W> &v,
+__device__ __forceinline__ bool attempt_begin(const Params &P, const AttemptTables &T, const DetView<W> &v,
                                               const unsigned char *occ, const HeavyTab *tab, const float *rcpf, unsigned a, unsigned iter,
                                               unsigned long long pol, unsigned long long *cnt, SpawnQueue<W> &out,
                                               int &i_out, int &a_out, unsigned &mallow_out, unsigned long long &q_out,
@@ -811,11 +850,11 @@ __device__ __forceinline__ bool attempt_begin(const Params &P, const Tables &T, 
     int ao;
     if (TAB) {
         const int e = (si == sj ? si : 2) * 8 + gij;
-        G = tab->G[e];
+        G = tab->GF[e].x;
         if (G == 0) { cnt[C_NULLS]++; return false; }
         const unsigned k2 = rank_next(rh, rl, G);
         if (!FQ_CHECK(k2 < (unsigned)MAXSO, P.st)) return false;
-        ao = tab->glist[e][k2];
+        ao = tab->glist[e & tab->row_mask][k2];
     } else {
         unsigned long long gm[W];
         G = good_set_t<W>(T, v, si, sj, gij, gm);
@@ -903,6 +942,130 @@ __device__ __forceinline__ bool attempt_begin(const Params &P, const Tables &T, 
     flip<W>(child, ao);
     flip<W>(child, bo);
     emit_spawn<W>(P, v, child, n, sgn_h, cnt, out);
+    return false;
+}
+
+// Whether attempts a, a + 32, ... of a heavily populated determinant can spawn at all, each from its draw, its electron
+// pair and its first virtual: p <= hb F for every b, with hb the largest |H| over the b (P.bnd) and F the entry's
+// bound of the 1 / P_gen factor, so an attempt whose type word is above hb F needs neither b nor an integral. Attempts
+// that pass, and singles, are evaluated from the start by attempt_begin; for the others the null excitations are
+// counted here. p averages 0.1 to 0.8% on 24e/60o and the bound lets 3 to 6% of the attempts through (an
+// electron-pair bound without the virtual lets 87% through: every pair has one large element). U attempts of a lane
+// are taken side by side without branches, so that one's table reads overlap the other's.
+template <int W, int MODE, int U>
+__device__ __forceinline__ void attempt_screen(const Params &P, const AttemptTables &T, const DetView<W> &v, const HeavyTab &tab,
+                                               unsigned row_mask, unsigned a, unsigned a1, unsigned iter, unsigned long long pol,
+                                               unsigned long long *cnt, bool (&live)[U]) {
+    unsigned long long t[U], rh[U];
+    unsigned rl[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        draw2(a + 32u * u, 0u, v.fp, P.seed, iter, t[u], rh[u]);
+        rl[u] = (unsigned)t[u] & 0x7FFu;
+        t[u] >>= 11;
+        live[u] = a + 32u * u < a1;
+    }
+    if (P.npairs == 0) return;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const unsigned short pr = T.pairs[rank_next(rh[u], rl[u], (unsigned)P.npairs)];
+        const unsigned oi = tab.occ2[pr & 0xFF], oj = tab.occ2[pr >> 8];
+        const int i = oi & 0xFF, j = oj & 0xFF, si = i & 1, sj = j & 1;
+        const int gij = (int)((oi ^ oj) >> 8);
+        const unsigned e = (unsigned)((si == sj ? si : 2) * 8 + gij);
+        const uint2 gf = tab.GF[e];
+        const unsigned k2 = rank_next(rh[u], rl[u], gf.x);
+        const int ao = gf.x != 0 && FQ_CHECK(k2 < (unsigned)MAXSO, P.st) ? tab.glist[e & row_mask][k2] : 0;
+        // the electron whose spin a takes comes first (either, for a pair of one spin)
+        const bool swap = si != sj && (ao & 1) != si;
+        const int I = (swap ? j : i) >> 1, J = (swap ? i : j) >> 1;
+        const int at = (((si == sj ? P.n_orb : 0) + I) * P.n_orb + J) * P.n_orb + (ao >> 1);
+        const float th = ld_keep(P.bnd + at, pol) * __uint_as_float(gf.y) * P.d53_f * (kUp * kUp);
+        const float q_lo = small_f((unsigned)(t[u] >> 30)) * 0x1p30f;  // q_lo <= t, exact
+        const bool twice = live[u] && t[u] < P.d53;  // a double excitation
+        const bool null = twice && gf.x == 0;
+        live[u] = live[u] && (!twice || (gf.x != 0 && q_lo < th));
+        cnt[C_NULLS] += null ? 1ull : 0ull;
+        if (MODE & 1) {  // rejected, but outside the permitted space it is a null excitation
+            if (twice && !null && !live[u]) {
+                const int ga = T.irrep[ao >> 1];
+                const int ca = ga * 2 + (ao & 1), cb = (gij ^ ga) * 2 + (si + sj - (ao & 1));
+                const unsigned same = ca == cb ? 1u : 0u;
+                int k3 = (int)rank_next(rh[u], rl[u], (unsigned)v.cnt[cb] - same);
+                if (same && k3 >= tab.urank[ao]) ++k3;
+                if (!FQ_CHECK(k3 < MAXSO / 2, P.st)) continue;
+                unsigned long long ch[W];
+#pragma unroll
+                for (int w = 0; w < W; ++w) ch[w] = v.d[w];
+                flip<W>(ch, i);
+                flip<W>(ch, j);
+                flip<W>(ch, ao);
+                flip<W>(ch, (int)tab.ulist[cb][k3]);
+                if (!in_space<W>(P, ch)) cnt[C_NULLS]++;
+            }
+        }
+    }
+}
+
+// attempt_screen for a light attempt, from the determinant's view. When every class keeps two unoccupied orbitals
+// (the irreps in use closed under products), all unoccupied orbitals of the allowed spins are good, which saves the
+// test of the irreps.
+template <int W, int MODE>
+__device__ __forceinline__ bool attempt_screen_light(const Params &P, const AttemptTables &T, const DetView<W> &v,
+                                                     const unsigned char *occ, const float *rcpf, unsigned a, unsigned iter,
+                                                     unsigned long long pol, unsigned long long *cnt) {
+    unsigned long long r0, rh;
+    draw2(a, 0u, v.fp, P.seed, iter, r0, rh);
+    const unsigned long long t = r0 >> 11;
+    unsigned rl = (unsigned)r0 & 0x7FFu;
+    if (t >= P.d53 || P.npairs == 0) return true;
+    const unsigned short pr = T.pairs[rank_next(rh, rl, (unsigned)P.npairs)];
+    const int i = occ[pr & 0xFF], j = occ[pr >> 8];
+    const int si = i & 1, sj = j & 1;
+    const int gij = T.irrep[i >> 1] ^ T.irrep[j >> 1];
+    unsigned long long gm[W];
+    unsigned G;
+    if (v.full) {
+        G = 0;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            unsigned long long m = 0ull;
+            if (si == sj) m = T.uh[((si * 2) * 16 + 15) * MAXW + w] | T.uh[((si * 2 + 1) * 16 + 15) * MAXW + w];
+            else m = T.all[w];
+            gm[w] = m & ~v.d[w];
+            G += __popcll(gm[w]);
+        }
+    } else {
+        G = good_set_t<W>(T, v, si, sj, gij, gm);
+    }
+    if (G == 0) { cnt[C_NULLS]++; return false; }
+    const int ao = select_bit<W>(gm, (int)rank_next(rh, rl, G));
+    const int ga = T.irrep[ao >> 1];
+    const int ca = ga * 2 + (ao & 1), cb = (gij ^ ga) * 2 + (si + sj - (ao & 1));
+    const unsigned same = ca == cb ? 1u : 0u;
+    const unsigned m_ba = v.cnt[cb] - same, m_ab = v.cnt[ca] - same;
+    const float F = P.cdn_f * small_f(G) * small_f(m_ba) * small_f(m_ab) * rcpf[m_ba + m_ab];
+    const bool swap = si != sj && (ao & 1) != si;
+    const int I = (swap ? j : i) >> 1, J = (swap ? i : j) >> 1;
+    const int at = (((si == sj ? P.n_orb : 0) + I) * P.n_orb + J) * P.n_orb + (ao >> 1);
+    const float th = ld_keep(P.bnd + at, pol) * F * P.d53_f * (kUp * kUp);
+    const float q_lo = small_f((unsigned)(t >> 30)) * 0x1p30f;  // q_lo <= t, exact
+    if (q_lo < th) return true;
+    if (MODE & 1) {  // rejected, but outside the permitted space it is a null excitation
+        unsigned long long bm[W], ch[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            bm[w] = ~v.d[w] & T.mask[cb * MAXW + w];
+            ch[w] = v.d[w];
+        }
+        clear_bit<W>(bm, ao);
+        const int bo = select_bit<W>(bm, (int)rank_next(rh, rl, m_ba));
+        flip<W>(ch, i);
+        flip<W>(ch, j);
+        flip<W>(ch, ao);
+        flip<W>(ch, bo);
+        if (!in_space<W>(P, ch)) cnt[C_NULLS]++;
+    }
     return false;
 }
 
@@ -1070,7 +1233,7 @@ __device__ __forceinline__ void hphf_single_end(const Params &P, const DetView<W
 
 // One spawning attempt per lane (active lanes only); called by all 32 lanes of a warp.
 template <int W, bool TAB, int MODE>
-__device__ __forceinline__ void spawn_attempt(const Params &P, const Tables &T, const DetView<W> &v,
+__device__ __forceinline__ void spawn_attempt(const Params &P, const AttemptTables &T, const DetView<W> &v,
                                               const unsigned char *occ, const HeavyTab *tab, const float *rcpf, bool active, unsigned a,
                                               unsigned iter, unsigned long long *cnt, SpawnQueue<W> &out,
                                               bool rtab = false) {
@@ -1172,11 +1335,6 @@ __device__ __forceinline__ double block_sum_f64(double v, double *s_red) {
 }
 
 // ---------------------------------------------------------------------------- kernels
-// Nearest floats of 1/L for the spawn bound, copied to shared memory.
-__device__ __forceinline__ void load_rcpf(const Params &P, float *s_rcpf) {
-    for (int k = threadIdx.x; k < 2 * MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
-}
-
 // MODE bit 0: the run has a permitted space; bit 1: walkers on spin-coupled functions (the code of
 // each is compiled in only for runs that use it).
 template <int W, int MODE>
@@ -1187,16 +1345,21 @@ __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) 
     extern __shared__ __align__(16) unsigned char s_queue[];
     unsigned char *const s_occ = s_queue + sizeof(SpawnQueue<W>) * (kTile / 32);
     const int ostride = occ_stride(P.n_elec);
-    __shared__ Tables T;
+    __shared__ AttemptTables T;
     __shared__ DetView<W> s_dv[kTile];
     __shared__ unsigned s_off[kTile];
     __shared__ unsigned s_wsum[kTile / 32];
-    __shared__ float s_rcpf[2 * MAXSO + 2];
+    __shared__ float s_rcpf[MAXSO + 2];  // two class counts (at most 64 each) add up to an index
     __shared__ unsigned long long s_red[(kTile / 32) * (NCNT + 4)];
-    load_tables(P, T);
-    load_rcpf(P, s_rcpf);
-    const int lb = st->lb, pp = st->pp;
+    __shared__ long long s_tile[2];
     const long long len = st->list_len;
+    const int tile = st->tile ? st->tile : kTile;  // determinants per tile this iteration
+    if (threadIdx.x == 0) s_tile[0] = (long long)atomicAdd(&st->sweep_next, 1ull) * tile;
+    __syncthreads();
+    if (s_tile[0] >= len) return;  // a short list: no tile for this block
+    load_tables(P, T);
+    for (int k = threadIdx.x; k < MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
+    const int lb = st->lb, pp = st->pp;
     const unsigned iter = (unsigned)st->iter;
     const double S = st->shift;
     const float S_f = __double2float_rn(S);
@@ -1222,17 +1385,18 @@ __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) 
     // static assignment left the blocks' last tiles as a tail. The next tile is claimed while this one is
     // worked on (two slots), so a tile takes three block barriers: after the per-determinant work, after the
     // attempt offsets, and after the attempts.
-    __shared__ long long s_tile[2];
     __shared__ double s_numw[kTile / 32];
-    if (tid == 0) s_tile[0] = (long long)atomicAdd(&st->sweep_next, 1ull) * kTile;
-    __syncthreads();
+    static_assert(kHeavy <= 256 && kTile <= 256, "a queued light attempt packs its determinant and number in 8 bits each");
+    __shared__ unsigned short s_pend[kTile / 32][64], s_left[kTile];  // attempts that passed the screen; the tile's rest
+    __shared__ unsigned s_nleft;
+    const unsigned long long pol = keep_policy();
     for (int slot = 0;; slot ^= 1) {
         const long long tb = s_tile[slot];
         if (tb >= len) break;
         double num = 0.0;  // this tile's share of the Eq. 2 numerator
         const long long s = tb + tid;
         unsigned att = 0;
-        if (s < len) {
+        if (tid < tile && s < len) {
             const int c = __ldcs(pop_in + s);
             if (c == 0) {
                 pop_out[s] = 0;
@@ -1257,7 +1421,14 @@ __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) 
                     pre[2] = p1.x;
                     pre[3] = p1.y;
                     const unsigned *os = reinterpret_cast<const unsigned *>(P.occa[lb] + s * ostride);
-                    for (int k = 0; k < ostride / 4; ++k) reinterpret_cast<unsigned *>(occ)[k] = __ldcs(os + k);
+                    for (int k = 0; k < ostride / 4; k += 8) {  // eight loads in flight
+                        unsigned o[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) o[u] = k + u < ostride / 4 ? __ldcs(os + k + u) : 0u;
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            if (k + u < ostride / 4) reinterpret_cast<unsigned *>(occ)[k + u] = o[u];
+                    }
                 }
                 fill_view<W>(P, v, pre, c);
                 const unsigned ac = (unsigned)(c < 0 ? -c : c);
@@ -1321,7 +1492,10 @@ __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) 
         const double wnum = warp_sum_f64(num);
         if (lane == 31) s_wsum[warp] = x;
         if (lane == 0) s_numw[warp] = wnum;
-        if (tid == 0) s_tile[slot ^ 1] = (long long)atomicAdd(&st->sweep_next, 1ull) * kTile;
+        if (tid == 0) {
+            s_tile[slot ^ 1] = (long long)atomicAdd(&st->sweep_next, 1ull) * tile;
+            s_nleft = 0;
+        }
         __syncthreads();
         unsigned woff = 0, total = 0;
 #pragma unroll
@@ -1336,52 +1510,121 @@ __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) 
             // took which tile
             double bs = 0.0;
             for (int w = 0; w < kTile / 32; ++w) bs = __dadd_rn(bs, s_numw[w]);
-            if (FQ_CHECK(tb / kTile < P.tiles_cap, P.st)) P.partial[tb / kTile] = bs;
+            if (FQ_CHECK(tb / tile < P.tiles_cap, P.st)) P.partial[tb / tile] = bs;
         }
         __syncthreads();
-        for (unsigned base = 0; base < total; base += kTile) {
-            const unsigned k = base + tid;
-            const bool act = k < total;
+        // Attempts are screened; those that can spawn collect in a queue of the warp and are evaluated 32 at a time, and
+        // what is left of the warps' queues at the end of the tile is evaluated by as few warps as it fills. (Spin-
+        // coupled functions are evaluated directly: the screen's bound does not cover them.)
+        unsigned np = 0;
+        bool last = false;
+        for (unsigned base = 0;;) {
+            bool act;
             int lo = 0;
-            if (act) {
-                int hi = kTile - 1;  // last d with s_off[d] <= k
-                while (lo < hi) {
-                    int mid = (lo + hi + 1) >> 1;
-                    if (s_off[mid] <= k) lo = mid; else hi = mid - 1;
+            unsigned a = 0;
+            if (base < total) {
+                const unsigned k = base + tid;
+                act = k < total;
+                base += kTile;
+                if (act) {
+                    int hi = kTile - 1;  // last d with s_off[d] <= k
+                    while (lo < hi) {
+                        int mid = (lo + hi + 1) >> 1;
+                        if (s_off[mid] <= k) lo = mid; else hi = mid - 1;
+                    }
+                    a = k - s_off[lo];
                 }
+                if (!(MODE & 2)) {
+                    const bool live = act && attempt_screen_light<W, MODE>(P, T, s_dv[lo], s_occ + lo * ostride, s_rcpf, a, iter, pol, acc);
+                    const unsigned m = __ballot_sync(0xFFFFFFFFu, live);
+                    if (live) s_pend[warp][np + __popc(m & ((1u << lane) - 1u))] = (unsigned short)(lo | (a << 8));
+                    np += __popc(m);
+                    if (np < 32) continue;
+                    __syncwarp();
+                    np -= 32;
+                    const unsigned e = s_pend[warp][np + lane];
+                    __syncwarp();
+                    act = true;
+                    lo = e & 0xFF;
+                    a = e >> 8;
+                }
+            } else {
+                if ((MODE & 2) || last) break;
+                last = true;
+                unsigned at = 0;
+                if (lane == 0 && np) at = atomicAdd(&s_nleft, np);
+                at = __shfl_sync(0xFFFFFFFFu, at, 0);
+                __syncwarp();
+                if (lane < (int)np) s_left[at + lane] = s_pend[warp][lane];
+                __syncthreads();
+                const unsigned nl = s_nleft;
+                if ((unsigned)warp * 32u >= nl) break;
+                act = (unsigned)tid < nl;
+                const unsigned e = act ? s_left[tid] : 0u;
+                lo = e & 0xFF;
+                a = e >> 8;
             }
-            spawn_attempt<W, false, MODE>(P, T, s_dv[lo], s_occ + lo * ostride, nullptr, s_rcpf, act, k - s_off[lo],
-                                          iter, acc, sq);
-            flush_queue<W>(P, sq, false, T.map1);
+            spawn_attempt<W, false, MODE>(P, T, s_dv[lo], s_occ + lo * ostride, nullptr, s_rcpf, act, a, iter, acc, sq);
+            flush_queue<W>(P, sq, false, P.map1);
         }
         __syncthreads();  // the tile's views and offsets are free again; the next tile's index is visible
     }
-    flush_queue<W>(P, sq, true, T.map1);
+    flush_queue<W>(P, sq, true, P.map1);
     unsigned long long *const dst[NCNT + 4] = {&st->cnt[0], &st->cnt[1], &st->cnt[2], &st->cnt[3], &st->cnt[4],
                                                &st->cnt[5], &st->cnt[6], &st->cnt[7], &st->cnt[8], &st->cnt[9],
                                                &st->nw_in, &st->nd_in, &st->d_nw, &st->d_nd};
     flush_counters<kTile, NCNT + 4>(acc, dst, s_red);
 }
 
-// Attempts of heavily populated determinants, split into chunks of kChunk attempts: warps take batches of
+// Attempts of heavily populated determinants, split into chunks of st->heavy_chunk attempts: warps take batches of
 // consecutive chunks from a counter (guided: a share of what is left, at most kChunkBatch), so a warp meets
-// few determinants, and build a determinant's tables once when they reach it.
+// few determinants, and build a determinant's tables once when they reach it. Attempts are screened first
+// (attempt_screen); those that can spawn collect in a queue of the warp and are evaluated 32 at a time, so the
+// expensive part runs with full warps. Not for spin-coupled functions (their element is a sum over two
+// determinants, which the bound does not cover) and not for the reference (its table gives p directly).
 template <int W, int MODE>
 __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
     DevState *st = P.st;
     if (st->status) return;
     extern __shared__ __align__(16) unsigned char s_queue[];  // one SpawnQueue per warp
     constexpr int NW = kTile / 32;
-    __shared__ Tables T;
+    constexpr int U = 2;  // attempts of a lane screened side by side
+    __shared__ AttemptTables T;
     __shared__ DetView<W> s_v[NW];
     __shared__ HeavyTab s_tab[NW];
-    __shared__ float s_rcpf[2 * MAXSO + 2];
-    __shared__ unsigned long long s_red[NW * NCNT];
-    load_tables(P, T);
-    load_rcpf(P, s_rcpf);
+    __shared__ __align__(8) unsigned s_pend[NW][31 + 32 * U];  // attempts that passed the screen; last the counters' sums
+    __shared__ float s_rcpf[MAXSO + 2];           // two class counts (at most 64 each) add up to an index
+    static_assert(sizeof(s_pend) >= sizeof(unsigned long long) * NW * NCNT, "room for the counters of every warp");
     const unsigned long long packed = st->heavy_packed;
     const long long nh = min((long long)(packed >> 40), P.heavy_cap);
     const unsigned long long nch = nh > 0 ? (packed & ((1ull << 40) - 1ull)) : 0ull;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // warps take batches of consecutive chunks from a counter by guided self-scheduling: a share of what is left, so
+    // batches are long while much is left (few determinant switches) and single chunks at the end (no tail); lane 0
+    // decides, so every lane of the warp holds the same batch
+    unsigned long long q = 0, qend = 0;  // the batch's next chunk and end
+    auto claim = [&]() {
+        unsigned long long b = 0, size = 1;
+        if (lane == 0) {
+            const unsigned long long taken = *(volatile unsigned long long *)&st->heavy_next;
+            const unsigned long long nwarps = (unsigned long long)gridDim.x * NW;
+            if (taken < nch) {
+                size = max(1ull, min((unsigned long long)kChunkBatch, (nch - taken) / (2ull * nwarps)));
+                b = atomicAdd(&st->heavy_next, size);
+            } else {
+                b = nch;
+            }
+        }
+        b = __shfl_sync(0xFFFFFFFFu, b, 0);
+        size = __shfl_sync(0xFFFFFFFFu, size, 0);
+        q = b;
+        qend = min(b + size, nch);
+        return b < nch;
+    };
+    bool done = !claim();
+    if (!__syncthreads_or(done ? 0 : 1)) return;  // a short list: nothing left for this block
+    load_tables(P, T);
+    for (int k = threadIdx.x; k < MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
     const unsigned iter = (unsigned)st->iter;
     const unsigned chunk = st->heavy_chunk ? st->heavy_chunk : (unsigned)kChunk;
     const DetView<W> *heavy = reinterpret_cast<const DetView<W> *>(P.heavy);
@@ -1389,75 +1632,108 @@ __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
 #pragma unroll
     for (int k = 0; k < NCNT; ++k) cnt[k] = 0;
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     long long cur = -1;
     DetView<W> &v = s_v[warp];
     HeavyTab &tab = s_tab[warp];
+    unsigned *const pend = s_pend[warp];
     SpawnQueue<W> &sq = reinterpret_cast<SpawnQueue<W> *>(s_queue)[warp];
     if (lane == 0) sq.n = 0;
     __syncwarp();
-    // warps take batches of consecutive chunks from a counter: consecutive chunks mostly belong to one
-    // determinant, so a warp still builds few tables, and no warp is left with a tail of work
-    unsigned long long q = 0, qend = 0;
+    const unsigned long long pol = keep_policy();
+    unsigned base = 0, a1 = 0;  // the current chunk's next attempt and end
+    unsigned np = 0;            // queued attempts, all of determinant cur
+    unsigned row_mask = 31u;
+    unsigned seen = 0, kept = 0;  // screened attempts of this warp and those that passed
+    bool direct = (MODE & 2) != 0;  // attempts are evaluated without the screen: where more than half pass it is a loss
+    bool rtab = false, fresh = true;  // fresh: a new batch, whose first record is not known yet
     for (;;) {
-        bool fresh = false;
-        if (q >= qend) {
-            // guided self-scheduling: a share of what is left, so batches are long while much is left (few
-            // determinant switches) and single chunks at the end (no tail); lane 0 decides, so every lane of
-            // the warp holds the same batch
-            unsigned long long b = 0, size = 1;
-            if (lane == 0) {
-                const unsigned long long taken = *(volatile unsigned long long *)&st->heavy_next;
-                const unsigned long long nwarps = (unsigned long long)gridDim.x * NW;
-                if (taken < nch)
-                    size = max(1ull, min((unsigned long long)kChunkBatch, (nch - taken) / (2ull * nwarps)));
-                b = atomicAdd(&st->heavy_next, size);
+        unsigned a = base + lane;
+        bool act = a < a1;
+        if (base < a1 && (direct || rtab)) {
+            base += 32;
+        } else if (!(MODE & 2) && (np >= 32 || base < a1)) {
+            if (np < 32) {
+                bool live[U];
+                attempt_screen<W, MODE, U>(P, T, v, tab, row_mask, a, a1, iter, pol, cnt, live);
+                seen += min(a1 - base, 32u * U);
+                kept -= np;
+                base += 32 * U;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const unsigned m = __ballot_sync(0xFFFFFFFFu, live[u]);
+                    if (live[u]) pend[np + __popc(m & ((1u << lane) - 1u))] = a + 32u * u;
+                    np += __popc(m);
+                }
+                kept += np;
+                direct = 2 * kept > seen;
+                if (np < 32) continue;
             }
-            b = __shfl_sync(0xFFFFFFFFu, b, 0);
-            size = __shfl_sync(0xFFFFFFFFu, size, 0);
-            if (b >= nch) break;
-            q = b;
-            qend = min(b + size, nch);
-            fresh = true;
-        }
-        // record holding chunk q: last record whose first chunk is <= q (searched at the start of a batch)
-        long long r;
-        if (cur < 0 || fresh) {
-            long long lo = 0, hi = nh - 1;
-            while (lo < hi) {
-                const long long mid = (lo + hi + 1) >> 1;
-                if ((unsigned long long)P.heavy_base[mid] <= q) lo = mid; else hi = mid - 1;
-            }
-            r = lo;
-        } else {
-            r = cur;
-            while (r + 1 < nh && (unsigned long long)P.heavy_base[r + 1] <= q) ++r;
-        }
-        if (r != cur) {
-            const unsigned long long *src = reinterpret_cast<const unsigned long long *>(heavy + r);
-            unsigned long long *dstv = reinterpret_cast<unsigned long long *>(&v);
-            for (int k = lane; k < (int)(sizeof(DetView<W>) / 8); k += 32) dstv[k] = src[k];
-            for (int k = lane; k < P.n_elec; k += 32) tab.occ[k] = P.heavy_occ[r * MAXN + k];
             __syncwarp();
-            build_heavy_tab<W>(P, T, v, tab, lane);
-            cur = r;
+            np -= 32;
+            a = pend[np + lane];
+            act = true;
+            __syncwarp();
+        } else {
+            // the next chunk
+            if (!done && q >= qend) {
+                done = !claim();
+                fresh = true;
+            }
+            // record holding chunk q: last record whose first chunk is <= q (searched at the start of a batch)
+            long long r = -1;
+            if (!done) {
+                if (fresh) {
+                    long long lo = 0, hi = nh - 1;
+                    while (lo < hi) {
+                        const long long mid = (lo + hi + 1) >> 1;
+                        if ((unsigned long long)P.heavy_base[mid] <= q) lo = mid; else hi = mid - 1;
+                    }
+                    r = lo;
+                } else {
+                    r = cur;
+                    while (r + 1 < nh && (unsigned long long)P.heavy_base[r + 1] <= q) ++r;
+                }
+            }
+            if (r != cur && np > 0) {
+                // the determinant changes: its queued attempts first (this chunk is taken up again after them)
+                __syncwarp();
+                act = lane < (int)np;
+                a = act ? pend[lane] : 0u;
+                np = 0;
+            } else {
+                if (done) break;
+                if (r != cur) {
+                    __syncwarp();
+                    const unsigned long long *src = reinterpret_cast<const unsigned long long *>(heavy + r);
+                    unsigned long long *dstv = reinterpret_cast<unsigned long long *>(&v);
+                    for (int k = lane; k < (int)(sizeof(DetView<W>) / 8); k += 32) dstv[k] = src[k];
+                    for (int k = lane; k < P.n_elec; k += 32) {
+                        const unsigned so = P.heavy_occ[r * MAXN + k];
+                        tab.occ[k] = (unsigned char)so;
+                        tab.occ2[k] = (unsigned short)(so | ((unsigned)T.irrep[so >> 1] << 8));
+                    }
+                    __syncwarp();
+                    build_heavy_tab<W>(P, T, v, s_rcpf, tab, lane);
+                    cur = r;
+                    rtab = P.ref_tab && v.isref;
+                    row_mask = tab.row_mask;
+                }
+                fresh = false;
+                base = (unsigned)(q - P.heavy_base[r]) * chunk;
+                a1 = min(base + chunk, P.heavy_att[r]);
+                ++q;
+                continue;
+            }
         }
-        const unsigned a0 = (unsigned)(q - P.heavy_base[r]) * chunk;
-        const unsigned a1 = min(a0 + chunk, P.heavy_att[r]);
-        const bool rtab = P.ref_tab && v.isref;
-        for (unsigned base = a0; base < a1; base += 32) {
-            const unsigned a = base + lane;
-            spawn_attempt<W, true, MODE>(P, T, v, tab.occ, &tab, s_rcpf, a < a1, a, iter, cnt, sq, rtab);
-            flush_queue<W>(P, sq, false, T.map1);
-        }
-        __syncwarp();
-        ++q;
+        spawn_attempt<W, true, MODE>(P, T, v, tab.occ, &tab, s_rcpf, act, a, iter, cnt, sq, rtab);
+        flush_queue<W>(P, sq, false, P.map1);
     }
-    flush_queue<W>(P, sq, true, T.map1);
+    flush_queue<W>(P, sq, true, P.map1);
     unsigned long long *const dst[NCNT] = {&st->cnt[0], &st->cnt[1], &st->cnt[2], &st->cnt[3], &st->cnt[4],
                                            &st->cnt[5], &st->cnt[6], &st->cnt[7], &st->cnt[8], &st->cnt[9]};
     cnt[C_ATTEMPTS] = 0;  // attempts are counted by the sweep
-    flush_counters<kTile, NCNT>(cnt, dst, s_red);
+    __syncthreads();
+    flush_counters<kTile, NCNT>(cnt, dst, reinterpret_cast<unsigned long long *>(s_pend));
 }
 
 }  // namespace fq

@@ -320,3 +320,31 @@ def test_compaction_preserves_parity(cap):
     compare_rows(g.history(150), rows_q)
     assert g.estimates()["compactions"] > 0
     g.close()
+
+
+@pytest.mark.parametrize("n_orb,n_elec,n_irrep,space", [
+    (40, 16, 1, {}),                        # one class a spin: every unoccupied orbital is good
+    (24, 12, 8, {}), (36, 20, 8, {}),       # eight irreps, both determinant widths
+    (20, 8, 3, {}),                         # irreps not closed under products
+    (10, 8, 8, {}), (9, 10, 4, {}),         # classes of one or two orbitals: empty good sets, null excitations
+    (34, 36, 2, {}),                        # more electrons than lanes
+    (24, 12, 8, dict(max_excitation=3)),    # rejected attempts outside the permitted space are null excitations
+    (36, 20, 8, dict(max_seniority=6)),
+])
+def test_screened_attempts_every_iteration(n_orb, n_elec, n_irrep, space):
+    """Attempts that the spawning kernels reject from a bound of the matrix element over the last virtual: light and
+    heavily populated determinants, lists, counters (null excitations among them) and merged spawns as the oracle's."""
+    s = synth.make_system(n_orb, n_elec, seed=7 * n_orb + n_elec, n_chol=12)
+    s.irrep = (np.arange(n_orb) % n_irrep).astype(np.int32)
+    g, q = make_pair(s, 0.004, 2, seed=9, main_capacity=1 << 18, spawn_capacity=1 << 18, **space)
+    dets, pops = synth.walker_snapshot(s, 6_000, seed=4)
+    keep = np.array([q.in_space(d) for d in dets])
+    dets, pops = dets[keep], pops[keep]
+    rng = np.random.default_rng(1)
+    pops = (pops * np.where(rng.random(len(pops)) < 0.1, 150, 1)).astype(np.int32)  # a tenth above the heavy threshold
+    for x in (g, q):
+        x.set_walkers(dets, pops, iteration=3, shift=0.3)
+    rows_g, rows_q = run_lockstep(g, q, 5)
+    compare_rows(rows_g, rows_q)
+    assert rows_g[0]["heavy_attempts"] > 0 and rows_g[0]["attempts"] > rows_g[0]["heavy_attempts"]
+    g.close()
