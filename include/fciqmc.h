@@ -442,8 +442,8 @@ void fciqmc_rdm_destroy(fciqmc_rdm *r);
  *                   beyond 2 n_orb (closed-shell with FCIQMC_STATIC_SPIN_COUPLED).
  *   dets_dev        device, n_dets x W words; pops_dev device, n_dets int32.
  *   flags           0 or FCIQMC_STATIC_SPIN_COUPLED.
- *   out_dev         device, 5 doubles, written by the last kernel.
- *   cuda_stream     stream the three kernels are enqueued on (asynchronous).
+ *   out_dev         device, 5 doubles, written by the call's kernel.
+ *   cuda_stream     stream the work is enqueued on (asynchronous).
  * Returns FCIQMC_ERR_CAPACITY, before launching anything, if n_dets >
  * FCIQMC_STATIC_MAX_DETS; FCIQMC_ERR_UNSUPPORTED for sizes beyond the
  * library's limits; FCIQMC_ERR_INVALID_ARG for null pointers, unknown flags or
