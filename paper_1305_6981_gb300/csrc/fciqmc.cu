@@ -436,6 +436,16 @@ int load_list(fciqmc_handle *h, const DevState &cur, DevState &st0, const uint64
     return FCIQMC_OK;
 }
 
+// The newest n of `total` rows written to a ring of cap rows, oldest first: one copy, or two around the ring's end
+// (a copy per row took 5 us each).
+int copy_rows(fciqmc_row *rows, const fciqmc_row *ring, long long total, long long n, long long cap, cudaStream_t s) {
+    const long long at = (total - n) % cap, first = std::min(n, cap - at);
+    if (first > 0) FQ_CUDA(cudaMemcpyAsync(rows, ring + at, sizeof(fciqmc_row) * first, cudaMemcpyDeviceToHost, s));
+    if (n > first) FQ_CUDA(cudaMemcpyAsync(rows + first, ring, sizeof(fciqmc_row) * (n - first), cudaMemcpyDeviceToHost, s));
+    FQ_CUDA(cudaStreamSynchronize(s));
+    return FCIQMC_OK;
+}
+
 int read_state(fciqmc_handle *h, DevState &st) {
     FQ_CUDA(cudaMemcpyAsync(&st, h->P.st, sizeof(DevState), cudaMemcpyDeviceToHost, h->stream));
     FQ_CUDA(cudaStreamSynchronize(h->stream));
@@ -960,11 +970,8 @@ int fciqmc_history(fciqmc_handle *h, fciqmc_row *rows, int64_t max_rows, int64_t
     if (rc != FCIQMC_OK) return rc;
     const long long avail = std::min<long long>(s.hist_n, h->z.hist_cap);
     const long long n = std::min<long long>(avail, max_rows);
-    for (long long k = 0; k < n; ++k) {
-        long long idx = (s.hist_n - n + k) % h->z.hist_cap;
-        FQ_CUDA(cudaMemcpyAsync(rows + k, h->P.hist + idx, sizeof(fciqmc_row), cudaMemcpyDeviceToHost, h->stream));
-    }
-    FQ_CUDA(cudaStreamSynchronize(h->stream));
+    rc = copy_rows(rows, h->P.hist, s.hist_n, n, h->z.hist_cap, h->stream);
+    if (rc != FCIQMC_OK) return rc;
     *n_rows = n;
     return FCIQMC_OK;
 }
@@ -1405,11 +1412,8 @@ int fciqmc_group_history(fciqmc_group *g, fciqmc_row *rows, int64_t max_rows, in
     FQ_CUDA(cudaStreamSynchronize(g->stream));
     const long long avail = std::min<long long>(d.hist_n, g->hist_cap);
     const long long n = std::min<long long>(avail, max_rows);
-    for (long long k = 0; k < n; ++k) {
-        const long long idx = (d.hist_n - n + k) % g->hist_cap;
-        FQ_CUDA(cudaMemcpyAsync(rows + k, g->ghist + idx, sizeof(fciqmc_row), cudaMemcpyDeviceToHost, g->stream));
-    }
-    FQ_CUDA(cudaStreamSynchronize(g->stream));
+    const int rc = copy_rows(rows, g->ghist, d.hist_n, n, g->hist_cap, g->stream);
+    if (rc != FCIQMC_OK) return rc;
     *n_rows = n;
     return FCIQMC_OK;
 }
