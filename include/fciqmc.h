@@ -350,19 +350,21 @@ int fciqmc_get_state(fciqmc_handle *h, fciqmc_state *st);
 /* Facts fixed at creation. Not synchronising. */
 int fciqmc_get_info(const fciqmc_handle *h, fciqmc_info *info);
 
-/* Kernels of one iteration, in launch order (indices into the kernel_ms array
+/* Steps of one iteration, in launch order (indices into the kernel_ms array
  * of fciqmc_profile). */
 #define FCIQMC_N_KERNELS 8
-/* 0 compact_copy, 1 index_clear (three launches: the whole index, or the old
- * list's entries located then emptied), 2 index_fill, 3 compact_finish (no-ops unless
- * a compaction is due), 4 sweep (estimators, death, spawning), 5 heavy
- * (spawning from determinants with more than 256 walkers), 6 annihilate (with
- * the diagonal elements of the determinants it placed in new slots: two
- * launches), 7 finish (reductions, shift). */
+/* 0 compact_copy (with the old list's index entries located, or the whole index
+ * emptied), 1 index_clear (the located entries emptied), 2 index_fill (whose
+ * last block makes the compacted list the active one), 3 compact_finish (part of
+ * 2: no launch); 0 to 3 are no-ops unless a compaction is due; 4 sweep (estimators,
+ * death, spawning), 5 heavy (spawning from heavily populated determinants), 6
+ * annihilate (and the diagonal elements of the determinants it placed in new
+ * slots: two launches, three with an occupation threshold), 7 finish
+ * (reductions, shift: part of 6, a launch with an occupation threshold). */
 
 /* Synchronising: runs n_iterations iterations exactly as fciqmc_step does, but
- * launching each kernel individually between CUDA events on the run's stream,
- * and adds each kernel's elapsed milliseconds, summed over the iterations,
+ * launching each step individually between CUDA events on the run's stream,
+ * and adds each step's elapsed milliseconds, summed over the iterations,
  * into kernel_ms[FCIQMC_N_KERNELS] (host array, not cleared). */
 int fciqmc_profile(fciqmc_handle *h, int32_t n_iterations, double *kernel_ms);
 

@@ -249,38 +249,46 @@ int configure_kernels(fciqmc_handle *h) {
 // The spawning kernels, instantiated with the permitted-space test only for runs that have one.
 int spawn_mode(const fciqmc_handle *h) { return (h->P.space ? 1 : 0) | (h->P.hphf ? 2 : 0); }
 template <int W>
-void launch_sweep(fciqmc_handle *h, cudaStream_t s) {
-    if (W == 1) fq::launch_sweep_w1(spawn_mode(h), h->sweep_grid, s, h->P);
-    else fq::launch_sweep_w2(spawn_mode(h), h->sweep_grid, s, h->P);
+void launch_sweep(fciqmc_handle *h, cudaStream_t s, bool next) {
+    if (W == 1) fq::launch_sweep_w1(spawn_mode(h), h->sweep_grid, s, next, h->P);
+    else fq::launch_sweep_w2(spawn_mode(h), h->sweep_grid, s, next, h->P);
 }
 template <int W>
-void launch_heavy(fciqmc_handle *h, cudaStream_t s) {
-    if (W == 1) fq::launch_heavy_w1(spawn_mode(h), h->heavy_grid, s, h->P);
-    else fq::launch_heavy_w2(spawn_mode(h), h->heavy_grid, s, h->P);
+void launch_heavy(fciqmc_handle *h, cudaStream_t s, bool next) {
+    if (W == 1) fq::launch_heavy_w1(spawn_mode(h), h->heavy_grid, s, next, h->P);
+    else fq::launch_heavy_w2(spawn_mode(h), h->heavy_grid, s, next, h->P);
 }
+
+// The steps of an iteration as fciqmc_profile names them (a step may be several launches or part of another's:
+// compact_finish is done by index_fill's last block, finish by annihilate's, except with hybrid walkers).
+enum { STEP_COPY = 0, STEP_CLEAR, STEP_FILL, STEP_COMPACT_FINISH, STEP_SWEEP, STEP_HEAVY, STEP_ANNIHILATE, STEP_FINISH };
+static_assert(STEP_FINISH + 1 == FCIQMC_N_KERNELS, "steps of fciqmc_profile");
+// next: each launch depends programmatically on the one before (launch_next); the first of an iteration never does.
 template <int W>
-void launch_spawning(fciqmc_handle *h, cudaStream_t s) {
-    launch_sweep<W>(h, s);
-    launch_heavy<W>(h, s);
-    // the sweep tiles' numerators are summed after k_heavy, which does not need them: the 32-block sum then
-    // does not sit between the two spawning kernels
-    fq::k_tile_sum<<<fq::kTileSums, 256, 0, s>>>(h->P);
+void enqueue_step(fciqmc_handle *h, cudaStream_t s, int step, bool next) {
+    const Params &P = h->P;
+    const bool rounds = P.occ_units > 1;
+    switch (step) {
+        case STEP_COPY: fq::launch_next(fq::k_compact_copy<W>, h->small_grid, 256, 0, s, false, P); break;
+        case STEP_CLEAR: fq::launch_next(fq::k_index_clear_old<W>, h->small_grid, 256, 0, s, next, P); break;
+        case STEP_FILL: fq::launch_next(fq::k_index_fill<W>, h->small_grid, 256, 0, s, next, P, 0); break;
+        case STEP_SWEEP: launch_sweep<W>(h, s, next); break;
+        case STEP_HEAVY: launch_heavy<W>(h, s, next); break;
+        case STEP_ANNIHILATE:
+            fq::launch_next(fq::k_annihilate<W>, h->ann_grid, 256, 0, s, next, P, rounds ? 0 : 1);
+            fq::launch_next(fq::k_new_diag<W>, h->diag_grid, fq::kDiagThreads, h->smem_d, s, next, P);
+            if (rounds) fq::launch_next(fq::k_round<W>, h->small_grid, 256, 0, s, next, P);
+            break;
+        case STEP_FINISH:
+            if (rounds) fq::launch_next(fq::k_finish, 1, 32, 0, s, next, P);
+            break;
+        default: break;
+    }
 }
 
 template <int W>
 void enqueue_iteration(fciqmc_handle *h, cudaStream_t s) {
-    const Params &P = h->P;
-    fq::k_compact_copy<W><<<h->small_grid, 256, 0, s>>>(P);
-    fq::k_index_clear<<<h->small_grid, 256, 0, s>>>(P, 0);
-    fq::k_index_locate_old<W><<<h->small_grid, 256, 0, s>>>(P);
-    fq::k_index_clear_old<W><<<h->small_grid, 256, 0, s>>>(P);
-    fq::k_index_fill<W><<<h->small_grid, 256, 0, s>>>(P, 0);
-    fq::k_compact_finish<<<1, 32, 0, s>>>(P);
-    launch_spawning<W>(h, s);
-    fq::k_annihilate<W><<<h->ann_grid, 256, 0, s>>>(P);
-    fq::k_new_diag<W><<<h->diag_grid, fq::kDiagThreads, h->smem_d, s>>>(P);
-    if (P.occ_units > 1) fq::k_round<W><<<h->small_grid, 256, 0, s>>>(P);
-    fq::k_finish<<<1, 32, 0, s>>>(P);
+    for (int step = 0; step < FCIQMC_N_KERNELS; ++step) enqueue_step<W>(h, s, step, true);
 }
 
 void enqueue(fciqmc_handle *h, cudaStream_t s) {
@@ -308,7 +316,7 @@ int build_graph(fciqmc_handle *h) {
 
 template <int W>
 void launch_index_rebuild(fciqmc_handle *h) {
-    fq::k_index_clear<<<h->small_grid, 256, 0, h->stream>>>(h->P, 1);
+    fq::k_index_clear<<<h->small_grid, 256, 0, h->stream>>>(h->P);
     fq::k_index_fill<W><<<h->small_grid, 256, 0, h->stream>>>(h->P, 1);
 }
 
@@ -364,7 +372,7 @@ int load_stage(fciqmc_handle *h, const DevState &cur, const uint64_t *dets, cons
         fq::k_index_locate<W><<<ob, 256, 0, a>>>(P, cur.lb, cur.list_len, pos);
         fq::k_index_clear_at<W><<<ob, 256, 0, a>>>(P, pos, cur.list_len);
     } else if (!sparse) {
-        fq::k_index_clear<<<h->small_grid, 256, 0, a>>>(P, 1);
+        fq::k_index_clear<<<h->small_grid, 256, 0, a>>>(P);
     }
     const int nchunk = (int)std::min<long long>(8, std::max<long long>(1, n >> 20));  // >= 2^20 keys a chunk
     for (int k = 0; k < nchunk; ++k) {
@@ -418,7 +426,7 @@ int load_list(fciqmc_handle *h, const DevState &cur, DevState &st0, const uint64
         cudaStreamSynchronize(h->aux);
         cudaStreamSynchronize(h->aux2);
         cudaStreamSynchronize(s);
-        fq::k_index_clear<<<h->small_grid, 256, 0, s>>>(P, 1);
+        fq::k_index_clear<<<h->small_grid, 256, 0, s>>>(P);
         fq::k_index_fill<W><<<h->small_grid, 256, 0, s>>>(P, 1);
         FQ_CUDA(cudaGetLastError());
         FQ_CUDA(cudaStreamSynchronize(s));
@@ -856,7 +864,6 @@ int fciqmc_profile(fciqmc_handle *h, int32_t n_iterations, double *kernel_ms) {
     if (!h || !kernel_ms || n_iterations < 0 || h->z.n_parts > 1) return FCIQMC_ERR_INVALID_ARG;
     cudaEvent_t ev[FCIQMC_N_KERNELS + 1];
     for (int k = 0; k <= FCIQMC_N_KERNELS; ++k) FQ_CUDA(cudaEventCreate(&ev[k]));
-    const Params &P = h->P;
     cudaStream_t s = h->stream;
     static const char *const kNames[FCIQMC_N_KERNELS] = {"compact_copy", "index_clear", "index_fill", "compact_finish",
                                                          "sweep", "heavy", "annihilate", "finish"};
@@ -864,51 +871,8 @@ int fciqmc_profile(fciqmc_handle *h, int32_t n_iterations, double *kernel_ms) {
         cudaEventRecord(ev[0], s);
         for (int k = 0; k < FCIQMC_N_KERNELS; ++k) {
             NvtxRange range(kNames[k]);
-            if (h->z.W == 1) {
-                switch (k) {
-                    case 0: fq::k_compact_copy<1><<<h->small_grid, 256, 0, s>>>(P); break;
-                    case 1:
-                        fq::k_index_clear<<<h->small_grid, 256, 0, s>>>(P, 0);
-                        fq::k_index_locate_old<1><<<h->small_grid, 256, 0, s>>>(P);
-                        fq::k_index_clear_old<1><<<h->small_grid, 256, 0, s>>>(P);
-                        break;
-                    case 2: fq::k_index_fill<1><<<h->small_grid, 256, 0, s>>>(P, 0); break;
-                    case 3: fq::k_compact_finish<<<1, 32, 0, s>>>(P); break;
-                    case 4:
-                        launch_sweep<1>(h, s);
-                        fq::k_tile_sum<<<fq::kTileSums, 256, 0, s>>>(P);
-                        break;
-                    case 5: launch_heavy<1>(h, s); break;
-                    case 6:
-                        fq::k_annihilate<1><<<h->ann_grid, 256, 0, s>>>(P);
-                        fq::k_new_diag<1><<<h->diag_grid, fq::kDiagThreads, h->smem_d, s>>>(P);
-                        if (P.occ_units > 1) fq::k_round<1><<<h->small_grid, 256, 0, s>>>(P);
-                        break;
-                    default: fq::k_finish<<<1, 32, 0, s>>>(P); break;
-                }
-            } else {
-                switch (k) {
-                    case 0: fq::k_compact_copy<2><<<h->small_grid, 256, 0, s>>>(P); break;
-                    case 1:
-                        fq::k_index_clear<<<h->small_grid, 256, 0, s>>>(P, 0);
-                        fq::k_index_locate_old<2><<<h->small_grid, 256, 0, s>>>(P);
-                        fq::k_index_clear_old<2><<<h->small_grid, 256, 0, s>>>(P);
-                        break;
-                    case 2: fq::k_index_fill<2><<<h->small_grid, 256, 0, s>>>(P, 0); break;
-                    case 3: fq::k_compact_finish<<<1, 32, 0, s>>>(P); break;
-                    case 4:
-                        launch_sweep<2>(h, s);
-                        fq::k_tile_sum<<<fq::kTileSums, 256, 0, s>>>(P);
-                        break;
-                    case 5: launch_heavy<2>(h, s); break;
-                    case 6:
-                        fq::k_annihilate<2><<<h->ann_grid, 256, 0, s>>>(P);
-                        fq::k_new_diag<2><<<h->diag_grid, fq::kDiagThreads, h->smem_d, s>>>(P);
-                        if (P.occ_units > 1) fq::k_round<2><<<h->small_grid, 256, 0, s>>>(P);
-                        break;
-                    default: fq::k_finish<<<1, 32, 0, s>>>(P); break;
-                }
-            }
+            if (h->z.W == 1) enqueue_step<1>(h, s, k, false);
+            else enqueue_step<2>(h, s, k, false);
             cudaEventRecord(ev[k + 1], s);
         }
         FQ_CUDA(cudaGetLastError());
@@ -1262,20 +1226,12 @@ GroupLayout group_layout(int n, long long hist_cap) {
 template <int W>
 void enqueue_group_iteration(fciqmc_group *g, cudaStream_t s) {
     const int n = (int)g->parts.size();
-    for (fciqmc_handle *h : g->parts) {
-        const Params &P = h->P;
-        fq::k_compact_copy<W><<<h->small_grid, 256, 0, s>>>(P);
-        fq::k_index_clear<<<h->small_grid, 256, 0, s>>>(P, 0);
-        fq::k_index_locate_old<W><<<h->small_grid, 256, 0, s>>>(P);
-        fq::k_index_clear_old<W><<<h->small_grid, 256, 0, s>>>(P);
-        fq::k_index_fill<W><<<h->small_grid, 256, 0, s>>>(P, 0);
-        fq::k_compact_finish<<<1, 32, 0, s>>>(P);
-    }
-    for (fciqmc_handle *h : g->parts) launch_spawning<W>(h, s);
+    for (fciqmc_handle *h : g->parts)
+        for (int step = STEP_COPY; step <= STEP_HEAVY; ++step) enqueue_step<W>(h, s, step, false);
     // the exchange: each partition merges the spawns the others routed to it
     for (fciqmc_handle *h : g->parts) fq::k_receive<W><<<h->ann_grid, 256, 0, s>>>(h->P, g->links);
     for (fciqmc_handle *h : g->parts) {
-        fq::k_annihilate<W><<<h->ann_grid, 256, 0, s>>>(h->P);
+        fq::k_annihilate<W><<<h->ann_grid, 256, 0, s>>>(h->P, 0);
         fq::k_new_diag<W><<<h->diag_grid, fq::kDiagThreads, h->smem_d, s>>>(h->P);
         if (h->P.occ_units > 1) fq::k_round<W><<<h->small_grid, 256, 0, s>>>(h->P);
     }

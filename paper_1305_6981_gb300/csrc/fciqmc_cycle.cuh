@@ -7,14 +7,186 @@
 
 namespace fq {
 
+// Natural logarithm from the atanh series (shift update); same operation order as the oracle's.
+__device__ double own_log(double x) {
+    const double LN2_HI = 0x1.62e42fe800000p-1;
+    const double LN2_LO = 0x1.e8e7bcd5e4f1ep-31;
+    const double SQRT2 = 0x1.6a09e667f3bcdp+0;
+    if (!(x > 0.0)) return x == 0.0 ? -CUDART_INF : CUDART_NAN;
+    if (isinf(x)) return x;
+    int e = 0;
+    if (x < 0x1.0p-1022) { x = __dmul_rn(x, 0x1.0p54); e = -54; }
+    unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+    e += (int)((bits >> 52) & 0x7FFull) - 1023;
+    bits = (bits & 0x000FFFFFFFFFFFFFull) | 0x3FF0000000000000ull;
+    double m = __longlong_as_double((long long)bits);
+    if (m > SQRT2) { m = __dmul_rn(m, 0.5); e += 1; }
+    double s = __ddiv_rn(__dsub_rn(m, 1.0), __dadd_rn(m, 1.0));
+    double z = __dmul_rn(s, s);
+    double poly = __ddiv_rn(1.0, 23.0);
+    for (int k = 10; k >= 0; --k) poly = __dadd_rn(__dmul_rn(poly, z), __ddiv_rn(1.0, (double)(2 * k + 1)));
+    double t = __dmul_rn(s, poly);
+    double lnm = __dadd_rn(t, t);
+    double de = (double)e;
+    double r = __dadd_rn(lnm, __dmul_rn(de, LN2_LO));
+    return __dadd_rn(__dmul_rn(de, LN2_HI), r);
+}
+
+// The iteration's row for one list: its estimators (start of the iteration) and counters; num is the
+// Eq. 2 numerator of the list.
+__device__ __forceinline__ fciqmc_row list_row(const volatile DevState *st, double num) {
+    fciqmc_row row;
+    const long long nw_in = (long long)st->nw_in, nd_in = (long long)st->nd_in;
+    row.iteration = st->iter;
+    row.shift = st->shift;
+    row.nw_in = nw_in;
+    row.nd_in = nd_in;
+    row.c0_in = st->c0_in;
+    row.num_in = num;
+    row.nw_out = nw_in + (long long)st->d_nw;
+    row.nd_out = nd_in + (long long)st->d_nd;
+    row.attempts = (long long)st->cnt[C_ATTEMPTS];
+    row.nulls = (long long)st->cnt[C_NULLS];
+    row.spawn_events = (long long)st->cnt[C_EVENTS];
+    row.spawned_walkers = (long long)st->cnt[C_SPAWNED];
+    row.death_walkers = (long long)st->cnt[C_DEATH];
+    row.clone_walkers = (long long)st->cnt[C_CLONE];
+    row.merged_entries = (long long)st->n_merged;
+    row.aborted_walkers = (long long)st->cnt[C_ABORTED];
+    row.inserted_dets = (long long)st->cnt[C_INSERTED];
+    row.heavy_attempts = (long long)st->cnt[C_HEAVY];
+    return row;
+}
+
+// Shift update of the run: S <- S - zeta/(A tau) ln(N_w(n) / N_w(n-A)) every A iterations once N_w reached
+// the target (nw_out: the whole run's walkers after the iteration).
+__device__ __forceinline__ void shift_update(DevState *st, long long nw_out, long long target, int period, double c_shift) {
+    if (!st->vary) {
+        if (nw_out >= target) { st->vary = 1; st->nw_prev = nw_out; st->n_since = 0; }
+    } else {
+        st->n_since++;
+        if (st->n_since == period) {
+            double ratio = __ddiv_rn((double)nw_out, (double)st->nw_prev);
+            st->shift = __dsub_rn(st->shift, __dmul_rn(c_shift, own_log(ratio)));
+            st->nw_prev = nw_out;
+            st->n_since = 0;
+        }
+    }
+}
+
+// Heavy chunk size for the next iteration from its expected attempts: the least that gives every k_heavy warp at most
+// one chunk, from kChunkLeast to kChunk (a warp that takes several small chunks pays for each claim: with eight chunks
+// per warp k_heavy took 112 us instead of 93 on 6e6 walkers of 24e/60o; chunks of 512 serial attempts for a
+// tenth of the warps took 90 instead of 47 on 3.6e4 walkers of 8e/8o), and on up to kChunkGrowth kChunk while every
+// warp gets kChunksPerWarp chunks (fewer table builds and batch claims).
+__device__ __forceinline__ unsigned next_chunk(long long attempts, long long warps) {
+    unsigned c = kChunkLeast;
+    while (c < (unsigned)kChunk && attempts > (long long)c * warps) c *= 2u;
+    while (c >= (unsigned)kChunk && c < (unsigned)(kChunkGrowth * kChunk) && attempts >= 2ll * c * kChunksPerWarp * warps) c *= 2u;
+    return c;
+}
+
+// Sweep tile for the next iteration: kTile, halved while there is not a tile for every fourth block, so that a list of
+// a few hundred determinants is spread over the SMs (8e/8o, 500 slots: 40 to 33 us). Longer lists keep whole tiles:
+// with two tiles for every block as the bound, 6e5 slots took 109 instead of 88 us.
+__device__ __forceinline__ int next_tile(long long slots, long long blocks) {
+    int t = kTile;
+    while (t > kTileLeast && (slots + t - 1) / t * 4 < blocks) t >>= 1;
+    return t;
+}
+
+// Makes the iteration's list the current one (new slots included, populations' parity flipped), decides a
+// compaction and the heavy chunk size for the next iteration (attempts: its expected spawning attempts) and
+// clears the per-iteration counters.
+__device__ __forceinline__ void commit_list(DevState *st, long long nd_out, long long cap, long long attempts,
+                                            long long heavy_warps, long long sweep_blocks) {
+    const long long new_len = (long long)*(volatile unsigned long long *)&st->claim;
+    st->list_len = new_len;
+    st->pp ^= 1;
+    st->iter++;
+    const long long vacated = new_len - nd_out;
+    if ((vacated > 64 && vacated * 4 > new_len) || (vacated > 0 && new_len * 4 > cap * 3))
+        st->compact_pending = 1;
+    st->n_merged = 0;
+    st->heavy_packed = 0;
+    st->nw_in = st->nd_in = 0;
+    st->c0_in = 0;
+    st->d_nw = st->d_nd = 0;
+    st->n_new = 0;
+    st->sweep_next = 0;
+    st->heavy_next = 0;
+    st->heavy_chunk = next_chunk(attempts, heavy_warps);
+    st->tile = next_tile(new_len, sweep_blocks);
+    // a short list leaves most sweep blocks without a tile, and each tile's light attempts run in one block:
+    // then the heavy path, whose chunks spread over every warp, takes determinants from 32 walkers on
+    st->heavy_thr = (new_len + kTile - 1) / kTile * 4 < sweep_blocks ? (unsigned)kHeavyShort : (unsigned)kHeavy;
+    for (int k = 0; k < NCNT; ++k) st->cnt[k] = 0;
+    for (int k = 0; k < MAXPARTS; ++k) st->ob_n[k] = 0;
+}
+
+// Range sums of the sweep tiles' numerators: range b holds the tiles [b n / kTileSums, (b + 1) n / kTileSums), added in a
+// fixed order (thread t takes tiles t, t + 256, ... of the range, then the block's fixed tree), so the run's
+// numerator is the same in every run; the FP64 adds are spread over kTileSums blocks (256 threads each).
+__device__ __forceinline__ void sum_tiles(const Params &P) {
+    __shared__ double s_sum[256 / 32];
+    const DevState *st = P.st;
+    const int tile = st->tile ? st->tile : kTile;
+    const long long n = (st->list_len + tile - 1) / tile;
+    for (int r = blockIdx.x; r < kTileSums; r += gridDim.x) {
+        const long long lo = n * r / kTileSums, hi = n * (r + 1) / kTileSums;
+        double v = 0.0;
+        for (long long t = lo + threadIdx.x; t < hi; t += blockDim.x) v = __dadd_rn(v, P.partial[t]);
+        const double bs = block_sum_f64<256>(v, s_sum);
+        if (threadIdx.x == 0) P.partial[P.tiles_cap + r] = bs;
+        __syncthreads();
+    }
+}
+
+// Eq. 2 numerator of one list: the kTileSums range sums added by one warp in a fixed order (lane k takes sum
+// k, then a fixed shuffle tree); lane 0 holds it.
+__device__ __forceinline__ double list_numerator(const double *range_sums) {
+    const int lane = threadIdx.x & 31;
+    double part = 0.0;
+    for (int b = lane; b < kTileSums; b += 32) part = __dadd_rn(part, __ldcg(range_sums + b));
+    return warp_sum_f64(part);
+}
+
+// End of an iteration of an unpartitioned run (one warp): history row, shift update, the list committed. The state is
+// read past L1: other blocks of the same kernel may have written it.
+__device__ __forceinline__ void end_iteration(const Params &P) {
+    DevState *st = P.st;
+    const double num = list_numerator(P.partial + P.tiles_cap);
+    if (threadIdx.x != 0) return;
+    const fciqmc_row row = list_row(st, num);
+    P.hist[st->hist_n % P.hist_cap] = row;
+    st->hist_n++;
+    shift_update(st, row.nw_out, P.target, P.period, P.c_shift);
+    commit_list(st, row.nd_out, P.cap, row.nw_out >> P.frac_bits, P.heavy_warps, P.sweep_blocks);
+}
+
+// The same as a launch of its own, after k_round.
+__global__ void k_finish(Params P) {
+    grid_next();
+    grid_wait();
+    if (P.st->status) return;
+    end_iteration(P);
+}
+
 // New determinants get a slot, their population and an index entry here; their diagonal elements are
 // computed by k_new_diag over the list of new slots, where every lane of a warp has one (inserting lanes
 // are a minority of each warp here, and H_ii is a long FP64 sum).
+//
+// Two things ride along, to save launches: the first kTileSums blocks add the sweep tiles' numerators (sum_tiles), and
+// with `commit` the last block to finish ends the iteration (end_iteration; hybrid walkers still have k_round to come,
+// and a partitioned run ends in k_group_finish).
 template <int W>
-__global__ void __launch_bounds__(256) k_annihilate(Params P) {
+__global__ void __launch_bounds__(256) k_annihilate(Params P, int commit) {
     __shared__ unsigned long long s_red[(256 / 32) * 4];
     DevState *st = P.st;
+    grid_next();
+    grid_wait();
     if (st->status) return;
+    sum_tiles(P);
     constexpr int S = Stride<W>::v;
     const unsigned long long nm = st->n_merged;
     const long long len = st->list_len;
@@ -119,6 +291,13 @@ __global__ void __launch_bounds__(256) k_annihilate(Params P) {
     unsigned long long accv[4] = {dnw, dnd, aborted, inserted};
     unsigned long long *const dst[4] = {&st->d_nw, &st->d_nd, &st->cnt[C_ABORTED], &st->cnt[C_INSERTED]};
     flush_counters<256, 4>(accv, dst, s_red);
+    if (!last_block(st)) return;
+    if (threadIdx.x == 0) {
+        st->diag_n = (long long)*(volatile unsigned long long *)&st->n_new;
+        st->diag_pp = pp;
+    }
+    __syncthreads();
+    if (commit && threadIdx.x < 32 && !*(volatile int *)&st->status) end_iteration(P);
 }
 
 // Threads of the kernels that evaluate diagonal elements, and their dynamic shared memory: the pair terms and h_pp, then
@@ -154,15 +333,17 @@ template <int W>
 __global__ void __launch_bounds__(kDiagThreads) k_new_diag(Params P) {
     extern __shared__ __align__(16) double s_w[];
     DevState *st = P.st;
-    if (st->status) return;
-    const long long n = (long long)st->n_new;
-    if ((long long)blockIdx.x * blockDim.x >= n) return;
     __shared__ Tables T;
+    grid_next();
     load_tables(P, T);
     unsigned char *occ = load_diag_tables(P, s_w);
+    grid_wait();
+    if (st->status) return;
+    const long long n = st->diag_n;
+    if ((long long)blockIdx.x * blockDim.x >= n) return;
     __syncthreads();
-    const int lb = st->lb, pp = st->pp;
-    const int *new_slots = P.pop[lb][pp];
+    const int lb = st->lb;
+    const int *new_slots = P.pop[lb][st->diag_pp];
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
         const long long s = new_slots[k];
         unsigned long long key[W];
@@ -182,6 +363,8 @@ template <int W>
 __global__ void __launch_bounds__(256) k_round(Params P) {
     __shared__ unsigned long long s_red[(256 / 32) * 2];
     DevState *st = P.st;
+    grid_next();
+    grid_wait();
     if (st->status) return;
     const int lb = st->lb, pp = st->pp;
     int *pop_out = P.pop[lb][pp ^ 1];
@@ -205,161 +388,6 @@ __global__ void __launch_bounds__(256) k_round(Params P) {
     unsigned long long accv[2] = {dnw, dnd};
     unsigned long long *const dst[2] = {&st->d_nw, &st->d_nd};
     flush_counters<256, 2>(accv, dst, s_red);
-}
-
-// Natural logarithm from the atanh series (shift update); same operation order as the oracle's.
-__device__ double own_log(double x) {
-    const double LN2_HI = 0x1.62e42fe800000p-1;
-    const double LN2_LO = 0x1.e8e7bcd5e4f1ep-31;
-    const double SQRT2 = 0x1.6a09e667f3bcdp+0;
-    if (!(x > 0.0)) return x == 0.0 ? -CUDART_INF : CUDART_NAN;
-    if (isinf(x)) return x;
-    int e = 0;
-    if (x < 0x1.0p-1022) { x = __dmul_rn(x, 0x1.0p54); e = -54; }
-    unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-    e += (int)((bits >> 52) & 0x7FFull) - 1023;
-    bits = (bits & 0x000FFFFFFFFFFFFFull) | 0x3FF0000000000000ull;
-    double m = __longlong_as_double((long long)bits);
-    if (m > SQRT2) { m = __dmul_rn(m, 0.5); e += 1; }
-    double s = __ddiv_rn(__dsub_rn(m, 1.0), __dadd_rn(m, 1.0));
-    double z = __dmul_rn(s, s);
-    double poly = __ddiv_rn(1.0, 23.0);
-    for (int k = 10; k >= 0; --k) poly = __dadd_rn(__dmul_rn(poly, z), __ddiv_rn(1.0, (double)(2 * k + 1)));
-    double t = __dmul_rn(s, poly);
-    double lnm = __dadd_rn(t, t);
-    double de = (double)e;
-    double r = __dadd_rn(lnm, __dmul_rn(de, LN2_LO));
-    return __dadd_rn(__dmul_rn(de, LN2_HI), r);
-}
-
-// The iteration's row for one list: its estimators (start of the iteration) and counters; num is the
-// Eq. 2 numerator of the list.
-__device__ __forceinline__ fciqmc_row list_row(const DevState *st, double num) {
-    fciqmc_row row;
-    const long long nw_in = (long long)st->nw_in, nd_in = (long long)st->nd_in;
-    row.iteration = st->iter;
-    row.shift = st->shift;
-    row.nw_in = nw_in;
-    row.nd_in = nd_in;
-    row.c0_in = st->c0_in;
-    row.num_in = num;
-    row.nw_out = nw_in + (long long)st->d_nw;
-    row.nd_out = nd_in + (long long)st->d_nd;
-    row.attempts = (long long)st->cnt[C_ATTEMPTS];
-    row.nulls = (long long)st->cnt[C_NULLS];
-    row.spawn_events = (long long)st->cnt[C_EVENTS];
-    row.spawned_walkers = (long long)st->cnt[C_SPAWNED];
-    row.death_walkers = (long long)st->cnt[C_DEATH];
-    row.clone_walkers = (long long)st->cnt[C_CLONE];
-    row.merged_entries = (long long)st->n_merged;
-    row.aborted_walkers = (long long)st->cnt[C_ABORTED];
-    row.inserted_dets = (long long)st->cnt[C_INSERTED];
-    row.heavy_attempts = (long long)st->cnt[C_HEAVY];
-    return row;
-}
-
-// Shift update of the run: S <- S - zeta/(A tau) ln(N_w(n) / N_w(n-A)) every A iterations once N_w reached
-// the target (nw_out: the whole run's walkers after the iteration).
-__device__ __forceinline__ void shift_update(DevState *st, long long nw_out, long long target, int period, double c_shift) {
-    if (!st->vary) {
-        if (nw_out >= target) { st->vary = 1; st->nw_prev = nw_out; st->n_since = 0; }
-    } else {
-        st->n_since++;
-        if (st->n_since == period) {
-            double ratio = __ddiv_rn((double)nw_out, (double)st->nw_prev);
-            st->shift = __dsub_rn(st->shift, __dmul_rn(c_shift, own_log(ratio)));
-            st->nw_prev = nw_out;
-            st->n_since = 0;
-        }
-    }
-}
-
-// Heavy chunk size for the next iteration from its expected attempts: the least that gives every k_heavy warp at most
-// one chunk, from kChunkLeast to kChunk (a warp that takes several small chunks pays for each claim: with eight chunks
-// per warp k_heavy took 112 us instead of 93 on 6e6 walkers of 24e/60o; chunks of 512 serial attempts for a
-// tenth of the warps took 90 instead of 47 on 3.6e4 walkers of 8e/8o), and on up to kChunkGrowth kChunk while every
-// warp gets kChunksPerWarp chunks (fewer table builds and batch claims).
-__device__ __forceinline__ unsigned next_chunk(long long attempts, long long warps) {
-    unsigned c = kChunkLeast;
-    while (c < (unsigned)kChunk && attempts > (long long)c * warps) c *= 2u;
-    while (c >= (unsigned)kChunk && c < (unsigned)(kChunkGrowth * kChunk) && attempts >= 2ll * c * kChunksPerWarp * warps) c *= 2u;
-    return c;
-}
-
-// Sweep tile for the next iteration: kTile, halved while there is not a tile for every fourth block, so that a list of
-// a few hundred determinants is spread over the SMs (8e/8o, 500 slots: 40 to 33 us). Longer lists keep whole tiles:
-// with two tiles for every block as the bound, 6e5 slots took 109 instead of 88 us.
-__device__ __forceinline__ int next_tile(long long slots, long long blocks) {
-    int t = kTile;
-    while (t > kTileLeast && (slots + t - 1) / t * 4 < blocks) t >>= 1;
-    return t;
-}
-
-// Makes the iteration's list the current one (new slots included, populations' parity flipped), decides a
-// compaction and the heavy chunk size for the next iteration (attempts: its expected spawning attempts) and
-// clears the per-iteration counters.
-__device__ __forceinline__ void commit_list(DevState *st, long long nd_out, long long cap, long long attempts,
-                                            long long heavy_warps, long long sweep_blocks) {
-    const long long new_len = (long long)st->claim;
-    st->list_len = new_len;
-    st->pp ^= 1;
-    st->iter++;
-    const long long vacated = new_len - nd_out;
-    if ((vacated > 64 && vacated * 4 > new_len) || (vacated > 0 && new_len * 4 > cap * 3))
-        st->compact_pending = 1;
-    st->n_merged = 0;
-    st->heavy_packed = 0;
-    st->nw_in = st->nd_in = 0;
-    st->c0_in = 0;
-    st->d_nw = st->d_nd = 0;
-    st->n_new = 0;
-    st->sweep_next = 0;
-    st->heavy_next = 0;
-    st->heavy_chunk = next_chunk(attempts, heavy_warps);
-    st->tile = next_tile(new_len, sweep_blocks);
-    // a short list leaves most sweep blocks without a tile, and each tile's light attempts run in one block:
-    // then the heavy path, whose chunks spread over every warp, takes determinants from 32 walkers on
-    st->heavy_thr = (new_len + kTile - 1) / kTile * 4 < sweep_blocks ? (unsigned)kHeavyShort : (unsigned)kHeavy;
-    for (int k = 0; k < NCNT; ++k) st->cnt[k] = 0;
-    for (int k = 0; k < MAXPARTS; ++k) st->ob_n[k] = 0;
-}
-
-// Range sums of the sweep tiles' numerators (after k_sweep): block b adds the tiles of its fixed range
-// [b n / kTileSums, (b + 1) n / kTileSums) in a fixed order (thread t takes tiles t, t + 256, ... of the range,
-// then the block's fixed tree), so the run's numerator is the same in every run; the FP64 adds are spread
-// over kTileSums SMs.
-__global__ void __launch_bounds__(256) k_tile_sum(Params P) {
-    __shared__ double s_red[256 / 32];
-    DevState *st = P.st;
-    if (st->status) return;
-    const int tile = st->tile ? st->tile : kTile;
-    const long long n = (st->list_len + tile - 1) / tile;
-    const long long lo = n * blockIdx.x / kTileSums, hi = n * (blockIdx.x + 1) / kTileSums;
-    double v = 0.0;
-    for (long long t = lo + threadIdx.x; t < hi; t += blockDim.x) v = __dadd_rn(v, P.partial[t]);
-    const double bs = block_sum_f64<256>(v, s_red);
-    if (threadIdx.x == 0) P.partial[P.tiles_cap + blockIdx.x] = bs;
-}
-
-// Eq. 2 numerator of one list: the kTileSums range sums added by one warp in a fixed order (lane k takes sum
-// k, then a fixed shuffle tree); lane 0 holds it.
-__device__ __forceinline__ double list_numerator(const double *range_sums) {
-    const int lane = threadIdx.x & 31;
-    double part = 0.0;
-    for (int b = lane; b < kTileSums; b += 32) part = __dadd_rn(part, range_sums[b]);
-    return warp_sum_f64(part);
-}
-
-__global__ void k_finish(Params P) {
-    DevState *st = P.st;
-    if (st->status) return;
-    const double num = list_numerator(P.partial + P.tiles_cap);
-    if (threadIdx.x != 0) return;
-    const fciqmc_row row = list_row(st, num);
-    P.hist[st->hist_n % P.hist_cap] = row;
-    st->hist_n++;
-    shift_update(st, row.nw_out, P.target, P.period, P.c_shift);
-    commit_list(st, row.nd_out, P.cap, row.nw_out >> P.frac_bits, P.heavy_warps, P.sweep_blocks);
 }
 
 // ---------------------------------------------------------------------------- hash-partitioned runs
@@ -461,19 +489,43 @@ __global__ void k_group_finish(const PartLink *links, int n_parts, GroupDev *g, 
 }
 
 // ---------------------------------------------------------------------------- compaction and index
+// A due compaction takes three kernels. The first copies the occupied slots to the other list buffer and, independently,
+// prepares the old entries' removal from the index: with a short list (len * 16 <= index capacity, positions held as
+// int) each old slot's entry is located, into the old buffer's idle population array (no probe chain is cut before
+// every key is found); otherwise the whole index is emptied.
+__device__ __forceinline__ bool sparse_index_clear(const Params &P, const DevState *st) {
+    return st->list_len * 16 <= P.idx_cap && P.idx_cap <= (1LL << 31);
+}
+__device__ __forceinline__ void empty_index(const Params &P) {
+    const long long nwords = P.idx_cap * (P.idx_stride);
+    ulonglong2 *p = reinterpret_cast<ulonglong2 *>(P.idx);
+    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < nwords / 2; k += (long long)gridDim.x * blockDim.x)
+        p[k] = make_ulonglong2(EMPTY, EMPTY);
+}
 template <int W>
 __global__ void k_compact_copy(Params P) {
     DevState *st = P.st;
+    grid_next();
+    grid_wait();
     if (!st->compact_pending || st->status) return;
+    constexpr int S = Stride<W>::v;
     const int lb = st->lb, pp = st->pp;
     const long long len = st->list_len;
+    const bool sparse = sparse_index_clear(P, st);
+    int *pos = P.pop[lb][pp ^ 1];
+    const unsigned long long imask = (unsigned long long)P.idx_cap - 1ull;
+    if (!sparse) empty_index(P);
     for (long long s0 = (long long)blockIdx.x * blockDim.x; s0 < len; s0 += (long long)gridDim.x * blockDim.x) {
         const long long s = s0 + threadIdx.x;
         int c = s < len ? P.pop[lb][pp][s] : 0;
         const long long ns = warp_append(&st->new_len, c != 0);
+        if (s >= len) continue;
+        unsigned long long key[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) key[w] = P.det[lb][s * W + w];
         if (c != 0) {
 #pragma unroll
-            for (int w = 0; w < W; ++w) P.det[lb ^ 1][ns * W + w] = P.det[lb][s * W + w];
+            for (int w = 0; w < W; ++w) P.det[lb ^ 1][ns * W + w] = key[w];
             P.hd[lb ^ 1][ns] = P.hd[lb][s];
             P.hdf[lb ^ 1][ns] = P.hdf[lb][s];
             P.pop[lb ^ 1][pp][ns] = c;
@@ -485,58 +537,31 @@ __global__ void k_compact_copy(Params P) {
             unsigned *od = reinterpret_cast<unsigned *>(P.occa[lb ^ 1] + ns * P.ostride);
             for (int k = 0; k < P.ostride / 4; ++k) od[k] = os[k];
         }
-    }
-}
-
-// Whether a due compaction empties the old list's index entries one by one (a short list: len * 16 <=
-// index capacity, positions held as int) rather than the whole index.
-__device__ __forceinline__ bool sparse_index_clear(const Params &P, const DevState *st) {
-    return st->list_len * 16 <= P.idx_cap && P.idx_cap <= (1LL << 31);
-}
-
-// Empties the whole index: forced (a rebuild, whatever the run's status), or for a due compaction whose
-// list is too long for the sparse clear below.
-__global__ void k_index_clear(Params P, int force) {
-    DevState *st = P.st;
-    if (!force && (st->status || !st->compact_pending || sparse_index_clear(P, st))) return;
-    const long long nwords = P.idx_cap * (P.idx_stride);
-    ulonglong2 *p = reinterpret_cast<ulonglong2 *>(P.idx);
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < nwords / 2; k += (long long)gridDim.x * blockDim.x)
-        p[k] = make_ulonglong2(EMPTY, EMPTY);
-}
-
-// A due compaction with a short list (len * 16 <= index capacity): the old list's entries are emptied one
-// by one instead of clearing the whole index. First every old slot's entry is located (into the old
-// buffer's idle population array: no probe chain is cut before every key is found), then emptied.
-template <int W>
-__global__ void k_index_locate_old(Params P) {
-    DevState *st = P.st;
-    if (st->status || !st->compact_pending || !sparse_index_clear(P, st)) return;
-    constexpr int S = Stride<W>::v;
-    const int lb = st->lb;
-    const long long n = st->list_len;
-    int *pos = P.pop[lb][st->pp ^ 1];
-    const unsigned long long imask = (unsigned long long)P.idx_cap - 1ull;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
-        unsigned long long key[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) key[w] = P.det[lb][s * W + w];
-        unsigned long long h = table_hash<W>(key, kSaltIndex) >> (64 - P.idx_bits);
-        int found = -1;
-        for (long long probe = 0; probe < P.idx_cap; ++probe) {
-            const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(P.idx + h * S);
-            const bool match = x.x == key[0] && (W == 1 || x.y == key[W - 1]);
-            const bool empty = x.x == EMPTY && (W == 1 || x.y == EMPTY);
-            if (match) { found = (int)h; break; }
-            if (empty) break;
-            h = (h + 1ull) & imask;
+        if (sparse) {
+            unsigned long long h = table_hash<W>(key, kSaltIndex) >> (64 - P.idx_bits);
+            int found = -1;
+            for (long long probe = 0; probe < P.idx_cap; ++probe) {
+                const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(P.idx + h * S);
+                const bool match = x.x == key[0] && (W == 1 || x.y == key[W - 1]);
+                const bool empty = x.x == EMPTY && (W == 1 || x.y == EMPTY);
+                if (match) { found = (int)h; break; }
+                if (empty) break;
+                h = (h + 1ull) & imask;
+            }
+            pos[s] = found;
         }
-        pos[s] = found;
     }
 }
+
+// Empties the whole index, whatever the run's status (a rebuild).
+__global__ void k_index_clear(Params P) { empty_index(P); }
+
+// Second kernel of a due compaction: the located entries are emptied.
 template <int W>
 __global__ void k_index_clear_old(Params P) {
     DevState *st = P.st;
+    grid_next();
+    grid_wait();
     if (st->status || !st->compact_pending || !sparse_index_clear(P, st)) return;
     constexpr int S = Stride<W>::v;
     const long long n = st->list_len;
@@ -551,11 +576,13 @@ __global__ void k_index_clear_old(Params P) {
 }
 
 // Inserts slots [0, n) of a list buffer into the (cleared) index. force: rebuild the active list (at
-// creation, or restoring it after a rejected set_walkers), whatever the run's status; otherwise the
-// compacted list in the other buffer.
+// creation, or restoring it after a rejected set_walkers), whatever the run's status; otherwise the third kernel of a
+// due compaction: the compacted list in the other buffer, which the last block then makes the active one.
 template <int W>
 __global__ void k_index_fill(Params P, int force) {
     DevState *st = P.st;
+    grid_next();
+    grid_wait();
     if (!force && (st->status || !st->compact_pending)) return;
     constexpr int S = Stride<W>::v;
     const int buf = force ? st->lb : (st->lb ^ 1);
@@ -580,6 +607,13 @@ __global__ void k_index_fill(Params P, int force) {
         }
         if (!done) set_status(st, FCIQMC_ERR_CAPACITY);
     }
+    if (force || !last_block(st) || threadIdx.x != 0 || *(volatile int *)&st->status) return;
+    st->lb ^= 1;
+    st->list_len = n;
+    st->claim = (unsigned long long)n;
+    st->new_len = 0;
+    st->compact_pending = 0;
+    st->compactions++;
 }
 
 // Inserts slots [lo, hi) of list buffer b (a list being loaded) into the index, the old list's entries
@@ -616,17 +650,6 @@ __global__ void k_mt_clear(Params P, int W) {
         for (int w = 0; w < W; ++w) P.mt[e * S + w] = EMPTY;
         P.mt[e * S + W] = 0ull;
     }
-}
-
-__global__ void k_compact_finish(Params P) {
-    DevState *st = P.st;
-    if (threadIdx.x != 0 || !st->compact_pending || st->status) return;
-    st->lb ^= 1;
-    st->list_len = (long long)st->new_len;
-    st->claim = st->new_len;
-    st->new_len = 0;
-    st->compact_pending = 0;
-    st->compactions++;
 }
 
 // ---------------------------------------------------------------------------- estimators, gather, setup

@@ -57,6 +57,11 @@ struct DevState {
     unsigned heavy_chunk;           // attempts per heavy chunk this iteration (0: kChunk)
     int tile;                       // determinants per sweep tile this iteration (0: kTile)
     unsigned heavy_thr;             // attempts above which a determinant takes the heavy path (0: kHeavy)
+    // new slots whose diagonal elements k_new_diag computes, and the population array that lists them (set by
+    // k_annihilate: by then the iteration may be committed and n_new cleared)
+    long long diag_n;
+    int diag_pp;
+    unsigned ticket;                // blocks of the running kernel that are done (its last block resets it)
     unsigned long long ob_n[MAXPARTS];  // partitioned runs: spawns routed to each other partition this iteration
 };
 
@@ -173,6 +178,31 @@ __device__ __forceinline__ void set_status(DevState *st, int code) { atomicCAS(&
 #else
 #define FQ_CHECK(cond, st) true
 #endif
+
+// ---------------------------------------------------------------------------
+// The kernels of an iteration are launched with programmatic dependencies (launch_next): a kernel's blocks may be
+// placed while its predecessor's last blocks still run. grid_wait() returns when the predecessor has finished and
+// its writes are visible; before it, a kernel reads only what no kernel of an iteration writes (tables made at
+// creation). Every block calls it, also those that have nothing to do, so that "the predecessor has finished" holds
+// for the whole chain. Without the launch attribute it returns at once.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the successor's blocks be placed from here on (as room allows).
+__device__ __forceinline__ void grid_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// True in the last block of the kernel to get here; all blocks' earlier writes are then visible to its later reads
+// that go past L1 (volatile, __ldcg). Every block of the grid has to call it.
+__device__ __forceinline__ bool last_block(DevState *st) {
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1u;
+        if (s_last) st->ticket = 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    return s_last;
+}
 
 // ---------------------------------------------------------------------------
 // 32 x 32 -> 64 bits in one instruction (written as a low and a high product, a Philox block took 6% longer).

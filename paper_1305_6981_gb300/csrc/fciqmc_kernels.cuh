@@ -1340,7 +1340,6 @@ __device__ __forceinline__ double block_sum_f64(double v, double *s_red) {
 template <int W, int MODE>
 __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) {
     DevState *st = P.st;
-    if (st->status) return;
     // dynamic: one SpawnQueue per warp, then the tile's occupied lists (occ_stride bytes each)
     extern __shared__ __align__(16) unsigned char s_queue[];
     unsigned char *const s_occ = s_queue + sizeof(SpawnQueue<W>) * (kTile / 32);
@@ -1352,13 +1351,16 @@ __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) 
     __shared__ float s_rcpf[MAXSO + 2];  // two class counts (at most 64 each) add up to an index
     __shared__ unsigned long long s_red[(kTile / 32) * (NCNT + 4)];
     __shared__ long long s_tile[2];
+    grid_next();
+    load_tables(P, T);
+    for (int k = threadIdx.x; k < MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
+    grid_wait();
+    if (st->status) return;
     const long long len = st->list_len;
     const int tile = st->tile ? st->tile : kTile;  // determinants per tile this iteration
     if (threadIdx.x == 0) s_tile[0] = (long long)atomicAdd(&st->sweep_next, 1ull) * tile;
     __syncthreads();
     if (s_tile[0] >= len) return;  // a short list: no tile for this block
-    load_tables(P, T);
-    for (int k = threadIdx.x; k < MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
     const int lb = st->lb, pp = st->pp;
     const unsigned iter = (unsigned)st->iter;
     const double S = st->shift;
@@ -1585,7 +1587,6 @@ __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) 
 template <int W, int MODE>
 __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
     DevState *st = P.st;
-    if (st->status) return;
     extern __shared__ __align__(16) unsigned char s_queue[];  // one SpawnQueue per warp
     constexpr int NW = kTile / 32;
     constexpr int U = 2;  // attempts of a lane screened side by side
@@ -1595,6 +1596,11 @@ __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
     __shared__ __align__(8) unsigned s_pend[NW][31 + 32 * U];  // attempts that passed the screen; last the counters' sums
     __shared__ float s_rcpf[MAXSO + 2];           // two class counts (at most 64 each) add up to an index
     static_assert(sizeof(s_pend) >= sizeof(unsigned long long) * NW * NCNT, "room for the counters of every warp");
+    grid_next();
+    load_tables(P, T);
+    for (int k = threadIdx.x; k < MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
+    grid_wait();
+    if (st->status) return;
     const unsigned long long packed = st->heavy_packed;
     const long long nh = min((long long)(packed >> 40), P.heavy_cap);
     const unsigned long long nch = nh > 0 ? (packed & ((1ull << 40) - 1ull)) : 0ull;
@@ -1623,8 +1629,6 @@ __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
     };
     bool done = !claim();
     if (!__syncthreads_or(done ? 0 : 1)) return;  // a short list: nothing left for this block
-    load_tables(P, T);
-    for (int k = threadIdx.x; k < MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
     const unsigned iter = (unsigned)st->iter;
     const unsigned chunk = st->heavy_chunk ? st->heavy_chunk : (unsigned)kChunk;
     const DetView<W> *heavy = reinterpret_cast<const DetView<W> *>(P.heavy);

@@ -28,24 +28,24 @@ cudaError_t configure_spawn_impl() {
 }
 
 template <int W>
-void launch_sweep_impl(int mode, int grid, cudaStream_t s, const Params &P) {
+void launch_sweep_impl(int mode, int grid, cudaStream_t s, bool next, const Params &P) {
     const size_t b = sweep_bytes<W>(P.n_elec);
     switch (mode) {
-        case 0: k_sweep<W, 0><<<grid, kTile, b, s>>>(P); break;
-        case 1: k_sweep<W, 1><<<grid, kTile, b, s>>>(P); break;
-        case 2: k_sweep<W, 2><<<grid, kTile, b, s>>>(P); break;
-        default: k_sweep<W, 3><<<grid, kTile, b, s>>>(P); break;
+        case 0: launch_next(k_sweep<W, 0>, grid, kTile, b, s, next, P); break;
+        case 1: launch_next(k_sweep<W, 1>, grid, kTile, b, s, next, P); break;
+        case 2: launch_next(k_sweep<W, 2>, grid, kTile, b, s, next, P); break;
+        default: launch_next(k_sweep<W, 3>, grid, kTile, b, s, next, P); break;
     }
 }
 
 template <int W>
-void launch_heavy_impl(int mode, int grid, cudaStream_t s, const Params &P) {
+void launch_heavy_impl(int mode, int grid, cudaStream_t s, bool next, const Params &P) {
     const size_t b = queue_bytes<W>();
     switch (mode) {
-        case 0: k_heavy<W, 0><<<grid, kTile, b, s>>>(P); break;
-        case 1: k_heavy<W, 1><<<grid, kTile, b, s>>>(P); break;
-        case 2: k_heavy<W, 2><<<grid, kTile, b, s>>>(P); break;
-        default: k_heavy<W, 3><<<grid, kTile, b, s>>>(P); break;
+        case 0: launch_next(k_heavy<W, 0>, grid, kTile, b, s, next, P); break;
+        case 1: launch_next(k_heavy<W, 1>, grid, kTile, b, s, next, P); break;
+        case 2: launch_next(k_heavy<W, 2>, grid, kTile, b, s, next, P); break;
+        default: launch_next(k_heavy<W, 3>, grid, kTile, b, s, next, P); break;
     }
 }
 
