@@ -166,7 +166,6 @@ __device__ __forceinline__ void end_iteration(const Params &P) {
 
 // The same as a launch of its own, after k_round.
 __global__ void k_finish(Params P) {
-    grid_next();
     grid_wait();
     if (P.st->status) return;
     end_iteration(P);
@@ -183,7 +182,6 @@ template <int W>
 __global__ void __launch_bounds__(256) k_annihilate(Params P, int commit) {
     __shared__ unsigned long long s_red[(256 / 32) * 4];
     DevState *st = P.st;
-    grid_next();
     grid_wait();
     if (st->status) return;
     sum_tiles(P);
@@ -334,7 +332,6 @@ __global__ void __launch_bounds__(kDiagThreads) k_new_diag(Params P) {
     extern __shared__ __align__(16) double s_w[];
     DevState *st = P.st;
     __shared__ Tables T;
-    grid_next();
     load_tables(P, T);
     unsigned char *occ = load_diag_tables(P, s_w);
     grid_wait();
@@ -363,7 +360,6 @@ template <int W>
 __global__ void __launch_bounds__(256) k_round(Params P) {
     __shared__ unsigned long long s_red[(256 / 32) * 2];
     DevState *st = P.st;
-    grid_next();
     grid_wait();
     if (st->status) return;
     const int lb = st->lb, pp = st->pp;
@@ -505,7 +501,6 @@ __device__ __forceinline__ void empty_index(const Params &P) {
 template <int W>
 __global__ void k_compact_copy(Params P) {
     DevState *st = P.st;
-    grid_next();
     grid_wait();
     if (!st->compact_pending || st->status) return;
     constexpr int S = Stride<W>::v;
@@ -560,7 +555,6 @@ __global__ void k_index_clear(Params P) { empty_index(P); }
 template <int W>
 __global__ void k_index_clear_old(Params P) {
     DevState *st = P.st;
-    grid_next();
     grid_wait();
     if (st->status || !st->compact_pending || !sparse_index_clear(P, st)) return;
     constexpr int S = Stride<W>::v;
@@ -581,7 +575,6 @@ __global__ void k_index_clear_old(Params P) {
 template <int W>
 __global__ void k_index_fill(Params P, int force) {
     DevState *st = P.st;
-    grid_next();
     grid_wait();
     if (!force && (st->status || !st->compact_pending)) return;
     constexpr int S = Stride<W>::v;

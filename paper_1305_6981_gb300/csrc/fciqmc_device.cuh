@@ -52,8 +52,8 @@ struct DevState {
     double est_num;
     int check_bad;             // set by the check of a list being loaded
     unsigned long long n_new;  // determinants placed in new slots this iteration (diagonal elements pending)
-    unsigned long long sweep_next;  // next sweep tile to hand out (tiles are taken dynamically by the blocks)
-    unsigned long long heavy_next;  // next batch of heavy chunks to hand out (taken dynamically by the warps)
+    unsigned long long sweep_next;  // sweep tiles handed out beyond the blocks' first (taken dynamically)
+    unsigned long long heavy_next;  // heavy chunks handed out beyond the warps' first (taken dynamically)
     unsigned heavy_chunk;           // attempts per heavy chunk this iteration (0: kChunk)
     int tile;                       // determinants per sweep tile this iteration (0: kTile)
     unsigned heavy_thr;             // attempts above which a determinant takes the heavy path (0: kHeavy)
@@ -181,14 +181,12 @@ __device__ __forceinline__ void set_status(DevState *st, int code) { atomicCAS(&
 
 // ---------------------------------------------------------------------------
 // The kernels of an iteration are launched with programmatic dependencies (launch_next): a kernel's blocks may be
-// placed while its predecessor's last blocks still run. grid_wait() returns when the predecessor has finished and
+// placed as its predecessor's blocks leave. (Placed from the predecessor's start on, by launch_dependents, the waiting
+// blocks got in its way: 232 instead of 217 us per iteration on 6e6 walkers of 24e/60o.) grid_wait() returns when the predecessor has finished and
 // its writes are visible; before it, a kernel reads only what no kernel of an iteration writes (tables made at
 // creation). Every block calls it, also those that have nothing to do, so that "the predecessor has finished" holds
 // for the whole chain. Without the launch attribute it returns at once.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// Lets the successor's blocks be placed from here on (as room allows).
-__device__ __forceinline__ void grid_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // True in the last block of the kernel to get here; all blocks' earlier writes are then visible to its later reads
 // that go past L1 (volatile, __ldcg). Every block of the grid has to call it.
 __device__ __forceinline__ bool last_block(DevState *st) {
@@ -381,18 +379,36 @@ __device__ __forceinline__ float eri_f(const Params &P, int p, int q, int r, int
     return ld_keep(P.eri_f + k, pol);
 }
 
-// Slater-Condon, single i -> a from source d (occupied list occ of d), exact FP64 in ascending order.
-template <int W>
-__device__ double hij_single(const Params &P, const unsigned long long (&d)[W], const unsigned char *occ, int i, int a) {
-    int I = i >> 1, A = a >> 1;
-    double v = __ldg(P.h + I * P.n_orb + A);
-    for (int x = 0; x < P.n_elec; ++x) {
-        int j = occ[x];
-        if (j == i) continue;
-        int J = j >> 1;
-        v = __dadd_rn(v, eri_d(P, I, A, J, J));
-        if ((j & 1) == (i & 1)) v = __dsub_rn(v, eri_d(P, I, J, J, A));
+// Slater-Condon, single i -> a without its parity, exact FP64 over the occupied list in ascending order. The integrals of
+// four electrons are read ahead of their additions (one at a time, the chain waited on L2 twice per electron). Not
+// inlined: the spawning kernels come here for one attempt in millions.
+static __device__ __noinline__ double single_element(const double *h, const double *eri, int n_orb, int n_elec, const unsigned char *occ,
+                                                     int i, int a) {
+    const int I = i >> 1, A = a >> 1;
+    double v = __ldg(h + I * n_orb + A);
+    for (int x0 = 0; x0 < n_elec; x0 += 4) {
+        double c[4], e[4];
+        int j[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            j[u] = x0 + u < n_elec ? occ[x0 + u] : i;
+            const int J = j[u] >> 1;
+            c[u] = __ldg(eri + eidx(I, A, J, J));
+            e[u] = __ldg(eri + eidx(I, J, J, A));
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (j[u] == i) continue;
+            v = __dadd_rn(v, c[u]);
+            if ((j[u] & 1) == (i & 1)) v = __dsub_rn(v, e[u]);
+        }
     }
+    return v;
+}
+// Slater-Condon, single i -> a from source d (occupied list occ of d).
+template <int W>
+__device__ __forceinline__ double hij_single(const Params &P, const unsigned long long (&d)[W], const unsigned char *occ, int i, int a) {
+    const double v = single_element(P.h, P.eri, P.n_orb, P.n_elec, occ, i, a);
     return (count_between<W>(d, i, a) & 1) ? -v : v;
 }
 

@@ -1,7 +1,7 @@
 // Kernels of one FCIQMC iteration (sm_103a).
 //
 // Per iteration, on the caller's stream (or as one CUDA graph):
-//   [compaction, only when flagged]  k_compact_copy -> k_index_clear -> k_index_fill -> k_compact_finish
+//   [compaction, only when flagged]  k_compact_copy -> k_index_clear_old -> k_index_fill
 //   k_sweep        estimators of the incoming list, death/cloning (Eq. 4), and every spawning
 //                  attempt (Eq. 3, Sec. VI) of determinants with |C_i| <= kHeavy, merged on the fly
 //                  into the spawn table (sum of signed amounts, initiator flags counted)
@@ -17,7 +17,7 @@
 namespace fq {
 
 constexpr int kTile = 256;          // threads per sweep block = most determinants of a sweep tile
-constexpr int kTileSums = 32;       // range sums of the per-tile numerators (blocks of k_tile_sum)
+constexpr int kTileSums = 32;       // range sums of the per-tile numerators (one block each)
 #ifndef FQ_SWEEP_MIN_BLOCKS
 #define FQ_SWEEP_MIN_BLOCKS 5          // resident sweep blocks per SM the register budget is sized for
 #endif
@@ -1069,14 +1069,54 @@ __device__ __forceinline__ bool attempt_screen_light(const Params &P, const Atte
     return false;
 }
 
+// Float value (x) and sum of absolute terms (y) of a single-excitation element without its parity, by one thread.
+static __device__ __noinline__ float2 single_sums(const float *h_f, const float *eri_f, int n_orb, int n_elec, const unsigned char *occ,
+                                                  int i, int a, unsigned long long pol) {
+    const int I = i >> 1, A = a >> 1;
+    float s = __ldg(h_f + I * n_orb + A), b = fabsf(s);
+    for (int x0 = 0; x0 < n_elec; x0 += 4) {
+        float c[4], e[4];
+        int j[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            j[u] = x0 + u < n_elec ? occ[x0 + u] : i;
+            const int J = j[u] >> 1;
+            c[u] = ld_keep(eri_f + eidx(I, A, J, J), pol);
+            e[u] = ld_keep(eri_f + eidx(I, J, J, A), pol);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (j[u] == i) continue;
+            s += c[u];
+            b += fabsf(c[u]);
+            if ((j[u] & 1) == (i & 1)) {
+                s -= e[u];
+                b += fabsf(e[u]);
+            }
+        }
+    }
+    return make_float2(s, b);
+}
+
 // Float value and sum of absolute terms of the single-excitation element h_ia + sum_j [(ia|jj) -
 // delta_spin (ij|ja)] (without the parity sign) for every lane with a pending single, each evaluated by
-// the whole warp: lane x takes electrons x, x + 32. Called by all 32 lanes.
+// the whole warp: lane x takes electrons x, x + 32. Where many lanes have one, each evaluates its own instead, four
+// electrons at a time: about 32 N instructions for the warp against 80 per single, and without a round trip
+// to L2 for each (8e/8o, three singles in 32 attempts: 85 to 55 us per iteration). Called by all 32 lanes.
 template <int W>
 __device__ __forceinline__ void single_elements_warp(const Params &P, const unsigned char *occp, bool pend, int i,
                                                      int a, unsigned long long pol, float &hs, float &hab) {
     unsigned need = __ballot_sync(0xFFFFFFFFu, pend);
     const int lane = threadIdx.x & 31;
+    if (5 * __popc(need) >= 2 * P.n_elec) {
+        if (pend) {
+            const float2 r = single_sums(P.h_f, P.eri_f, P.n_orb, P.n_elec, occp, i, a, pol);
+            hs = r.x;
+            hab = r.y;
+        }
+        __syncwarp();
+        return;
+    }
     while (need) {
         const int src = __ffs(need) - 1;
         need &= need - 1;
@@ -1351,16 +1391,14 @@ __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) 
     __shared__ float s_rcpf[MAXSO + 2];  // two class counts (at most 64 each) add up to an index
     __shared__ unsigned long long s_red[(kTile / 32) * (NCNT + 4)];
     __shared__ long long s_tile[2];
-    grid_next();
     load_tables(P, T);
     for (int k = threadIdx.x; k < MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
     grid_wait();
     if (st->status) return;
     const long long len = st->list_len;
     const int tile = st->tile ? st->tile : kTile;  // determinants per tile this iteration
-    if (threadIdx.x == 0) s_tile[0] = (long long)atomicAdd(&st->sweep_next, 1ull) * tile;
-    __syncthreads();
-    if (s_tile[0] >= len) return;  // a short list: no tile for this block
+    if ((long long)blockIdx.x * tile >= len) return;  // a short list: no tile for this block
+    if (threadIdx.x == 0) s_tile[0] = (long long)blockIdx.x * tile;
     const int lb = st->lb, pp = st->pp;
     const unsigned iter = (unsigned)st->iter;
     const double S = st->shift;
@@ -1399,39 +1437,41 @@ __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) 
         const long long s = tb + tid;
         unsigned att = 0;
         if (tid < tile && s < len) {
+            // everything of the slot is read at once, its population with the rest (a vacated slot, one in four at
+            // most, costs its bytes; waiting for the population first cost every tile a round trip)
+            DetView<W> &v = s_dv[tid];
+            unsigned char *occ = s_occ + tid * ostride;
             const int c = __ldcs(pop_in + s);
-            if (c == 0) {
-                pop_out[s] = 0;
-            } else {
-                DetView<W> &v = s_dv[tid];
+            const float hf = __ldcs(hdf + s);
+            unsigned long long pre[PRE_WORDS];
+            {
+                const ulonglong2 *ps = reinterpret_cast<const ulonglong2 *>(P.pre[lb] + s * PRE_WORDS);
+                const ulonglong2 p0 = __ldcs(ps), p1 = __ldcs(ps + 1);
+                pre[0] = p0.x;
+                pre[1] = p0.y;
+                pre[2] = p1.x;
+                pre[3] = p1.y;
                 if (W == 2) {
-                    ulonglong2 dd = __ldcs(reinterpret_cast<const ulonglong2 *>(det) + s);
+                    const ulonglong2 dd = __ldcs(reinterpret_cast<const ulonglong2 *>(det) + s);
                     v.d[0] = dd.x;
                     v.d[W - 1] = dd.y;
                 } else {
                     v.d[0] = __ldcs(det + s);
                 }
-                const float hf = __ldcs(hdf + s);
-                // the determinant's derived words and occupied list, stored when it entered the list
-                unsigned char *occ = s_occ + tid * ostride;
-                unsigned long long pre[PRE_WORDS];
-                {
-                    const ulonglong2 *ps = reinterpret_cast<const ulonglong2 *>(P.pre[lb] + s * PRE_WORDS);
-                    const ulonglong2 p0 = __ldcs(ps), p1 = __ldcs(ps + 1);
-                    pre[0] = p0.x;
-                    pre[1] = p0.y;
-                    pre[2] = p1.x;
-                    pre[3] = p1.y;
-                    const unsigned *os = reinterpret_cast<const unsigned *>(P.occa[lb] + s * ostride);
-                    for (int k = 0; k < ostride / 4; k += 8) {  // eight loads in flight
-                        unsigned o[8];
+                // the determinant's occupied list, stored when it entered the list
+                const unsigned *os = reinterpret_cast<const unsigned *>(P.occa[lb] + s * ostride);
+                for (int k = 0; k < ostride / 4; k += 8) {  // eight loads in flight
+                    unsigned o[8];
 #pragma unroll
-                        for (int u = 0; u < 8; ++u) o[u] = k + u < ostride / 4 ? __ldcs(os + k + u) : 0u;
+                    for (int u = 0; u < 8; ++u) o[u] = k + u < ostride / 4 ? __ldcs(os + k + u) : 0u;
 #pragma unroll
-                        for (int u = 0; u < 8; ++u)
-                            if (k + u < ostride / 4) reinterpret_cast<unsigned *>(occ)[k + u] = o[u];
-                    }
+                    for (int u = 0; u < 8; ++u)
+                        if (k + u < ostride / 4) reinterpret_cast<unsigned *>(occ)[k + u] = o[u];
                 }
+            }
+            if (c == 0) {
+                pop_out[s] = 0;
+            } else {
                 fill_view<W>(P, v, pre, c);
                 const unsigned ac = (unsigned)(c < 0 ? -c : c);
                 acc[NCNT] += ac;
@@ -1495,7 +1535,7 @@ __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) 
         if (lane == 31) s_wsum[warp] = x;
         if (lane == 0) s_numw[warp] = wnum;
         if (tid == 0) {
-            s_tile[slot ^ 1] = (long long)atomicAdd(&st->sweep_next, 1ull) * tile;
+            s_tile[slot ^ 1] = (long long)(gridDim.x + atomicAdd(&st->sweep_next, 1ull)) * tile;
             s_nleft = 0;
         }
         __syncthreads();
@@ -1596,7 +1636,6 @@ __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
     __shared__ __align__(8) unsigned s_pend[NW][31 + 32 * U];  // attempts that passed the screen; last the counters' sums
     __shared__ float s_rcpf[MAXSO + 2];           // two class counts (at most 64 each) add up to an index
     static_assert(sizeof(s_pend) >= sizeof(unsigned long long) * NW * NCNT, "room for the counters of every warp");
-    grid_next();
     load_tables(P, T);
     for (int k = threadIdx.x; k < MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
     grid_wait();
@@ -1608,26 +1647,27 @@ __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
     // warps take batches of consecutive chunks from a counter by guided self-scheduling: a share of what is left, so
     // batches are long while much is left (few determinant switches) and single chunks at the end (no tail); lane 0
     // decides, so every lane of the warp holds the same batch
-    unsigned long long q = 0, qend = 0;  // the batch's next chunk and end
+    // (every warp's first chunk is its own number: 4,864 warps on one counter waited 2 to 5 us each)
+    const unsigned long long nwarps = (unsigned long long)gridDim.x * NW;
+    unsigned long long q = (unsigned long long)blockIdx.x * NW + warp, qend = q + 1;  // the batch's next chunk and end
     auto claim = [&]() {
-        unsigned long long b = 0, size = 1;
+        if (nch <= nwarps) return false;
+        const unsigned long long rest = nch - nwarps;
+        unsigned long long b = rest, size = 1;
         if (lane == 0) {
             const unsigned long long taken = *(volatile unsigned long long *)&st->heavy_next;
-            const unsigned long long nwarps = (unsigned long long)gridDim.x * NW;
-            if (taken < nch) {
-                size = max(1ull, min((unsigned long long)kChunkBatch, (nch - taken) / (2ull * nwarps)));
+            if (taken < rest) {
+                size = max(1ull, min((unsigned long long)kChunkBatch, (rest - taken) / (2ull * nwarps)));
                 b = atomicAdd(&st->heavy_next, size);
-            } else {
-                b = nch;
             }
         }
         b = __shfl_sync(0xFFFFFFFFu, b, 0);
         size = __shfl_sync(0xFFFFFFFFu, size, 0);
-        q = b;
-        qend = min(b + size, nch);
-        return b < nch;
+        q = nwarps + b;
+        qend = min(q + size, nch);
+        return b < rest;
     };
-    bool done = !claim();
+    bool done = q >= nch;
     if (!__syncthreads_or(done ? 0 : 1)) return;  // a short list: nothing left for this block
     const unsigned iter = (unsigned)st->iter;
     const unsigned chunk = st->heavy_chunk ? st->heavy_chunk : (unsigned)kChunk;
@@ -1687,10 +1727,14 @@ __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
             long long r = -1;
             if (!done) {
                 if (fresh) {
-                    long long lo = 0, hi = nh - 1;
-                    while (lo < hi) {
-                        const long long mid = (lo + hi + 1) >> 1;
-                        if ((unsigned long long)P.heavy_base[mid] <= q) lo = mid; else hi = mid - 1;
+                    // 32 places at a time (two or three dependent reads for a few thousand records, not eleven)
+                    long long lo = 0, n = nh;  // the record is in [lo, lo + n), and heavy_base[lo] <= q
+                    while (n > 1) {
+                        const long long step = (n + 31) >> 5, at = lo + step * lane;
+                        const bool le = at < lo + n && (unsigned long long)P.heavy_base[at] <= q;
+                        const int last = 31 - __clz(__ballot_sync(0xFFFFFFFFu, le) | 1u);
+                        n = min(step, lo + n - (lo + step * last));
+                        lo += step * last;
                     }
                     r = lo;
                 } else {
@@ -1710,12 +1754,16 @@ __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
                     __syncwarp();
                     const unsigned long long *src = reinterpret_cast<const unsigned long long *>(heavy + r);
                     unsigned long long *dstv = reinterpret_cast<unsigned long long *>(&v);
-                    for (int k = lane; k < (int)(sizeof(DetView<W>) / 8); k += 32) dstv[k] = src[k];
-                    for (int k = lane; k < P.n_elec; k += 32) {
-                        const unsigned so = P.heavy_occ[r * MAXN + k];
-                        tab.occ[k] = (unsigned char)so;
-                        tab.occ2[k] = (unsigned short)(so | ((unsigned)T.irrep[so >> 1] << 8));
-                    }
+                    static_assert(sizeof(DetView<W>) <= 8 * 32, "one word per lane");
+                    // all reads at once
+                    const unsigned long long x = lane < (int)(sizeof(DetView<W>) / 8) ? src[lane] : 0ull;
+                    const unsigned so0 = lane < P.n_elec ? P.heavy_occ[r * MAXN + lane] : 0u;
+                    const unsigned so1 = lane + 32 < P.n_elec ? P.heavy_occ[r * MAXN + lane + 32] : 0u;
+                    if (lane < (int)(sizeof(DetView<W>) / 8)) dstv[lane] = x;
+                    tab.occ[lane] = (unsigned char)so0;
+                    tab.occ[lane + 32] = (unsigned char)so1;
+                    tab.occ2[lane] = (unsigned short)(so0 | ((unsigned)T.irrep[so0 >> 1] << 8));
+                    tab.occ2[lane + 32] = (unsigned short)(so1 | ((unsigned)T.irrep[so1 >> 1] << 8));
                     __syncwarp();
                     build_heavy_tab<W>(P, T, v, s_rcpf, tab, lane);
                     cur = r;
