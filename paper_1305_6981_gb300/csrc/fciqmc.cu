@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstddef>
 #include <cstdint>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -38,6 +39,7 @@ struct NvtxRange {
 
 constexpr size_t kAlign = 256;
 constexpr int kMaxGrid = 4096;
+constexpr int kCompThreads = 512;  // threads of the compaction kernels of an iteration
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 long long next_pow2(long long x) {
@@ -189,7 +191,7 @@ struct fciqmc_handle {
     char *ws;
     cudaStream_t stream;
     fciqmc_info info;
-    int sweep_grid, heavy_grid, ann_grid, diag_grid, small_grid;
+    int sweep_grid, heavy_grid, ann_grid, diag_grid, small_grid, comp_grid;
     size_t smem_w, smem_d;   // dynamic shared memory: pair terms; pair terms and occupied lists
     double e_core;
     cudaGraph_t graph_tmpl;  // one iteration, kept for composing batch graphs
@@ -230,6 +232,17 @@ int configure_kernels(fciqmc_handle *h) {
     FQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fq::k_new_diag<W>, fq::kDiagThreads, h->smem_d));
     h->diag_grid = std::min(kMaxGrid, std::max(1, sms * std::max(per_sm, 1)));
     h->heavy_grid = std::min(kMaxGrid, sms * 4);
+    // no more blocks than a list at capacity has tiles or entries for (small runs advanced side by side share the SMs'
+    // block slots)
+    auto at_most = [](int grid, long long n, int per) { return (int)std::max<long long>(1, std::min<long long>(grid, (n + per - 1) / per)); };
+    h->sweep_grid = at_most(h->sweep_grid, h->z.cap, fq::kTileLeast);
+    h->ann_grid = at_most(h->ann_grid, h->z.mt_cap, 256);
+    h->diag_grid = at_most(h->diag_grid, h->z.cap, fq::kDiagThreads);
+    // k_heavy: the smallest chunk for every warp at four times the target population (where one is set)
+    const long long target = h->opt.target_walkers;
+    if (target > 0 && target < (1LL << 40))
+        h->heavy_grid = at_most(h->heavy_grid, 4 * std::max<long long>(target, std::llabs((long long)h->opt.initial_population)),
+                                fq::kChunkLeast * (fq::kTile / 32));
     if (h->grid_request > 0) {
         const int g = std::min(kMaxGrid, h->grid_request);
         h->sweep_grid = std::min(h->sweep_grid, g);
@@ -240,6 +253,9 @@ int configure_kernels(fciqmc_handle *h) {
     h->P.heavy_warps = (long long)h->heavy_grid * (fq::kTile / 32);
     h->P.sweep_blocks = h->sweep_grid;
     h->small_grid = std::min(kMaxGrid, sms * 8);
+    // the compaction kernels mostly return at once, and placing 1,216 blocks for that takes longer than the rest of the
+    // launch: two blocks an SM, fewer for a list that four slots a thread cover with less
+    h->comp_grid = (int)std::max<long long>(1, std::min<long long>(sms * 2, (h->z.cap + 4 * kCompThreads - 1) / (4 * kCompThreads)));
     h->info.num_sms = sms;
     h->info.grid_blocks = h->sweep_grid;
     h->P.sweep_grid = h->sweep_grid;
@@ -269,9 +285,9 @@ void enqueue_step(fciqmc_handle *h, cudaStream_t s, int step, bool next) {
     const Params &P = h->P;
     const bool rounds = P.occ_units > 1;
     switch (step) {
-        case STEP_COPY: fq::launch_next(fq::k_compact_copy<W>, h->small_grid, 256, 0, s, false, P); break;
-        case STEP_CLEAR: fq::launch_next(fq::k_index_clear_old<W>, h->small_grid, 256, 0, s, next, P); break;
-        case STEP_FILL: fq::launch_next(fq::k_index_fill<W>, h->small_grid, 256, 0, s, next, P, 0); break;
+        case STEP_COPY: fq::launch_next(fq::k_compact_copy<W>, h->comp_grid, kCompThreads, 0, s, false, P); break;
+        case STEP_CLEAR: fq::launch_next(fq::k_index_clear_old<W>, h->comp_grid, kCompThreads, 0, s, next, P); break;
+        case STEP_FILL: fq::launch_next(fq::k_index_fill<W>, h->comp_grid, kCompThreads, 0, s, next, P, 0); break;
         case STEP_SWEEP: launch_sweep<W>(h, s, next); break;
         case STEP_HEAVY: launch_heavy<W>(h, s, next); break;
         case STEP_ANNIHILATE:
@@ -1223,20 +1239,42 @@ GroupLayout group_layout(int n, long long hist_cap) {
     return L;
 }
 
+// One iteration of the group under capture: the partitions are independent of one another up to the exchange and again
+// after it, so each has a branch of its own (a partition of a million walkers fills no GPU: on one stream four of them
+// took four times as long). streams[0] is the capturing one.
 template <int W>
-void enqueue_group_iteration(fciqmc_group *g, cudaStream_t s) {
-    const int n = (int)g->parts.size();
-    for (fciqmc_handle *h : g->parts)
-        for (int step = STEP_COPY; step <= STEP_HEAVY; ++step) enqueue_step<W>(h, s, step, false);
-    // the exchange: each partition merges the spawns the others routed to it
-    for (fciqmc_handle *h : g->parts) fq::k_receive<W><<<h->ann_grid, 256, 0, s>>>(h->P, g->links);
-    for (fciqmc_handle *h : g->parts) {
-        fq::k_annihilate<W><<<h->ann_grid, 256, 0, s>>>(h->P, 0);
-        fq::k_new_diag<W><<<h->diag_grid, fq::kDiagThreads, h->smem_d, s>>>(h->P);
-        if (h->P.occ_units > 1) fq::k_round<W><<<h->small_grid, 256, 0, s>>>(h->P);
+cudaError_t enqueue_group_iteration(fciqmc_group *g, const std::vector<cudaStream_t> &streams, cudaEvent_t ev) {
+    const size_t n = g->parts.size();
+    cudaError_t e = cudaSuccess;
+    auto ok = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
+    auto fork = [&]() {
+        ok(cudaEventRecord(ev, streams[0]));
+        for (size_t r = 1; r < n; ++r) ok(cudaStreamWaitEvent(streams[r], ev, 0));
+    };
+    auto join = [&]() {
+        for (size_t r = 1; r < n; ++r) {
+            ok(cudaEventRecord(ev, streams[r]));
+            ok(cudaStreamWaitEvent(streams[0], ev, 0));
+        }
+    };
+    fork();
+    for (size_t r = 0; r < n; ++r)
+        for (int step = STEP_COPY; step <= STEP_HEAVY; ++step) enqueue_step<W>(g->parts[r], streams[r], step, step != STEP_COPY);
+    join();
+    fork();
+    for (size_t r = 0; r < n; ++r) {
+        fciqmc_handle *h = g->parts[r];
+        // the exchange: each partition merges the spawns the others routed to it
+        fq::k_receive<W><<<h->ann_grid, 256, 0, streams[r]>>>(h->P, g->links);
+        fq::launch_next(fq::k_annihilate<W>, h->ann_grid, 256, 0, streams[r], true, h->P, 0);
+        fq::launch_next(fq::k_new_diag<W>, h->diag_grid, fq::kDiagThreads, h->smem_d, streams[r], true, h->P);
+        if (h->P.occ_units > 1) fq::launch_next(fq::k_round<W>, h->small_grid, 256, 0, streams[r], true, h->P);
     }
+    join();
     const Params &P0 = g->parts[0]->P;
-    fq::k_group_finish<<<1, 32, 0, s>>>(g->links, n, g->gdev, g->ghist, g->hist_cap, P0.target, P0.period, P0.c_shift);
+    fq::k_group_finish<<<1, 32, 0, streams[0]>>>(g->links, (int)n, g->gdev, g->ghist, g->hist_cap, P0.target, P0.period, P0.c_shift);
+    ok(cudaGetLastError());
+    return e;
 }
 
 bool same_run(const fciqmc_handle *a, const fciqmc_handle *b) {
@@ -1300,7 +1338,8 @@ int fciqmc_group_create(fciqmc_handle *const *parts, int32_t n_partitions, int64
         links[r].frac_bits = P.frac_bits;
     }
     int rc = FCIQMC_OK;
-    cudaStream_t cs = nullptr;
+    std::vector<cudaStream_t> cs(n_partitions, nullptr);  // for the capture only
+    cudaEvent_t ev = nullptr;
     do {
         // the partitions' own streams finish their work (creation, loads) before the group starts
         for (fciqmc_handle *h : g->parts)
@@ -1310,13 +1349,16 @@ int fciqmc_group_create(fciqmc_handle *const *parts, int32_t n_partitions, int64
             cudaMemcpyAsync(g->links, links.data(), sizeof(fq::PartLink) * n_partitions, cudaMemcpyHostToDevice,
                             g->stream) != cudaSuccess ||
             cudaStreamSynchronize(g->stream) != cudaSuccess) { rc = FCIQMC_ERR_CUDA; break; }
-        if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) { rc = FCIQMC_ERR_CUDA; break; }
+        for (int r = 0; r < n_partitions && rc == FCIQMC_OK; ++r)
+            if (cudaStreamCreateWithFlags(&cs[r], cudaStreamNonBlocking) != cudaSuccess) rc = FCIQMC_ERR_CUDA;
+        if (rc == FCIQMC_OK && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) rc = FCIQMC_ERR_CUDA;
+        if (rc != FCIQMC_OK) break;
         cudaGraph_t graph = nullptr;
-        cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+        cudaError_t e = cudaStreamBeginCapture(cs[0], cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            if (parts[0]->z.W == 1) enqueue_group_iteration<1>(g, cs);
-            else enqueue_group_iteration<2>(g, cs);
-            e = cudaStreamEndCapture(cs, &graph);
+            const cudaError_t q = parts[0]->z.W == 1 ? enqueue_group_iteration<1>(g, cs, ev) : enqueue_group_iteration<2>(g, cs, ev);
+            e = cudaStreamEndCapture(cs[0], &graph);
+            if (e == cudaSuccess) e = q;
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&g->exec, graph, 0);
         if (e == cudaSuccess) g->graph = graph;
@@ -1328,7 +1370,9 @@ int fciqmc_group_create(fciqmc_handle *const *parts, int32_t n_partitions, int64
         if (rc == FCIQMC_OK && cudaEventCreateWithFlags(&g->done, cudaEventDisableTiming) != cudaSuccess)
             rc = FCIQMC_ERR_CUDA;
     } while (false);
-    if (cs) cudaStreamDestroy(cs);
+    for (cudaStream_t c : cs)
+        if (c) cudaStreamDestroy(c);
+    if (ev) cudaEventDestroy(ev);
     if (rc != FCIQMC_OK) {
         cudaGetLastError();
         if (g->exec) cudaGraphExecDestroy(g->exec);

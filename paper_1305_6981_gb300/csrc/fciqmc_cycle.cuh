@@ -332,12 +332,12 @@ __global__ void __launch_bounds__(kDiagThreads) k_new_diag(Params P) {
     extern __shared__ __align__(16) double s_w[];
     DevState *st = P.st;
     __shared__ Tables T;
-    load_tables(P, T);
-    unsigned char *occ = load_diag_tables(P, s_w);
     grid_wait();
     if (st->status) return;
     const long long n = st->diag_n;
     if ((long long)blockIdx.x * blockDim.x >= n) return;
+    load_tables(P, T);
+    unsigned char *occ = load_diag_tables(P, s_w);
     __syncthreads();
     const int lb = st->lb;
     const int *new_slots = P.pop[lb][st->diag_pp];
@@ -409,6 +409,7 @@ struct GroupDev {
 template <int W>
 __global__ void __launch_bounds__(256) k_receive(Params P, const PartLink *links) {
     DevState *st = P.st;
+    grid_wait();
     if (st->status) return;
     constexpr int S = Stride<W>::v;
     for (int r = 0; r < P.n_parts; ++r) {

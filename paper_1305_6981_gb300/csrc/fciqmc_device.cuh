@@ -180,12 +180,11 @@ __device__ __forceinline__ void set_status(DevState *st, int code) { atomicCAS(&
 #endif
 
 // ---------------------------------------------------------------------------
-// The kernels of an iteration are launched with programmatic dependencies (launch_next): a kernel's blocks may be
-// placed as its predecessor's blocks leave. (Placed from the predecessor's start on, by launch_dependents, the waiting
-// blocks got in its way: 232 instead of 217 us per iteration on 6e6 walkers of 24e/60o.) grid_wait() returns when the predecessor has finished and
-// its writes are visible; before it, a kernel reads only what no kernel of an iteration writes (tables made at
-// creation). Every block calls it, also those that have nothing to do, so that "the predecessor has finished" holds
-// for the whole chain. Without the launch attribute it returns at once.
+// The kernels of an iteration are launched with programmatic dependencies (launch_next): a kernel's blocks are placed as
+// its predecessor's blocks leave, and grid_wait() returns when the predecessor has finished and its writes are visible.
+// Every block calls it first, also those that have nothing to do, so that "the predecessor has finished" holds for the
+// whole chain. Without the launch attribute it returns at once. (Blocks placed from the predecessor's start on, by
+// launch_dependents, got in its way: 232 instead of 217 us per iteration on 6e6 walkers of 24e/60o.)
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // True in the last block of the kernel to get here; all blocks' earlier writes are then visible to its later reads
 // that go past L1 (volatile, __ldcg). Every block of the grid has to call it.

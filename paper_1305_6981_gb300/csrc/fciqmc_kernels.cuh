@@ -1391,13 +1391,13 @@ __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) 
     __shared__ float s_rcpf[MAXSO + 2];  // two class counts (at most 64 each) add up to an index
     __shared__ unsigned long long s_red[(kTile / 32) * (NCNT + 4)];
     __shared__ long long s_tile[2];
-    load_tables(P, T);
-    for (int k = threadIdx.x; k < MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
     grid_wait();
     if (st->status) return;
     const long long len = st->list_len;
     const int tile = st->tile ? st->tile : kTile;  // determinants per tile this iteration
     if ((long long)blockIdx.x * tile >= len) return;  // a short list: no tile for this block
+    load_tables(P, T);
+    for (int k = threadIdx.x; k < MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
     if (threadIdx.x == 0) s_tile[0] = (long long)blockIdx.x * tile;
     const int lb = st->lb, pp = st->pp;
     const unsigned iter = (unsigned)st->iter;
@@ -1636,8 +1636,6 @@ __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
     __shared__ __align__(8) unsigned s_pend[NW][31 + 32 * U];  // attempts that passed the screen; last the counters' sums
     __shared__ float s_rcpf[MAXSO + 2];           // two class counts (at most 64 each) add up to an index
     static_assert(sizeof(s_pend) >= sizeof(unsigned long long) * NW * NCNT, "room for the counters of every warp");
-    load_tables(P, T);
-    for (int k = threadIdx.x; k < MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
     grid_wait();
     if (st->status) return;
     const unsigned long long packed = st->heavy_packed;
@@ -1669,6 +1667,8 @@ __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
     };
     bool done = q >= nch;
     if (!__syncthreads_or(done ? 0 : 1)) return;  // a short list: nothing left for this block
+    load_tables(P, T);
+    for (int k = threadIdx.x; k < MAXSO + 2; k += blockDim.x) s_rcpf[k] = P.rcpf[k];
     const unsigned iter = (unsigned)st->iter;
     const unsigned chunk = st->heavy_chunk ? st->heavy_chunk : (unsigned)kChunk;
     const DetView<W> *heavy = reinterpret_cast<const DetView<W> *>(P.heavy);

@@ -10,8 +10,8 @@ namespace fq {
 struct Params;
 
 // Launches a kernel of an iteration. next: with a programmatic dependency on the launch before it on the stream, so
-// that its blocks are placed while that one drains and its table loads overlap (the kernels call grid_wait() before
-// they read anything an iteration changes). Captured into a graph, the dependency becomes a programmatic edge.
+// that its blocks are placed while that one drains (the kernels call grid_wait() before they read anything). Captured
+// into a graph, the dependency becomes a programmatic edge.
 template <typename... K, typename... A>
 cudaError_t launch_next(void (*kernel)(K...), int grid, int block, size_t smem, cudaStream_t s, bool next, A... args) {
     cudaLaunchConfig_t cfg = {};
