@@ -85,7 +85,8 @@ int log2i(long long x) {
 }
 
 constexpr int kSms = 152;                     // blocks of the passes that take one block per SM
-constexpr int kPairGrid = kSms * 8;           // blocks of the pair passes
+constexpr int kPairGrid = kSms * 32;          // most blocks of the pair passes (several waves: partitions differ in cost)
+constexpr int kPairThreads = 128;
 constexpr int kNormGrid = kSms;
 
 struct Dims {
@@ -952,9 +953,9 @@ __device__ __forceinline__ RowRange row_range(unsigned packed, int local) {
 // within one partition (a handful of rows), compensated across partitions, the blocks' sums in a fixed tree. A
 // row is an FMA chain of at most half a small group, or of eight partners of a large one at a time.
 // Bound by the FP64 pipe (one FMA per pair, charged per warp instruction) and the table reads from L2.
-__global__ void __launch_bounds__(kThreads) k_pair_energy(const Member *members, const unsigned *base_p, const unsigned *count_p,
+__global__ void __launch_bounds__(kPairThreads) k_pair_energy(const Member *members, const unsigned *base_p, const unsigned *count_p,
                                                           int parts, int n1, int n2, const double *table, double *partial) {
-    __shared__ CSum s_red[kThreads / 32];
+    __shared__ CSum s_red[kPairThreads / 32];
     CSum acc{0.0, 0.0};
     const double *mixed = table + (size_t)n1 * n1;
     for (int p = blockIdx.x; p < parts; p += gridDim.x) {
@@ -962,7 +963,7 @@ __global__ void __launch_bounds__(kThreads) k_pair_energy(const Member *members,
         const int cnt = (int)count_p[p];
         if ((int)threadIdx.x >= cnt) continue;
         double sum = 0.0;
-        for (int j = threadIdx.x; j < cnt; j += kThreads) {
+        for (int j = threadIdx.x; j < cnt; j += kPairThreads) {
             const Member u = mem[j];
             const Member *grp = mem + u.first;
             const RowRange r = row_range(u.code, j - (int)u.first);
@@ -1023,13 +1024,13 @@ __global__ void __launch_bounds__(1024) k_energy_finish(const double *pp, int np
 
 // The two-body density matrix over pair codes: v v' of every pair of members added at (smaller code, larger code) with
 // one FP64 reduction in L2. Large groups walk a triangle, so a warp's reductions fall in one table row.
-__global__ void __launch_bounds__(kThreads) k_pair_grad(const Member *members, const unsigned *base_p, const unsigned *count_p,
+__global__ void __launch_bounds__(kPairThreads) k_pair_grad(const Member *members, const unsigned *base_p, const unsigned *count_p,
                                                         int parts, int n1, int n2, double *table) {
     double *mixed = table + (size_t)n1 * n1;
     for (int p = blockIdx.x; p < parts; p += gridDim.x) {
         const Member *mem = members + base_p[p];
         const int cnt = (int)count_p[p];
-        for (int j = threadIdx.x; j < cnt; j += kThreads) {
+        for (int j = threadIdx.x; j < cnt; j += kPairThreads) {
             const Member u = mem[j];
             const Member *grp = mem + u.first;
             const RowRange r = row_range(u.code, j - (int)u.first);
@@ -1234,7 +1235,7 @@ void launch_energy(fciqmc_rdm *r, const double *h, const double *eri, double *e)
     double *partial = ptr<double>(r, r->L.partial), *table = ptr<double>(r, r->L.table);
     const int g = pair_grid(d);
     k_pair_table<<<table_grid(d, 0), kThreads, 0, s>>>(h, eri, d.n_orb, d.n1, d.n2, 1.0 / (d.n_elec - 1), table);
-    k_pair_energy<<<g, kThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p), ptr<unsigned>(r, r->L.count_p),
+    k_pair_energy<<<g, kPairThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p), ptr<unsigned>(r, r->L.count_p),
                                          d.parts, d.n1, d.n2, table, partial);
     k_energy_finish<<<1, 1024, 0, s>>>(partial, g, ptr<double>(r, r->L.occ_pair), h, eri, d.n_orb, st, e);
 }
@@ -1246,7 +1247,7 @@ void launch_rdm(fciqmc_rdm *r) {
     cudaMemsetAsync(gh, 0, sizeof(double) * d.n_orb * d.n_orb, s);
     cudaMemsetAsync(ge, 0, sizeof(double) * d.n_eri, s);
     cudaMemsetAsync(table, 0, sizeof(double) * ((size_t)d.n1 * d.n1 + (size_t)d.n2 * d.n2), s);
-    k_pair_grad<<<pair_grid(d), kThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p),
+    k_pair_grad<<<pair_grid(d), kPairThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p),
                                                   ptr<unsigned>(r, r->L.count_p), d.parts, d.n1, d.n2, table);
     k_fold<<<table_grid(d, d.n_so), kThreads, 0, s>>>(table, ptr<double>(r, r->L.occ_pair), d.n_orb, d.n1, d.n2,
                                                       1.0 / (d.n_elec - 1), gh, ge);
