@@ -306,15 +306,20 @@ constexpr int kDiagThreads = 128;
 __host__ __device__ constexpr size_t diag_bytes(int n_orb, int ostride) {
     return sizeof(double) * ((size_t)2 * n_orb * n_orb + n_orb) + (size_t)kDiagThreads * ostride;
 }
-// Copies the pair terms and h_pp to shared memory (16 bytes at a time); returns the thread's occupied list.
+// Starts the copy of the pair terms to shared memory (asynchronous, 16 bytes at a time; wait_diag_tables ends it) and
+// copies h_pp; returns the thread's occupied list.
 __device__ __forceinline__ unsigned char *load_diag_tables(const Params &P, double *s_w) {
     const int M = P.n_orb;
     const double2 *src = reinterpret_cast<const double2 *>(P.wpair);
-    double2 *dst = reinterpret_cast<double2 *>(s_w);
-#pragma unroll 4
-    for (int k = threadIdx.x; k < M * M; k += blockDim.x) dst[k] = src[k];
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(s_w);
+    for (int k = threadIdx.x; k < M * M; k += blockDim.x)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * (unsigned)k), "l"(src + k) : "memory");
     for (int k = threadIdx.x; k < M; k += blockDim.x) s_w[2 * M * M + k] = P.h[k * M + k];
     return reinterpret_cast<unsigned char *>(s_w + 2 * M * M + M) + threadIdx.x * P.ostride;
+}
+__device__ __forceinline__ void wait_diag_tables() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
 }
 // H_ii - E0 of a determinant with its occupied list.
 template <int W>
@@ -331,22 +336,24 @@ template <int W>
 __global__ void __launch_bounds__(kDiagThreads) k_new_diag(Params P) {
     extern __shared__ __align__(16) double s_w[];
     DevState *st = P.st;
-    __shared__ Tables T;
     grid_wait();
     if (st->status) return;
     const long long n = st->diag_n;
     if ((long long)blockIdx.x * blockDim.x >= n) return;
-    load_tables(P, T);
     unsigned char *occ = load_diag_tables(P, s_w);
-    __syncthreads();
     const int lb = st->lb;
     const int *new_slots = P.pop[lb][st->diag_pp];
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const long long s = new_slots[k];
+    bool ready = false;  // the tables are needed after the first slot's derived data
+    for (long long k0 = (long long)blockIdx.x * blockDim.x; k0 < n; k0 += (long long)gridDim.x * blockDim.x) {
+        const long long k = k0 + threadIdx.x;
+        const long long s = new_slots[min(k, n - 1)];  // (threads past the end read the last slot and write nothing)
         unsigned long long key[W];
 #pragma unroll
         for (int w = 0; w < W; ++w) key[w] = P.det[lb][s * W + w];
-        store_derived<W>(P, T, lb, s, key, occ);
+        if (k < n) store_derived<W>(P, lb, s, key, occ);
+        if (!ready) wait_diag_tables();
+        ready = true;
+        if (k >= n) continue;
         const double hdv = diag_element<W>(P, key, occ, s_w);
         P.hd[lb][s] = hdv;
         P.hdf[lb][s] = __double2float_rn(hdv);
@@ -789,16 +796,14 @@ __global__ void k_index_clear_at(Params P, const int *pos, long long n) {
 template <int W>
 __global__ void __launch_bounds__(kDiagThreads) k_prepare_list(Params P, int b, long long lo, long long n, int compute) {
     extern __shared__ __align__(16) double s_w[];
-    __shared__ Tables T;
-    load_tables(P, T);
     unsigned char *occ = compute ? load_diag_tables(P, s_w)
                                  : reinterpret_cast<unsigned char *>(s_w) + threadIdx.x * P.ostride;
-    __syncthreads();
+    if (compute) wait_diag_tables();
     for (long long s = lo + (long long)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
         unsigned long long d[W];
 #pragma unroll
         for (int w = 0; w < W; ++w) d[w] = P.det[b][s * W + w];
-        store_derived<W>(P, T, b, s, d, occ);
+        store_derived<W>(P, b, s, d, occ);
         if (compute) {
             const double v = diag_element<W>(P, d, occ, s_w);
             P.hd[b][s] = v;
@@ -893,7 +898,7 @@ __global__ void __launch_bounds__(256) k_bounds(Params P, float *bnd) {
 template <int W>
 __global__ void __launch_bounds__(256) k_ref_table(Params P, unsigned *pinfo, unsigned *off2, RefExc *ex,
                                                    long long cap, long long *out) {
-    __shared__ Tables T;
+    __shared__ AttemptTables T;
     __shared__ DetView<W> v;
     __shared__ unsigned char occ[MAXN];
     __shared__ unsigned s_g[MAXPAIRS], s_go[MAXPAIRS], s_eo[MAXPAIRS];
@@ -903,7 +908,7 @@ __global__ void __launch_bounds__(256) k_ref_table(Params P, unsigned *pinfo, un
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int w = 0; w < W; ++w) v.d[w] = P.ref[w];
-        prepare_det<W>(P, T, v, occ, 1);
+        prepare_det<W>(P, v, occ, 1);
     }
     __syncthreads();
     const int np = P.npairs;

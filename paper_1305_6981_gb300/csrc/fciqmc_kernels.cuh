@@ -92,11 +92,6 @@ struct AttemptTables {
     unsigned char irrep[MAXSO / 2];
     unsigned short pairs[MAXPAIRS];
 };
-// With the orbital map of Algorithm 1, for the kernels that derive a determinant's data.
-struct Tables : AttemptTables {
-    unsigned long long map1[MAXSO];
-};
-
 __device__ __forceinline__ void load_tables(const Params &P, AttemptTables &T) {
     for (int k = threadIdx.x; k < NCLASS * MAXW; k += blockDim.x) T.mask[k] = P.cmask[k];
     for (int k = threadIdx.x; k < 2 * 2 * 16 * MAXW; k += blockDim.x) {
@@ -109,11 +104,6 @@ __device__ __forceinline__ void load_tables(const Params &P, AttemptTables &T) {
     for (int k = threadIdx.x; k < MAXW; k += blockDim.x) T.all[k] = k * 64 >= P.n_so ? 0ull : low_bits(min(P.n_so - 64 * k, 64));
     for (int k = threadIdx.x; k < P.n_orb; k += blockDim.x) T.irrep[k] = P.irrep[k];
     for (int k = threadIdx.x; k < P.npairs; k += blockDim.x) T.pairs[k] = P.pairs[k];
-}
-
-__device__ __forceinline__ void load_tables(const Params &P, Tables &T) {
-    for (int k = threadIdx.x; k < P.n_so; k += blockDim.x) T.map1[k] = P.map1[k];
-    load_tables(P, static_cast<AttemptTables &>(T));
 }
 
 // ---------------------------------------------------------------------------- float bounds
@@ -184,17 +174,18 @@ enum { PRE_FP = 0, PRE_OKM, PRE_CB0, PRE_CB1, PRE_WORDS };
 
 // Class counts first (population counts against the class masks); then one pass over the occupied spin
 // orbitals in ascending order gives the occupied list, the electrons with an allowed single and the
-// fingerprint.
+// fingerprint. The class masks and the orbital map come from global memory (two kilobytes, the masks the same for all
+// lanes), so that a kernel can derive while its other tables are on their way.
 template <int W>
-__device__ __forceinline__ void derive_det(const Params &P, const Tables &T, const unsigned long long (&d)[W],
+__device__ __forceinline__ void derive_det(const Params &P, const unsigned long long (&d)[W],
                                            unsigned long long (&pre)[PRE_WORDS], unsigned char *occ) {
     unsigned long long cb0 = 0, cb1 = 0;
     for (int g = 0; g < P.n_irrep_used; ++g) {
         int u0 = 0, u1 = 0;
 #pragma unroll
         for (int w = 0; w < W; ++w) {
-            u0 += __popcll(~d[w] & T.mask[(2 * g) * MAXW + w]);
-            u1 += __popcll(~d[w] & T.mask[(2 * g + 1) * MAXW + w]);
+            u0 += __popcll(~d[w] & __ldg(P.cmask + (2 * g) * MAXW + w));
+            u1 += __popcll(~d[w] & __ldg(P.cmask + (2 * g + 1) * MAXW + w));
         }
         cb0 |= (unsigned long long)u0 << (8 * g);
         cb1 |= (unsigned long long)u1 << (8 * g);
@@ -215,7 +206,7 @@ __device__ __forceinline__ void derive_det(const Params &P, const Tables &T, con
             if (!FQ_CHECK(n < MAXN, P.st)) break;
             occ[n] = (unsigned char)k;
             okm |= ((ok[w] >> b) & 1ull) << n;
-            h = 1099511628211ull * h + T.map1[k] * (unsigned long long)(n + 1);
+            h = 1099511628211ull * h + __ldg(P.map1 + k) * (unsigned long long)(n + 1);
             ++n;
             m &= m - 1;
         }
@@ -251,21 +242,20 @@ __device__ __forceinline__ void fill_view(const Params &P, DetView<W> &v, const 
 
 // The view of v.d (its bits already set), derived on the spot.
 template <int W>
-__device__ __forceinline__ void prepare_det(const Params &P, const Tables &T, DetView<W> &v, unsigned char *occ,
-                                            int c) {
+__device__ __forceinline__ void prepare_det(const Params &P, DetView<W> &v, unsigned char *occ, int c) {
     unsigned long long pre[PRE_WORDS];
-    derive_det<W>(P, T, v.d, pre, occ);
+    derive_det<W>(P, v.d, pre, occ);
     fill_view<W>(P, v, pre, c);
 }
 
 // Derived words and occupied list of slot s of list buffer b, computed and stored; the list is left in occ
 // (P.ostride bytes, 4-byte aligned).
 template <int W>
-__device__ __forceinline__ void store_derived(const Params &P, const Tables &T, int b, long long s,
+__device__ __forceinline__ void store_derived(const Params &P, int b, long long s,
                                               const unsigned long long (&d)[W], unsigned char *occ) {
     unsigned long long pre[PRE_WORDS];
     for (int k = P.n_elec; k < P.ostride; ++k) occ[k] = 0;
-    derive_det<W>(P, T, d, pre, occ);
+    derive_det<W>(P, d, pre, occ);
     ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(P.pre[b] + s * PRE_WORDS);
     dst[0] = make_ulonglong2(pre[0], pre[1]);
     dst[1] = make_ulonglong2(pre[2], pre[3]);
