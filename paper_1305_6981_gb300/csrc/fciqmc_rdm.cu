@@ -866,7 +866,8 @@ __global__ void __launch_bounds__(256) k_occ_pairs(const unsigned long long *det
     }
 }
 
-// Sums of the blocks' occupation pairs (compensated, in block order); the last block adds the partial sums of c^2.
+// Sums of the blocks' occupation pairs (compensated): a warp adds 8 entries, four lanes each taking every fourth block in
+// order, merged in a fixed tree. The last block adds the partial sums of c^2.
 __global__ void __launch_bounds__(kMergeThreads) k_occ_merge(const double *occ_part, int nblocks, int nent, double *occ_pair,
                                                              const double *norm_part, int n_norm, RdmState *st) {
     if (blockIdx.x == gridDim.x - 1) {
@@ -877,11 +878,22 @@ __global__ void __launch_bounds__(kMergeThreads) k_occ_merge(const double *occ_p
         if (threadIdx.x == 0) st->norm = __dadd_rn(a.s, a.c);
         return;
     }
-    const int k = blockIdx.x * kMergeThreads + threadIdx.x;
-    if (k >= nent) return;
+    const int lane = threadIdx.x & 31, part = lane >> 3;
+    const int k = (blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5)) * 8 + (lane & 7);
     CSum a{0.0, 0.0};
-    for (int b = 0; b < nblocks; ++b) csum_add(a, occ_part[(size_t)b * nent + k]);
-    occ_pair[k] = __dadd_rn(a.s, a.c);
+    if (k < nent)
+        for (int b0 = part; b0 < nblocks; b0 += 16) {  // four reads in flight
+            double x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = b0 + 4 * u < nblocks ? occ_part[(size_t)(b0 + 4 * u) * nent + k] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) csum_add(a, x[u]);
+        }
+    for (int o = 16; o >= 8; o >>= 1) {
+        const CSum b{__shfl_down_sync(0xFFFFFFFFu, a.s, o), __shfl_down_sync(0xFFFFFFFFu, a.c, o)};
+        csum_merge(a, b);
+    }
+    if (k < nent && part == 0) occ_pair[k] = __dadd_rn(a.s, a.c);
 }
 
 __global__ void __launch_bounds__(kThreads) k_norm(const double *c, long long n, double *partial) {
@@ -1215,7 +1227,7 @@ int construct(fciqmc_rdm *r) {
     const int go = (int)std::min<long long>(kSms, (d.n + nw - 1) / nw), gn = (int)std::min<long long>(kNormGrid, (d.n + kThreads - 1) / kThreads);
     k_norm<<<gn, kThreads, 0, s>>>(c, d.n, norm_part);
     k_occ_pairs<W><<<go, 32 * nw, sm_occ, s>>>(dets, c, d.n, d.n_elec, d.n_so, ptr<double>(r, r->L.occ_part));
-    k_occ_merge<<<(unsigned)((nent + kMergeThreads - 1) / kMergeThreads) + 1, kMergeThreads, 0, s>>>(
+    k_occ_merge<<<(unsigned)((nent + kMergeThreads / 4 - 1) / (kMergeThreads / 4)) + 1, kMergeThreads, 0, s>>>(
         ptr<double>(r, r->L.occ_part), go, (int)nent, ptr<double>(r, r->L.occ_pair), norm_part, gn, st);
     if (cudaGetLastError() != cudaSuccess) return FCIQMC_ERR_CUDA;
     if (cudaMemcpyAsync(&r->host, st, sizeof(RdmState), cudaMemcpyDeviceToHost, s) != cudaSuccess) return FCIQMC_ERR_CUDA;

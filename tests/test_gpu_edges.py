@@ -88,3 +88,19 @@ def test_empty_walker_list():
     assert all(r["nw_out"] == 0 and r["attempts"] == 0 for r in rows)
     assert len(g.walkers()[1]) == 0
     g.close()
+
+
+@pytest.mark.parametrize("steps,want", [(5, 16), (16, 16), (21, 16), (40, 7)])
+def test_history_ring_in_one_or_two_pieces(steps, want):
+    """The newest rows, oldest first, before and after the ring of 16 rows has wrapped."""
+    from paper_1305_6981_gb300 import Fciqmc
+    runs = [Fciqmc(synth.tiny_8e8o(), 0.01, -1, initial_population=50, seed=3, main_capacity=1 << 12, history_capacity=c)
+            for c in (16, 64)]
+    for g in runs:
+        g.step(steps)
+    short, full = (g.history(want) for g in runs)
+    assert [r["iteration"] for r in short] == list(range(max(0, steps - want), steps)) and len(short) == min(steps, want, 16)
+    ints = [k for k in short[0] if k != "num_in"]  # (the numerator is summed in slot order)
+    assert [[r[k] for k in ints] for r in short] == [[r[k] for k in ints] for r in full]
+    for g in runs:
+        g.close()
