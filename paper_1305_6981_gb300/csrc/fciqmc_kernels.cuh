@@ -7,9 +7,11 @@
 //                  into the spawn table (sum of signed amounts, initiator flags counted)
 //   k_heavy        the attempts of determinants with |C_i| > kHeavy, split into chunks
 //   k_annihilate   the merged spawns against the post-death main list through the hash index, with
-//                  the initiator filter and H_ii on insertion (Sec. V B)
-//   k_finish       deterministic reduction of the projected-energy numerator, history row, shift
-//                  update, population parity flip
+//                  the initiator filter (Sec. V B); its last block sums the projected-energy numerator
+//                  in a fixed order, writes the history row, updates the shift and commits the list
+//   k_new_diag     H_ii and the derived words of the determinants inserted
+// Hybrid walkers have k_round and k_finish between these and the next iteration (the threshold changes the
+// populations that the row counts); partitions have k_receive and k_group_finish.
 #pragma once
 
 #include "fciqmc_device.cuh"
@@ -495,6 +497,39 @@ __device__ __forceinline__ int decide_spawn(float p_lo, float p_hi, unsigned lon
     return -1;
 }
 
+// The exact decisions (FP64) of a double and a single, for about one attempt in three million: the number spawned,
+// with the sign of the element before its parity. They are calls, because in line they lie in the middle of loops that
+// already miss the instruction cache (k_heavy waited 3.2 warps an issue for instructions, more than for memory):
+// k_heavy 1.00 to 1.11 ms before, 0.88 to 0.90 after on 1.2e8 walkers of 24e/60o, 94 and 88 us on 6e6. (The queue's
+// flush as a call, or Philox rounds in a loop, gave nothing or lost it again.)
+static __device__ __noinline__ int exact_double(const double *eri, const double *recip, DevState *st, int i, int j, int A, int B,
+                                                double cd, double d53, long long K, unsigned L, unsigned long long t) {
+    atomicAdd(&st->exact_spawn, 1ull);
+    double v = 0.0;
+    if ((i & 1) == (A & 1) && (j & 1) == (B & 1)) v = __dadd_rn(v, __ldg(eri + eidx(i >> 1, A >> 1, j >> 1, B >> 1)));
+    if ((i & 1) == (B & 1) && (j & 1) == (A & 1)) v = __dsub_rn(v, __ldg(eri + eidx(i >> 1, B >> 1, j >> 1, A >> 1)));
+    if (v == 0.0) return 0;
+    // p = ((|H| (tau / P_double)) (npairs G M^(b|a) M^(a|b))) (1 / (M^(b|a) + M^(a|b)))
+    const double p = __dmul_rn(__dmul_rn(__dmul_rn(fabs(v), cd), (double)K), recip[L]);
+    const double fl = floor(p);
+    if (fl >= 2147483647.0) { set_status(st, FCIQMC_ERR_NUMERIC); return 0; }
+    const int n = (int)fl + (__ull2double_rn(t) < __dmul_rn(__dsub_rn(p, fl), d53) ? 1 : 0);
+    return v > 0.0 ? n : -n;
+}
+static __device__ __noinline__ int exact_single(const double *h, const double *eri, DevState *st, int n_orb, int n_elec,
+                                                const unsigned char *occ, int i, int a, double cs, double d53, long long K,
+                                                unsigned long long q) {
+    atomicAdd(&st->exact_spawn, 1ull);
+    const double v = single_element(h, eri, n_orb, n_elec, occ, i, a);
+    if (v == 0.0) return 0;
+    // p = (|H| (tau / P_single)) (M_allow (N - delta_s))
+    const double p = __dmul_rn(__dmul_rn(fabs(v), cs), (double)K);
+    const double fl = floor(p);
+    if (fl >= 2147483647.0) { set_status(st, FCIQMC_ERR_NUMERIC); return 0; }
+    const int n = (int)fl + (__ull2double_rn(q) < __dmul_rn(__dsub_rn(p, fl), __dsub_rn(9007199254740992.0, d53)) ? 1 : 0);
+    return v > 0.0 ? n : -n;
+}
+
 // Counters and queued merge-table entry of an attempt that spawns n > 0 walkers onto child.
 template <int W>
 __device__ __forceinline__ void emit_spawn(const Params &P, const DetView<W> &v, const unsigned long long (&child)[W],
@@ -906,24 +941,15 @@ __device__ __forceinline__ bool attempt_begin(const Params &P, const AttemptTabl
     const float ah_lo = fabsf(hf) - eh, ah_hi = fabsf(hf) + eh;
     const float F = P.cdn_f * small_f(G) * small_f(m_ba) * small_f(m_ab) * rcpf[L];
     int n = decide_spawn(ah_lo * F * kDown, ah_hi * F * kUp, t, P.d53_f);
-    int sgn_h;
-    if (n >= 0) {
-        if (n == 0) return false;
-        sgn_h = hf > 0.f ? 1 : -1;  // |hf| > eh: same sign as H
-        if (double_parity<W>(v.d, i, j, A, B)) sgn_h = -sgn_h;
-    } else {
-        atomicAdd(&P.st->exact_spawn, 1ull);
-        const double hd = hij_double<W>(P, v.d, i, j, A, B);
-        if (hd == 0.0) return false;
-        // p = ((|H| (tau / P_double)) (npairs G M^(b|a) M^(a|b))) (1 / (M^(b|a) + M^(a|b)))
-        const long long K = (long long)P.npairs * (long long)G * (long long)m_ba * (long long)m_ab;
-        const double p = __dmul_rn(__dmul_rn(__dmul_rn(fabs(hd), P.cd), (double)K), P.recip[L]);
-        const double fl = floor(p);
-        if (fl >= 2147483647.0) { set_status(P.st, FCIQMC_ERR_NUMERIC); return false; }
-        n = (int)fl + (__ull2double_rn(t) < __dmul_rn(__dsub_rn(p, fl), P.d53_d) ? 1 : 0);
-        sgn_h = hd > 0.0 ? 1 : -1;
-        if (n == 0) return false;
+    int sgn_h = hf > 0.f ? 1 : -1;  // where n > 0, |hf| > eh: same sign as H
+    if (n < 0) {
+        n = exact_double(P.eri, P.recip, P.st, i, j, A, B, P.cd, P.d53_d,
+                         (long long)P.npairs * (long long)G * (long long)m_ba * (long long)m_ab, L, t);
+        sgn_h = n > 0 ? 1 : -1;
+        n = abs(n);
     }
+    if (n == 0) return false;
+    if (double_parity<W>(v.d, i, j, A, B)) sgn_h = -sgn_h;
     unsigned long long child[W];
 #pragma unroll
     for (int w = 0; w < W; ++w) child[w] = v.d[w];
@@ -1158,24 +1184,14 @@ __device__ __forceinline__ void attempt_single_end(const Params &P, const DetVie
     const float ah_lo = fabsf(hs) - eh, ah_hi = fabsf(hs) + eh;
     const float F = P.cs_f * small_f(mallow * v.nok);
     int n = decide_spawn(ah_lo * F * kDown, ah_hi * F * kUp, q, P.srange_f);
-    int sgn_h;
-    if (n >= 0) {
-        if (n == 0) return;
-        sgn_h = hs > 0.f ? 1 : -1;
-        if (count_between<W>(v.d, i, ao) & 1) sgn_h = -sgn_h;
-    } else {
-        atomicAdd(&P.st->exact_spawn, 1ull);
-        const double hv = hij_single<W>(P, v.d, occ, i, ao);
-        if (hv == 0.0) return;
-        // p = (|H| (tau / P_single)) (M_allow (N - delta_s))
-        const double p = __dmul_rn(__dmul_rn(fabs(hv), P.cs), (double)((long long)mallow * (long long)v.nok));
-        const double fl = floor(p);
-        if (fl >= 2147483647.0) { set_status(P.st, FCIQMC_ERR_NUMERIC); return; }
-        const double range = __dsub_rn(9007199254740992.0, P.d53_d);
-        n = (int)fl + (__ull2double_rn(q) < __dmul_rn(__dsub_rn(p, fl), range) ? 1 : 0);
-        sgn_h = hv > 0.0 ? 1 : -1;
-        if (n == 0) return;
+    int sgn_h = hs > 0.f ? 1 : -1;
+    if (n < 0) {
+        n = exact_single(P.h, P.eri, P.st, P.n_orb, P.n_elec, occ, i, ao, P.cs, P.d53_d, (long long)mallow * (long long)v.nok, q);
+        sgn_h = n > 0 ? 1 : -1;
+        n = abs(n);
     }
+    if (n == 0) return;
+    if (count_between<W>(v.d, i, ao) & 1) sgn_h = -sgn_h;
     unsigned long long child[W];
 #pragma unroll
     for (int w = 0; w < W; ++w) child[w] = v.d[w];
