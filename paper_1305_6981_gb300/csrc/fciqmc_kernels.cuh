@@ -1118,13 +1118,15 @@ static __device__ __noinline__ float2 single_sums(const float *h_f, const float 
 // delta_spin (ij|ja)] (without the parity sign) for every lane with a pending single, each evaluated by
 // the whole warp: lane x takes electrons x, x + 32. Where many lanes have one, each evaluates its own instead, four
 // electrons at a time: about 32 N instructions for the warp against 80 per single, and without a round trip
-// to L2 for each (8e/8o, three singles in 32 attempts: 85 to 55 us per iteration). Called by all 32 lanes.
-template <int W>
+// to L2 for each (8e/8o, three singles in 32 attempts: 85 to 55 us per iteration); not on spin-coupled functions
+// (EACH false), whose longer loop loses more by the call than their rare singles gain (9.2e7 walkers of 24e/60o:
+// k_heavy 2.91 ms with it, 2.70 without). Called by all 32 lanes.
+template <int W, bool EACH>
 __device__ __forceinline__ void single_elements_warp(const Params &P, const unsigned char *occp, bool pend, int i,
                                                      int a, unsigned long long pol, float &hs, float &hab) {
     unsigned need = __ballot_sync(0xFFFFFFFFu, pend);
     const int lane = threadIdx.x & 31;
-    if (5 * __popc(need) >= 2 * P.n_elec) {
+    if (EACH && 5 * __popc(need) >= 2 * P.n_elec) {
         if (pend) {
             const float2 r = single_sums(P.h_f, P.eri_f, P.n_orb, P.n_elec, occp, i, a, pol);
             hs = r.x;
@@ -1292,10 +1294,10 @@ __device__ __forceinline__ void spawn_attempt(const Params &P, const AttemptTabl
         pend = attempt_begin<W, TAB, MODE>(P, T, v, occ, tab, rcpf, a, iter, pol, cnt, out, i, ao, mallow, q, i1, a1, i2, a2,
                                            rtab);
     float hs = 0.f, hab = 0.f;
-    single_elements_warp<W>(P, occ, pend, i1, a1, pol, hs, hab);
+    single_elements_warp<W, (MODE & 2) == 0>(P, occ, pend, i1, a1, pol, hs, hab);
     if (MODE & 2) {
         float hs2 = 0.f, hab2 = 0.f;
-        single_elements_warp<W>(P, occ, pend && i2 >= 0, i2, a2, pol, hs2, hab2);
+        single_elements_warp<W, (MODE & 2) == 0>(P, occ, pend && i2 >= 0, i2, a2, pol, hs2, hab2);
         if (pend) hphf_single_end<W>(P, v, tab, i, ao, i1, a1, i2, a2, mallow, q, hs, hab, hs2, hab2, cnt, out);
     } else if (pend) {
         attempt_single_end<W>(P, v, occ, i, ao, mallow, q, hs, hab, cnt, out);
