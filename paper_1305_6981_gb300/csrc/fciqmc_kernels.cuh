@@ -499,9 +499,9 @@ __device__ __forceinline__ int decide_spawn(float p_lo, float p_hi, unsigned lon
 
 // The exact decisions (FP64) of a double and a single, for about one attempt in three million: the number spawned,
 // with the sign of the element before its parity. They are calls, because in line they lie in the middle of loops that
-// already miss the instruction cache (k_heavy waited 3.2 warps an issue for instructions, more than for memory):
-// k_heavy 1.00 to 1.11 ms before, 0.88 to 0.90 after on 1.2e8 walkers of 24e/60o, 94 and 88 us on 6e6. (The queue's
-// flush as a call, or Philox rounds in a loop, gave nothing or lost it again.)
+// already miss the instruction cache (k_heavy waited 3.2 warps an issue for instructions, as many as for memory):
+// k_heavy 0.99 to 1.11 ms before, 0.88 to 0.98 after on 1.2e8 walkers of 24e/60o, 94 and 88 us on 6e6. (The queue's
+// flush or the table build as calls, or Philox rounds in a loop, gave nothing or lost it again.)
 static __device__ __noinline__ int exact_double(const double *eri, const double *recip, DevState *st, int i, int j, int A, int B,
                                                 double cd, double d53, long long K, unsigned L, unsigned long long t) {
     atomicAdd(&st->exact_spawn, 1ull);
