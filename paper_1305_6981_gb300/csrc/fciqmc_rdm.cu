@@ -161,6 +161,16 @@ __device__ __forceinline__ void load_det(const unsigned long long *dets, long lo
     }
 }
 
+// A key's hash as it is used. -DFQ_RDM_HASH_BITS=b leaves 2^b different ones, so that a test can have keys that share
+// all hash bits in every partition of a small list.
+__device__ __forceinline__ unsigned long long used_hash(unsigned long long h) {
+#ifdef FQ_RDM_HASH_BITS
+    return fq::mix64(h & ((1ull << FQ_RDM_HASH_BITS) - 1ull));
+#else
+    return h;
+#endif
+}
+
 // The hash word of a spin orbital.
 __device__ __forceinline__ unsigned long long orbital_word(int k) { return fq::mix64(0x9E3779B97F4A7C15ull * (unsigned long long)(k + 1)); }
 
@@ -258,7 +268,7 @@ __device__ __forceinline__ void for_keys(HashShared &s, const unsigned long long
         const unsigned t0 = (unsigned)(I * npairs);
         for (int k = lane; k < npairs; k += 32) {
             const unsigned short pr = s.pairs[k];
-            f(t0 + (unsigned)k, H ^ zo[pr & 0xFF] ^ zo[pr >> 8]);
+            f(t0 + (unsigned)k, used_hash(H ^ zo[pr & 0xFF] ^ zo[pr >> 8]));
         }
     }
 }
@@ -468,21 +478,22 @@ struct GroupShared {
     unsigned long long lo, hi;         // smallest and largest hash of a selection
     unsigned long long leader[kBigLeaders][W];
     unsigned long long acc[3];
-    unsigned n, min_t, kept, bad;
+    unsigned n, min_t, kept;
 };
 
 // Records s.rec[0, s.n) grouped by key; groups of two and more go to out + s.kept, longer groups first (four size
 // classes), members in the order of their codes, so that the lanes of the pair passes have rows of similar length
 // and neighbouring table columns. Grouping goes by the hash bits; every member's key is then compared with its
-// group's first, and in the rare case that two keys share the hash, false is returned and nothing is written:
-// called again with `exact`, the keys themselves are compared on insertion.
+// group's first, and where two keys share the hash, false is returned to the whole block and nothing is written:
+// called again with `exact`, the keys themselves are compared on insertion. That happens to about
+// 2850^2 / 2 / 2^30 = 0.4% of the partitions of 1.2e8 keys (2,850 distinct keys, 30 hash bits left in a
+// partition), 120 of 32,768.
 template <int W>
 __device__ __forceinline__ bool group_shared(GroupShared<W> &s, const unsigned long long *dets, const double *c, int npairs,
                                              int n_orb, int tbits, Member *out, bool exact) {
     constexpr unsigned kFree = 0xFFFFFFFFu;
     const unsigned n = s.n;
     for (int h = threadIdx.x; h < kGroupSlots; h += kGroupThreads) s.table[h] = kFree;
-    if (threadIdx.x == 0) s.bad = 0;
     __syncthreads();
     for (unsigned i = threadIdx.x; i < n; i += kGroupThreads) {
         const unsigned long long r = s.rec[i];
@@ -562,6 +573,7 @@ __device__ __forceinline__ bool group_shared(GroupShared<W> &s, const unsigned l
     __syncthreads();
     if (!exact) {
         // the same key: the determinants differ by the two pairs
+        bool bad = false;
         for (unsigned at = threadIdx.x; at < placed; at += kGroupThreads) {
             const unsigned i = s.order[at], first = s.table[s.slot[i]] >> 16;
             if (first == at) continue;
@@ -573,10 +585,11 @@ __device__ __forceinline__ bool group_shared(GroupShared<W> &s, const unsigned l
             fq::flip<W>(a, x >> 8);
             fq::flip<W>(b, y & 0xFF);
             fq::flip<W>(b, y >> 8);
-            if (!same_key<W>(a, b)) s.bad = 1;
+            if (!same_key<W>(a, b)) bad = true;
         }
-        __syncthreads();
-        if (s.bad) return false;
+        // one verdict for the block, and the barrier after which the caller may fill the table again (a flag in shared
+        // memory would be cleared by the next call while slower warps still read it)
+        if (__syncthreads_or(bad)) return false;
     }
     const unsigned kept = s.kept;
     for (unsigned at = threadIdx.x; at < placed; at += kGroupThreads) {

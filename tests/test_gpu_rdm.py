@@ -4,12 +4,17 @@ brute-force count of connected pairs, and central finite differences (E is linea
 differences are exact up to rounding)."""
 from __future__ import annotations
 
+import ctypes
+import functools
+import os
+import subprocess
+
 import numpy as np
 import pytest
 
 import bruteforce as bf
 from oracle.oracle import Oracle
-from paper_1305_6981_gb300 import synth
+from paper_1305_6981_gb300 import _native, synth
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -206,3 +211,70 @@ def test_grouping_edges_match_oracle(case):
     if len(ints) <= 1000:  # connected or not: the counts are of pairs one and two spin orbitals apart
         assert (info["single_pairs"], info["double_pairs"]) == _count_pairs(dets)
     f.close()
+
+
+def _matches_oracle(n_orb, n_elec, dets, c, want):
+    """E and both density matrices of the library against the oracle's; want: (h, eri, gh, ge) of the oracle."""
+    h, eri, ghq, geq = want
+    from paper_1305_6981_gb300 import EnergyFunctional
+    f = EnergyFunctional(n_elec, n_orb, dets, c)
+    E = float(f.energy(_dev(h), _dev(eri)))
+    gh, ge = f.gradient(torch.ones((), dtype=torch.float64, device="cuda"))
+    Eq = float((h * ghq).sum() + (eri * geq).sum())
+    assert abs(E - Eq) <= 1e-12 * max(1.0, abs(Eq))
+    assert np.abs(gh.cpu().numpy() - ghq).max() < 1e-12 and np.abs(ge.cpu().numpy() - geq).max() < 1e-12
+    if len(c) <= 1000:  # connected or not: the counts are of pairs one and two spin orbitals apart
+        info = f.info()
+        assert (info["single_pairs"], info["double_pairs"]) == _count_pairs(dets)
+    f.close()
+
+
+@functools.cache
+def _short_hash_case(name):
+    """(n_orb, n_elec, dets, c, oracle's values) of the lists that are grouped with short hashes."""
+    if name in ("16e-600", "64e-2100"):  # the second: 4.2e6 keys, 2,048 partitions, the records scattered in two passes
+        n_orb, n_elec, n = (40, 16, 600) if name == "16e-600" else (64, 64, 2100)
+        s = synth.make_system(n_orb, n_elec, seed=5, n_chol=8, fock_diagonal=False)
+        dets, c = synth.sampled_vector(s, n, seed=5)
+        c = c / np.linalg.norm(c)
+    else:
+        _, n_orb, n_elec, ints = next(x for x in _grouping_cases() if x[0] == name)
+        s = synth.make_system(n_orb, n_elec, seed=n_orb + n_elec, n_chol=8, fock_diagonal=False)
+        dets = np.array([bf.to_words(d, (2 * n_orb + 63) // 64) for d in ints], dtype=np.uint64)
+        c = np.random.default_rng(len(ints)).normal(size=len(ints))
+        c /= np.linalg.norm(c)
+    _, gh, ge = Oracle(s, tau=0.01, ms2=n_elec % 2).rdm_energy(dets, c)
+    return n_orb, n_elec, dets, c, (s.h, s.eri_s8, gh, ge)
+
+
+@pytest.fixture(scope="module")
+def short_hash_library(tmp_path_factory):
+    """bits -> the energy functional compiled with that many bits of a key's hash."""
+    return functools.cache(lambda bits: _short_hash_build(bits, str(tmp_path_factory.mktemp("rdm"))))
+
+
+def _short_hash_build(bits, where):
+    so = os.path.join(where, f"librdm{bits}.so")
+    subprocess.check_call([_native.nvcc(), _native.ARCH, *_native.NVCC_FLAGS, f"-DFQ_RDM_HASH_BITS={bits}", "-I" + _native.INCLUDE,
+                           "-o", so, os.path.join(_native.CSRC, "fciqmc_rdm.cu")])
+    full, L = _native.load(), ctypes.CDLL(so)
+    for name in _native.SYMBOLS:
+        if name.startswith("fciqmc_rdm_"):
+            getattr(L, name).argtypes = getattr(full, name).argtypes
+            getattr(L, name).restype = getattr(full, name).restype
+    return L
+
+
+@pytest.mark.parametrize("bits,name", [
+    (5, "16e-600"),                  # every partition regrouped by the keys themselves
+    (5, "3e-one-orbital-common"),    # a key of 5,151 determinants that shares its hash with other keys
+    (5, "2e-whole-52-orbitals"),     # the same alone
+    (5, "3e-5o-whole"), (5, "33e-40o"),
+    (12, "64e-2100"),                # two scatter passes, partitions of several hashes taken in parts
+])
+def test_keys_that_share_their_hash(bits, name, short_hash_library, monkeypatch):
+    """Keys that agree in every hash bit are told apart: the library compiled with 2^5 or 2^12 different hashes, so that
+    in every partition many keys share one, against the oracle."""
+    library = short_hash_library(bits)
+    monkeypatch.setattr(_native, "load", lambda *a: library)
+    _matches_oracle(*_short_hash_case(name))
