@@ -177,7 +177,8 @@ enum { PRE_FP = 0, PRE_OKM, PRE_CB0, PRE_CB1, PRE_WORDS };
 // Class counts first (population counts against the class masks); then one pass over the occupied spin
 // orbitals in ascending order gives the occupied list, the electrons with an allowed single and the
 // fingerprint. The class masks and the orbital map come from global memory (two kilobytes, the masks the same for all
-// lanes), so that a kernel can derive while its other tables are on their way.
+// lanes), so that a kernel can derive while its other tables are on their way. A list being loaded is derived before
+// its check has ended, so d may have any bits: at most n_elec of them go to occ.
 template <int W>
 __device__ __forceinline__ void derive_det(const Params &P, const unsigned long long (&d)[W],
                                            unsigned long long (&pre)[PRE_WORDS], unsigned char *occ) {
@@ -202,10 +203,9 @@ __device__ __forceinline__ void derive_det(const Params &P, const unsigned long 
 #pragma unroll
     for (int w = 0; w < W; ++w) {
         unsigned long long m = d[w];
-        while (m) {
+        while (m && n < P.n_elec) {
             const int b = __ffsll((long long)m) - 1;
             const int k = 64 * w + b;
-            if (!FQ_CHECK(n < MAXN, P.st)) break;
             occ[n] = (unsigned char)k;
             okm |= ((ok[w] >> b) & 1ull) << n;
             h = 1099511628211ull * h + __ldg(P.map1 + k) * (unsigned long long)(n + 1);

@@ -184,6 +184,29 @@ def test_reloads_and_invalid_lists():
     g.close()
 
 
+@pytest.mark.parametrize("n_orb,n_elec", [(24, 12), (32, 6), (60, 24), (64, 4)])
+def test_lists_of_too_many_electrons(n_orb, n_elec):
+    """Determinants with more electrons than the run's, up to every spin orbital, in all slots or the last of a block:
+    rejected, and the run advances as the oracle does (the derived data of a list is made before its check has ended)."""
+    from paper_1305_6981_gb300._native import FciqmcError
+    s = synth.make_system(n_orb, n_elec, seed=n_orb, n_chol=8)
+    g, q = make_pair(s, 0.005, 3, initial_population=500, seed=2, main_capacity=1 << 12)
+    full = np.array(bf.to_words((1 << 2 * n_orb) - 1, g.W), dtype=np.uint64)
+    one_more = np.array(bf.to_words((1 << n_elec + 1) - 1, g.W), dtype=np.uint64)
+    dets, pops = synth.walker_snapshot(s, 1500, seed=1)
+    for bad in (full, one_more):
+        for at in (slice(None), slice(127, None, 128), slice(len(dets) - 1, None)):
+            d = dets.copy()
+            d[at] = bad
+            with pytest.raises(FciqmcError):
+                g.set_walkers(d, pops)
+    rows_q = q.iterate(10)
+    g.step(10)
+    compare_rows(g.history(10), rows_q)
+    assert same_lists(g.walkers(), q.walkers())
+    g.close()
+
+
 def test_reloads_and_invalid_lists_dense_index():
     """The same with lists long against the index (more than 1/16 of its entries), where loading empties the
     whole index instead of the old list's entries one by one: synthetic lists of 1.9e3 and 2.6e3
