@@ -43,16 +43,31 @@ constexpr int kGroupThreads = 512;
 constexpr int kGroupCap = 4608;
 constexpr int kGroupSlots = 8192;
 constexpr int kBigLeaders = 16;       // distinct keys of one hash value that the oversized path tells apart
-constexpr int kTriangle = 48;         // groups from this size on are walked as a triangle (see row_range)
+constexpr int kTriangle = 48;         // groups from this size on are large: walked as triangles, by warps of all blocks
+constexpr int kTaskPartners = 128;    // partners of a row beyond which more warps share it
+constexpr int kTaskShares = 16;       // most warps that do
 constexpr int kMergeThreads = 128;
 
 // A determinant in the group of a key: its signed amplitude, its pair code (bits 0..12 the index within the
-// class, 13..14 the class: 0 alpha alpha, 1 beta beta, 2 mixed; bits 15..20 the group size, 63 from kTriangle
+// class, 13..14 the class: 0 alpha alpha, 1 beta beta, 2 mixed; bits 15..20 the group size, kLarge from kTriangle
 // on), and the position of the group's first member in the partition.
+constexpr unsigned kLarge = 63;
 struct alignas(16) Member {
     double v;
     unsigned code;
     unsigned first;
+};
+
+// A large group: its first member (of all) and size.
+struct Head {
+    unsigned first, m;
+};
+
+// A warp's share of a large group of m members from `first` on: rows row0 + lane, each with the members before it, of
+// those the blocks of 64 numbered share, share + n_shares, ...
+struct alignas(16) Task {
+    unsigned first, m, row0;
+    unsigned short share, n_shares;
 };
 
 struct RdmState {
@@ -61,13 +76,16 @@ struct RdmState {
     unsigned long long n_pairs;    // candidate pairs
     unsigned long long n_shared;   // pairs of members that share one spin orbital (counted on request)
     unsigned long long n_apart;    // pairs that share none
+    unsigned long long n_tasks;
+    unsigned n_heads;
+    unsigned pad0;
     double norm;
     int status;
     int pad;
 };
 
 struct RdmLayout {
-    size_t dets, c, total_p, base_p, cursor_p, coarse_p, count_p, records, members, state, gh, ge, table, occ_part,
+    size_t dets, c, total_p, base_p, cursor_p, coarse_p, count_p, records, members, heads, state, gh, ge, table, occ_part,
         occ_pair, partial;
     size_t total;
 };
@@ -87,6 +105,7 @@ int log2i(long long x) {
 constexpr int kSms = 152;                     // blocks of the passes that take one block per SM
 constexpr int kPairGrid = kSms * 32;          // most blocks of the pair passes (several waves: partitions differ in cost)
 constexpr int kPairThreads = 128;
+constexpr int kLargeGrid = kSms * 16;         // most blocks of the pair passes for large groups
 constexpr int kNormGrid = kSms;
 
 struct Dims {
@@ -138,13 +157,14 @@ RdmLayout layout_of(const Dims &d) {
     L.count_p = take(sizeof(unsigned) * d.parts);
     L.records = take(sizeof(unsigned long long) * d.n_keys);
     L.members = take(sizeof(Member) * d.n_keys);
+    L.heads = take(sizeof(Head) * (d.n_keys / kTriangle + 1));
     L.state = take(sizeof(RdmState));
     L.gh = take(sizeof(double) * d.n_orb * d.n_orb);
     L.ge = take(sizeof(double) * d.n_eri);
     L.table = take(sizeof(double) * ((size_t)d.n1 * d.n1 + (size_t)d.n2 * d.n2));
     L.occ_part = take(sizeof(double) * kSms * ((size_t)d.n_so * (d.n_so + 1) / 2));
     L.occ_pair = take(sizeof(double) * ((size_t)d.n_so * (d.n_so + 1) / 2));
-    L.partial = take(sizeof(double) * 2 * (kPairGrid + kNormGrid));
+    L.partial = take(sizeof(double) * 2 * (kPairGrid + kLargeGrid + kNormGrid));
     L.total = off;
     return L;
 }
@@ -481,7 +501,7 @@ struct GroupShared {
     unsigned n, min_t, kept;
 };
 
-// Records s.rec[0, s.n) grouped by key; groups of two and more go to out + s.kept, longer groups first (four size
+// Records s.rec[0, s.n) grouped by key; groups of two and more go to members + base + s.kept, longer groups first (four size
 // classes), members in the order of their codes, so that the lanes of the pair passes have rows of similar length
 // and neighbouring table columns. Grouping goes by the hash bits; every member's key is then compared with its
 // group's first, and where two keys share the hash, false is returned to the whole block and nothing is written:
@@ -490,7 +510,9 @@ struct GroupShared {
 // partition), 120 of 32,768.
 template <int W>
 __device__ __forceinline__ bool group_shared(GroupShared<W> &s, const unsigned long long *dets, const double *c, int npairs,
-                                             int n_orb, int tbits, Member *out, bool exact) {
+                                             int n_orb, int tbits, Member *members, unsigned base, Head *heads, RdmState *st,
+                                             bool exact) {
+    Member *out = members + base;
     constexpr unsigned kFree = 0xFFFFFFFFu;
     const unsigned n = s.n;
     for (int h = threadIdx.x; h < kGroupSlots; h += kGroupThreads) s.table[h] = kFree;
@@ -603,9 +625,10 @@ __device__ __forceinline__ bool group_shared(GroupShared<W> &s, const unsigned l
         const double v = __ldg(c + rec_t(s.rec[i], tbits) / (unsigned)npairs);
         Member o;
         o.v = code == kNoPair ? 0.0 : (ci & 0x8000u) ? -v : v;
-        o.code = (code == kNoPair ? 0u : code) | ((m >= kTriangle ? 63u : m) << 15);
+        o.code = (code == kNoPair ? 0u : code) | ((m >= kTriangle ? kLarge : m) << 15);
         o.first = kept + first;
         out[kept + first + rank] = o;
+        if (at == first && m >= kTriangle) heads[atomicAdd(&st->n_heads, 1u)] = Head{base + kept + first, m};
     }
     for (int o = 16; o > 0; o >>= 1) {
         buckets += __shfl_down_sync(0xFFFFFFFFu, buckets, o);
@@ -629,7 +652,9 @@ __device__ __forceinline__ bool group_shared(GroupShared<W> &s, const unsigned l
 // over the partition; its members are written in the order the threads meet them.
 template <int W>
 __device__ void group_big(GroupShared<W> &s, const unsigned long long *rec, unsigned size, unsigned long long hash,
-                          const unsigned long long *dets, const double *c, int npairs, int n_orb, int tbits, Member *out, RdmState *st) {
+                          const unsigned long long *dets, const double *c, int npairs, int n_orb, int tbits, Member *members, unsigned base,
+                          Head *heads, RdmState *st) {
+    Member *out = members + base;
     for (int nl = 0;; ++nl) {
         if (threadIdx.x == 0) {
             s.min_t = 0xFFFFFFFFu;
@@ -673,6 +698,7 @@ __device__ void group_big(GroupShared<W> &s, const unsigned long long *rec, unsi
                 s.acc[1] += m;
                 s.acc[2] += (unsigned long long)m * (m - 1) / 2;
                 s.kept = kept + m;
+                if (m >= kTriangle) heads[atomicAdd(&st->n_heads, 1u)] = Head{base + kept, m};
             }
         }
         __syncthreads();
@@ -686,7 +712,7 @@ __device__ void group_big(GroupShared<W> &s, const unsigned long long *rec, unsi
             Member o;
             const unsigned code = pair_code(q.ox, q.oy, n_orb);
             o.v = code == kNoPair ? 0.0 : signed_c(c, q.I, s.pairs[q.k], q.ox, q.oy);
-            o.code = (code == kNoPair ? 0u : code) | ((m >= kTriangle ? 63u : m) << 15);
+            o.code = (code == kNoPair ? 0u : code) | ((m >= kTriangle ? kLarge : m) << 15);
             o.first = kept;
             out[kept + atomicAdd(&s.n, 1u)] = o;
         }
@@ -699,7 +725,7 @@ __device__ void group_big(GroupShared<W> &s, const unsigned long long *rec, unsi
 template <int W>
 __global__ void __launch_bounds__(kGroupThreads, 2) k_group(const unsigned long long *dets, const double *c, int n_elec, int n_orb,
                                                             int tbits, const unsigned long long *records, const unsigned *base_p,
-                                                            Member *members, unsigned *count_p, RdmState *st) {
+                                                            Member *members, unsigned *count_p, Head *heads, RdmState *st) {
     extern __shared__ __align__(16) unsigned char s_raw[];
     GroupShared<W> &s = *reinterpret_cast<GroupShared<W> *>(s_raw);
     const int npairs = n_elec * (n_elec - 1) / 2;
@@ -708,12 +734,11 @@ __global__ void __launch_bounds__(kGroupThreads, 2) k_group(const unsigned long 
     if (threadIdx.x == 0) s.kept = 0;
     const unsigned base = base_p[blockIdx.x], size = base_p[blockIdx.x + 1] - base;
     const unsigned long long *rec = records + base;
-    Member *out = members + base;
     if (size <= (unsigned)kGroupCap) {
         for (unsigned i = threadIdx.x; i < size; i += kGroupThreads) s.rec[i] = rec[i];
         if (threadIdx.x == 0) s.n = size;
         __syncthreads();
-        if (size && !group_shared<W>(s, dets, c, npairs, n_orb, tbits, out, false)) group_shared<W>(s, dets, c, npairs, n_orb, tbits, out, true);
+        if (size && !group_shared<W>(s, dets, c, npairs, n_orb, tbits, members, base, heads, st, false)) group_shared<W>(s, dets, c, npairs, n_orb, tbits, members, base, heads, st, true);
     } else {
         // sub-partitions by the leading `depth` bits of the hash, deeper where one is still too long
         int d0 = 1;
@@ -745,8 +770,8 @@ __global__ void __launch_bounds__(kGroupThreads, 2) k_group(const unsigned long 
             }
             const unsigned long long hash = s.lo;
             __syncthreads();
-            if (m > (unsigned)kGroupCap) group_big<W>(s, rec, size, hash, dets, c, npairs, n_orb, tbits, out, st);
-            else if (m && !group_shared<W>(s, dets, c, npairs, n_orb, tbits, out, false)) group_shared<W>(s, dets, c, npairs, n_orb, tbits, out, true);
+            if (m > (unsigned)kGroupCap) group_big<W>(s, rec, size, hash, dets, c, npairs, n_orb, tbits, members, base, heads, st);
+            else if (m && !group_shared<W>(s, dets, c, npairs, n_orb, tbits, members, base, heads, st, false)) group_shared<W>(s, dets, c, npairs, n_orb, tbits, members, base, heads, st, true);
             __syncthreads();
             ++sub;
             while (depth > d0 && !(sub & 1ull)) {
@@ -761,6 +786,29 @@ __global__ void __launch_bounds__(kGroupThreads, 2) k_group(const unsigned long 
         if (s.acc[0]) atomicAdd(&st->n_buckets, s.acc[0]);
         if (s.acc[1]) atomicAdd(&st->n_members, s.acc[1]);
         if (s.acc[2]) atomicAdd(&st->n_pairs, s.acc[2]);
+    }
+}
+
+// The tasks of the large groups, a warp per group. They lie where the records were: at most m / 2 of 16 bytes for a
+// group of m (one for 32 rows up to kTaskPartners, kTaskShares at most), and a record is 8 bytes.
+__device__ __forceinline__ void make_tasks(const Head *heads, Task *tasks, RdmState *st, unsigned g, unsigned warps) {
+    const int lane = threadIdx.x & 31;
+    const unsigned n = st->n_heads;
+    for (; g < n; g += warps) {
+        const Head q = heads[g];
+        for (unsigned t0 = 0; t0 * 32u < q.m; t0 += 32) {  // a tile of 32 rows per lane
+            const unsigned row0 = 32u * (t0 + (unsigned)lane);
+            const unsigned mine = row0 < q.m ? min((row0 + 32u + kTaskPartners - 1) / kTaskPartners, (unsigned)kTaskShares) : 0u;
+            unsigned x = mine;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+                if (lane >= o) x += y;
+            }
+            unsigned long long at = 0;
+            if (lane == 31) at = atomicAdd(&st->n_tasks, (unsigned long long)x);
+            at = __shfl_sync(0xFFFFFFFFu, at, 31) + (x - mine);
+            for (unsigned k = 0; k < mine; ++k) tasks[at + k] = Task{q.first, q.m, row0, (unsigned short)k, (unsigned short)mine};
+        }
     }
 }
 
@@ -880,10 +928,17 @@ __global__ void __launch_bounds__(256) k_occ_pairs(const unsigned long long *det
 }
 
 // Sums of the blocks' occupation pairs (compensated): a warp adds 8 entries, four lanes each taking every fourth block in
-// order, merged in a fixed tree. The last block adds the partial sums of c^2.
-__global__ void __launch_bounds__(kMergeThreads) k_occ_merge(const double *occ_part, int nblocks, int nent, double *occ_pair,
-                                                             const double *norm_part, int n_norm, RdmState *st) {
-    if (blockIdx.x == gridDim.x - 1) {
+// order, merged in a fixed tree (the first n_merge blocks). The next block adds the partial sums of c^2, the others make
+// the tasks of the large groups, which need k_group's heads only and here cost no launch and no time.
+__global__ void __launch_bounds__(kMergeThreads) k_occ_merge(const double *occ_part, int nblocks, int nent, double *occ_pair, int n_merge,
+                                                             const double *norm_part, int n_norm, const Head *heads, Task *tasks,
+                                                             RdmState *st) {
+    if ((int)blockIdx.x > n_merge) {
+        constexpr unsigned kWarps = kMergeThreads / 32;
+        make_tasks(heads, tasks, st, (blockIdx.x - n_merge - 1) * kWarps + (threadIdx.x >> 5), (gridDim.x - n_merge - 1) * kWarps);
+        return;
+    }
+    if ((int)blockIdx.x == n_merge) {
         __shared__ CSum s[kMergeThreads / 32];
         CSum a{0.0, 0.0};
         for (int b = threadIdx.x; b < n_norm; b += kMergeThreads) csum_merge(a, CSum{norm_part[2 * b], norm_part[2 * b + 1]});
@@ -960,30 +1015,72 @@ __global__ void __launch_bounds__(kThreads) k_pair_table(const double *h, const 
 
 // The partners of member j of a group of m starting at `first`, so that every pair is met once: small groups
 // cyclically (each member takes about half of the others, so the lanes of a warp, in groups of similar size,
-// finish together), large ones (m >= kTriangle) as a triangle, in which the lanes of a warp meet the same partner
-// at the same time and read neighbouring columns of its table row.
+// finish together). Large ones (m >= kTriangle) are not a partition's business: their rows are triangles, in which
+// the lanes of a warp meet the same partner at the same time and read neighbouring columns of its table row, and
+// they are dealt out to the warps of all blocks (Task). A list of few keys is a few large groups (two electrons: one), and
+// in a vector around a reference they hold most pairs; as rows of the block that has the partition, the 3.3e7 pairs of
+// 8,128 determinants of two electrons took E 68.6 ms and its gradient 24.1 (0.41 and 0.25 as tasks), those of 1e6
+// determinants of 16e/40o 1.86 and 1.59 (1.33 and 1.40; shares of 512 partners instead of 128, in launches of their own:
+// 1.47 and 1.62, and 12 us more for 3e3 determinants, whose longest share was the launch).
 struct RowRange {
     int n;        // partners
     int at;       // first partner, counted from the group's start
-    int wrap;     // group size for the cyclic walk (never reached by the triangle)
+    int wrap;     // group size
 };
 __device__ __forceinline__ RowRange row_range(unsigned packed, int local) {
     const int m = (int)(packed >> 15);
-    if (m == 63) return RowRange{local, 0, 0x7FFFFFFF};
+    if (m == (int)kLarge) return RowRange{0, 0, 0};
     const int half = (m - 1) >> 1, even = (m & 1) == 0 && local < (m >> 1) ? 1 : 0;
     return RowRange{half + even, local + 1 < m ? local + 1 : 0, m};
 }
 
-// 2 c_I c_J H_IJ summed over the pairs of members, without the factor 2: per thread the rows of its members, plain
-// within one partition (a handful of rows), compensated across partitions, the blocks' sums in a fixed tree. A
-// row is an FMA chain of at most half a small group, or of eight partners of a large one at a time.
+// The tasks of warp g of `warps`, a lane per row: f(its member, the group, k0, k1) for the task's blocks of 64 members
+// before it.
+template <typename F>
+__device__ __forceinline__ void for_task_rows(const Member *members, const Task *tasks, unsigned long long n_tasks, unsigned g,
+                                              unsigned warps, F f) {
+    for (unsigned long long i = g; i < n_tasks; i += warps) {
+        const Task t = tasks[i];
+        const Member *grp = members + t.first;
+        const unsigned row = t.row0 + (threadIdx.x & 31u);
+        if (row >= t.m) continue;
+        const Member u = grp[row];
+        for (unsigned k0 = 64u * t.share; k0 < row; k0 += 64u * t.n_shares) f(u, grp, k0, min(k0 + 64u, row));
+    }
+}
+
+// 2 c_I c_J H_IJ summed over the pairs of members, without the factor 2. The first `large` blocks take the tasks of the
+// large groups, a warp each, the others the partitions' small groups; per thread plain sums of a task's or a partition's
+// rows, compensated across those, the blocks' sums in a fixed tree. A row is an FMA chain of eight partners at a time.
 // Bound by the FP64 pipe (one FMA per pair, charged per warp instruction) and the table reads from L2.
 __global__ void __launch_bounds__(kPairThreads) k_pair_energy(const Member *members, const unsigned *base_p, const unsigned *count_p,
-                                                          int parts, int n1, int n2, const double *table, double *partial) {
+                                                          int parts, const Task *tasks, unsigned long long n_tasks, int large,
+                                                          int n1, int n2, const double *table, double *partial) {
     __shared__ CSum s_red[kPairThreads / 32];
     CSum acc{0.0, 0.0};
     const double *mixed = table + (size_t)n1 * n1;
-    for (int p = blockIdx.x; p < parts; p += gridDim.x) {
+    if ((int)blockIdx.x < large) {
+        constexpr unsigned kWarps = kPairThreads / 32;
+        for_task_rows(members, tasks, n_tasks, blockIdx.x * kWarps + (threadIdx.x >> 5), (unsigned)large * kWarps,
+                      [&](const Member &u, const Member *grp, unsigned k0, unsigned k1) {
+            const unsigned cls = (u.code >> 13) & 3u;
+            const double *col = (cls == 2u ? mixed : table) + (u.code & 0x1FFFu);
+            const int stride = cls == 2u ? n2 : n1;
+            double row = 0.0;
+            for (; k0 < k1; k0 += 8) {
+                double part = 0.0;
+                const unsigned end = min(k0 + 8u, k1);
+#pragma unroll 4
+                for (unsigned k = k0; k < end; ++k) {
+                    const Member w = grp[k];
+                    if (((w.code >> 13) & 3u) == cls) part = __fma_rn(__ldg(col + (size_t)(w.code & 0x1FFFu) * stride), w.v, part);
+                }
+                row = __dadd_rn(row, part);
+            }
+            csum_add(acc, __dmul_rn(u.v, row));
+        });
+    }
+    for (int p = (int)blockIdx.x - large; p >= 0 && p < parts; p += (int)gridDim.x - large) {
         const Member *mem = members + base_p[p];
         const int cnt = (int)count_p[p];
         if ((int)threadIdx.x >= cnt) continue;
@@ -1048,28 +1145,38 @@ __global__ void __launch_bounds__(1024) k_energy_finish(const double *pp, int np
 }
 
 // The two-body density matrix over pair codes: v v' of every pair of members added at (smaller code, larger code) with
-// one FP64 reduction in L2. Large groups walk a triangle, so a warp's reductions fall in one table row.
+// one FP64 reduction in L2. Blocks as in k_pair_energy; in large groups a warp's reductions fall in one table row.
 __global__ void __launch_bounds__(kPairThreads) k_pair_grad(const Member *members, const unsigned *base_p, const unsigned *count_p,
-                                                        int parts, int n1, int n2, double *table) {
+                                                        int parts, const Task *tasks, unsigned long long n_tasks, int large,
+                                                        int n1, int n2, double *table) {
     double *mixed = table + (size_t)n1 * n1;
-    for (int p = blockIdx.x; p < parts; p += gridDim.x) {
+    auto add = [&](const Member &u, const Member &w) {
+        const unsigned cls = (u.code >> 13) & 3u, cu = u.code & 0x1FFFu, cw = w.code & 0x1FFFu;
+        if (((w.code >> 13) & 3u) == cls)
+            atomicAdd((cls == 2u ? mixed : table) + (size_t)min(cu, cw) * (cls == 2u ? n2 : n1) + max(cu, cw), __dmul_rn(u.v, w.v));
+    };
+    if ((int)blockIdx.x < large) {
+        constexpr unsigned kWarps = kPairThreads / 32;
+        for_task_rows(members, tasks, n_tasks, blockIdx.x * kWarps + (threadIdx.x >> 5), (unsigned)large * kWarps,
+                      [&](const Member &u, const Member *grp, unsigned k0, unsigned k1) {
+#pragma unroll 4
+            for (unsigned k = k0; k < k1; ++k) add(u, grp[k]);
+        });
+        return;
+    }
+    for (int p = (int)blockIdx.x - large; p < parts; p += (int)gridDim.x - large) {
         const Member *mem = members + base_p[p];
         const int cnt = (int)count_p[p];
         for (int j = threadIdx.x; j < cnt; j += kPairThreads) {
             const Member u = mem[j];
             const Member *grp = mem + u.first;
             const RowRange r = row_range(u.code, j - (int)u.first);
-            const unsigned cls = (u.code >> 13) & 3u, cu = u.code & 0x1FFFu;
-            double *t = cls == 2u ? mixed : table;
-            const int stride = cls == 2u ? n2 : n1;
             int at = r.at;
 #pragma unroll 4
             for (int k = 0; k < r.n; ++k) {
                 const Member w = grp[at];
                 at = at + 1 == r.wrap ? 0 : at + 1;
-                const unsigned cw = w.code & 0x1FFFu;
-                if (((w.code >> 13) & 3u) == cls)
-                    atomicAdd(t + (size_t)min(cu, cw) * stride + max(cu, cw), __dmul_rn(u.v, w.v));
+                add(u, w);
             }
         }
     }
@@ -1234,14 +1341,16 @@ int construct(fciqmc_rdm *r) {
         k_refine<<<dim3((unsigned)std::min<long long>(tiles + 1, 1024), 1u << cbits), kHashThreads, 0, s>>>(first, d.tbits, base, cursor, records);
     }
     k_group<W><<<d.parts, kGroupThreads, sm_group, s>>>(dets, c, d.n_elec, d.n_orb, d.tbits, records, base, ptr<Member>(r, r->L.members),
-                                                        ptr<unsigned>(r, r->L.count_p), st);
-    double *norm_part = ptr<double>(r, r->L.partial) + 2 * kPairGrid;
+                                                        ptr<unsigned>(r, r->L.count_p), ptr<Head>(r, r->L.heads), st);
+    double *norm_part = ptr<double>(r, r->L.partial) + 2 * (kPairGrid + kLargeGrid);
     const int nw = occ_warps(d);
     const int go = (int)std::min<long long>(kSms, (d.n + nw - 1) / nw), gn = (int)std::min<long long>(kNormGrid, (d.n + kThreads - 1) / kThreads);
     k_norm<<<gn, kThreads, 0, s>>>(c, d.n, norm_part);
     k_occ_pairs<W><<<go, 32 * nw, sm_occ, s>>>(dets, c, d.n, d.n_elec, d.n_so, ptr<double>(r, r->L.occ_part));
-    k_occ_merge<<<(unsigned)((nent + kMergeThreads / 4 - 1) / (kMergeThreads / 4)) + 1, kMergeThreads, 0, s>>>(
-        ptr<double>(r, r->L.occ_part), go, (int)nent, ptr<double>(r, r->L.occ_pair), norm_part, gn, st);
+    const int n_merge = (int)((nent + kMergeThreads / 4 - 1) / (kMergeThreads / 4));
+    k_occ_merge<<<n_merge + 1 + kSms, kMergeThreads, 0, s>>>(ptr<double>(r, r->L.occ_part), go, (int)nent, ptr<double>(r, r->L.occ_pair),
+                                                             n_merge, norm_part, gn, ptr<Head>(r, r->L.heads),
+                                                             ptr<Task>(r, r->L.records), st);
     if (cudaGetLastError() != cudaSuccess) return FCIQMC_ERR_CUDA;
     if (cudaMemcpyAsync(&r->host, st, sizeof(RdmState), cudaMemcpyDeviceToHost, s) != cudaSuccess) return FCIQMC_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return FCIQMC_ERR_CUDA;
@@ -1252,17 +1361,22 @@ dim3 table_grid(const Dims &d, int extra_rows) {
     return dim3((unsigned)std::max(1, (std::max(d.n1, d.n2) + 4 * kThreads - 1) / (4 * kThreads)), (unsigned)(d.n1 + d.n2 + extra_rows));
 }
 int pair_grid(const Dims &d) { return std::min(kPairGrid, d.parts); }
+int large_grid(const fciqmc_rdm *r) {
+    constexpr unsigned long long kWarps = kPairThreads / 32;
+    return (int)std::min<unsigned long long>(kLargeGrid, (r->host.n_tasks + kWarps - 1) / kWarps);
+}
 
 void launch_energy(fciqmc_rdm *r, const double *h, const double *eri, double *e) {
     const Dims &d = r->d;
     cudaStream_t s = r->s;
     const RdmState *st = ptr<RdmState>(r, r->L.state);
     double *partial = ptr<double>(r, r->L.partial), *table = ptr<double>(r, r->L.table);
-    const int g = pair_grid(d);
+    const int g = pair_grid(d), gl = large_grid(r);
     k_pair_table<<<table_grid(d, 0), kThreads, 0, s>>>(h, eri, d.n_orb, d.n1, d.n2, 1.0 / (d.n_elec - 1), table);
-    k_pair_energy<<<g, kPairThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p), ptr<unsigned>(r, r->L.count_p),
-                                         d.parts, d.n1, d.n2, table, partial);
-    k_energy_finish<<<1, 1024, 0, s>>>(partial, g, ptr<double>(r, r->L.occ_pair), h, eri, d.n_orb, st, e);
+    k_pair_energy<<<g + gl, kPairThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p),
+                                              ptr<unsigned>(r, r->L.count_p), d.parts, ptr<Task>(r, r->L.records), r->host.n_tasks, gl,
+                                              d.n1, d.n2, table, partial);
+    k_energy_finish<<<1, 1024, 0, s>>>(partial, g + gl, ptr<double>(r, r->L.occ_pair), h, eri, d.n_orb, st, e);
 }
 
 void launch_rdm(fciqmc_rdm *r) {
@@ -1272,8 +1386,10 @@ void launch_rdm(fciqmc_rdm *r) {
     cudaMemsetAsync(gh, 0, sizeof(double) * d.n_orb * d.n_orb, s);
     cudaMemsetAsync(ge, 0, sizeof(double) * d.n_eri, s);
     cudaMemsetAsync(table, 0, sizeof(double) * ((size_t)d.n1 * d.n1 + (size_t)d.n2 * d.n2), s);
-    k_pair_grad<<<pair_grid(d), kPairThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p),
-                                                  ptr<unsigned>(r, r->L.count_p), d.parts, d.n1, d.n2, table);
+    const int gl = large_grid(r);
+    k_pair_grad<<<pair_grid(d) + gl, kPairThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p),
+                                                       ptr<unsigned>(r, r->L.count_p), d.parts, ptr<Task>(r, r->L.records),
+                                                       r->host.n_tasks, gl, d.n1, d.n2, table);
     k_fold<<<table_grid(d, d.n_so), kThreads, 0, s>>>(table, ptr<double>(r, r->L.occ_pair), d.n_orb, d.n1, d.n2,
                                                       1.0 / (d.n_elec - 1), gh, ge);
 }

@@ -278,3 +278,41 @@ def test_keys_that_share_their_hash(bits, name, short_hash_library, monkeypatch)
     library = short_hash_library(bits)
     monkeypatch.setattr(_native, "load", lambda *a: library)
     _matches_oracle(*_short_hash_case(name))
+
+
+@pytest.mark.parametrize("n", [48, 64, 65, 128, 129, 161, 2049, 2081])
+def test_large_groups_in_shares(n):
+    """One key of n determinants: the rows of a large group are dealt to warps 32 at a time, in shares from 128 partners on
+    and at most 16 of them. The counts as well, up to 161."""
+    s = synth.make_system(33, 2, seed=n, n_chol=8, fock_diagonal=False)
+    dets = np.array([bf.to_words(d, 2) for d in _some_pairs(33, 2, n, n)], dtype=np.uint64)
+    c = np.random.default_rng(n).normal(size=n)
+    c /= np.linalg.norm(c)
+    _, gh, ge = Oracle(s, tau=0.01).rdm_energy(dets, c)
+    _matches_oracle(33, 2, dets, c, (s.h, s.eri_s8, gh, ge))
+
+
+def test_one_key_is_spread_over_the_device():
+    """E of the 5,356 determinants of two electrons in 52 orbitals, 1.4e7 pairs of one key, takes no longer than a few times
+    that of a list of 4.7e7 pairs over many keys (it took 55 times as long when a key belonged to one block)."""
+    from itertools import combinations
+
+    def time_of(n_orb, n_elec):
+        s = synth.make_system(n_orb, n_elec, seed=1, n_chol=8, fock_diagonal=False)
+        dets = np.array([bf.to_words(sum(1 << k for k in occ), (2 * n_orb + 63) // 64) for occ in combinations(range(2 * n_orb), n_elec)],
+                        dtype=np.uint64)
+        f = _functional(s, dets, np.random.default_rng(1).normal(size=len(dets)))
+        h, eri = _dev(s.h), _dev(s.eri_s8)
+        f.energy(h, eri)
+        best = np.inf
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            f.energy(h, eri)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        f.close()
+        return best
+
+    assert time_of(52, 2) < 5 * time_of(16, 4)
