@@ -85,8 +85,8 @@ struct RdmState {
 };
 
 struct RdmLayout {
-    size_t dets, c, total_p, base_p, cursor_p, coarse_p, count_p, records, members, heads, state, gh, ge, table, occ_part,
-        occ_pair, partial;
+    size_t dets, c, total_p, base_p, cursor_p, coarse_p, count_p, records, members, heads, state, gh, ge, share, table,
+        occ_part, occ_pair, partial;
     size_t total;
 };
 
@@ -161,6 +161,7 @@ RdmLayout layout_of(const Dims &d) {
     L.state = take(sizeof(RdmState));
     L.gh = take(sizeof(double) * d.n_orb * d.n_orb);
     L.ge = take(sizeof(double) * d.n_eri);
+    L.share = take(sizeof(double) * d.n_orb * d.n_orb);
     L.table = take(sizeof(double) * ((size_t)d.n1 * d.n1 + (size_t)d.n2 * d.n2));
     L.occ_part = take(sizeof(double) * kSms * ((size_t)d.n_so * (d.n_so + 1) / 2));
     L.occ_pair = take(sizeof(double) * ((size_t)d.n_so * (d.n_so + 1) / 2));
@@ -815,7 +816,8 @@ __device__ __forceinline__ void make_tasks(const Head *heads, Task *tasks, RdmSt
 // ------------------------------------------------------------------------------------ compensated sums
 // Sum and running error of a sequence of FP64 additions (Knuth's TwoSum per addition, Neumaier's
 // compensated summation): the result is the rounded exact sum up to a few ulp whatever the number of
-// terms, so finite differences of E are not swamped by accumulated rounding.
+// additions, so finite differences of E are not swamped by accumulated rounding. A compensated addition costs
+// seven plain ones, so terms are added plainly first, a bounded number at a time (k_pair_energy).
 struct CSum {
     double s, c;
 };
@@ -977,9 +979,15 @@ __global__ void __launch_bounds__(kThreads) k_norm(const double *c, long long n,
 }
 
 // ------------------------------------------------------------------------------------ pairs
+// h / (N - 1), the share of one key in a one-electron element (divided for each entry that needs it, k_pair_table and k_fold
+// took far longer; a product with the rounded inverse has two roundings, the same ones at all N - 1 keys).
+__global__ void __launch_bounds__(kThreads) k_share(const double *h, int n, double keys, double *share) {
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) share[k] = __ddiv_rn(h[k], keys);
+}
+
 // T over pair codes: the same-spin block (n1 x n1, rows and columns p < q), then the mixed block (n2 x n2, alpha
 // first); the diagonals stay zero (the diagonal of H comes from the occupation-pair sums).
-__global__ void __launch_bounds__(kThreads) k_pair_table(const double *h, const double *eri, int n_orb, int n1, int n2, double inv,
+__global__ void __launch_bounds__(kThreads) k_pair_table(const double *share, const double *eri, int n_orb, int n1, int n2,
                                                          double *table) {
     const int row = blockIdx.y;
     if (row < n1) {
@@ -991,10 +999,10 @@ __global__ void __launch_bounds__(kThreads) k_pair_table(const double *h, const 
             double v = 0.0;
             if (col != row) {
                 v = __dsub_rn(__ldg(eri + fq::eidx(p, r, q, s)), __ldg(eri + fq::eidx(p, s, q, r)));
-                if (q == s) v = __dadd_rn(v, __dmul_rn(inv, __ldg(h + p * n_orb + r)));
-                if (p == r) v = __dadd_rn(v, __dmul_rn(inv, __ldg(h + q * n_orb + s)));
-                if (q == r) v = __dsub_rn(v, __dmul_rn(inv, __ldg(h + p * n_orb + s)));
-                if (p == s) v = __dsub_rn(v, __dmul_rn(inv, __ldg(h + q * n_orb + r)));
+                if (q == s) v = __dadd_rn(v, __ldg(share + p * n_orb + r));
+                if (p == r) v = __dadd_rn(v, __ldg(share + q * n_orb + s));
+                if (q == r) v = __dsub_rn(v, __ldg(share + p * n_orb + s));
+                if (p == s) v = __dsub_rn(v, __ldg(share + q * n_orb + r));
             }
             table[(size_t)row * n1 + col] = v;
         }
@@ -1005,8 +1013,8 @@ __global__ void __launch_bounds__(kThreads) k_pair_table(const double *h, const 
             double v = 0.0;
             if (col != row2) {
                 v = __ldg(eri + fq::eidx(p, r, q, s));
-                if (q == s) v = __dadd_rn(v, __dmul_rn(inv, __ldg(h + p * n_orb + r)));
-                if (p == r) v = __dadd_rn(v, __dmul_rn(inv, __ldg(h + q * n_orb + s)));
+                if (q == s) v = __dadd_rn(v, __ldg(share + p * n_orb + r));
+                if (p == r) v = __dadd_rn(v, __ldg(share + q * n_orb + s));
             }
             table[(size_t)n1 * n1 + (size_t)row2 * n2 + col] = v;
         }
@@ -1050,9 +1058,13 @@ __device__ __forceinline__ void for_task_rows(const Member *members, const Task 
 }
 
 // 2 c_I c_J H_IJ summed over the pairs of members, without the factor 2. The first `large` blocks take the tasks of the
-// large groups, a warp each, the others the partitions' small groups; per thread plain sums of a task's or a partition's
-// rows, compensated across those, the blocks' sums in a fixed tree. A row is an FMA chain of eight partners at a time.
+// large groups, a warp each, the others the partitions' small groups. A row is an FMA chain of eight partners at a time;
+// per thread these parts are added plainly, at most eight of a large group's row or the three of kPlainRows rows of small
+// ones, and then compensated, the blocks' sums in a fixed tree. So a pair is followed by at most 8 + 3 + kPlainRows plain
+// additions whatever the length of the list (with one plain sum per row, thread and partition, 8.4e6 equal pairs of one
+// key came out 48 times 2^-53 off).
 // Bound by the FP64 pipe (one FMA per pair, charged per warp instruction) and the table reads from L2.
+constexpr int kPlainRows = 16;
 __global__ void __launch_bounds__(kPairThreads) k_pair_energy(const Member *members, const unsigned *base_p, const unsigned *count_p,
                                                           int parts, const Task *tasks, unsigned long long n_tasks, int large,
                                                           int n1, int n2, const double *table, double *partial) {
@@ -1084,30 +1096,33 @@ __global__ void __launch_bounds__(kPairThreads) k_pair_energy(const Member *memb
         const Member *mem = members + base_p[p];
         const int cnt = (int)count_p[p];
         if ((int)threadIdx.x >= cnt) continue;
-        double sum = 0.0;
-        for (int j = threadIdx.x; j < cnt; j += kPairThreads) {
-            const Member u = mem[j];
-            const Member *grp = mem + u.first;
-            const RowRange r = row_range(u.code, j - (int)u.first);
-            const unsigned cls = (u.code >> 13) & 3u, cu = u.code & 0x1FFFu;
-            const double *col = (cls == 2u ? mixed : table) + cu;
-            const int stride = cls == 2u ? n2 : n1;
-            double row = 0.0;
-            int at = r.at;
-            for (int k0 = 0; k0 < r.n; k0 += 8) {
-                double part = 0.0;
-                const int k1 = min(k0 + 8, r.n);
+        for (int j0 = threadIdx.x; j0 < cnt; j0 += kPlainRows * kPairThreads) {
+            const int j1 = min(j0 + kPlainRows * kPairThreads, cnt);
+            double sum = 0.0;
+            for (int j = j0; j < j1; j += kPairThreads) {
+                const Member u = mem[j];
+                const Member *grp = mem + u.first;
+                const RowRange r = row_range(u.code, j - (int)u.first);
+                const unsigned cls = (u.code >> 13) & 3u, cu = u.code & 0x1FFFu;
+                const double *col = (cls == 2u ? mixed : table) + cu;
+                const int stride = cls == 2u ? n2 : n1;
+                double row = 0.0;
+                int at = r.at;
+                for (int k0 = 0; k0 < r.n; k0 += 8) {
+                    double part = 0.0;
+                    const int k1 = min(k0 + 8, r.n);
 #pragma unroll 4
-                for (int k = k0; k < k1; ++k) {
-                    const Member w = grp[at];
-                    at = at + 1 == r.wrap ? 0 : at + 1;
-                    if (((w.code >> 13) & 3u) == cls) part = __fma_rn(__ldg(col + (size_t)(w.code & 0x1FFFu) * stride), w.v, part);
+                    for (int k = k0; k < k1; ++k) {
+                        const Member w = grp[at];
+                        at = at + 1 == r.wrap ? 0 : at + 1;
+                        if (((w.code >> 13) & 3u) == cls) part = __fma_rn(__ldg(col + (size_t)(w.code & 0x1FFFu) * stride), w.v, part);
+                    }
+                    row = __dadd_rn(row, part);
                 }
-                row = __dadd_rn(row, part);
+                sum = __fma_rn(u.v, row, sum);
             }
-            sum = __fma_rn(u.v, row, sum);
+            csum_add(acc, sum);
         }
-        csum_add(acc, sum);
     }
     acc = block_csum(acc, s_red);
     if (threadIdx.x == 0) {
@@ -1182,8 +1197,9 @@ __global__ void __launch_bounds__(kPairThreads) k_pair_grad(const Member *member
     }
 }
 
-// Maps the density matrix over pair codes (rows < columns) and the occupation-pair sums onto h and the packed ERIs.
-__global__ void __launch_bounds__(kThreads) k_fold(const double *table, const double *occ_pair, int n_orb, int n1, int n2, double inv,
+// Maps the density matrix over pair codes (rows < columns) and the occupation-pair sums onto h and the packed ERIs. A
+// one-electron element comes once per shared key: gh holds N - 1 times its value off the diagonal (k_scale_out divides).
+__global__ void __launch_bounds__(kThreads) k_fold(const double *table, const double *occ_pair, int n_orb, int n1, int n2,
                                                    double *gh, double *ge) {
     auto one_body = [&](int a, int b, double v) {  // both h[a][b] and h[b][a]
         atomicAdd(&gh[a * n_orb + b], v);
@@ -1198,13 +1214,12 @@ __global__ void __launch_bounds__(kThreads) k_fold(const double *table, const do
             if (g == 0.0) continue;
             int r, s;
             triangle_of(col, r, s);
-            const double g1 = __dmul_rn(inv, g);
             atomicAdd(&ge[fq::eidx(p, r, q, s)], 2.0 * g);
             atomicAdd(&ge[fq::eidx(p, s, q, r)], -2.0 * g);
-            if (q == s) one_body(p, r, g1);
-            if (p == r) one_body(q, s, g1);
-            if (q == r) one_body(p, s, -g1);
-            if (p == s) one_body(q, r, -g1);
+            if (q == s) one_body(p, r, g);
+            if (p == r) one_body(q, s, g);
+            if (q == r) one_body(p, s, -g);
+            if (p == s) one_body(q, r, -g);
         }
     } else if (row < n1 + n2) {
         const int row2 = row - n1, p = row2 / n_orb, q = row2 - p * n_orb;
@@ -1212,10 +1227,9 @@ __global__ void __launch_bounds__(kThreads) k_fold(const double *table, const do
             const double g = table[(size_t)n1 * n1 + (size_t)row2 * n2 + col];
             if (g == 0.0) continue;
             const int r = col / n_orb, s = col - r * n_orb;
-            const double g1 = __dmul_rn(inv, g);
             atomicAdd(&ge[fq::eidx(p, r, q, s)], 2.0 * g);
-            if (q == s) one_body(p, r, g1);
-            if (p == r) one_body(q, s, g1);
+            if (q == s) one_body(p, r, g);
+            if (p == r) one_body(q, s, g);
         }
     } else if (blockIdx.x == 0) {  // spin orbital q: O_pq for p <= q
         const int q = row - n1 - n2, Q = q >> 1;
@@ -1276,11 +1290,12 @@ __global__ void __launch_bounds__(kThreads) k_pair_count(const Member *members, 
     }
 }
 
-__global__ void k_scale_out(const double *gh, const double *ge, long long n_h, long long n_e, const double *scale,
+__global__ void k_scale_out(const double *gh, const double *ge, int n_orb, long long n_e, double keys, const double *scale,
                             const RdmState *st, double *out_h, double *out_e) {
     const double f = __ddiv_rn(*scale, st->norm);
+    const int n_h = n_orb * n_orb;
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n_h + n_e; k += (long long)gridDim.x * blockDim.x) {
-        if (k < n_h) out_h[k] = __dmul_rn(gh[k], f);
+        if (k < n_h) out_h[k] = __dmul_rn((int)k / n_orb == (int)k % n_orb ? gh[k] : __ddiv_rn(gh[k], keys), f);
         else out_e[k - n_h] = __dmul_rn(ge[k - n_h], f);
     }
 }
@@ -1370,9 +1385,10 @@ void launch_energy(fciqmc_rdm *r, const double *h, const double *eri, double *e)
     const Dims &d = r->d;
     cudaStream_t s = r->s;
     const RdmState *st = ptr<RdmState>(r, r->L.state);
-    double *partial = ptr<double>(r, r->L.partial), *table = ptr<double>(r, r->L.table);
+    double *partial = ptr<double>(r, r->L.partial), *table = ptr<double>(r, r->L.table), *share = ptr<double>(r, r->L.share);
     const int g = pair_grid(d), gl = large_grid(r);
-    k_pair_table<<<table_grid(d, 0), kThreads, 0, s>>>(h, eri, d.n_orb, d.n1, d.n2, 1.0 / (d.n_elec - 1), table);
+    k_share<<<(d.n_orb * d.n_orb + kThreads - 1) / kThreads, kThreads, 0, s>>>(h, d.n_orb * d.n_orb, (double)(d.n_elec - 1), share);
+    k_pair_table<<<table_grid(d, 0), kThreads, 0, s>>>(share, eri, d.n_orb, d.n1, d.n2, table);
     k_pair_energy<<<g + gl, kPairThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p),
                                               ptr<unsigned>(r, r->L.count_p), d.parts, ptr<Task>(r, r->L.records), r->host.n_tasks, gl,
                                               d.n1, d.n2, table, partial);
@@ -1391,7 +1407,7 @@ void launch_rdm(fciqmc_rdm *r) {
                                                        ptr<unsigned>(r, r->L.count_p), d.parts, ptr<Task>(r, r->L.records),
                                                        r->host.n_tasks, gl, d.n1, d.n2, table);
     k_fold<<<table_grid(d, d.n_so), kThreads, 0, s>>>(table, ptr<double>(r, r->L.occ_pair), d.n_orb, d.n1, d.n2,
-                                                      1.0 / (d.n_elec - 1), gh, ge);
+                                                      gh, ge);
 }
 }  // namespace
 
@@ -1447,8 +1463,8 @@ int fciqmc_rdm_gradient(fciqmc_rdm *r, const double *scale_dev, double *grad_h_d
     }
     const long long nh = (long long)r->d.n_orb * r->d.n_orb;
     const int g = (int)std::min<long long>(kSms * 4, (nh + r->d.n_eri + kThreads - 1) / kThreads);
-    k_scale_out<<<g, kThreads, 0, r->s>>>(ptr<double>(r, r->L.gh), ptr<double>(r, r->L.ge), nh, r->d.n_eri, scale_dev,
-                                          ptr<RdmState>(r, r->L.state), grad_h_dev, grad_eri_dev);
+    k_scale_out<<<g, kThreads, 0, r->s>>>(ptr<double>(r, r->L.gh), ptr<double>(r, r->L.ge), r->d.n_orb, r->d.n_eri, (double)(r->d.n_elec - 1),
+                                          scale_dev, ptr<RdmState>(r, r->L.state), grad_h_dev, grad_eri_dev);
     return cudaGetLastError() == cudaSuccess ? FCIQMC_OK : FCIQMC_ERR_CUDA;
 }
 

@@ -316,3 +316,22 @@ def test_one_key_is_spread_over_the_device():
         return best
 
     assert time_of(52, 2) < 5 * time_of(16, 4)
+
+
+def test_pair_sums_of_equal_terms():
+    """All 4,096 opposite-spin pairs of two electrons in 64 orbitals with equal amplitudes (of the alpha electron before
+    the beta one: the sign changes where the beta orbital is the lower) and every integral 1: E = 4096. The 8.4e6 pairs
+    share one key and their terms are equal, so plain additions err in one direction (48 times 2^-53 in all where a
+    thread's are plain); a pair is followed by at most 8 + 3 + 16 of them, each within 2^-53, and the amplitudes' squares
+    in c^T c and the last operations add four more."""
+    M = 64
+    dets = np.array([bf.to_words((1 << 2 * p) | (1 << 2 * q + 1), 2) for p in range(M) for q in range(M)], dtype=np.uint64)
+    npair = M * (M + 1) // 2
+    from paper_1305_6981_gb300 import EnergyFunctional
+    sign = np.array([1.0 if p <= q else -1.0 for p in range(M) for q in range(M)])
+    for c in (0.1, 0.3, 0.7):
+        f = EnergyFunctional(2, M, dets, c * sign)
+        E = float(f.energy(torch.zeros((M, M), dtype=torch.float64, device="cuda"),
+                           torch.ones(npair * (npair + 1) // 2, dtype=torch.float64, device="cuda")))
+        assert abs(E / 4096 - 1) <= (8 + 3 + 16 + 4) * 2.0 ** -53
+        f.close()
