@@ -163,7 +163,7 @@ RdmLayout layout_of(const Dims &d) {
     L.ge = take(sizeof(double) * d.n_eri);
     L.share = take(sizeof(double) * d.n_orb * d.n_orb);
     L.table = take(sizeof(double) * ((size_t)d.n1 * d.n1 + (size_t)d.n2 * d.n2));
-    L.occ_part = take(sizeof(double) * kSms * ((size_t)d.n_so * (d.n_so + 1) / 2));
+    L.occ_part = take(2 * sizeof(double) * kSms * ((size_t)d.n_so * (d.n_so + 1) / 2));
     L.occ_pair = take(sizeof(double) * ((size_t)d.n_so * (d.n_so + 1) / 2));
     L.partial = take(sizeof(double) * 2 * (kPairGrid + kLargeGrid + kNormGrid));
     L.total = off;
@@ -818,7 +818,7 @@ __device__ __forceinline__ void make_tasks(const Head *heads, Task *tasks, RdmSt
 // compensated summation): the result is the rounded exact sum up to a few ulp whatever the number of
 // additions, so finite differences of E are not swamped by accumulated rounding. A compensated addition costs
 // seven plain ones, so terms are added plainly first, a bounded number at a time (k_pair_energy).
-struct CSum {
+struct alignas(16) CSum {
     double s, c;
 };
 __device__ __forceinline__ void csum_add(CSum &a, double x) {
@@ -861,20 +861,26 @@ __device__ __forceinline__ CSum block_csum(CSum acc, CSum *s) {
 // occupations). One determinant per warp at a time: the lanes hold its occupied list and take its pairs, which are
 // distinct, so each warp adds into a copy of its own in shared memory without atomics (shared FP64 atomics are
 // compare-and-swap loops, and the core pairs, occupied in nearly every determinant, made all lanes retry on
-// one word). Block copies are added up in warp order into occ_part[block].
+// one word). A warp adds kOccPlain determinants plainly; then the block adds its copies, in warp order, to its compensated
+// sums in occ_part[block] (all of a warp's determinants added plainly, the occupation of a core orbital came out 188 times
+// 2^-53 off for 4e5 equal amplitudes in 64 orbitals, and E of 1e6 determinants of 16e/40o 1.7e-13; now 13 times and 5e-15).
+// Bound by the FP64 pipe: construction for 1e6 determinants of 16e/40o and 3e5 of 24e/60o 5.48 and 4.12 ms without the
+// compensated sums, 5.60 and 4.20 with 128 determinants between them, 5.70 and 4.29 with 64.
+constexpr int kOccPlain = 64;
+constexpr int kOccThreads = 256;
 template <int W>
-__global__ void __launch_bounds__(256) k_occ_pairs(const unsigned long long *dets, const double *c, long long n, int n_elec,
-                                                   int n_so, double *occ_part) {
+__global__ void __launch_bounds__(kOccThreads) k_occ_pairs(const unsigned long long *dets, const double *c, long long n, int n_elec,
+                                                           int n_so, int nw, CSum *occ_part) {
     extern __shared__ double s_o[];
     __shared__ unsigned short s_pairs[fq::MAXPAIRS];
     fill_pairs(n_elec, s_pairs);
     const int nent = n_so * (n_so + 1) / 2, npairs = n_elec * (n_elec - 1) / 2;
-    const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int k = threadIdx.x; k < nent * nw; k += blockDim.x) s_o[k] = 0.0;
     __syncthreads();
     double *o = s_o + nent * warp;
     const long long step = (long long)gridDim.x * nw;
-    long long I = (long long)blockIdx.x * nw + warp;
+    long long I = warp < nw ? (long long)blockIdx.x * nw + warp : n;
     // the lane's occupied orbitals (ranks lane and lane + 32; ranks beyond the electrons are not used) and c^2, of the
     // next determinant while the current one's sums are in flight
     auto decode = [&](long long i, int &k0, int &k1, double &c2) {
@@ -888,51 +894,75 @@ __global__ void __launch_bounds__(256) k_occ_pairs(const unsigned long long *det
     int k0 = 0, k1 = 0, nk0 = 0, nk1 = 0;
     double c2 = 0.0, nc2 = 0.0;
     if (I < n) decode(I, k0, k1, c2);
-    for (; I < n; I += step, k0 = nk0, k1 = nk1, c2 = nc2) {
-        if (I + step < n) decode(I + step, nk0, nk1, nc2);
-        // four pairs of a lane at a time: their words are distinct, so the loads need not wait for the stores
-        for (int k0s = 0; k0s < npairs; k0s += 128) {
-            double *e[4], x[4];
+    CSum *sums = occ_part + (size_t)blockIdx.x * nent;
+    for (long long i0 = (long long)blockIdx.x * nw; i0 < n; i0 += step * kOccPlain) {
+        for (int left = kOccPlain; left > 0 && I < n; --left, I += step, k0 = nk0, k1 = nk1, c2 = nc2) {
+            if (I + step < n) decode(I + step, nk0, nk1, nc2);
+            // four pairs of a lane at a time: their words are distinct, so the loads need not wait for the stores
+            for (int k0s = 0; k0s < npairs; k0s += 128) {
+                double *e[4], x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int k = k0s + 32 * u + lane;
+                    const unsigned short pr = k < npairs ? s_pairs[k] : 0;
+                    const int rx = pr & 0xFF, ry = pr >> 8;
+                    int p = __shfl_sync(0xFFFFFFFFu, k0, rx & 31), q = __shfl_sync(0xFFFFFFFFu, k0, ry & 31);
+                    if (n_elec > 32) {
+                        const int p1 = __shfl_sync(0xFFFFFFFFu, k1, rx & 31), q1 = __shfl_sync(0xFFFFFFFFu, k1, ry & 31);
+                        if (rx >= 32) p = p1;
+                        if (ry >= 32) q = q1;
+                    }
+                    e[u] = k < npairs && p <= q && q < n_so ? o + q * (q + 1) / 2 + p : nullptr;
+                    x[u] = e[u] ? *e[u] : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (e[u]) *e[u] = __dadd_rn(x[u], c2);
+            }
+            if (lane < n_elec && k0 < n_so) {
+                double *e = o + k0 * (k0 + 1) / 2 + k0;
+                *e = __dadd_rn(*e, c2);
+            }
+            if (lane + 32 < n_elec && k1 < n_so) {
+                double *e = o + k1 * (k1 + 1) / 2 + k1;
+                *e = __dadd_rn(*e, c2);
+            }
+            __syncwarp();
+        }
+        __syncthreads();
+        const bool first = i0 < step, last = i0 + step * kOccPlain >= n;
+        for (int k0 = threadIdx.x; k0 < nent; k0 += 4 * kOccThreads) {  // four entries in flight
+            CSum a[4];
+            double t[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int k = k0s + 32 * u + lane;
-                const unsigned short pr = k < npairs ? s_pairs[k] : 0;
-                const int rx = pr & 0xFF, ry = pr >> 8;
-                int p = __shfl_sync(0xFFFFFFFFu, k0, rx & 31), q = __shfl_sync(0xFFFFFFFFu, k0, ry & 31);
-                if (n_elec > 32) {
-                    const int p1 = __shfl_sync(0xFFFFFFFFu, k1, rx & 31), q1 = __shfl_sync(0xFFFFFFFFu, k1, ry & 31);
-                    if (rx >= 32) p = p1;
-                    if (ry >= 32) q = q1;
-                }
-                e[u] = k < npairs && p <= q && q < n_so ? o + q * (q + 1) / 2 + p : nullptr;
-                x[u] = e[u] ? *e[u] : 0.0;
+                const int k = k0 + u * kOccThreads;
+                a[u] = !first && k < nent ? sums[k] : CSum{0.0, 0.0};
+                t[u] = k < nent ? s_o[k] : 0.0;
             }
+            for (int w = 1; w < nw; ++w)
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (e[u]) *e[u] = __dadd_rn(x[u], c2);
+                for (int u = 0; u < 4; ++u)
+                    if (k0 + u * kOccThreads < nent) t[u] = __dadd_rn(t[u], s_o[nent * w + k0 + u * kOccThreads]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = k0 + u * kOccThreads;
+                if (k >= nent) continue;
+                if (first) a[u].s = t[u];
+                else csum_add(a[u], t[u]);
+                sums[k] = a[u];
+                if (!last)
+                    for (int w = 0; w < nw; ++w) s_o[nent * w + k] = 0.0;
+            }
         }
-        if (lane < n_elec && k0 < n_so) {
-            double *e = o + k0 * (k0 + 1) / 2 + k0;
-            *e = __dadd_rn(*e, c2);
-        }
-        if (lane + 32 < n_elec && k1 < n_so) {
-            double *e = o + k1 * (k1 + 1) / 2 + k1;
-            *e = __dadd_rn(*e, c2);
-        }
-        __syncwarp();
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < nent; k += blockDim.x) {
-        double t = 0.0;
-        for (int w = 0; w < nw; ++w) t = __dadd_rn(t, s_o[nent * w + k]);
-        occ_part[(size_t)blockIdx.x * nent + k] = t;
+        __syncthreads();
     }
 }
 
 // Sums of the blocks' occupation pairs (compensated): a warp adds 8 entries, four lanes each taking every fourth block in
 // order, merged in a fixed tree (the first n_merge blocks). The next block adds the partial sums of c^2, the others make
 // the tasks of the large groups, which need k_group's heads only and here cost no launch and no time.
-__global__ void __launch_bounds__(kMergeThreads) k_occ_merge(const double *occ_part, int nblocks, int nent, double *occ_pair, int n_merge,
+__global__ void __launch_bounds__(kMergeThreads) k_occ_merge(const CSum *occ_part, int nblocks, int nent, double *occ_pair, int n_merge,
                                                              const double *norm_part, int n_norm, const Head *heads, Task *tasks,
                                                              RdmState *st) {
     if ((int)blockIdx.x > n_merge) {
@@ -953,11 +983,11 @@ __global__ void __launch_bounds__(kMergeThreads) k_occ_merge(const double *occ_p
     CSum a{0.0, 0.0};
     if (k < nent)
         for (int b0 = part; b0 < nblocks; b0 += 16) {  // four reads in flight
-            double x[4];
+            CSum x[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = b0 + 4 * u < nblocks ? occ_part[(size_t)(b0 + 4 * u) * nent + k] : 0.0;
+            for (int u = 0; u < 4; ++u) x[u] = b0 + 4 * u < nblocks ? occ_part[(size_t)(b0 + 4 * u) * nent + k] : CSum{0.0, 0.0};
 #pragma unroll
-            for (int u = 0; u < 4; ++u) csum_add(a, x[u]);
+            for (int u = 0; u < 4; ++u) csum_merge(a, x[u]);
         }
     for (int o = 16; o >= 8; o >>= 1) {
         const CSum b{__shfl_down_sync(0xFFFFFFFFu, a.s, o), __shfl_down_sync(0xFFFFFFFFu, a.c, o)};
@@ -1317,10 +1347,11 @@ T *ptr(const fciqmc_rdm *r, size_t off) {
     return reinterpret_cast<T *>(r->ws + off);
 }
 
-// Warps of a k_occ_pairs block: as many copies of the occupation triangle as fit in 208 KB, at most eight.
+// Warps of a k_occ_pairs block that add determinants: as many copies of the occupation triangle as fit in 208 KB, at most
+// all of them.
 int occ_warps(const Dims &d) {
     const size_t nent = (size_t)d.n_so * (d.n_so + 1) / 2;
-    return (int)std::max<size_t>(1, std::min<size_t>(8, (208u << 10) / (sizeof(double) * nent)));
+    return (int)std::max<size_t>(1, std::min<size_t>(kOccThreads / 32, (208u << 10) / (sizeof(double) * nent)));
 }
 
 template <int W>
@@ -1361,9 +1392,9 @@ int construct(fciqmc_rdm *r) {
     const int nw = occ_warps(d);
     const int go = (int)std::min<long long>(kSms, (d.n + nw - 1) / nw), gn = (int)std::min<long long>(kNormGrid, (d.n + kThreads - 1) / kThreads);
     k_norm<<<gn, kThreads, 0, s>>>(c, d.n, norm_part);
-    k_occ_pairs<W><<<go, 32 * nw, sm_occ, s>>>(dets, c, d.n, d.n_elec, d.n_so, ptr<double>(r, r->L.occ_part));
+    k_occ_pairs<W><<<go, kOccThreads, sm_occ, s>>>(dets, c, d.n, d.n_elec, d.n_so, nw, ptr<CSum>(r, r->L.occ_part));
     const int n_merge = (int)((nent + kMergeThreads / 4 - 1) / (kMergeThreads / 4));
-    k_occ_merge<<<n_merge + 1 + kSms, kMergeThreads, 0, s>>>(ptr<double>(r, r->L.occ_part), go, (int)nent, ptr<double>(r, r->L.occ_pair),
+    k_occ_merge<<<n_merge + 1 + kSms, kMergeThreads, 0, s>>>(ptr<CSum>(r, r->L.occ_part), go, (int)nent, ptr<double>(r, r->L.occ_pair),
                                                              n_merge, norm_part, gn, ptr<Head>(r, r->L.heads),
                                                              ptr<Task>(r, r->L.records), st);
     if (cudaGetLastError() != cudaSuccess) return FCIQMC_ERR_CUDA;

@@ -335,3 +335,28 @@ def test_pair_sums_of_equal_terms():
                            torch.ones(npair * (npair + 1) // 2, dtype=torch.float64, device="cuda")))
         assert abs(E / 4096 - 1) <= (8 + 3 + 16 + 4) * 2.0 ** -53
         f.close()
+
+
+@pytest.mark.parametrize("c", [0.1, 0.3, 1 / 3])
+def test_occupation_sums_of_equal_terms(c):
+    """4e5 determinants of seven electrons in 64 orbitals with equal amplitudes, the first spin orbital always occupied, and
+    h = 1 on its orbital alone: E and the density matrix element are one plus the other spin's share. The c^2 are equal,
+    so plain additions err in one direction (by 188 times 2^-53 where a warp's are plain); a term is followed by at most
+    64 + 3 of them (a warp's determinants, the block's three copies) before it is compensated, and six operations more."""
+    from paper_1305_6981_gb300 import EnergyFunctional
+    M, n = 64, 400_000
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    occ = torch.rand((n, 2 * M - 1), generator=gen, device="cuda").argsort(1)[:, :6] + 1
+    bits = torch.zeros((n, 128), dtype=torch.bool, device="cuda").scatter_(1, occ, True)
+    bits[:, 0] = True
+    dets = torch.unique((bits.view(n, 2, 64).to(torch.int64) << torch.arange(64, device="cuda")).sum(-1), dim=0).contiguous()
+    both = 1 + float((dets[:, 0] >> 1 & 1).double().mean())
+    f = EnergyFunctional(7, M, dets, torch.full((len(dets),), c, dtype=torch.float64, device="cuda"))
+    h = torch.zeros((M, M), dtype=torch.float64, device="cuda")
+    h[0, 0] = 1
+    npair = M * (M + 1) // 2
+    E = float(f.energy(h, torch.zeros(npair * (npair + 1) // 2, dtype=torch.float64, device="cuda")))
+    gh, _ = f.gradient(torch.ones((), dtype=torch.float64, device="cuda"))
+    for x in (E, float(gh[0, 0])):
+        assert abs(x / both - 1) <= (64 + 3 + 6) * 2.0 ** -53
+    f.close()
