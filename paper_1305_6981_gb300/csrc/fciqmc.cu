@@ -8,7 +8,6 @@
 #include <cmath>
 #include <cstddef>
 #include <cstdint>
-#include <cstdlib>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -238,11 +237,7 @@ int configure_kernels(fciqmc_handle *h) {
     h->sweep_grid = at_most(h->sweep_grid, h->z.cap, fq::kTileLeast);
     h->ann_grid = at_most(h->ann_grid, h->z.mt_cap, 256);
     h->diag_grid = at_most(h->diag_grid, h->z.cap, fq::kDiagThreads);
-    // k_heavy: the smallest chunk for every warp at four times the target population (where one is set)
-    const long long target = h->opt.target_walkers;
-    if (target > 0 && target < (1LL << 40))
-        h->heavy_grid = at_most(h->heavy_grid, 4 * std::max<long long>(target, std::llabs((long long)h->opt.initial_population)),
-                                fq::kChunkLeast * (fq::kTile / 32));
+    // (not k_heavy's: its attempts are walkers, which neither the capacity nor the target bounds)
     if (h->grid_request > 0) {
         const int g = std::min(kMaxGrid, h->grid_request);
         h->sweep_grid = std::min(h->sweep_grid, g);

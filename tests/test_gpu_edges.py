@@ -104,3 +104,29 @@ def test_history_ring_in_one_or_two_pieces(steps, want):
     assert [[r[k] for k in ints] for r in short] == [[r[k] for k in ints] for r in full]
     for g in runs:
         g.close()
+
+
+def test_target_does_not_size_the_run():
+    """A run made for a target of one walker (the shift varies from the start) and loaded with a list of 1e6 advances as
+    fast as one made for 1e6 (20 times slower when the grid for heavily populated determinants followed the target)."""
+    from paper_1305_6981_gb300 import Fciqmc
+    s = synth.large_24e60o()
+    dets, pops = synth.walker_snapshot(s, 1_000_000, seed=2)
+
+    def best(target):
+        g = Fciqmc(s, 0.001, 3, target_walkers=target, seed=1, main_capacity=1 << 20, spawn_capacity=1 << 18)
+        g.set_walkers(dets, 8 * pops, iteration=5, shift=0.0, vary=0)
+        g.step(3)
+        times = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            g.step(5)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        assert g.history(1)[0]["heavy_attempts"] > 100_000
+        g.close()
+        return min(times)
+
+    assert best(1) < 2 * best(1_000_000)
