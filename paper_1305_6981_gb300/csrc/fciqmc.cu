@@ -71,8 +71,9 @@ bool sizes_of(int n_elec, int n_orb, const fciqmc_options &o, Sizes &z) {
     z.idx_cap = next_pow2(std::max<long long>((long long)std::ceil((double)z.cap / load), 1 << 12));
     z.mt_cap = next_pow2(std::max<long long>(o.spawn_capacity > 0 ? o.spawn_capacity : z.cap / 2, 1 << 12));
     if (z.mt_cap > (1LL << 32)) return false;
-    // records of determinants with |C| > 256 (a run that needs more stops with FCIQMC_ERR_CAPACITY)
-    z.heavy_cap = std::max<long long>(1 << 14, std::min<long long>(z.cap / 2, 1 << 22));
+    // records of determinants with |C| > 256 (a run that needs more stops with FCIQMC_ERR_CAPACITY); a short list can have
+    // all its determinants there (kHeavyShort)
+    z.heavy_cap = std::max<long long>({1 << 14, std::min<long long>(z.cap / 2, 1 << 22), std::min<long long>(z.cap, 1 << 16)});
     z.hist_cap = std::max<long long>(o.history_capacity > 0 ? o.history_capacity : (1LL << 16), 16);
     // the reference's double excitations: at most npairs x virtuals x virtuals choices
     const long long nv = z.n_so - n_elec;
@@ -1328,6 +1329,7 @@ int fciqmc_group_create(fciqmc_handle *const *parts, int32_t n_partitions, int64
         links[r].hist = P.hist;
         links[r].hist_cap = P.hist_cap;
         links[r].cap = P.cap;
+        links[r].heavy_cap = P.heavy_cap;
         links[r].heavy_warps = P.heavy_warps;
         links[r].sweep_blocks = P.sweep_blocks;
         links[r].frac_bits = P.frac_bits;

@@ -104,7 +104,7 @@ __device__ __forceinline__ int next_tile(long long slots, long long blocks) {
 // compaction and the heavy chunk size for the next iteration (attempts: its expected spawning attempts) and
 // clears the per-iteration counters.
 __device__ __forceinline__ void commit_list(DevState *st, long long nd_out, long long cap, long long attempts,
-                                            long long heavy_warps, long long sweep_blocks) {
+                                            long long heavy_cap, long long heavy_warps, long long sweep_blocks) {
     const long long new_len = (long long)*(volatile unsigned long long *)&st->claim;
     st->list_len = new_len;
     st->pp ^= 1;
@@ -123,8 +123,10 @@ __device__ __forceinline__ void commit_list(DevState *st, long long nd_out, long
     st->heavy_chunk = next_chunk(attempts, heavy_warps);
     st->tile = next_tile(new_len, sweep_blocks);
     // a short list leaves most sweep blocks without a tile, and each tile's light attempts run in one block:
-    // then the heavy path, whose chunks spread over every warp, takes determinants from 32 walkers on
-    st->heavy_thr = (new_len + kTile - 1) / kTile * 4 < sweep_blocks ? (unsigned)kHeavyShort : (unsigned)kHeavy;
+    // then the heavy path, whose chunks spread over every warp, takes determinants from 32 walkers on, where its
+    // buffer has room for the whole list
+    const bool few = (new_len + kTile - 1) / kTile * 4 < sweep_blocks && new_len <= heavy_cap;
+    st->heavy_thr = few ? (unsigned)kHeavyShort : (unsigned)kHeavy;
     for (int k = 0; k < NCNT; ++k) st->cnt[k] = 0;
     for (int k = 0; k < MAXPARTS; ++k) st->ob_n[k] = 0;
 }
@@ -166,7 +168,7 @@ __device__ __forceinline__ void end_iteration(const Params &P) {
     P.hist[st->hist_n % P.hist_cap] = row;
     st->hist_n++;
     shift_update(st, row.nw_out, P.target, P.period, P.c_shift);
-    commit_list(st, row.nd_out, P.cap, row.nw_out >> P.frac_bits, P.heavy_warps, P.sweep_blocks);
+    commit_list(st, row.nd_out, P.cap, row.nw_out >> P.frac_bits, P.heavy_cap, P.heavy_warps, P.sweep_blocks);
 }
 
 // The same as a launch of its own, after k_round.
@@ -407,6 +409,7 @@ struct PartLink {
     const double *partial;       // range sums of the sweep tiles' numerators (kTileSums)
     fciqmc_row *hist;            // the partition's own rows (its list's counters)
     long long hist_cap, cap;
+    long long heavy_cap;         // records its heavy buffer holds
     long long heavy_warps;       // warps of the partition's k_heavy launch
     long long sweep_blocks;      // blocks of the partition's k_sweep launch
     int frac_bits;               // hybrid walkers: populations in units of 2^-frac_bits
@@ -493,7 +496,7 @@ __global__ void k_group_finish(const PartLink *links, int n_parts, GroupDev *g, 
         shift_update(st, tot.nw_out, target, period, c_shift);  // the same state and input in every partition
         const long long nw_part = (long long)st->nw_in + (long long)st->d_nw;
         commit_list(st, (long long)st->nd_in + (long long)st->d_nd, links[r].cap, nw_part >> links[r].frac_bits,
-                    links[r].heavy_warps, links[r].sweep_blocks);
+                    links[r].heavy_cap, links[r].heavy_warps, links[r].sweep_blocks);
     }
 }
 

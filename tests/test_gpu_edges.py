@@ -130,3 +130,24 @@ def test_target_does_not_size_the_run():
         return min(times)
 
     assert best(1) < 2 * best(1_000_000)
+
+
+@pytest.mark.parametrize("walkers,tau", [(40, 0.0005), (300, 0.0001)])
+def test_every_determinant_of_a_short_list_heavily_populated(walkers, tau):
+    """20,000 determinants in a capacity of 32,768, all above the threshold of heavily populated determinants (32 walkers
+    for a list as short as this, from its second iteration on): as the oracle, and no capacity is exceeded."""
+    s = synth.make_system(20, 10, seed=4, n_chol=8)
+    g, q = make_pair(s, tau, 3, seed=6, main_capacity=1 << 15, spawn_capacity=1 << 18)
+    dets, _ = synth.walker_snapshot(s, 200_000, seed=3)
+    dets = dets[:20_000]
+    assert len(dets) == 20_000
+    pops = np.where(np.random.default_rng(1).random(20_000) < 0.5, -walkers, walkers).astype(np.int32)
+    for x in (g, q):
+        x.set_walkers(dets, pops, iteration=3, shift=0.0)
+    rows_q = q.iterate(3)
+    g.step(3)
+    rows_g = g.history(3)
+    compare_rows(rows_g, rows_q)
+    assert rows_g[1]["heavy_attempts"] > 0.9 * rows_g[1]["attempts"]
+    assert same_lists(g.walkers(), q.walkers())
+    g.close()
