@@ -43,7 +43,10 @@ constexpr int kGroupThreads = 512;
 constexpr int kGroupCap = 4608;
 constexpr int kGroupSlots = 8192;
 constexpr int kBigLeaders = 16;       // distinct keys of one hash value that the oversized path tells apart
-constexpr int kTriangle = 48;         // groups from this size on are large: walked as triangles, by warps of all blocks
+// Groups from this size on are large: walked as triangles, by warps of all blocks. The largest that a member's code can
+// tell apart; E and gradient of 1e6 determinants of 16e/40o 1.27 and 1.40 ms with 62, 1.32 and 1.47 with 48, 1.52 and 1.48
+// with 24; 3e5 of 24e/60o 0.51, 0.53 and 0.62 (E).
+constexpr int kTriangle = 63;
 constexpr int kTaskPartners = 128;    // partners of a row beyond which more warps share it
 constexpr int kTaskShares = 16;       // most warps that do
 constexpr int kMergeThreads = 128;
@@ -52,6 +55,7 @@ constexpr int kMergeThreads = 128;
 // class, 13..14 the class: 0 alpha alpha, 1 beta beta, 2 mixed; bits 15..20 the group size, kLarge from kTriangle
 // on), and the position of the group's first member in the partition.
 constexpr unsigned kLarge = 63;
+static_assert(kTriangle <= kLarge, "a small group's size is not kLarge");
 struct alignas(16) Member {
     double v;
     unsigned code;
@@ -1089,8 +1093,8 @@ __device__ __forceinline__ void for_task_rows(const Member *members, const Task 
 
 // 2 c_I c_J H_IJ summed over the pairs of members, without the factor 2. The first `large` blocks take the tasks of the
 // large groups, a warp each, the others the partitions' small groups. A row is an FMA chain of eight partners at a time;
-// per thread these parts are added plainly, at most eight of a large group's row or the three of kPlainRows rows of small
-// ones, and then compensated, the blocks' sums in a fixed tree. So a pair is followed by at most 8 + 3 + kPlainRows plain
+// per thread these parts are added plainly, at most eight of a large group's row or the four of kPlainRows rows of small
+// ones, and then compensated, the blocks' sums in a fixed tree. So a pair is followed by at most 8 + 4 + kPlainRows plain
 // additions whatever the length of the list (with one plain sum per row, thread and partition, 8.4e6 equal pairs of one
 // key came out 48 times 2^-53 off).
 // Bound by the FP64 pipe (one FMA per pair, charged per warp instruction) and the table reads from L2.

@@ -280,10 +280,10 @@ def test_keys_that_share_their_hash(bits, name, short_hash_library, monkeypatch)
     _matches_oracle(*_short_hash_case(name))
 
 
-@pytest.mark.parametrize("n", [48, 64, 65, 128, 129, 161, 2049, 2081])
+@pytest.mark.parametrize("n", [48, 62, 63, 64, 65, 128, 129, 161, 2049, 2081])
 def test_large_groups_in_shares(n):
-    """One key of n determinants: the rows of a large group are dealt to warps 32 at a time, in shares from 128 partners on
-    and at most 16 of them. The counts as well, up to 161."""
+    """One key of n determinants: a group is large from 63 on, and its rows are dealt to warps 32 at a time, in shares from
+    128 partners on and at most 16 of them. The counts as well, up to 161."""
     s = synth.make_system(33, 2, seed=n, n_chol=8, fock_diagonal=False)
     dets = np.array([bf.to_words(d, 2) for d in _some_pairs(33, 2, n, n)], dtype=np.uint64)
     c = np.random.default_rng(n).normal(size=n)
@@ -322,7 +322,7 @@ def test_pair_sums_of_equal_terms():
     """All 4,096 opposite-spin pairs of two electrons in 64 orbitals with equal amplitudes (of the alpha electron before
     the beta one: the sign changes where the beta orbital is the lower) and every integral 1: E = 4096. The 8.4e6 pairs
     share one key and their terms are equal, so plain additions err in one direction (48 times 2^-53 in all where a
-    thread's are plain); a pair is followed by at most 8 + 3 + 16 of them, each within 2^-53, and the amplitudes' squares
+    thread's are plain); a pair is followed by at most 8 + 4 + 16 of them, each within 2^-53, and the amplitudes' squares
     in c^T c and the last operations add four more."""
     M = 64
     dets = np.array([bf.to_words((1 << 2 * p) | (1 << 2 * q + 1), 2) for p in range(M) for q in range(M)], dtype=np.uint64)
@@ -333,7 +333,7 @@ def test_pair_sums_of_equal_terms():
         f = EnergyFunctional(2, M, dets, c * sign)
         E = float(f.energy(torch.zeros((M, M), dtype=torch.float64, device="cuda"),
                            torch.ones(npair * (npair + 1) // 2, dtype=torch.float64, device="cuda")))
-        assert abs(E / 4096 - 1) <= (8 + 3 + 16 + 4) * 2.0 ** -53
+        assert abs(E / 4096 - 1) <= (8 + 4 + 16 + 4) * 2.0 ** -53
         f.close()
 
 
