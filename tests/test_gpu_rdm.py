@@ -360,3 +360,37 @@ def test_occupation_sums_of_equal_terms(c):
     for x in (E, float(gh[0, 0])):
         assert abs(x / both - 1) <= (64 + 3 + 6) * 2.0 ** -53
     f.close()
+
+
+def test_two_scatter_passes_match_oracle():
+    """The same list above the 1,024 partitions that one scatter pass covers, with the library as it is."""
+    _matches_oracle(*_short_hash_case("64e-2100"))
+
+
+def _pair_counts(dets):
+    """Numbers of pairs of determinants that are a single and a double excitation apart."""
+    d = _dev(dets.view(np.int64))
+    n_so = 64 * d.shape[1]
+    occ = (d[:, :, None] >> torch.arange(64, device="cuda") & 1).reshape(len(d), n_so).half()
+    ns = nd = 0
+    for part in occ.split(4000):
+        common = part @ occ.T  # whole numbers up to 64: exact
+        apart = occ[0].sum() - common
+        ns += int((apart == 1).sum())
+        nd += int((apart == 2).sum())
+    return ns // 2, nd // 2
+
+
+@pytest.mark.parametrize("n_orb,n_elec,n", [(60, 24, 40_000), (32, 32, 9_000)])
+def test_connected_pairs_above_one_scatter_pass(n_orb, n_elec, n):
+    """More than 4.2e6 keys, so that the records are scattered in two passes, in two-word and one-word determinants: the
+    pairs of members found through the keys are the connected pairs that the overlaps of the occupations give, each
+    single N - 1 times and each double once."""
+    assert n * n_elec * (n_elec - 1) // 2 > 1024 * 4096
+    s = synth.make_system(n_orb, n_elec, seed=3, n_chol=8, fock_diagonal=False)
+    dets, c = synth.sampled_vector(s, n, seed=8)
+    f = _functional(s, dets, c)
+    f.gradient(torch.ones((), dtype=torch.float64, device="cuda"))
+    info = f.info()
+    assert (info["single_pairs"], info["double_pairs"]) == _pair_counts(dets)
+    f.close()
