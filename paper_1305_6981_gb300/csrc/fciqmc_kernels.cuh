@@ -1118,7 +1118,8 @@ static __device__ __noinline__ float2 single_sums(const float *h_f, const float 
 // delta_spin (ij|ja)] (without the parity sign) for every lane with a pending single, each evaluated by
 // the whole warp: lane x takes electrons x, x + 32. Where many lanes have one, each evaluates its own instead, four
 // electrons at a time: about 32 N instructions for the warp against 80 per single, and without a round trip
-// to L2 for each (8e/8o, three singles in 32 attempts: 85 to 55 us per iteration); not on spin-coupled functions
+// to L2 for each. us per iteration with this rule, by the warp always, and each its own always: 8e/8o (16,384 walkers)
+// 58.8, 87.7 and 53.7; 12e/24o (1e6) 90.5, 96.7 and 99.7; 24e/60o (5e6) 204.5, 206.0 and 209.9. Not on spin-coupled functions
 // (EACH false), whose longer loop loses more by the call than their rare singles gain (9.2e7 walkers of 24e/60o:
 // k_heavy 2.91 ms with it, 2.70 without). Called by all 32 lanes.
 template <int W, bool EACH>
@@ -1631,7 +1632,10 @@ __global__ void __launch_bounds__(kTile, FQ_SWEEP_MIN_BLOCKS) k_sweep(Params P) 
 // few determinants, and build a determinant's tables once when they reach it. Attempts are screened first
 // (attempt_screen); those that can spawn collect in a queue of the warp and are evaluated 32 at a time, so the
 // expensive part runs with full warps. Not for spin-coupled functions (their element is a sum over two
-// determinants, which the bound does not cover) and not for the reference (its table gives p directly).
+// determinants, which the bound does not cover) and not for the reference (its table gives p directly). A warp that has
+// seen more than half of its attempts pass evaluates the rest of them unscreened. k_heavy in us, all screened, none, and
+// by this rule: 24e/60o with 2.3e6 attempts at tau 0.001 51.1, 53.6 and 51.2; at 0.016 57.3, 61.0 and 59.4; at 0.064
+// (4 spawns in 100 attempts) 67.6, 65.5 and 67.2; 8e/8o at 0.01, where fewer than half pass, 20.6, 16.3 and 20.6.
 template <int W, int MODE>
 __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
     DevState *st = P.st;
@@ -1696,7 +1700,7 @@ __global__ void __launch_bounds__(kTile, 4) k_heavy(Params P) {
     unsigned np = 0;            // queued attempts, all of determinant cur
     unsigned row_mask = 31u;
     unsigned seen = 0, kept = 0;  // screened attempts of this warp and those that passed
-    bool direct = (MODE & 2) != 0;  // attempts are evaluated without the screen: where more than half pass it is a loss
+    bool direct = (MODE & 2) != 0;  // attempts are evaluated without the screen
     bool rtab = false, fresh = true;  // fresh: a new batch, whose first record is not known yet
     for (;;) {
         unsigned a = base + lane;
