@@ -109,6 +109,7 @@ int log2i(long long x) {
 constexpr int kSms = 152;                     // blocks of the passes that take one block per SM
 constexpr int kPairGrid = kSms * 32;          // most blocks of the pair passes (several waves: partitions differ in cost)
 constexpr int kPairThreads = 128;
+constexpr int kDiagBlocks = 16;               // blocks of the energy's diagonal
 constexpr int kLargeGrid = kSms * 16;         // most blocks of the pair passes for large groups
 constexpr int kNormGrid = kSms;
 
@@ -169,7 +170,7 @@ RdmLayout layout_of(const Dims &d) {
     L.table = take(sizeof(double) * ((size_t)d.n1 * d.n1 + (size_t)d.n2 * d.n2));
     L.occ_part = take(2 * sizeof(double) * kSms * ((size_t)d.n_so * (d.n_so + 1) / 2));
     L.occ_pair = take(sizeof(double) * ((size_t)d.n_so * (d.n_so + 1) / 2));
-    L.partial = take(sizeof(double) * 2 * (kPairGrid + kLargeGrid + kNormGrid));
+    L.partial = take(sizeof(double) * 2 * (kPairGrid + kLargeGrid + kDiagBlocks + kNormGrid));
     L.total = off;
     return L;
 }
@@ -1020,14 +1021,16 @@ __global__ void __launch_bounds__(kThreads) k_share(const double *h, int n, doub
 }
 
 // T over pair codes: the same-spin block (n1 x n1, rows and columns p < q), then the mixed block (n2 x n2, alpha
-// first); the diagonals stay zero (the diagonal of H comes from the occupation-pair sums).
+// first); zero on the diagonals (the diagonal of H comes from the occupation-pair sums), and only columns from the
+// diagonal on: T is symmetric and the pair passes read and add at (smaller code, larger code). The table grows with the
+// basis and not with the list: E of 5,000 determinants of 8e/64o, 2.1e7 entries, took 228 us with whole rows, 163 so.
 __global__ void __launch_bounds__(kThreads) k_pair_table(const double *share, const double *eri, int n_orb, int n1, int n2,
                                                          double *table) {
     const int row = blockIdx.y;
     if (row < n1) {
         int p, q;
         triangle_of(row, p, q);
-        for (int col = blockIdx.x * blockDim.x + threadIdx.x; col < n1; col += gridDim.x * blockDim.x) {
+        for (int col = row + blockIdx.x * blockDim.x + threadIdx.x; col < n1; col += gridDim.x * blockDim.x) {
             int r, s;
             triangle_of(col, r, s);
             double v = 0.0;
@@ -1042,7 +1045,7 @@ __global__ void __launch_bounds__(kThreads) k_pair_table(const double *share, co
         }
     } else {
         const int row2 = row - n1, p = row2 / n_orb, q = row2 - p * n_orb;
-        for (int col = blockIdx.x * blockDim.x + threadIdx.x; col < n2; col += gridDim.x * blockDim.x) {
+        for (int col = row2 + blockIdx.x * blockDim.x + threadIdx.x; col < n2; col += gridDim.x * blockDim.x) {
             const int r = col / n_orb, s = col - r * n_orb;
             double v = 0.0;
             if (col != row2) {
@@ -1076,6 +1079,10 @@ __device__ __forceinline__ RowRange row_range(unsigned packed, int local) {
     return RowRange{half + even, local + 1 < m ? local + 1 : 0, m};
 }
 
+__device__ __forceinline__ double pair_entry(const double *t, int stride, unsigned a, unsigned b) {
+    return __ldg(t + (size_t)min(a, b) * stride + max(a, b));
+}
+
 // The tasks of warp g of `warps`, a lane per row: f(its member, the group, k0, k1) for the task's blocks of 64 members
 // before it.
 template <typename F>
@@ -1091,8 +1098,29 @@ __device__ __forceinline__ void for_task_rows(const Member *members, const Task 
     }
 }
 
+// Thread t of n: half of its share of the diagonal, sum_p O_pp h_pp + sum_{p<q} O_pq ((pp|qq) - delta_spin (pq|qp)).
+__device__ __forceinline__ CSum diagonal_energy(const double *occ_pair, const double *h, const double *eri, int n_orb, int t, int n) {
+    CSum acc{0.0, 0.0};
+    for (int k = t; k < n_orb * (2 * n_orb + 1); k += n) {
+        int q = (int)((sqrtf(8.0f * (float)k + 1.0f) - 1.0f) * 0.5f);
+        while (q * (q + 1) / 2 > k) --q;
+        while ((q + 1) * (q + 2) / 2 <= k) ++q;
+        const int p = k - q * (q + 1) / 2, P = p >> 1, Q = q >> 1;
+        double x;
+        if (p == q) {
+            x = __ldg(h + P * n_orb + P);
+        } else {
+            x = __ldg(eri + fq::eidx(P, P, Q, Q));
+            if ((p & 1) == (q & 1)) x = __dsub_rn(x, __ldg(eri + fq::eidx(P, Q, Q, P)));
+        }
+        csum_add(acc, 0.5 * __dmul_rn(occ_pair[k], x));
+    }
+    return acc;
+}
+
 // 2 c_I c_J H_IJ summed over the pairs of members, without the factor 2. The first `large` blocks take the tasks of the
-// large groups, a warp each, the others the partitions' small groups. A row is an FMA chain of eight partners at a time;
+// large groups, a warp each, the last kDiagBlocks half of the diagonal (in the one block that merges the sums it took 8 us in 40
+// orbitals and 24 in 64), those between the partitions' small groups. A row is an FMA chain of eight partners at a time;
 // per thread these parts are added plainly, at most eight of a large group's row or the four of kPlainRows rows of small
 // ones, and then compensated, the blocks' sums in a fixed tree. So a pair is followed by at most 8 + 4 + kPlainRows plain
 // additions whatever the length of the list (with one plain sum per row, thread and partition, 8.4e6 equal pairs of one
@@ -1101,16 +1129,18 @@ __device__ __forceinline__ void for_task_rows(const Member *members, const Task 
 constexpr int kPlainRows = 16;
 __global__ void __launch_bounds__(kPairThreads) k_pair_energy(const Member *members, const unsigned *base_p, const unsigned *count_p,
                                                           int parts, const Task *tasks, unsigned long long n_tasks, int large,
-                                                          int n1, int n2, const double *table, double *partial) {
+                                                          int n1, int n2, const double *table, const double *occ_pair,
+                                                          const double *h, const double *eri, int n_orb, double *partial) {
     __shared__ CSum s_red[kPairThreads / 32];
     CSum acc{0.0, 0.0};
     const double *mixed = table + (size_t)n1 * n1;
+    const int small = (int)gridDim.x - large - kDiagBlocks;
     if ((int)blockIdx.x < large) {
         constexpr unsigned kWarps = kPairThreads / 32;
         for_task_rows(members, tasks, n_tasks, blockIdx.x * kWarps + (threadIdx.x >> 5), (unsigned)large * kWarps,
                       [&](const Member &u, const Member *grp, unsigned k0, unsigned k1) {
-            const unsigned cls = (u.code >> 13) & 3u;
-            const double *col = (cls == 2u ? mixed : table) + (u.code & 0x1FFFu);
+            const unsigned cls = (u.code >> 13) & 3u, cu = u.code & 0x1FFFu;
+            const double *t = cls == 2u ? mixed : table;
             const int stride = cls == 2u ? n2 : n1;
             double row = 0.0;
             for (; k0 < k1; k0 += 8) {
@@ -1119,43 +1149,46 @@ __global__ void __launch_bounds__(kPairThreads) k_pair_energy(const Member *memb
 #pragma unroll 4
                 for (unsigned k = k0; k < end; ++k) {
                     const Member w = grp[k];
-                    if (((w.code >> 13) & 3u) == cls) part = __fma_rn(__ldg(col + (size_t)(w.code & 0x1FFFu) * stride), w.v, part);
+                    if (((w.code >> 13) & 3u) == cls) part = __fma_rn(pair_entry(t, stride, cu, w.code & 0x1FFFu), w.v, part);
                 }
                 row = __dadd_rn(row, part);
             }
             csum_add(acc, __dmul_rn(u.v, row));
         });
-    }
-    for (int p = (int)blockIdx.x - large; p >= 0 && p < parts; p += (int)gridDim.x - large) {
-        const Member *mem = members + base_p[p];
-        const int cnt = (int)count_p[p];
-        if ((int)threadIdx.x >= cnt) continue;
-        for (int j0 = threadIdx.x; j0 < cnt; j0 += kPlainRows * kPairThreads) {
-            const int j1 = min(j0 + kPlainRows * kPairThreads, cnt);
-            double sum = 0.0;
-            for (int j = j0; j < j1; j += kPairThreads) {
-                const Member u = mem[j];
-                const Member *grp = mem + u.first;
-                const RowRange r = row_range(u.code, j - (int)u.first);
-                const unsigned cls = (u.code >> 13) & 3u, cu = u.code & 0x1FFFu;
-                const double *col = (cls == 2u ? mixed : table) + cu;
-                const int stride = cls == 2u ? n2 : n1;
-                double row = 0.0;
-                int at = r.at;
-                for (int k0 = 0; k0 < r.n; k0 += 8) {
-                    double part = 0.0;
-                    const int k1 = min(k0 + 8, r.n);
+    } else if ((int)blockIdx.x >= large + small) {
+        acc = diagonal_energy(occ_pair, h, eri, n_orb, ((int)blockIdx.x - large - small) * kPairThreads + threadIdx.x, kDiagBlocks * kPairThreads);
+    } else {
+        for (int p = (int)blockIdx.x - large; p < parts; p += small) {
+            const Member *mem = members + base_p[p];
+            const int cnt = (int)count_p[p];
+            if ((int)threadIdx.x >= cnt) continue;
+            for (int j0 = threadIdx.x; j0 < cnt; j0 += kPlainRows * kPairThreads) {
+                const int j1 = min(j0 + kPlainRows * kPairThreads, cnt);
+                double sum = 0.0;
+                for (int j = j0; j < j1; j += kPairThreads) {
+                    const Member u = mem[j];
+                    const Member *grp = mem + u.first;
+                    const RowRange r = row_range(u.code, j - (int)u.first);
+                    const unsigned cls = (u.code >> 13) & 3u, cu = u.code & 0x1FFFu;
+                    const double *t = cls == 2u ? mixed : table;
+                    const int stride = cls == 2u ? n2 : n1;
+                    double row = 0.0;
+                    int at = r.at;
+                    for (int k0 = 0; k0 < r.n; k0 += 8) {
+                        double part = 0.0;
+                        const int k1 = min(k0 + 8, r.n);
 #pragma unroll 4
-                    for (int k = k0; k < k1; ++k) {
-                        const Member w = grp[at];
-                        at = at + 1 == r.wrap ? 0 : at + 1;
-                        if (((w.code >> 13) & 3u) == cls) part = __fma_rn(__ldg(col + (size_t)(w.code & 0x1FFFu) * stride), w.v, part);
+                        for (int k = k0; k < k1; ++k) {
+                            const Member w = grp[at];
+                            at = at + 1 == r.wrap ? 0 : at + 1;
+                            if (((w.code >> 13) & 3u) == cls) part = __fma_rn(pair_entry(t, stride, cu, w.code & 0x1FFFu), w.v, part);
+                        }
+                        row = __dadd_rn(row, part);
                     }
-                    row = __dadd_rn(row, part);
+                    sum = __fma_rn(u.v, row, sum);
                 }
-                sum = __fma_rn(u.v, row, sum);
+                csum_add(acc, sum);
             }
-            csum_add(acc, sum);
         }
     }
     acc = block_csum(acc, s_red);
@@ -1165,30 +1198,11 @@ __global__ void __launch_bounds__(kPairThreads) k_pair_energy(const Member *memb
     }
 }
 
-// One block: the pair sums (twice: both orders of a pair), then the diagonal from the occupation pairs,
-// sum_p O_pp h_pp + sum_{p<q} O_pq ((pp|qq) - delta_spin (pq|qp)), all compensated in a fixed order; over c^T c.
-__global__ void __launch_bounds__(1024) k_energy_finish(const double *pp, int npp, const double *occ_pair, const double *h,
-                                                        const double *eri, int n_orb, const RdmState *st, double *e) {
+// One block: the blocks' sums (pairs twice: both orders), merged in a fixed order; over c^T c.
+__global__ void __launch_bounds__(1024) k_energy_finish(const double *partial, int n, const RdmState *st, double *e) {
     __shared__ CSum s_red[32];
     CSum tot{0.0, 0.0};
-    for (int b = threadIdx.x; b < npp; b += blockDim.x) csum_merge(tot, CSum{2.0 * pp[2 * b], 2.0 * pp[2 * b + 1]});
-    const int nent = n_orb * (2 * n_orb + 1);
-    for (int k = threadIdx.x; k < nent; k += blockDim.x) {
-        int q = (int)((sqrtf(8.0f * (float)k + 1.0f) - 1.0f) * 0.5f);
-        while (q * (q + 1) / 2 > k) --q;
-        while ((q + 1) * (q + 2) / 2 <= k) ++q;
-        const int p = k - q * (q + 1) / 2;
-        const double o = occ_pair[k];
-        const int P = p >> 1, Q = q >> 1;
-        double x;
-        if (p == q) {
-            x = __ldg(h + P * n_orb + P);
-        } else {
-            x = __ldg(eri + fq::eidx(P, P, Q, Q));
-            if ((p & 1) == (q & 1)) x = __dsub_rn(x, __ldg(eri + fq::eidx(P, Q, Q, P)));
-        }
-        csum_add(tot, __dmul_rn(o, x));
-    }
+    for (int b = threadIdx.x; b < n; b += blockDim.x) csum_merge(tot, CSum{2.0 * partial[2 * b], 2.0 * partial[2 * b + 1]});
     tot = block_csum(tot, s_red);
     if (threadIdx.x == 0) *e = __ddiv_rn(__dadd_rn(tot.s, tot.c), st->norm);
 }
@@ -1392,7 +1406,7 @@ int construct(fciqmc_rdm *r) {
     }
     k_group<W><<<d.parts, kGroupThreads, sm_group, s>>>(dets, c, d.n_elec, d.n_orb, d.tbits, records, base, ptr<Member>(r, r->L.members),
                                                         ptr<unsigned>(r, r->L.count_p), ptr<Head>(r, r->L.heads), st);
-    double *norm_part = ptr<double>(r, r->L.partial) + 2 * (kPairGrid + kLargeGrid);
+    double *norm_part = ptr<double>(r, r->L.partial) + 2 * (kPairGrid + kLargeGrid + kDiagBlocks);
     const int nw = occ_warps(d);
     const int go = (int)std::min<long long>(kSms, (d.n + nw - 1) / nw), gn = (int)std::min<long long>(kNormGrid, (d.n + kThreads - 1) / kThreads);
     k_norm<<<gn, kThreads, 0, s>>>(c, d.n, norm_part);
@@ -1424,10 +1438,11 @@ void launch_energy(fciqmc_rdm *r, const double *h, const double *eri, double *e)
     const int g = pair_grid(d), gl = large_grid(r);
     k_share<<<(d.n_orb * d.n_orb + kThreads - 1) / kThreads, kThreads, 0, s>>>(h, d.n_orb * d.n_orb, (double)(d.n_elec - 1), share);
     k_pair_table<<<table_grid(d, 0), kThreads, 0, s>>>(share, eri, d.n_orb, d.n1, d.n2, table);
-    k_pair_energy<<<g + gl, kPairThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p),
-                                              ptr<unsigned>(r, r->L.count_p), d.parts, ptr<Task>(r, r->L.records), r->host.n_tasks, gl,
-                                              d.n1, d.n2, table, partial);
-    k_energy_finish<<<1, 1024, 0, s>>>(partial, g + gl, ptr<double>(r, r->L.occ_pair), h, eri, d.n_orb, st, e);
+    k_pair_energy<<<g + gl + kDiagBlocks, kPairThreads, 0, s>>>(ptr<Member>(r, r->L.members), ptr<unsigned>(r, r->L.base_p),
+                                                            ptr<unsigned>(r, r->L.count_p), d.parts, ptr<Task>(r, r->L.records),
+                                                            r->host.n_tasks, gl, d.n1, d.n2, table, ptr<double>(r, r->L.occ_pair),
+                                                            h, eri, d.n_orb, partial);
+    k_energy_finish<<<1, 1024, 0, s>>>(partial, g + gl + kDiagBlocks, st, e);
 }
 
 void launch_rdm(fciqmc_rdm *r) {
