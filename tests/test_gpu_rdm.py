@@ -394,3 +394,25 @@ def test_connected_pairs_above_one_scatter_pass(n_orb, n_elec, n):
     info = f.info()
     assert (info["single_pairs"], info["double_pairs"]) == _pair_counts(dets)
     f.close()
+
+
+def test_counts_of_one_key_are_spread_over_the_device():
+    """info() of the 8,128 determinants of two electrons in 64 orbitals (one key, 3.3e7 pairs): singles and doubles as the
+    space gives them, and in a few milliseconds (27 when the key belonged to one block)."""
+    import time
+    from itertools import combinations
+    M = 64
+    dets = np.array([bf.to_words(1 << a | 1 << b, 2) for a, b in combinations(range(2 * M), 2)], dtype=np.uint64)
+    s = synth.make_system(M, 2, seed=1, n_chol=4, fock_diagonal=False)
+    f = _functional(s, dets, np.ones(len(dets)))
+    f.gradient(torch.ones((), dtype=torch.float64, device="cuda"))
+    times = []
+    for _ in range(4):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        info = f.info()
+        times.append(time.perf_counter() - t)
+    n = len(dets)
+    assert info["single_pairs"] == n * 2 * (2 * M - 2) // 2 and info["single_pairs"] + info["double_pairs"] == n * (n - 1) // 2
+    assert min(times) < 5e-3
+    f.close()
